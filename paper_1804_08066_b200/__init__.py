@@ -21,6 +21,7 @@ import os
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libmqgrad.so")
+_NOT_BUILT = "%s is not built (%s); run `python paper_1804_08066_b200/build.py`. There is no fallback path."
 
 MQG_OK = 0
 MQG_ERR_INVALID = -1
@@ -41,9 +42,7 @@ class MqgError(RuntimeError):
 
 def _load() -> C.CDLL:
     if not os.path.exists(LIB_PATH):
-        raise ImportError(
-            "libmqgrad.so is not built (%s); run `python paper_1804_08066_b200/build.py`. "
-            "There is no fallback path." % LIB_PATH)
+        raise ImportError(_NOT_BUILT % ("libmqgrad.so", LIB_PATH))
     lib = C.CDLL(LIB_PATH)
     u64, u32, i32, vp, f32 = C.c_uint64, C.c_uint32, C.c_int, C.c_void_p, C.c_float
     sigs = {
@@ -103,28 +102,40 @@ def _check(status: int) -> None:
         raise MqgError(status, _lib.mqg_last_error().decode())
 
 
-def _dev_ptr(t, what: str) -> int:
-    import torch
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
-        raise TypeError("%s must be a CUDA tensor (libmqgrad has no CPU path)" % what)
-    if not t.is_contiguous():
-        raise ValueError("%s must be contiguous" % what)
-    return t.data_ptr()
-
-
-def _stream() -> int:
-    import torch
-    return torch.cuda.current_stream().cuda_stream
-
-
-def _ptr_table(tensors, what: str):
-    return (C.c_void_p * len(tensors))(*[_dev_ptr(t, "%s[%d]" % (what, i))
-                                         for i, t in enumerate(tensors)])
-
-
 def _u64_table(values):
     vals = [int(v) for v in values]
     return (C.c_uint64 * len(vals))(*vals)
+
+
+# The calls that enqueue work are native functions (csrc/mqg_binding.cpp, built as _binding.so): the device is
+# done with a small gradient in less time than Python and ctypes need to marshal a call's arguments.
+_NATIVE = frozenset((
+    "mqg_quantize", "mqg_quantize_workers", "mqg_dequant_accumulate", "mqg_apply", "mqg_server_step",
+    "mqg_server_requantize", "mqg_quantize_segments", "mqg_quantize_segments_workers", "mqg_server_step_segments",
+    "mqg_quantize_minmax", "mqg_quantize_workers_minmax", "mqg_dequant_accumulate_minmax", "mqg_server_step_minmax",
+    "mqg_quantize_l2", "mqg_quantize_workers_l2", "mqg_quantize_segments_l2", "mqg_quantize_segments_l2_static",
+    "mqg_quantize_1bit_ef"))
+
+
+def __getattr__(name):
+    """Loads the native functions when the first of them is asked for, not at import (as _LazyLibrary)."""
+    if name not in _NATIVE:
+        raise AttributeError("module %r has no attribute %r" % (__name__, name))
+    for path in (LIB_PATH, os.path.join(_HERE, "_binding.so")):
+        if not os.path.exists(path):
+            raise ImportError(_NOT_BUILT % (os.path.basename(path), path))
+    import importlib
+
+    import torch  # noqa: F401  (its libraries have to be loaded before the native module's)
+    native = importlib.import_module(__name__ + "._binding")
+    native._set_error_class(MqgError)
+    for fn in _NATIVE:
+        globals()[fn] = getattr(native, fn)
+    return globals()[name]
+
+
+def __dir__():
+    return sorted({*globals(), *_NATIVE})
 
 
 def mqg_code_words(n: int, bits: int) -> int:
@@ -168,187 +179,11 @@ def mqg_test_wait_override(poll_limit: int = 0, arm_only: bool = False) -> None:
     _check(_lib.mqg_test_wait_override(poll_limit, 1 if arm_only else 0))
 
 
-def _grad_dtype(grad) -> int:
-    import torch
-    if grad.dtype == torch.float32:
-        return MQG_F32
-    if grad.dtype == torch.bfloat16:
-        return MQG_BF16
-    raise TypeError("grad must be float32 or bfloat16, got %s" % grad.dtype)
-
-
-def mqg_quantize(grad, n: int, bits: int, bucket: int, seed: int, codes, scales,
-                 worker: int = 0, step: int = 0, elem_offset: int = 0) -> None:
-    """Quantize(g, K): writes `codes` (uint32/int32 words) and `scales` (float32)."""
-    _check(_lib.mqg_quantize(_dev_ptr(grad, "grad") if n else None, n, bits, bucket,
-                             seed & 0xFFFFFFFFFFFFFFFF,
-                             _dev_ptr(codes, "codes") if n else None,
-                             _dev_ptr(scales, "scales") if n else None,
-                             _grad_dtype(grad), worker, step, elem_offset, _stream()))
-
-
-def mqg_quantize_workers(grads, W: int, n: int, bits: int, bucket: int, seed: int, codes, scales,
-                         first_worker: int = 0, step: int = 0, elem_offset: int = 0) -> None:
-    """Quantize(g_p, K) for W workers' gradients (lists of W tensors) in one launch."""
-    if len(grads) != W or len(codes) != W or len(scales) != W:
-        raise ValueError("grads, codes and scales must each hold W tensors")
-    dtypes = {_grad_dtype(g) for g in grads}
-    if len(dtypes) != 1:
-        raise TypeError("all gradients must have the same dtype")
-    _check(_lib.mqg_quantize_workers(_ptr_table(grads, "grads"), W, n, bits, bucket,
-                                     seed & 0xFFFFFFFFFFFFFFFF, _ptr_table(codes, "codes"),
-                                     _ptr_table(scales, "scales"), dtypes.pop(), first_worker, step,
-                                     elem_offset, _stream()))
-
-
-def mqg_quantize_workers_l2(grads, W: int, n: int, bits: int, bucket: int, seed: int, codes, scales,
-                            first_worker: int = 0, step: int = 0, elem_offset: int = 0) -> None:
-    """The L2-norm scale variant for W workers' gradients (lists of W tensors) in one launch."""
-    if len(grads) != W or len(codes) != W or len(scales) != W:
-        raise ValueError("grads, codes and scales must each hold W tensors")
-    dtypes = {_grad_dtype(g) for g in grads}
-    if len(dtypes) != 1:
-        raise TypeError("all gradients must have the same dtype")
-    _check(_lib.mqg_quantize_workers_l2(_ptr_table(grads, "grads"), W, n, bits, bucket,
-                                        seed & 0xFFFFFFFFFFFFFFFF, _ptr_table(codes, "codes"),
-                                        _ptr_table(scales, "scales"), dtypes.pop(), first_worker, step,
-                                        elem_offset, _stream()))
-
-
-def mqg_dequant_accumulate(codes, scales, W: int, bits: int, n: int, acc, bucket: int,
-                           add_into_acc: bool = False) -> None:
-    _check(_lib.mqg_dequant_accumulate(_ptr_table(codes, "codes"), _ptr_table(scales, "scales"),
-                                       W, bits, n, _dev_ptr(acc, "acc") if n else None, bucket,
-                                       1 if add_into_acc else 0, _stream()))
-
-
-def mqg_apply(params, acc, lr: float, n: int) -> None:
-    _check(_lib.mqg_apply(_dev_ptr(params, "params") if n else None,
-                          _dev_ptr(acc, "acc") if n else None, lr, n, _stream()))
-
-
-def mqg_server_step(codes, scales, W: int, bits: int, n: int, bucket: int, params, lr: float,
-                    acc_out=None) -> None:
-    _check(_lib.mqg_server_step(_ptr_table(codes, "codes"), _ptr_table(scales, "scales"), W, bits,
-                                n, bucket, _dev_ptr(params, "params") if n else None, lr,
-                                _dev_ptr(acc_out, "acc_out") if acc_out is not None else None,
-                                _stream()))
-
-
-def mqg_quantize_workers_minmax(grads, W: int, n: int, bits: int, bucket: int, codes, ranges) -> None:
-    """The (min, max) variant for W workers' gradients (lists of W tensors) in one launch."""
-    if len(grads) != W or len(codes) != W or len(ranges) != W:
-        raise ValueError("grads, codes and ranges must each hold W tensors")
-    dtypes = {_grad_dtype(g) for g in grads}
-    if len(dtypes) != 1:
-        raise TypeError("all gradients must have the same dtype")
-    _check(_lib.mqg_quantize_workers_minmax(_ptr_table(grads, "grads"), W, n, bits, bucket,
-                                            _ptr_table(codes, "codes"), _ptr_table(ranges, "ranges"),
-                                            dtypes.pop(), _stream()))
-
-
-def mqg_quantize_minmax(grad, n: int, bits: int, bucket: int, codes, ranges) -> None:
-    """(min, max) nearest-rounding variant: writes `codes` and `ranges` (lo, hi per bucket)."""
-    _check(_lib.mqg_quantize_minmax(_dev_ptr(grad, "grad") if n else None, n, bits, bucket,
-                                    _dev_ptr(codes, "codes") if n else None,
-                                    _dev_ptr(ranges, "ranges") if n else None, _grad_dtype(grad), _stream()))
-
-
-def mqg_dequant_accumulate_minmax(codes, ranges, W: int, bits: int, n: int, acc, bucket: int,
-                                  add_into_acc: bool = False) -> None:
-    _check(_lib.mqg_dequant_accumulate_minmax(_ptr_table(codes, "codes"), _ptr_table(ranges, "ranges"),
-                                              W, bits, n, _dev_ptr(acc, "acc") if n else None, bucket,
-                                              1 if add_into_acc else 0, _stream()))
-
-
-def mqg_server_step_minmax(codes, ranges, W: int, bits: int, n: int, bucket: int, params, lr: float,
-                           acc_out=None) -> None:
-    _check(_lib.mqg_server_step_minmax(_ptr_table(codes, "codes"), _ptr_table(ranges, "ranges"), W, bits,
-                                       n, bucket, _dev_ptr(params, "params") if n else None, lr,
-                                       _dev_ptr(acc_out, "acc_out") if acc_out is not None else None,
-                                       _stream()))
-
-
-def mqg_server_requantize(codes, scales, W: int, bits: int, n: int, bucket: int, mean_scale: float,
-                          seed: int, codes_out, scales_out, worker: int = 0, step: int = 0) -> None:
-    """Downlink: de-quantize + sum + scale to the mean + quantize again, in one pass."""
-    _check(_lib.mqg_server_requantize(_ptr_table(codes, "codes"), _ptr_table(scales, "scales"), W, bits,
-                                      n, bucket, mean_scale, seed & 0xFFFFFFFFFFFFFFFF,
-                                      _dev_ptr(codes_out, "codes_out") if n else None,
-                                      _dev_ptr(scales_out, "scales_out") if n else None,
-                                      worker, step, _stream()))
-
-
-def mqg_quantize_segments(grad, seg_off, code_off, bits: int, seed: int, codes, scales,
-                          worker: int = 0, step: int = 0, elem_offset: int = 0) -> None:
-    nseg = len(seg_off) - 1
-    _check(_lib.mqg_quantize_segments(_dev_ptr(grad, "grad"), nseg, _u64_table(seg_off),
-                                      _u64_table(code_off), bits, seed & 0xFFFFFFFFFFFFFFFF,
-                                      _dev_ptr(codes, "codes"), _dev_ptr(scales, "scales"),
-                                      _grad_dtype(grad), worker, step, elem_offset, _stream()))
-
-
-def mqg_quantize_segments_workers(grads, W: int, seg_off, code_off, bits: int, seed: int, codes, scales,
-                                  first_worker: int = 0, step: int = 0, elem_offset: int = 0) -> None:
-    nseg = len(seg_off) - 1
-    _check(_lib.mqg_quantize_segments_workers(_ptr_table(grads, "grads"), W, nseg, _u64_table(seg_off),
-                                              _u64_table(code_off), bits, seed & 0xFFFFFFFFFFFFFFFF,
-                                              _ptr_table(codes, "codes"), _ptr_table(scales, "scales"),
-                                              _grad_dtype(grads[0]), first_worker, step, elem_offset, _stream()))
-
-
-def mqg_server_step_segments(codes, scales, W: int, bits: int, seg_off, code_off, params,
-                             lr: float, acc_out=None) -> None:
-    nseg = len(seg_off) - 1
-    _check(_lib.mqg_server_step_segments(_ptr_table(codes, "codes"), _ptr_table(scales, "scales"),
-                                         W, bits, nseg, _u64_table(seg_off), _u64_table(code_off),
-                                         _dev_ptr(params, "params"), lr,
-                                         _dev_ptr(acc_out, "acc_out") if acc_out is not None else None,
-                                         _stream()))
-
-
-def mqg_quantize_1bit_ef(grad, residual, n: int, bucket: int, codes, ranges) -> None:
-    """`residual` (float32, n elements) is read and updated in place."""
-    _check(_lib.mqg_quantize_1bit_ef(_dev_ptr(grad, "grad"), _dev_ptr(residual, "residual"), n, bucket,
-                                     _dev_ptr(codes, "codes"), _dev_ptr(ranges, "ranges"),
-                                     _grad_dtype(grad), _stream()))
-
-
-def mqg_quantize_l2(grad, n: int, bits: int, bucket: int, seed: int, codes, scales,
-                    worker: int = 0, step: int = 0, elem_offset: int = 0) -> None:
-    _check(_lib.mqg_quantize_l2(_dev_ptr(grad, "grad"), n, bits, bucket, seed & 0xFFFFFFFFFFFFFFFF,
-                                _dev_ptr(codes, "codes"), _dev_ptr(scales, "scales"),
-                                _grad_dtype(grad), worker, step, elem_offset, _stream()))
-
-
 def mqg_l2_workspace_floats(seg_off) -> int:
     return int(_lib.mqg_l2_workspace_floats(len(seg_off) - 1, _u64_table(seg_off)))
 
 
-def mqg_quantize_segments_l2(grad, seg_off, code_off, bits: int, seed: int, codes, scales, workspace,
-                             worker: int = 0, step: int = 0, elem_offset: int = 0) -> None:
-    """`workspace`: float32 CUDA tensor of at least mqg_l2_workspace_floats(seg_off) elements."""
-    nseg = len(seg_off) - 1
-    _check(_lib.mqg_quantize_segments_l2(_dev_ptr(grad, "grad"), nseg, _u64_table(seg_off),
-                                         _u64_table(code_off), bits, seed & 0xFFFFFFFFFFFFFFFF,
-                                         _dev_ptr(codes, "codes"), _dev_ptr(scales, "scales"),
-                                         _grad_dtype(grad), worker, step, elem_offset,
-                                         _dev_ptr(workspace, "workspace"), workspace.numel(), _stream()))
-
-
 MQG_L2_STATIC_WORKSPACE_FLOATS = 65536
-
-
-def mqg_quantize_segments_l2_static(grad, seg_off, code_off, bits: int, seed: int, codes, scales,
-                                    worker: int = 0, step: int = 0, elem_offset: int = 0) -> None:
-    """mqg_quantize_segments_l2 for callers that cannot supply a workspace: the partial sums use an
-    array inside the library (at most MQG_L2_STATIC_WORKSPACE_FLOATS of them); calls that may
-    overlap on the device must be ordered by the caller."""
-    nseg = len(seg_off) - 1
-    _check(_lib.mqg_quantize_segments_l2_static(_dev_ptr(grad, "grad"), nseg, _u64_table(seg_off),
-                                                _u64_table(code_off), bits, seed & 0xFFFFFFFFFFFFFFFF,
-                                                _dev_ptr(codes, "codes"), _dev_ptr(scales, "scales"),
-                                                _grad_dtype(grad), worker, step, elem_offset, _stream()))
 
 
 def raw_library() -> C.CDLL:
