@@ -1,9 +1,8 @@
 // General (any shape) kernels of the (min, max) nearest-rounding codec variant: the scheme the
 // footnote of Section 3.2 refers to, a bucket's range [min, max] mapped linearly onto the 2^K
-// codes.  The fast paths are the TMA kernels in mqg_quantize.cu (RANGE tile) and
-// mqg_server_tma.cu; the kernels here take every other shape: buckets above 4096 elements, tiny
-// inputs, small buckets on the server side, an extra accumulator output.  A thread owns a row of
-// 32 elements throughout; buckets are whole rows (multiples of 32 elements, or one bucket).
+// codes.  The fast path is the TMA kernel in mqg_quantize.cu (RANGE tile); the kernels here take
+// every other shape: buckets above 4096 elements, tiny inputs.  A thread owns a row of 32 elements
+// throughout; buckets are whole rows (multiples of 32 elements, or one bucket).
 #include "mqg_common.cuh"
 #include "mqg_internal.h"
 
@@ -164,93 +163,6 @@ cudaError_t launch_quantize_range_general(const void* grad, uint64_t n, int bits
         case 6: launch_encode<6>(a, dtype, grid, stream); break;
         case 7: launch_encode<7>(a, dtype, grid, stream); break;
         case 8: launch_encode<8>(a, dtype, grid, stream); break;
-        default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
-// ---- server side, any shape ---------------------------------------------------------------
-struct RangeServerArgs {
-    WorkerPtrs ptrs;             // scales[w] = worker w's ranges
-    float* params;               // may be null
-    float* acc;                  // may be null when params is given
-    uint64_t n, nrows, ncode_words, rows_per_bucket;
-    int W, add_into;
-    float neg_lr;
-    uint32_t bias_bits;
-};
-
-template <int BITS>
-__global__ void __launch_bounds__(kRangeThreads)
-range_server_kernel(const __grid_constant__ RangeServerArgs a)
-{
-    const uint64_t row = (uint64_t)blockIdx.x * kRangeThreads + threadIdx.x;
-    if (row >= a.nrows) return;
-    const uint64_t e0 = row * 32, word0 = row * BITS, bucket = row / a.rows_per_bucket;
-    const bool full = e0 + 32 <= a.n;
-    float2 v2[16];
-#pragma unroll
-    for (int p = 0; p < 16; ++p) {
-        v2[p] = make_float2(0.0f, 0.0f);
-        if (a.add_into) {                                    // the sum continues from the accumulator
-            if (e0 + 2 * p < a.n) v2[p].x = a.acc[e0 + 2 * p];
-            if (e0 + 2 * p + 1 < a.n) v2[p].y = a.acc[e0 + 2 * p + 1];
-        }
-    }
-    for (int w = 0; w < a.W; ++w) {
-        uint32_t cw[BITS];
-        if (full) {
-            load_row_words<BITS>(a.ptrs.codes[w], word0, cw);
-        } else {
-#pragma unroll
-            for (int j = 0; j < BITS; ++j)
-                cw[j] = (word0 + j < a.ncode_words) ? __ldg(a.ptrs.codes[w] + word0 + j) : 0u;
-        }
-        const DecodeScale2 d = widen(range_decode_scale<BITS>(__ldg(a.ptrs.scales[w] + 2 * bucket),
-                                                              __ldg(a.ptrs.scales[w] + 2 * bucket + 1)));
-        add_decoded_row<BITS, true>(cw, d, v2, a.bias_bits);
-    }
-    float v[32];
-    floats_from_pairs(v2, v);
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-        if (e0 + j < a.n) {
-            if (a.acc) a.acc[e0 + j] = v[j];
-            if (a.params) a.params[e0 + j] = __fmaf_rn(a.neg_lr, v[j], a.params[e0 + j]);
-        }
-    }
-}
-
-cudaError_t launch_server_range(const WorkerPtrs& ptrs, int W, int bits, uint64_t n, uint64_t bucket,
-                                float* params, float lr, float* acc, int add_into, cudaStream_t stream)
-{
-    if (server_tma_applies(n, bucket, W)) {
-        if (params != nullptr && acc == nullptr)
-            return launch_server_range_tma(ptrs, W, bits, n, bucket, params, lr, 1, stream);
-        if (params == nullptr)
-            return launch_server_range_tma(ptrs, W, bits, n, bucket, acc, 0.0f, add_into ? 2 : 0, stream);
-    }
-    RangeServerArgs a;
-    a.ptrs = ptrs; a.params = params; a.acc = acc;
-    a.n = n;
-    a.nrows = (n + 31) / 32;
-    a.ncode_words = (n * (uint64_t)bits + 31) / 32;
-    a.rows_per_bucket = bucket >= n ? a.nrows : bucket / 32;
-    a.W = W; a.add_into = add_into;
-    a.neg_lr = -lr;
-    a.bias_bits = 0x4B000000u;
-    const uint64_t blocks = (a.nrows + kRangeThreads - 1) / kRangeThreads;
-    if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    const unsigned grid = (unsigned)blocks;
-    switch (bits) {
-        case 1: range_server_kernel<1><<<grid, kRangeThreads, 0, stream>>>(a); break;
-        case 2: range_server_kernel<2><<<grid, kRangeThreads, 0, stream>>>(a); break;
-        case 3: range_server_kernel<3><<<grid, kRangeThreads, 0, stream>>>(a); break;
-        case 4: range_server_kernel<4><<<grid, kRangeThreads, 0, stream>>>(a); break;
-        case 5: range_server_kernel<5><<<grid, kRangeThreads, 0, stream>>>(a); break;
-        case 6: range_server_kernel<6><<<grid, kRangeThreads, 0, stream>>>(a); break;
-        case 7: range_server_kernel<7><<<grid, kRangeThreads, 0, stream>>>(a); break;
-        case 8: range_server_kernel<8><<<grid, kRangeThreads, 0, stream>>>(a); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

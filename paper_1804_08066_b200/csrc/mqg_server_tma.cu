@@ -253,39 +253,45 @@ constexpr int server_min_ctas() { return 4; }
 // MODE 1: dst = params, dst <- fma(-lr, sum, dst).  MODE 0: dst = acc, dst <- sum.
 // MODE 2: dst = acc, the sum continues from the value already there.
 // RANGE: the (min, max) nearest-rounding variant (x^ = fma(q, step, lo)).
-// The one row of a gradient that has fewer than 32 elements (row `row`, the last one): plain loads and
-// stores by a single thread.  `params` is the gradient's first parameter, n its length, its bit stream
-// the words [code_word0, words_end) of every worker's buffer, `bucket` the index of the row's scale.
+// The one row of a gradient that has fewer than 32 elements (row `row`, the last one): a warp, lane j on
+// element j, with plain loads and stores; the code words and scales of eight workers are requested at a
+// time.  (One thread on the whole row, worker after worker, took about 1 us per worker at the end of the
+// launch.)  `params` is the gradient's first parameter, n its length, its bit stream the words
+// [code_word0, words_end) of every worker's buffer, `bucket` the index of the row's scale.
 template <int BITS, int MODE, bool RANGE>
 __device__ __noinline__ void server_ragged_row(const ServerTmaArgs& a, float* params, uint32_t row, uint64_t n,
-                                               uint64_t code_word0, uint64_t words_end, uint32_t bucket)
+                                               uint64_t code_word0, uint64_t words_end, uint32_t bucket, uint32_t lane)
 {
-    const uint64_t e0 = (uint64_t)row * 32;
-    const uint64_t word0 = code_word0 + (uint64_t)row * BITS;
-    float2 v2[16];
+    const uint64_t e = (uint64_t)row * 32 + lane;
+    if (e >= n) return;
+    const uint32_t bit = lane * BITS, shift = bit & 31u;
+    const uint64_t word = code_word0 + (uint64_t)row * BITS + (bit >> 5);
+    const bool two = shift + BITS > 32 && word + 1 < words_end;
+    const float old = MODE != 0 ? params[e] : 0.0f;
+    float2 v = make_float2(MODE == 2 ? old : 0.0f, 0.0f);
+    constexpr int kBatch = 8;
+#pragma unroll 1
+    for (int w0 = 0; w0 < a.W; w0 += kBatch) {
+        uint32_t lo[kBatch], hi[kBatch];
+        float2 sc[kBatch];
 #pragma unroll
-    for (int p = 0; p < 16; ++p) {
-        v2[p] = make_float2(0.0f, 0.0f);
-        if constexpr (MODE == 2) {
-            if (e0 + 2 * p < n) v2[p].x = params[e0 + 2 * p];
-            if (e0 + 2 * p + 1 < n) v2[p].y = params[e0 + 2 * p + 1];
+        for (int i = 0; i < kBatch; ++i) {
+            if (w0 + i >= a.W) break;
+            lo[i] = __ldg(a.ptrs.codes[w0 + i] + word);
+            hi[i] = two ? __ldg(a.ptrs.codes[w0 + i] + word + 1) : 0u;
+            if (RANGE) sc[i] = __ldg(reinterpret_cast<const float2*>(a.ptrs.scales[w0 + i]) + bucket);
+            else sc[i] = make_float2(__ldg(a.ptrs.scales[w0 + i] + bucket), 0.0f);
+        }
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+            if (w0 + i >= a.W) break;
+            const DecodeScale d = RANGE ? range_decode_scale<BITS>(sc[i].x, sc[i].y) : decode_scale<BITS>(sc[i].x);
+            const uint32_t q = __funnelshift_r(lo[i], hi[i], shift) & ((1u << BITS) - 1u);
+            v = accumulate2<BITS, RANGE>(v, make_float2(__uint_as_float(q | 0x4B000000u), 8388608.0f),
+                                         make_float2(d.two_h, d.two_h), make_float2(d.minus_h, d.minus_h));
         }
     }
-    for (int w = 0; w < a.W; ++w) {
-        uint32_t cw[BITS];
-#pragma unroll
-        for (int j = 0; j < BITS; ++j)
-            cw[j] = (word0 + j < words_end) ? __ldg(a.ptrs.codes[w] + word0 + j) : 0u;
-        const DecodeScale2 d = widen(RANGE ? range_decode_scale<BITS>(__ldg(a.ptrs.scales[w] + 2 * bucket),
-                                                                      __ldg(a.ptrs.scales[w] + 2 * bucket + 1))
-                                           : decode_scale<BITS>(__ldg(a.ptrs.scales[w] + bucket)));
-        add_decoded_row<BITS, RANGE>(cw, d, v2);
-    }
-    float v[32];
-    floats_from_pairs(v2, v);
-#pragma unroll
-    for (int j = 0; j < 32; ++j)
-        if (e0 + j < n) params[e0 + j] = MODE == 1 ? __fmaf_rn(a.neg_lr, v[j], params[e0 + j]) : v[j];
+    params[e] = MODE == 1 ? __fmaf_rn(a.neg_lr, v.x, old) : v.x;
 }
 
 template <int BITS, int MODE, bool RANGE, bool SEGS>
@@ -343,17 +349,21 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
     constexpr int kIssueAt = 4;
     const int issue_at = min(kIssueAt, a.W - 1);
 
+    // (a long launch gains nothing from it and loses 1 % at two bits, 45.6 against 46.1 us: the parameter tiles
+    // of all warps then stand in front of the codes of all warps)
+    const bool params_first = ntiles < 4;
+
     bool failed = false;
     uint32_t k = 0, u = 0;                         // tile and code stage in use
     if (ntiles > 0) {
-        float2 s0[2];
+        // with a few tiles per warp, everything the first tile needs is requested before any of it is waited for
         const TileLoc first = locate_srv_tile<SEGS>(map_full, a, segs, t_begin, next_e);
-        load_tile_scales<RANGE, SEGS>(a, first, lane, wide, s0);
-        store_tile_scales<BITS, RANGE>(a, table, lane, wide, s0);
-        if (MODE == 2 && lane == 0) {
+        if ((MODE == 2 || (MODE == 1 && params_first)) && lane == 0) {
             mbar_expect_tx(bar, kSrvTileBytes);
             if (!a.arm_only) tma_load_2d(smem_u32(stage), first.map, 0, (int)first.row0, bar);
         }
+        float2 s0[2];
+        load_tile_scales<RANGE, SEGS>(a, first, lane, wide, s0);
         // the first kCodeDepth code stages (u2 = stage number, tile u2 / groups, group u2 % groups);
         // one copy group per stage, empty when there is no such stage
 #pragma unroll
@@ -364,6 +374,7 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
                                       (int)(u2 % groups) * kGroup, lane_off);
             cp_async_commit();
         }
+        store_tile_scales<BITS, RANGE>(a, table, lane, wide, s0);
         __syncwarp();
     }
     // position of the code stage kCodeDepth ahead of the one in use, kept incrementally
@@ -433,7 +444,7 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
             // box is clipped by the tensor's bounds and the rows beyond arrive as zeros, still counted
             // in the bytes.
             auto load_params = [&]() {
-                if (lane == 0) {
+                if (lane == 0 && (k != 0 || !params_first)) {
                     bulk_wait_read<0>();
                     mbar_expect_tx(bar, kSrvTileBytes);
                     if (!a.arm_only) tma_load_2d(smem_u32(stage), loc.map, 0, (int)row0, bar);
@@ -528,21 +539,21 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
         bulk_wait_all<0>();                                    // stores done before the stage goes away
     }
 
-    // A last row of fewer than 32 elements is not covered by the tensor map: one lane of the
-    // grid's last CTA handles it (SEGS: one lane per segment that has such a row).
-    if (blockIdx.x == gridDim.x - 1) {
-        if constexpr (SEGS) {
-            for (int j = (int)threadIdx.x; j < segs->nseg; j += kSrvThreads) {
-                const ServerSegEntry& e = segs->e[j];
-                if (e.ragged == 0) continue;
-                const uint64_t n = (uint64_t)e.nrows_full * 32 + e.ragged;
-                server_ragged_row<BITS, MODE, RANGE>(a, a.params + e.elem0, e.nrows_full, n, e.code_word0,
-                                                     e.code_word0 + (n * BITS + 31) / 32, e.scale_idx);
-            }
-        } else if (a.nrows > a.nrows_full && threadIdx.x == kSrvThreads - 1) {
-            server_ragged_row<BITS, MODE, RANGE>(a, a.params, a.nrows_full, a.n, 0, a.ncode_words,
-                                                 bucket_of_row(a, a.nrows_full));
+    // A last row of fewer than 32 elements is not covered by the tensor map: the grid's last warp takes it
+    // (SEGS: the segments that have such a row go to the grid's last warps in turn; those have a tile less than
+    // the first ones, unless all have the same number).
+    const uint32_t from_end = nwarps - 1 - gwarp;
+    if constexpr (SEGS) {
+        for (uint32_t j = from_end; j < (uint32_t)segs->nseg; j += nwarps) {
+            const ServerSegEntry& e = segs->e[j];
+            if (e.ragged == 0) continue;
+            const uint64_t n = (uint64_t)e.nrows_full * 32 + e.ragged;
+            server_ragged_row<BITS, MODE, RANGE>(a, a.params + e.elem0, e.nrows_full, n, e.code_word0,
+                                                 e.code_word0 + (n * BITS + 31) / 32, e.scale_idx, lane);
         }
+    } else if (a.nrows > a.nrows_full && from_end == 0) {
+        server_ragged_row<BITS, MODE, RANGE>(a, a.params, a.nrows_full, a.n, 0, a.ncode_words,
+                                             bucket_of_row(a, a.nrows_full), lane);
     }
 }
 
@@ -652,10 +663,13 @@ static cudaError_t launch_server_tma_inst(const void* params, ServerTmaArgs& a, 
         cap = sms * (occ > 0 ? occ : 1);
         grid_cap[dev].store(cap, std::memory_order_relaxed);   // every thread computes the same value
     }
-    // the tiles are split evenly over the warps of the grid; tiny inputs are not spread too thin
+    // The tiles are split evenly over the warps of the grid, down to one tile per warp: a warp's tiles follow one
+    // another, so a short gradient is done soonest when it is spread as thin as it goes.  Per step at two bits
+    // against at least four tiles per warp (and the parameter tile, the scales and the codes of a warp's first
+    // tile requested in turn): 3.4 against 7.4 us at n = 2^20, W = 4, 5.4 against 12.5 us at W = 16, 6.7 against
+    // 8.8 us at n = 2^22, W = 4.
     uint64_t grid = (uint64_t)cap;
-    const uint64_t max_warps = (a.ntiles + 3) / 4;
-    if (grid * kSrvWarps > max_warps) grid = (max_warps + kSrvWarps - 1) / kSrvWarps;
+    if (grid * kSrvWarps > a.ntiles) grid = (a.ntiles + kSrvWarps - 1) / kSrvWarps;
     CUtensorMap map_full;
     const char* why = nullptr;
     if (!encode_rows_map(&map_full, params, a.nrows_full, 4, 32, kSrvTileRows, &why)) return cudaErrorNotSupported;
@@ -1048,8 +1062,8 @@ static cudaError_t launch_server_segs_inst(const ServerSegTable& tab, const Serv
         grid_cap[dev].store(cap, std::memory_order_relaxed);   // every thread computes the same value
     }
     uint64_t grid = (uint64_t)cap;
-    const uint64_t max_warps = (a.ntiles + 3) / 4;
-    if (grid * kSrvWarps > max_warps) grid = (max_warps + kSrvWarps - 1) / kSrvWarps;
+    const uint64_t warps = (uint64_t)a.ntiles + ss.pieces;          // at least one tile or short piece per warp
+    if (grid * kSrvWarps > warps) grid = (warps + kSrvWarps - 1) / kSrvWarps;
     return launch_pdl_smem(kernel, (unsigned)grid, kSrvThreads, kSmemBytes, stream, tab, ss, a, timeouts);
 }
 
