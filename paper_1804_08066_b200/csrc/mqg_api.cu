@@ -67,15 +67,16 @@ mqg_status check_workers(const uint32_t* const* codes, const float* const* scale
     return MQG_OK;
 }
 
-// Validates a segment table and cuts it into chunks of at most kMaxSegmentsPerLaunch segments;
-// calls fn(table, first_segment_index) for each chunk.  Segments for which skip(j) holds get no
-// tiles in the tables, exactly like empty segments: another launch takes care of them.  skip is
-// only called once the table has been checked.
-struct SkipNone { bool operator()(int) const { return false; } };
+uint64_t eff_bucket(uint64_t n, uint64_t bucket) { return bucket < n ? bucket : n; }
 
-template <typename Fn, typename Skip = SkipNone>
-mqg_status for_each_chunk(int nseg, const uint64_t* seg_off, const uint64_t* code_off, int bits,
-                          Fn&& fn, Skip&& skip = Skip())
+// (min, max) shapes outside the one-pass kernel: a bucket per CTA where it fills the CTA's warps, or where the
+// gradient is so short that one launch instead of four decides.
+bool range_spans_preferred(uint64_t n, uint64_t bucket)
+{
+    return mqg::bucket_spans_apply(n, bucket) && (eff_bucket(n, bucket) > 4096 || n < 65536);
+}
+
+mqg_status check_segments(int nseg, const uint64_t* seg_off, const uint64_t* code_off, int bits)
 {
     if (nseg < 0) return fail(MQG_ERR_INVALID, "nseg = %d is negative", nseg);
     if (nseg == 0) return MQG_OK;
@@ -88,6 +89,33 @@ mqg_status for_each_chunk(int nseg, const uint64_t* seg_off, const uint64_t* cod
             return fail(MQG_ERR_INVALID, "code_off leaves segment %d fewer than %llu words", j,
                         (unsigned long long)need);
     }
+    return MQG_OK;
+}
+
+// The per-layer quantizers: max-abs scales (workspace == nullptr), or L2-norm scales of one worker.
+mqg_status quantize_segments(const void* const* grads, int W, int nseg, const uint64_t* seg_off, const uint64_t* code_off,
+                             int bits, uint64_t seed, uint32_t* const* codes, float* const* scales, mqg_dtype dtype,
+                             uint32_t first_worker, uint32_t step, uint64_t elem_offset, float* workspace,
+                             cudaStream_t stream, const char* what)
+{
+    if (mqg_status st = check_segments(nseg, seg_off, code_off, bits)) return st;
+    if (nseg == 0) return MQG_OK;
+    const cudaError_t err = mqg::launch_quantize_segments(grads, W, nseg, seg_off, code_off, bits, seed, codes, scales,
+                                                          (int)dtype, first_worker, step, elem_offset, workspace, stream);
+    return err == cudaSuccess ? MQG_OK : cuda_fail(what, err);
+}
+
+// Validates a segment table and cuts it into chunks of at most kMaxSegmentsPerLaunch segments;
+// calls fn(table, first_segment_index) for each chunk.  Segments for which skip(j) holds get no
+// tiles in the tables, exactly like empty segments: another launch takes care of them.  skip is
+// only called once the table has been checked.
+struct SkipNone { bool operator()(int) const { return false; } };
+
+template <typename Fn, typename Skip = SkipNone>
+mqg_status for_each_chunk(int nseg, const uint64_t* seg_off, const uint64_t* code_off, int bits,
+                          Fn&& fn, Skip&& skip = Skip())
+{
+    if (mqg_status st = check_segments(nseg, seg_off, code_off, bits)) return st;
     const uint64_t tile_elems = (uint64_t)mqg::kMaxTileRows * 32;
     int j = 0;
     while (j < nseg) {
@@ -187,6 +215,9 @@ mqg_status mqg_quantize(const void* grad, uint64_t n, int bits, uint64_t bucket,
     if (eff <= (uint64_t)mqg::kMaxFusedBucket)
         err = mqg::launch_quantize_fused(grad, n, bits, bucket, seed, codes, scales, (int)dtype,
                                          worker, step, elem_offset, stream);
+    else if (mqg::bucket_spans_apply(n, bucket))
+        err = mqg::launch_bucket_spans(&grad, 1, n, bits, bucket, seed, &codes, &scales, 0, (int)dtype, worker, step,
+                                       elem_offset, stream);
     else
         err = mqg::launch_quantize_big_buckets(grad, n, bits, bucket, seed, codes, scales, (int)dtype,
                                                worker, step, elem_offset, stream);
@@ -221,7 +252,13 @@ mqg_status mqg_quantize_workers(const void* const* grads, int W, uint64_t n, int
         if (err != cudaSuccess) return cuda_fail("mqg_quantize_workers", err);
         return MQG_OK;
     }
-    // shapes the batched kernel does not take: one launch per worker, same results
+    if (W > 1 && eff_bucket(n, bucket) > (uint64_t)mqg::kMaxFusedBucket && mqg::bucket_spans_apply(n, bucket)) {
+        const cudaError_t err = mqg::launch_bucket_spans(grads, W, n, bits, bucket, seed, codes, scales, 0, (int)dtype,
+                                                         first_worker, step, elem_offset, stream);
+        if (err != cudaSuccess) return cuda_fail("mqg_quantize_workers", err);
+        return MQG_OK;
+    }
+    // shapes the batched kernels do not take: one launch per worker, same results
     for (int w = 0; w < W; ++w) {
         const mqg_status st = mqg_quantize(grads[w], n, bits, bucket, seed, codes[w], scales[w], dtype,
                                            first_worker + (uint32_t)w, step, elem_offset, cuda_stream);
@@ -244,6 +281,8 @@ mqg_status mqg_quantize_minmax(const void* grad, uint64_t n, int bits, uint64_t 
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const cudaError_t err = mqg::quantize_range_fused_applies(n, bucket)
         ? mqg::launch_quantize_range_fused(grad, n, bits, bucket, codes, ranges, (int)dtype, stream)
+        : range_spans_preferred(n, bucket)
+        ? mqg::launch_bucket_spans(&grad, 1, n, bits, bucket, 0, &codes, &ranges, 1, (int)dtype, 0, 0, 0, stream)
         : mqg::launch_quantize_range_general(grad, n, bits, bucket, codes, ranges, (int)dtype, stream);
     if (err != cudaSuccess) return cuda_fail("mqg_quantize_minmax", err);
     return MQG_OK;
@@ -274,7 +313,13 @@ mqg_status mqg_quantize_workers_minmax(const void* const* grads, int W, uint64_t
         if (err != cudaSuccess) return cuda_fail("mqg_quantize_workers_minmax", err);
         return MQG_OK;
     }
-    // shapes the batched kernel does not take: one call per worker, same results
+    if (range_spans_preferred(n, bucket)) {
+        const cudaError_t err = mqg::launch_bucket_spans(grads, W, n, bits, bucket, 0, codes, ranges, 1, (int)dtype, 0, 0, 0,
+                                                         stream);
+        if (err != cudaSuccess) return cuda_fail("mqg_quantize_workers_minmax", err);
+        return MQG_OK;
+    }
+    // shapes the batched kernels do not take: one call per worker, same results
     for (int w = 0; w < W; ++w) {
         const mqg_status st = mqg_quantize_minmax(grads[w], n, bits, bucket, codes[w], ranges[w], dtype, cuda_stream);
         if (st != MQG_OK) return st;
@@ -413,38 +458,8 @@ mqg_status mqg_quantize_segments(const void* grad, int nseg, const uint64_t* seg
         if (!aligned4(scales)) return fail(MQG_ERR_ALIGN, "scales not 4-byte aligned");
     }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    // Max pass over every segment; then the encode pass.  A long segment whose buffers are aligned
-    // for bulk copies is encoded by the TMA-fed quantize kernel in a launch of its own (its scale is
-    // final by then); in the table-driven encode launch it has no tiles.  Same results bit for bit.
-    const size_t esz = dtype == MQG_BF16 ? 2 : 4;
-    auto own = [&](int j) {
-        return mqg::quantize_given_scale_applies(static_cast<const char*>(grad) + seg_off[j] * esz,
-                                                 seg_off[j + 1] - seg_off[j], codes + code_off[j],
-                                                 elem_offset + seg_off[j]);
-    };
-    mqg_status st = for_each_chunk(nseg, seg_off, code_off, bits,
-        [&](const mqg::SegmentTable& tab, int first) -> mqg_status {
-            const cudaError_t err = mqg::launch_segments_absmax(grad, tab, scales + first, (int)dtype, stream);
-            if (err != cudaSuccess) return cuda_fail("mqg_quantize_segments", err);
-            return MQG_OK;
-        });
-    if (st != MQG_OK) return st;
-    st = for_each_chunk(nseg, seg_off, code_off, bits,
-        [&](const mqg::SegmentTable& tab, int first) -> mqg_status {
-            const cudaError_t err = mqg::launch_segments_encode(grad, tab, bits, seed, codes, scales + first,
-                                                                (int)dtype, worker, step, elem_offset, stream);
-            if (err != cudaSuccess) return cuda_fail("mqg_quantize_segments", err);
-            return MQG_OK;
-        }, own);
-    if (st != MQG_OK) return st;
-    for (int j = 0; j < nseg; ++j) {
-        if (!own(j)) continue;
-        const cudaError_t err = mqg::launch_quantize_given_scale(
-            static_cast<const char*>(grad) + seg_off[j] * esz, seg_off[j + 1] - seg_off[j], bits, seed,
-            codes + code_off[j], scales + j, (int)dtype, worker, step, elem_offset + seg_off[j], stream);
-        if (err != cudaSuccess) return cuda_fail("mqg_quantize_segments", err);
-    }
-    return MQG_OK;
+    return quantize_segments(&grad, 1, nseg, seg_off, code_off, bits, seed, &codes, &scales, dtype, worker, step,
+                             elem_offset, nullptr, stream, "mqg_quantize_segments");
 }
 
 mqg_status mqg_quantize_segments_workers(const void* const* grads, int W, int nseg, const uint64_t* seg_off,
@@ -468,66 +483,8 @@ mqg_status mqg_quantize_segments_workers(const void* const* grads, int W, int ns
         if (!aligned4(scales[w])) return fail(MQG_ERR_ALIGN, "worker %d: scales not 4-byte aligned", w);
     }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    const size_t esz = dtype == MQG_BF16 ? 2 : 4;
-    // a long segment whose buffers are aligned for bulk copies with every worker is an entry of the
-    // TMA-fed part of the encode launch; all other segments go through its table-driven part
-    auto own = [&](int j) {
-        for (int w = 0; w < W; ++w)
-            if (!mqg::quantize_given_scale_applies(static_cast<const char*>(grads[w]) + seg_off[j] * esz,
-                                                   seg_off[j + 1] - seg_off[j], codes[w] + code_off[j],
-                                                   elem_offset + seg_off[j], mqg::kEntrySegmentElems))
-                return false;
-        return true;
-    };
-    bool zeroed = false;
-    mqg_status st = for_each_chunk(nseg, seg_off, code_off, bits,
-        [&](const mqg::SegmentTable& tab, int first) -> mqg_status {
-            if (!zeroed) {                 // after the table has been validated
-                const cudaError_t err = mqg::launch_zero_scales(scales, W, nseg, stream);
-                if (err != cudaSuccess) return cuda_fail("mqg_quantize_segments_workers", err);
-                zeroed = true;
-            }
-            const cudaError_t err = mqg::launch_absmax_workers(grads, scales, first, W, tab, (int)dtype, stream);
-            if (err != cudaSuccess) return cuda_fail("mqg_quantize_segments_workers", err);
-            return MQG_OK;
-        });
-    if (st != MQG_OK) return st;
-
-    std::vector<mqg::SegEntryHost> entries;
-    for (int j = 0; j < nseg; ++j) {
-        if (seg_off[j + 1] == seg_off[j] || !own(j)) continue;
-        for (int w = 0; w < W; ++w) {
-            mqg::SegEntryHost e;
-            e.grad = static_cast<const char*>(grads[w]) + seg_off[j] * esz;
-            e.codes = codes[w] + code_off[j];
-            e.scale = scales[w] + j;
-            e.n = seg_off[j + 1] - seg_off[j];
-            e.elem_offset = elem_offset + seg_off[j];
-            e.worker = first_worker + (uint32_t)w;
-            entries.push_back(e);
-        }
-    }
-    std::vector<std::pair<mqg::SegmentTable, int>> short_tabs;
-    st = for_each_chunk(nseg, seg_off, code_off, bits,
-        [&](const mqg::SegmentTable& tab, int first) -> mqg_status {
-            if (tab.tile_start[tab.nseg] != 0) short_tabs.emplace_back(tab, first);
-            return MQG_OK;
-        }, own);
-    if (st != MQG_OK) return st;
-    const size_t per = (size_t)mqg::kMaxSegEntriesPerLaunch;
-    const size_t entry_launches = (entries.size() + per - 1) / per;
-    const size_t launches = entry_launches > short_tabs.size() ? entry_launches : short_tabs.size();
-    for (size_t i = 0; i < launches; ++i) {
-        const size_t e0 = i * per;
-        const int nent = e0 < entries.size() ? (int)(entries.size() - e0 < per ? entries.size() - e0 : per) : 0;
-        const mqg::SegmentTable* tab = i < short_tabs.size() ? &short_tabs[i].first : nullptr;
-        const int first = i < short_tabs.size() ? short_tabs[i].second : 0;
-        const cudaError_t err = mqg::launch_encode_workers(nent ? entries.data() + e0 : nullptr, nent, tab, grads,
-                                                           codes, scales, first, W, bits, seed, (int)dtype,
-                                                           first_worker, step, elem_offset, stream);
-        if (err != cudaSuccess) return cuda_fail("mqg_quantize_segments_workers", err);
-    }
-    return MQG_OK;
+    return quantize_segments(grads, W, nseg, seg_off, code_off, bits, seed, codes, scales, dtype, first_worker, step,
+                             elem_offset, nullptr, stream, "mqg_quantize_segments_workers");
 }
 
 mqg_status mqg_quantize_l2(const void* grad, uint64_t n, int bits, uint64_t bucket, uint64_t seed,
@@ -644,40 +601,9 @@ mqg_status mqg_quantize_segments_l2(const void* grad, int nseg, const uint64_t* 
         if (!aligned4(workspace)) return fail(MQG_ERR_ALIGN, "workspace not 4-byte aligned");
     }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    // Sums and scales of every segment first; then the encode, where a long segment with buffers
-    // aligned for bulk copies takes a launch of the TMA-fed quantize kernel of its own.
-    const size_t esz = dtype == MQG_BF16 ? 2 : 4;
-    auto own = [&](int j) {
-        return mqg::quantize_given_scale_applies(static_cast<const char*>(grad) + seg_off[j] * esz,
-                                                 seg_off[j + 1] - seg_off[j], codes + code_off[j],
-                                                 elem_offset + seg_off[j]);
-    };
-    size_t used = 0;                      // tiles of the chunks already launched
-    mqg_status st = for_each_chunk(nseg, seg_off, code_off, bits,
-        [&](const mqg::SegmentTable& tab, int first) -> mqg_status {
-            const cudaError_t err = mqg::launch_segments_l2_scales(grad, tab, scales + first, (int)dtype,
-                                                                   workspace + used, stream);
-            if (err != cudaSuccess) return cuda_fail("mqg_quantize_segments_l2", err);
-            used += tab.tile_start[tab.nseg];
-            return MQG_OK;
-        });
-    if (st != MQG_OK) return st;
-    st = for_each_chunk(nseg, seg_off, code_off, bits,
-        [&](const mqg::SegmentTable& tab, int first) -> mqg_status {
-            const cudaError_t err = mqg::launch_segments_encode(grad, tab, bits, seed, codes, scales + first,
-                                                                (int)dtype, worker, step, elem_offset, stream);
-            if (err != cudaSuccess) return cuda_fail("mqg_quantize_segments_l2", err);
-            return MQG_OK;
-        }, own);
-    if (st != MQG_OK) return st;
-    for (int j = 0; j < nseg; ++j) {
-        if (!own(j)) continue;
-        const cudaError_t err = mqg::launch_quantize_given_scale(
-            static_cast<const char*>(grad) + seg_off[j] * esz, seg_off[j + 1] - seg_off[j], bits, seed,
-            codes + code_off[j], scales + j, (int)dtype, worker, step, elem_offset + seg_off[j], stream);
-        if (err != cudaSuccess) return cuda_fail("mqg_quantize_segments_l2", err);
-    }
-    return MQG_OK;
+    float none = 0.0f;                    // a table of empty segments needs no workspace, but a pointer that says which codec
+    return quantize_segments(&grad, 1, nseg, seg_off, code_off, bits, seed, &codes, &scales, dtype, worker, step,
+                             elem_offset, workspace ? workspace : &none, stream, "mqg_quantize_segments_l2");
 }
 
 mqg_status mqg_server_step_segments(const uint32_t* const* codes, const float* const* scales, int W,

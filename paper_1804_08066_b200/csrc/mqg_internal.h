@@ -80,46 +80,26 @@ cudaError_t launch_segments_l2_scales(const void* grad, const SegmentTable& tab,
 cudaError_t launch_quantize_onebit_ef(const void* grad, float* residual, uint64_t n, uint64_t bucket,
                                       uint32_t* codes, float* ranges, int dtype, cudaStream_t stream);
 
-// The two passes of the per-layer quantizer (scales_base points at the scale of the table's first
-// segment), and the encode of ONE long segment (= one
-// bucket whose scale already stands at *scale) on the TMA-fed quantize kernel.
-cudaError_t launch_segments_absmax(const void* grad, const SegmentTable& tab, float* scales_base, int dtype,
-                                   cudaStream_t stream);
-cudaError_t launch_segments_encode(const void* grad, const SegmentTable& tab, int bits, uint64_t seed,
-                                   uint32_t* codes, float* scales_base, int dtype, uint32_t worker,
-                                   uint32_t step, uint64_t elem_offset, cudaStream_t stream);
-// Shortest segment that gets a launch of its own on the bulk-copy kernels (one-worker per-layer calls), and
-// shortest segment that becomes one entry of a launch shared by many segments (the all-workers quantizer,
-// the per-layer server step): 8 tiles of 128 rows.  Shorter segments go through the table-driven code.
-// (Entries from 2^15 instead of 2^20 elements on the AlexNet-shaped gradient, W = 8: the five convolution
-// tensors join the three large ones; quantize call 620 against 631 us, server step 137 against 140 us at K = 4.)
-constexpr uint64_t kOwnLaunchSegmentElems = 1ull << 20;
-constexpr uint64_t kEntrySegmentElems = 1ull << 15;
-bool quantize_given_scale_applies(const void* grad, uint64_t n, const uint32_t* codes, uint64_t elem_offset,
-                                  uint64_t min_elems = kOwnLaunchSegmentElems);
-cudaError_t launch_quantize_given_scale(const void* grad, uint64_t n, int bits, uint64_t seed, uint32_t* codes,
-                                        float* scale, int dtype, uint32_t worker, uint32_t step,
-                                        uint64_t elem_offset, cudaStream_t stream);
+// Whether a segment's buffers are aligned for the bulk-copy encode of the per-layer quantizer.
+bool quantize_given_scale_applies(const void* grad, uint64_t n, const uint32_t* codes, uint64_t elem_offset);
 
-// Per-layer quantization of several workers in three launches (mqg_segments_workers.cu): zero the
-// scale arrays, max pass over all (worker, segment) pairs, one encode pass.  A SegEntryHost is one
-// (worker, long segment) pair for which quantize_given_scale_applies() holds.
-struct SegEntryHost {
-    const void* grad;        // the segment's first element
-    uint32_t* codes;         // its first code word
-    float* scale;            // its scale
-    uint64_t n;              // its length
-    uint64_t elem_offset;    // flat position of its first element (for the draws)
-    uint32_t worker;         // worker id of the draws
-};
-constexpr int kMaxSegEntriesPerLaunch = 64;
-cudaError_t launch_zero_scales(float* const* scales, int W, int nseg, cudaStream_t stream);
-cudaError_t launch_absmax_workers(const void* const* grads, float* const* scales, int first, int W,
-                                  const SegmentTable& tab, int dtype, cudaStream_t stream);
-cudaError_t launch_encode_workers(const SegEntryHost* entries, int nent, const SegmentTable* short_tab,
-                                  const void* const* grads, uint32_t* const* codes, float* const* scales,
-                                  int scale_first, int W, int bits, uint64_t seed, int dtype,
-                                  uint32_t first_worker, uint32_t step, uint64_t elem_offset, cudaStream_t stream);
+// Per-layer quantization of W >= 1 workers that share a (checked) segment table: mqg_segments_workers.cu.
+// workspace != nullptr: L2-norm scales (one worker), the partial sums of its long segments go there.
+cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, const uint64_t* seg_off,
+                                     const uint64_t* code_off, int bits, uint64_t seed, uint32_t* const* codes,
+                                     float* const* scales, int dtype, uint32_t first_worker, uint32_t step,
+                                     uint64_t elem_offset, float* workspace, cudaStream_t stream);
+
+// Shortest segment that the per-layer server step gives to its bulk-copy kernel.  (From 2^15 instead of 2^20
+// elements on the AlexNet-shaped gradient, W = 8: server step 137 against 140 us at K = 4.)
+constexpr uint64_t kEntrySegmentElems = 1ull << 15;
+
+// Buckets (or a single bucket n) that one CTA quantizes as a whole, for W >= 1 workers; mode: 0 = main codec,
+// 1 = (min, max) variant (`scales` are ranges).
+bool bucket_spans_apply(uint64_t n, uint64_t bucket);
+cudaError_t launch_bucket_spans(const void* const* grads, int W, uint64_t n, int bits, uint64_t bucket, uint64_t seed,
+                                uint32_t* const* codes, float* const* scales, int mode, int dtype, uint32_t first_worker,
+                                uint32_t step, uint64_t elem_offset, cudaStream_t stream);
 
 // Two-pass quantize with uniform large buckets (bucket > kMaxFusedBucket, or a single bucket
 // whose length is not a multiple of 32).

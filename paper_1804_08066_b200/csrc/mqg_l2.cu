@@ -11,6 +11,7 @@
 // Adding +0 is exact, so evaluating more (all-zero) leaves or levels than the padded tree has
 // does not change the result; that is what lets a fixed 256-row tile serve every bucket shape.
 #include "mqg_segments.cuh"
+#include "mqg_tma.cuh"
 #include "mqg_tree.cuh"
 
 namespace mqg {
@@ -94,12 +95,14 @@ l2_quantize_kernel(const L2Args a)
 // rows) goes to partial[blockIdx.x].
 template <int DTYPE>
 __global__ void __launch_bounds__(kMaxTileRows)
-l2_partials_kernel(const void* __restrict__ grad, const SegmentTable tab, float* __restrict__ partial)
+l2_partials_kernel(const void* __restrict__ grad, const __grid_constant__ SegmentTable tab, float* __restrict__ partial)
 {
     __shared__ __align__(1024) float4 tile[kMaxTileRows * 8];
     __shared__ float s_part[kMaxTileRows / 32];
     const uint32_t t = threadIdx.x;
     const TileGeom g = locate_tile<1>(tab, blockIdx.x);
+    grid_dependency_release();
+    grid_dependency_wait();
     if constexpr (DTYPE == 0)
         load_tile_f32<kMaxTileRows>(tile, static_cast<const float*>(grad) + g.elem0, g.valid, g.rows);
     else
@@ -117,20 +120,40 @@ l2_partials_kernel(const void* __restrict__ grad, const SegmentTable tab, float*
     if (t == 0) partial[blockIdx.x] = tree8(s_part, 0, kMaxTileRows / 32);
 }
 
-// Pass 2: one CTA per segment folds the segment's tile sums, in place, one tree level per
-// barrier, and writes the segment's scale.
-__global__ void __launch_bounds__(256)
-l2_finish_kernel(const SegmentTable tab, float* __restrict__ partial, float* __restrict__ scales)
+// Pass 2: one CTA per segment folds the segment's tile sums, in place, and writes the segment's scale.  A turn folds
+// aligned groups of 1024 sums to one each (two levels in a thread, five in a warp, three over the warps); zero
+// leaves beyond the last add exactly.  (One level per turn, through memory, was 13 round trips for 2^25 elements.)
+constexpr int kFinishThreads = 256;
+__global__ void __launch_bounds__(kFinishThreads)
+l2_finish_kernel(const __grid_constant__ SegmentTable tab, float* __restrict__ partial, float* __restrict__ scales)
 {
-    const uint32_t seg = blockIdx.x;
-    const uint64_t first = tab.tile_start[seg], count = tab.tile_start[seg + 1] - first;
+    __shared__ float s_part[2][kFinishThreads / 32];
+    const uint32_t seg = blockIdx.x, t = threadIdx.x;
+    const uint64_t first = tab.tile_start[seg];
+    uint64_t count = tab.tile_start[seg + 1] - first;
+    grid_dependency_release();
+    grid_dependency_wait();
+    if (count == 0) return;                        // a segment that another kernel has taken
     float* p = partial + first;
-    for (uint64_t d = 1; d < count; d <<= 1) {
-        for (uint64_t j = (uint64_t)threadIdx.x * 2 * d; j < count; j += 256ull * 2 * d)
-            if (j + d < count) p[j] = __fadd_rn(p[j], p[j + d]);   // a missing partner is a zero leaf
+    uint32_t k = 0;
+    float sum;
+    do {
+        const uint64_t groups = (count + 1023) / 1024;
+        for (uint64_t g = 0; g < groups; ++g, ++k) {
+            const uint64_t j = g * 1024 + 4 * t;
+            float v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = j + i < count ? __ldcg(p + j + i) : 0.0f;
+            sum = warp_tree(__fadd_rn(__fadd_rn(v[0], v[1]), __fadd_rn(v[2], v[3])), 32);
+            if ((t & 31) == 0) s_part[k & 1][t >> 5] = sum;
+            __syncthreads();                       // group g has been read: its sum may go to p[g]
+            sum = tree8(s_part[k & 1], 0, kFinishThreads / 32);
+            if (t == 0 && groups > 1) __stcg(p + g, sum);
+        }
         __syncthreads();
-    }
-    if (threadIdx.x == 0) scales[seg] = count ? norm_from_sum(p[0]) : 0.0f;
+        count = groups;
+    } while (count > 1);
+    if (t == 0) scales[seg] = norm_from_sum(sum);
 }
 
 template <int BITS>
@@ -138,22 +161,6 @@ cudaError_t launch_l2_bits(const L2Args& a, int dtype, unsigned grid, cudaStream
 {
     if (dtype == 0) l2_quantize_kernel<BITS, 0><<<grid, kMaxTileRows, 0, stream>>>(a);
     else l2_quantize_kernel<BITS, 1><<<grid, kMaxTileRows, 0, stream>>>(a);
-    return cudaGetLastError();
-}
-
-// partials -> scales for one table; `partial` has room for the table's tiles.
-cudaError_t sums_and_scales(const void* grad, const SegmentTable& tab, float* scales, int dtype, float* partial,
-                            cudaStream_t stream)
-{
-    const uint32_t ntiles = tab.tile_start[tab.nseg];
-    if (tab.nseg == 0) return cudaSuccess;
-    if (ntiles != 0) {
-        if (dtype == 0) l2_partials_kernel<0><<<ntiles, kMaxTileRows, 0, stream>>>(grad, tab, partial);
-        else l2_partials_kernel<1><<<ntiles, kMaxTileRows, 0, stream>>>(grad, tab, partial);
-        const cudaError_t err = cudaGetLastError();
-        if (err != cudaSuccess) return err;
-    }
-    l2_finish_kernel<<<(unsigned)tab.nseg, 256, 0, stream>>>(tab, partial, scales);
     return cudaGetLastError();
 }
 
@@ -196,10 +203,17 @@ cudaError_t launch_quantize_l2(const void* grad, uint64_t n, int bits, uint64_t 
     return cudaErrorInvalidValue;
 }
 
+// partials -> scales of the table's segments that have tiles; `partial` has room for the table's tiles.
 cudaError_t launch_segments_l2_scales(const void* grad, const SegmentTable& tab, float* scales_base, int dtype,
                                       float* partial, cudaStream_t stream)
 {
-    return sums_and_scales(grad, tab, scales_base, dtype, partial, stream);
+    const uint32_t ntiles = tab_tiles(tab);
+    if (ntiles == 0) return cudaSuccess;
+    const cudaError_t err =
+        dtype == 0 ? launch_pdl(l2_partials_kernel<0>, ntiles, kMaxTileRows, stream, grad, tab, partial)
+                   : launch_pdl(l2_partials_kernel<1>, ntiles, kMaxTileRows, stream, grad, tab, partial);
+    if (err != cudaSuccess) return err;
+    return launch_pdl(l2_finish_kernel, (unsigned)tab.nseg, kFinishThreads, stream, tab, partial, scales_base);
 }
 
 }  // namespace mqg

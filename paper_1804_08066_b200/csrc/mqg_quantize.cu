@@ -183,9 +183,8 @@ __device__ __forceinline__ bool range_quantize_tile(TmaQuantizeShared<DTYPE, THR
     return true;
 }
 
-// MODE: kMaxAbs = the main codec, kRange = the (min, max) variant, kNorm = the L2-norm scale variant,
-// kGiven = encode against a scale computed by an earlier pass (long segments of the per-layer quantizers).
-enum : int { kMaxAbs = 0, kRange = 1, kNorm = 2, kGiven = 3 };
+// MODE: kMaxAbs = the main codec, kRange = the (min, max) variant, kNorm = the L2-norm scale variant.
+enum : int { kMaxAbs = 0, kRange = 1, kNorm = 2 };
 
 template <int BITS, int DTYPE, int THREADS, bool SHUFFLE, int MODE = kMaxAbs>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS)
@@ -244,13 +243,13 @@ quantize_tma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
                 ok = range_quantize_tile<BITS, DTYPE, THREADS, false, SHUFFLE>(sh, wv, a, k, rot, tile, refill,
                                                                                 local_bucket, scale_writer);
         } else {
-            constexpr bool NORM = MODE == kNorm, GIVEN = MODE == kGiven;
+            constexpr bool NORM = MODE == kNorm;
             if (tile < c.full_tiles)
-                ok = quantize_tile<BITS, DTYPE, THREADS, true, SHUFFLE, NORM, GIVEN>(sh, wv, a, c, k, rot, tile, refill,
-                                                                                      local_bucket, scale_writer);
+                ok = quantize_tile<BITS, DTYPE, THREADS, true, SHUFFLE, NORM>(sh, wv, a, c, k, rot, tile, refill,
+                                                                               local_bucket, scale_writer);
             else
-                ok = quantize_tile<BITS, DTYPE, THREADS, false, SHUFFLE, NORM, GIVEN>(sh, wv, a, c, k, rot, tile, refill,
-                                                                                       local_bucket, scale_writer);
+                ok = quantize_tile<BITS, DTYPE, THREADS, false, SHUFFLE, NORM>(sh, wv, a, c, k, rot, tile, refill,
+                                                                                local_bucket, scale_writer);
         }
     }
     if (!ok) {
@@ -734,39 +733,12 @@ cudaError_t launch_quantize_norm_fused(const void* grad, uint64_t n, int bits, u
     return cudaErrorInvalidValue;
 }
 
-// ---- encode against a given scale on the TMA kernel: one long segment (= one bucket) per launch ----
-bool quantize_given_scale_applies(const void* grad, uint64_t n, const uint32_t* codes, uint64_t elem_offset,
-                                  uint64_t min_elems)
+// ---- encode against a given scale (mqg_segments_workers.cu): whole rows, block-aligned draws, bulk copies ----
+bool quantize_given_scale_applies(const void* grad, uint64_t n, const uint32_t* codes, uint64_t elem_offset)
 {
-    return n >= min_elems && n / 32 <= 0x7FFFFFFFull && (elem_offset & 7u) == 0 &&
+    return n >= 32 * 64 && n / 32 <= 0x7FFFFFFFull && (elem_offset & 7u) == 0 &&
            blocks_share_high_half(n, elem_offset) &&
            (reinterpret_cast<uintptr_t>(grad) & 15u) == 0 && (reinterpret_cast<uintptr_t>(codes) & 15u) == 0;
-}
-
-cudaError_t launch_quantize_given_scale(const void* grad, uint64_t n, int bits, uint64_t seed, uint32_t* codes,
-                                        float* scale, int dtype, uint32_t worker, uint32_t step,
-                                        uint64_t elem_offset, cudaStream_t stream)
-{
-    QuantizeArgs a;
-    fill_args(a, grad, n, bits, 128 * 32, seed, codes, scale, worker, step, elem_offset);   // tiles of 128 rows
-    a.nbuckets = 1;
-    TmaQuantizeConsts c;
-    if (fill_tma_args(a, c, 128) != 128) return cudaErrorInvalidValue;
-    unsigned int* timeouts = wait_timeout_counter();
-    if (timeouts == nullptr) return cudaErrorNotSupported;
-    CUtensorMap map;
-    const char* why = nullptr;
-    if (!encode_rows_map(&map, grad, a.nrows_full, dtype == 0 ? 4 : 2, 32, a.tile_rows, &why))
-        return cudaErrorNotSupported;
-#define MQG_GIVEN_CASE(B) \
-    case B: return dtype == 0 ? launch_tma_inst<B, 0, 128, false, kGiven>(map, a, c, timeouts, stream) \
-                              : launch_tma_inst<B, 1, 128, false, kGiven>(map, a, c, timeouts, stream)
-    switch (bits) {
-        MQG_GIVEN_CASE(1); MQG_GIVEN_CASE(2); MQG_GIVEN_CASE(3); MQG_GIVEN_CASE(4);
-        MQG_GIVEN_CASE(5); MQG_GIVEN_CASE(6); MQG_GIVEN_CASE(7); MQG_GIVEN_CASE(8);
-    }
-#undef MQG_GIVEN_CASE
-    return cudaErrorInvalidValue;
 }
 
 }  // namespace mqg

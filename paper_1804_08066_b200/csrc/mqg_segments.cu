@@ -1,183 +1,358 @@
-// Worker side with one scale per segment (per-layer scale) or with buckets larger than a CTA
-// tile: the max and the encode cannot share one pass over on-chip storage, so the gradient
-// is read twice -- a max pass that folds every tile's max (if it reaches the flush limit) into
-// scales[] with an atomic max on the float's bit pattern, then an encode pass identical to the
-// one-pass kernel's.
+// Worker side with one scale per segment (per-layer scale) or with buckets longer than the tiles of the
+// one-pass kernels.  Two ways:
+//   * span_kernel - a span is a segment or a bucket that fits one CTA's shared memory: the CTA stages all of it,
+//     finds the scale and encodes from there, so the gradient is read once and every span of every worker
+//     is one launch's work;
+//   * absmax_table_kernel, encode_table_kernel - longer ones: a max pass that folds every tile's maximum into
+//     scales[] with an atomic max on the float's bit pattern, then an encode pass.
+// Worker w of W is blockIdx.y in all of them; its results do not depend on W or on the way taken.
+#include <string.h>
+
+#include <atomic>
+#include <type_traits>
+
 #include "mqg_segments.cuh"
+#include "mqg_tma.cuh"
+#include "mqg_tree.cuh"
 
 namespace mqg {
 
+// The encode of one row: elements `left` (>= 1) long at flat position g0, words word0 .. of a stream that ends at
+// words_end.  VEC: the row's words start where store_row_words may use its widest access.
+template <int BITS, bool RANGE, typename Scale>
+__device__ __forceinline__ void encode_store_row(const float (&x)[32], const Scale& es, const TableArgs& a, uint32_t w,
+                                                 uint64_t g0, uint64_t left, uint64_t word0, uint64_t words_end, bool vec)
+{
+    uint32_t cw[BITS];
+    if constexpr (RANGE) {
+        range_encode_pack_row<BITS>(x, es, cw);
+    } else {
+        uint32_t h[16];
+        if ((g0 & 7u) == 0) {
+            const uint64_t blk = g0 >> 3;
+            draw_row_blocks((uint32_t)blk, (uint32_t)(blk >> 32), a.first_worker + w, a.rk, h);
+        } else {
+            const DrawKey key = {a.rk.k0[0], a.rk.k1[0], a.first_worker + w, a.rk.step};
+            draw_row_unaligned(g0, key, h);
+        }
+        encode_pack_row_packed<BITS>(x, es, h, cw);
+    }
+    if (vec && left >= 32) {
+        store_row_words<BITS>(a.codes[w], word0, cw);
+    } else {
+        if (left < 32) mask_row_words<BITS>(cw, (int)left * BITS);
+#pragma unroll
+        for (int k = 0; k < BITS; ++k)
+            if (word0 + k < words_end) a.codes[w][word0 + k] = cw[k];
+    }
+}
+
+// ---- spans ---------------------------------------------------------------------------------------
+// What bounds it: a short launch its latency (one staging copy, one reduction, one encode), a long one the
+// encode's instructions; CTAs on an SM are in different phases, which overlaps the copies with the encode.
+// Up to 512 rows: 256 threads (one or two rows each) and the registers of three CTAs per SM; longer spans: 512
+// threads, one CTA per SM.
+template <int BITS, int DTYPE, int MODE, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 3 : 1)
+span_kernel(const __grid_constant__ TableArgs a, const __grid_constant__ SpanTable tab)
+{
+    extern __shared__ uint8_t smem_raw[];
+    float4* tile = reinterpret_cast<float4*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
+    constexpr int kWarps = THREADS / 32;
+    __shared__ uint32_t s_a[kMaxSpanRows / 32], s_b[kWarps];   // kSpanNorm: a sum per 32 rows, else a word per warp
+    const uint32_t t = threadIdx.x, lane = t & 31u, wid = t >> 5, w = blockIdx.y;
+    grid_dependency_release();
+    grid_dependency_wait();
+
+    uint64_t elem0, len, code0, scale_idx;
+    if (tab.bucket != 0) {
+        scale_idx = blockIdx.x;
+        elem0 = scale_idx * tab.bucket;
+        len = tab.n - elem0 < tab.bucket ? tab.n - elem0 : tab.bucket;
+        code0 = elem0 / 32 * BITS;
+    } else {
+        if (blockIdx.x == 0 && t < (uint32_t)kMaxSegmentsPerLaunch && ((tab.clear[t >> 5] >> (t & 31u)) & 1u))
+            a.scales[w][tab.first + t] = 0.0f;
+        if (blockIdx.x >= (uint32_t)tab.nspan) return;
+        elem0 = tab.elem0[blockIdx.x];
+        len = tab.len[blockIdx.x];
+        code0 = tab.code0[blockIdx.x];
+        scale_idx = tab.scale_idx[blockIdx.x];
+    }
+    const int rows = (int)((len + 31) / 32);
+    if constexpr (DTYPE == 0) load_tile_f32<THREADS>(tile, static_cast<const float*>(a.grad[w]) + elem0, len, rows);
+    else load_tile_bf16<THREADS>(tile, static_cast<const uint16_t*>(a.grad[w]) + elem0, len, rows);
+    __syncthreads();
+
+    const int turns = (rows + THREADS - 1) / THREADS;
+    float x[32];
+    uint32_t lo = kOrderedMinIdentity, hi = MODE == kSpanRange ? kOrderedMaxIdentity : 0u;
+    for (int k = 0; k < turns; ++k) {
+        const int r = k * THREADS + (int)t;
+        const bool active = r < rows;
+        if (active) read_row(tile, r, x);                     // elements beyond the span were staged as zeros
+        if constexpr (MODE == kSpanNorm) {
+            const float s = warp_tree(active ? row_sum_squares(x) : 0.0f, 32);
+            if (lane == 0) s_a[k * kWarps + wid] = __float_as_uint(s);
+        } else if (active) {
+            if constexpr (MODE == kSpanRange) {
+                const uint64_t left = len - 32ull * r;        // the elements a ragged row lacks repeat its first one
+#pragma unroll
+                for (int j = 1; j < 32; ++j) x[j] = (uint64_t)j < left ? x[j] : x[0];
+                float l, h;
+                row_min_max(x, l, h);
+                lo = min(lo, ordered_bits(l));
+                hi = max(hi, ordered_bits(h));
+            } else {
+                hi = max(hi, __float_as_uint(row_abs_max(x)));
+            }
+        }
+    }
+    float scale = 0.0f;
+    RangeEncodeScale range = {0.0f, 0.0f};
+    if constexpr (MODE == kSpanNorm) {
+        __syncthreads();
+        // the tree over the sums of 32 rows: lane l on leaves 2l, 2l + 1 of 64, zeros beyond the last
+        const uint32_t n32 = (uint32_t)(turns * kWarps);
+        const float p = 2 * lane < n32 ? __uint_as_float(s_a[2 * lane]) : 0.0f;
+        const float q = 2 * lane + 1 < n32 ? __uint_as_float(s_a[2 * lane + 1]) : 0.0f;
+        const float S = warp_tree(__fadd_rn(p, q), 32);
+        scale = S < flush_limit() ? 0.0f : __fsqrt_rn(S);
+        if (t == 0) a.scales[w][scale_idx] = scale;
+    } else {
+        hi = __reduce_max_sync(0xFFFFFFFFu, hi);
+        if (MODE == kSpanRange) lo = __reduce_min_sync(0xFFFFFFFFu, lo);
+        if (lane == 0) { s_a[wid] = hi; s_b[wid] = lo; }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kWarps; ++i) { hi = max(hi, s_a[i]); lo = min(lo, s_b[i]); }
+        if constexpr (MODE == kSpanRange) {
+            // a zero of either sign is stored as +0
+            const float l = __fadd_rn(from_ordered_bits(lo), 0.0f), h = __fadd_rn(from_ordered_bits(hi), 0.0f);
+            if (t == 0) reinterpret_cast<float2*>(a.scales[w])[scale_idx] = make_float2(l, h);
+            range = range_encode_scale<BITS>(l, h);
+        } else {
+            scale = __uint_as_float(hi);
+            if (scale < flush_limit()) scale = 0.0f;
+            if (t == 0) a.scales[w][scale_idx] = scale;
+        }
+    }
+    const EncodeScale es = encode_scale<BITS>(scale);
+    const uint64_t words_end = code0 + (len * BITS + 31) / 32;
+    const bool vec = (reinterpret_cast<uintptr_t>(a.codes[w] + code0) & 15u) == 0;
+    for (int r = (int)t; r < rows; r += THREADS) {
+        read_row(tile, r, x);
+        const uint64_t g0 = a.elem_offset + elem0 + 32ull * r, left = len - 32ull * r, word0 = code0 + (uint64_t)r * BITS;
+        if constexpr (MODE == kSpanRange) encode_store_row<BITS, true>(x, range, a, w, g0, left, word0, words_end, vec);
+        else encode_store_row<BITS, false>(x, es, a, w, g0, left, word0, words_end, vec);
+    }
+}
+
+// ---- two passes over tiles of 256 rows ---------------------------------------------------------------
 template <int DTYPE>
 __global__ void __launch_bounds__(kMaxTileRows)
-absmax_segments_kernel(const SegQuantArgs a, const SegmentTable tab)
+absmax_table_kernel(const __grid_constant__ TableArgs a, const __grid_constant__ SegmentTable tab)
 {
-    __shared__ uint32_t s_warp[kMaxTileRows / 32];
+    constexpr int THREADS = kMaxTileRows;
+    __shared__ uint32_t s_warp[THREADS / 32];
     const TileGeom g = locate_tile<1>(tab, blockIdx.x);
     const uint64_t count = g.valid < (uint64_t)(kMaxTileRows * 32) ? g.valid : (uint64_t)(kMaxTileRows * 32);
-    float mx = 0.0f;
-    if constexpr (DTYPE == 0) {
-        const float* src = static_cast<const float*>(a.grad) + g.elem0;
-        if ((reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
-            const uint64_t n4 = count / 4;
-            for (uint64_t i = threadIdx.x; i < n4; i += kMaxTileRows) {
-                const float4 v = __ldg(reinterpret_cast<const float4*>(src) + i);
-                mx = fmaxf(fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
-            }
-            for (uint64_t i = n4 * 4 + threadIdx.x; i < count; i += kMaxTileRows)
-                mx = fmaxf(mx, fabsf(__ldg(src + i)));
-        } else {
-            for (uint64_t i = threadIdx.x; i < count; i += kMaxTileRows)
-                mx = fmaxf(mx, fabsf(__ldg(src + i)));
+    grid_dependency_release();
+    grid_dependency_wait();
+
+    using T = typename std::conditional<DTYPE == 0, float, uint16_t>::type;
+    const T* src = static_cast<const T*>(a.grad[blockIdx.y]) + g.elem0;
+    auto value = [&](uint64_t i) {
+        if constexpr (DTYPE == 0) return fabsf(__ldcg(src + i));
+        else return fabsf(bf16_lo(__ldcg(src + i)));
+    };
+    // 16-byte accesses from the tile's first 16-byte boundary on
+    constexpr uint64_t kPer = 16 / sizeof(T);
+    const uint64_t to_align = (kPer - (reinterpret_cast<uintptr_t>(src) / sizeof(T)) % kPer) % kPer;
+    const uint64_t head = to_align < count ? to_align : count, nvec = (count - head) / kPer;
+    const uint4* v4 = reinterpret_cast<const uint4*>(src + head);
+    float m = 0.0f;
+    auto take = [&](const uint4& v) {
+        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int k = 0; k < 4; k += DTYPE == 0 ? 2 : 1) {
+            if constexpr (DTYPE == 0) m = max3_abs(m, __uint_as_float(u[k]), __uint_as_float(u[k + 1]));
+            else m = max3_abs(m, bf16_lo(u[k]), bf16_hi(u[k]));
         }
+    };
+    constexpr int kFull = kMaxTileRows * 32 / kPer / THREADS;          // accesses per thread of a whole tile
+    if (nvec == (uint64_t)kFull * THREADS) {
+        uint4 v[kFull];
+#pragma unroll
+        for (int k = 0; k < kFull; ++k) v[k] = __ldcg(v4 + k * THREADS + threadIdx.x);
+#pragma unroll
+        for (int k = 0; k < kFull; ++k) take(v[k]);
     } else {
-        const uint16_t* src = static_cast<const uint16_t*>(a.grad) + g.elem0;
-        if ((reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
-            const uint64_t n8 = count / 8;
-            for (uint64_t i = threadIdx.x; i < n8; i += kMaxTileRows) {
-                const uint4 v = __ldg(reinterpret_cast<const uint4*>(src) + i);
-                const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    mx = fmaxf(mx, fmaxf(fabsf(bf16_lo(u[k])), fabsf(bf16_hi(u[k]))));
-            }
-            for (uint64_t i = n8 * 8 + threadIdx.x; i < count; i += kMaxTileRows)
-                mx = fmaxf(mx, fabsf(bf16_lo(__ldg(src + i))));
-        } else {
-            for (uint64_t i = threadIdx.x; i < count; i += kMaxTileRows)
-                mx = fmaxf(mx, fabsf(bf16_lo(__ldg(src + i))));
-        }
+        if (threadIdx.x < head) m = value(threadIdx.x);
+#pragma unroll 4
+        for (uint64_t i = threadIdx.x; i < nvec; i += THREADS) take(__ldcg(v4 + i));
+        const uint64_t tail = head + nvec * kPer + threadIdx.x;
+        if (tail < count) m = fmaxf(m, value(tail));
     }
-    uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(mx));
-    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = m;
+    uint32_t r = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(m));
+    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = r;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        m = threadIdx.x < kMaxTileRows / 32 ? s_warp[threadIdx.x] : 0u;
-        m = __reduce_max_sync(0xFFFFFFFFu, m);
-        // a tile's maximum below the flush limit does not count: a segment whose every tile stays below
-        // it keeps the scale 0 the pass started from, so the scale that stands after the pass is final
-        if (threadIdx.x == 0 && m >= __float_as_uint(flush_limit()))
-            atomicMax(reinterpret_cast<unsigned int*>(a.scales) + g.seg, m);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int i = 1; i < THREADS / 32; ++i) r = max(r, s_warp[i]);
+        // a tile's maximum below the flush limit does not count: a segment whose every tile stays below it
+        // keeps the scale 0 the pass started from, so the scale that stands after the pass is final
+        if (r >= __float_as_uint(flush_limit()))
+            atomicMax(reinterpret_cast<unsigned int*>(a.scales[blockIdx.y]) + g.seg, r);
     }
 }
 
+// A 256-row tile of the table is two CTAs' work.
+constexpr int kEncodeThreads = 128;
 template <int BITS, int DTYPE>
-__global__ void __launch_bounds__(kMaxTileRows)
-encode_segments_kernel(const SegQuantArgs a, const SegmentTable tab)
+__global__ void __launch_bounds__(kEncodeThreads)
+encode_table_kernel(const __grid_constant__ TableArgs a, const __grid_constant__ SegmentTable tab)
 {
-    __shared__ __align__(1024) float4 tile[kMaxTileRows * 8];
-    const uint32_t t = threadIdx.x;
-    const TileGeom g = locate_tile<BITS>(tab, blockIdx.x);
-
-    if constexpr (DTYPE == 0)
-        load_tile_f32<kMaxTileRows>(tile, static_cast<const float*>(a.grad) + g.elem0, g.valid, g.rows);
-    else
-        load_tile_bf16<kMaxTileRows>(tile, static_cast<const uint16_t*>(a.grad) + g.elem0, g.valid, g.rows);
-
-    const float s = a.scales[g.seg];        // final: the max pass has applied the flush
+    __shared__ __align__(1024) float4 tile[kEncodeThreads * 8];
+    const TileGeom g = locate_tile<BITS>(tab, blockIdx.x >> 1);
+    const int r0 = (int)(blockIdx.x & 1u) * kEncodeThreads, t = (int)threadIdx.x;
+    const uint32_t w = blockIdx.y;
+    grid_dependency_release();
+    grid_dependency_wait();
+    if (r0 >= g.rows) return;
+    const uint64_t elem0 = g.elem0 + 32ull * r0, valid = g.valid - 32ull * r0;
+    const int rows = min(kEncodeThreads, g.rows - r0);
+    if constexpr (DTYPE == 0) load_tile_f32<kEncodeThreads>(tile, static_cast<const float*>(a.grad[w]) + elem0, valid, rows);
+    else load_tile_bf16<kEncodeThreads>(tile, static_cast<const uint16_t*>(a.grad[w]) + elem0, valid, rows);
+    const EncodeScale es = encode_scale<BITS>(__ldcg(a.scales[w] + g.seg));   // final: the max pass applied the flush
     __syncthreads();
-    if (t >= (uint32_t)g.rows) return;
-
+    if (t >= rows) return;
     float x[32];
-    read_row(tile, (int)t, x);
-    const EncodeScale es = encode_scale<BITS>(s);
-    const uint64_t g0 = a.elem_offset + g.elem0 + 32ull * t;
-    uint32_t h[16];
-    if ((g0 & 7u) == 0) draw_row_aligned(g0, make_round_keys(a.key), h);
-    else draw_row_unaligned(g0, a.key, h);
-
-    uint32_t w[BITS];
-    encode_pack_row<BITS>(x, es, h, w);
-
-    const uint64_t word0 = g.word0 + (uint64_t)t * BITS;
-    const uint64_t left = g.valid - 32ull * t;          // elements of the segment from this row on
-    if (left < 32) mask_row_words<BITS>(w, (int)left * BITS);
-#pragma unroll
-    for (int k = 0; k < BITS; ++k)
-        if (word0 + k < g.words_end) a.codes[word0 + k] = w[k];
+    read_row(tile, t, x);
+    const uint64_t word0 = g.word0 + (uint64_t)(r0 + t) * BITS;
+    const bool vec = (reinterpret_cast<uintptr_t>(a.codes[w] + g.word0) & 15u) == 0;
+    encode_store_row<BITS, false>(x, es, a, w, a.elem_offset + elem0 + 32ull * t, valid - 32ull * t, word0, g.words_end, vec);
 }
 
-template <int BITS>
-static cudaError_t launch_encode_bits(const SegQuantArgs& a, const SegmentTable& tab, int dtype,
-                                      unsigned grid, cudaStream_t stream)
+// ---- host side -------------------------------------------------------------------------------------
+TableArgs make_table_args(const void* const* grads, int W, uint32_t* const* codes, float* const* scales, uint64_t seed,
+                          uint32_t first_worker, uint32_t step, uint64_t elem_offset)
 {
-    if (dtype == 0) encode_segments_kernel<BITS, 0><<<grid, kMaxTileRows, 0, stream>>>(a, tab);
-    else encode_segments_kernel<BITS, 1><<<grid, kMaxTileRows, 0, stream>>>(a, tab);
-    return cudaGetLastError();
+    TableArgs a;
+    memset(&a, 0, sizeof(a));
+    for (int w = 0; w < W; ++w) { a.grad[w] = grads[w]; a.codes[w] = codes[w]; a.scales[w] = scales[w]; }
+    a.elem_offset = elem_offset;
+    a.first_worker = first_worker;
+    a.W = W;
+    uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+    for (int r = 0; r < 10; ++r) {
+        a.rk.k0[r] = k0; a.rk.k1[r] = k1;
+        k0 += 0x9E3779B9u; k1 += 0xBB67AE85u;
+    }
+    a.rk.worker = first_worker; a.rk.step = step;
+    return a;
 }
 
-cudaError_t launch_encode_segments(const SegQuantArgs& a, const SegmentTable& tab, int bits, int dtype,
-                                   unsigned grid, cudaStream_t stream)
+template <int BITS, int DTYPE, int MODE, int THREADS>
+static cudaError_t launch_span_inst(const TableArgs& a, const SpanTable& tab, unsigned nspan, uint64_t most,
+                                    cudaStream_t stream)
 {
+    auto kernel = span_kernel<BITS, DTYPE, MODE, THREADS>;
+    const size_t smem = (size_t)((most + 31) / 32) * 128 + 1024;       // + slack to round the base up
+    static std::atomic<bool> ready[64];                                // per device (zero-initialised)
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return err;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!ready[dev].load(std::memory_order_relaxed)) {
+        constexpr int kMost = (THREADS == 256 ? 512 : kMaxSpanRows) * 128 + 1024;
+        err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+        if (err != cudaSuccess) return err;
+        ready[dev].store(true, std::memory_order_relaxed);
+    }
+    return launch_pdl_grid(kernel, dim3(nspan, (unsigned)a.W), THREADS, smem, stream, a, tab);
+}
+
+template <int MODE>
+static cudaError_t launch_span_mode(const TableArgs& a, const SpanTable& tab, unsigned nspan, uint64_t most, int bits,
+                                    int dtype, cudaStream_t stream)
+{
+    const bool wide = most > 512 * 32;
     switch (bits) {
-        case 1: return launch_encode_bits<1>(a, tab, dtype, grid, stream);
-        case 2: return launch_encode_bits<2>(a, tab, dtype, grid, stream);
-        case 3: return launch_encode_bits<3>(a, tab, dtype, grid, stream);
-        case 4: return launch_encode_bits<4>(a, tab, dtype, grid, stream);
-        case 5: return launch_encode_bits<5>(a, tab, dtype, grid, stream);
-        case 6: return launch_encode_bits<6>(a, tab, dtype, grid, stream);
-        case 7: return launch_encode_bits<7>(a, tab, dtype, grid, stream);
-        case 8: return launch_encode_bits<8>(a, tab, dtype, grid, stream);
+#define MQG_SPAN_CASE(B) \
+        case B: return dtype == 0 ? (wide ? launch_span_inst<B, 0, MODE, 512>(a, tab, nspan, most, stream)  \
+                                          : launch_span_inst<B, 0, MODE, 256>(a, tab, nspan, most, stream)) \
+                                  : (wide ? launch_span_inst<B, 1, MODE, 512>(a, tab, nspan, most, stream)  \
+                                          : launch_span_inst<B, 1, MODE, 256>(a, tab, nspan, most, stream))
+        MQG_SPAN_CASE(1); MQG_SPAN_CASE(2); MQG_SPAN_CASE(3); MQG_SPAN_CASE(4);
+        MQG_SPAN_CASE(5); MQG_SPAN_CASE(6); MQG_SPAN_CASE(7); MQG_SPAN_CASE(8);
+#undef MQG_SPAN_CASE
     }
     return cudaErrorInvalidValue;
 }
 
-static cudaError_t two_pass(const SegQuantArgs& a, const SegmentTable& tab, uint64_t ntiles,
-                            uint64_t nscales, int bits, int dtype, cudaStream_t stream)
+cudaError_t launch_spans(const TableArgs& a, const SpanTable& tab, unsigned nspan, uint64_t most, int mode, int bits,
+                         int dtype, cudaStream_t stream)
 {
-    cudaError_t err = cudaMemsetAsync(a.scales, 0, nscales * sizeof(float), stream);
-    if (err != cudaSuccess) return err;
-    if (ntiles == 0) return cudaSuccess;
-    if (ntiles > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    const unsigned grid = (unsigned)ntiles;
-    if (dtype == 0) absmax_segments_kernel<0><<<grid, kMaxTileRows, 0, stream>>>(a, tab);
-    else absmax_segments_kernel<1><<<grid, kMaxTileRows, 0, stream>>>(a, tab);
-    err = cudaGetLastError();
-    if (err != cudaSuccess) return err;
-    return launch_encode_segments(a, tab, bits, dtype, grid, stream);
+    if (most > (uint64_t)kMaxSpanRows * 32) return cudaErrorInvalidValue;
+    if (mode == kSpanRange) return launch_span_mode<kSpanRange>(a, tab, nspan, most, bits, dtype, stream);
+    if (mode == kSpanNorm) return launch_span_mode<kSpanNorm>(a, tab, nspan, most, bits, dtype, stream);
+    return launch_span_mode<kSpanMaxAbs>(a, tab, nspan, most, bits, dtype, stream);
 }
 
-// The two passes of the per-layer quantizer as separate launches (the caller may give some segments'
-// encode to another kernel): the max pass over every segment of `tab`, and the encode pass over the
-// tiles `tab` lists.
-cudaError_t launch_segments_absmax(const void* grad, const SegmentTable& tab, float* scales_base, int dtype,
-                                   cudaStream_t stream)
+bool bucket_spans_apply(uint64_t n, uint64_t bucket)
 {
-    SegQuantArgs a;
-    a.grad = grad; a.codes = nullptr; a.scales = scales_base; a.elem_offset = 0;
-    a.key.seed_lo = a.key.seed_hi = a.key.worker = a.key.step = 0;
-    cudaError_t err = cudaMemsetAsync(scales_base, 0, (size_t)tab.nseg * sizeof(float), stream);
-    if (err != cudaSuccess) return err;
-    const uint32_t ntiles = tab.tile_start[tab.nseg];
-    if (ntiles == 0) return cudaSuccess;
-    if (dtype == 0) absmax_segments_kernel<0><<<ntiles, kMaxTileRows, 0, stream>>>(a, tab);
-    else absmax_segments_kernel<1><<<ntiles, kMaxTileRows, 0, stream>>>(a, tab);
-    return cudaGetLastError();
+    const uint64_t b = bucket < n ? bucket : n;
+    return b <= (uint64_t)kMaxSpanRows * 32 && (n + b - 1) / b <= 0x7FFFFFFFull;
 }
 
-cudaError_t launch_segments_encode(const void* grad, const SegmentTable& tab, int bits, uint64_t seed,
-                                   uint32_t* codes, float* scales_base, int dtype, uint32_t worker,
-                                   uint32_t step, uint64_t elem_offset, cudaStream_t stream)
+cudaError_t launch_bucket_spans(const void* const* grads, int W, uint64_t n, int bits, uint64_t bucket, uint64_t seed,
+                                uint32_t* const* codes, float* const* scales, int mode, int dtype, uint32_t first_worker,
+                                uint32_t step, uint64_t elem_offset, cudaStream_t stream)
 {
-    SegQuantArgs a;
-    a.grad = grad; a.codes = codes; a.scales = scales_base; a.elem_offset = elem_offset;
-    a.key.seed_lo = (uint32_t)seed; a.key.seed_hi = (uint32_t)(seed >> 32);
-    a.key.worker = worker; a.key.step = step;
-    const uint32_t ntiles = tab.tile_start[tab.nseg];
-    if (ntiles == 0) return cudaSuccess;
-    return launch_encode_segments(a, tab, bits, dtype, ntiles, stream);
+    const TableArgs a = make_table_args(grads, W, codes, scales, seed, first_worker, step, elem_offset);
+    SpanTable tab;
+    tab.bucket = bucket < n ? bucket : n;
+    tab.n = n;
+    tab.nspan = 0;
+    return launch_spans(a, tab, (unsigned)((n + tab.bucket - 1) / tab.bucket), tab.bucket, mode, bits, dtype, stream);
 }
 
+cudaError_t launch_absmax_table(const TableArgs& a, const SegmentTable& tab, int dtype, cudaStream_t stream)
+{
+    const uint32_t tiles = tab_tiles(tab);
+    if (tiles == 0) return cudaSuccess;
+    const dim3 grid(tiles, (unsigned)a.W);
+    return dtype == 0 ? launch_pdl_grid(absmax_table_kernel<0>, grid, kMaxTileRows, 0, stream, a, tab)
+                      : launch_pdl_grid(absmax_table_kernel<1>, grid, kMaxTileRows, 0, stream, a, tab);
+}
+
+cudaError_t launch_encode_table(const TableArgs& a, const SegmentTable& tab, int bits, int dtype, cudaStream_t stream)
+{
+    const uint32_t tiles = tab_tiles(tab);
+    if (tiles == 0) return cudaSuccess;
+    if (tiles > 0x3FFFFFFFu) return cudaErrorInvalidValue;
+    const dim3 grid(2 * tiles, (unsigned)a.W);
+    switch (bits) {
+#define MQG_TAB_CASE(B) \
+        case B: return dtype == 0 ? launch_pdl_grid(encode_table_kernel<B, 0>, grid, kEncodeThreads, 0, stream, a, tab) \
+                                  : launch_pdl_grid(encode_table_kernel<B, 1>, grid, kEncodeThreads, 0, stream, a, tab)
+        MQG_TAB_CASE(1); MQG_TAB_CASE(2); MQG_TAB_CASE(3); MQG_TAB_CASE(4);
+        MQG_TAB_CASE(5); MQG_TAB_CASE(6); MQG_TAB_CASE(7); MQG_TAB_CASE(8);
+#undef MQG_TAB_CASE
+    }
+    return cudaErrorInvalidValue;
+}
+
+// Buckets longer than a span: two passes per worker.
 cudaError_t launch_quantize_big_buckets(const void* grad, uint64_t n, int bits, uint64_t bucket,
                                         uint64_t seed, uint32_t* codes, float* scales, int dtype,
                                         uint32_t worker, uint32_t step, uint64_t elem_offset,
                                         cudaStream_t stream)
 {
-    SegQuantArgs a;
-    a.grad = grad; a.codes = codes; a.scales = scales; a.elem_offset = elem_offset;
-    a.key.seed_lo = (uint32_t)seed; a.key.seed_hi = (uint32_t)(seed >> 32);
-    a.key.worker = worker; a.key.step = step;
+    const TableArgs a = make_table_args(&grad, 1, &codes, &scales, seed, worker, step, elem_offset);
     SegmentTable tab;
-    tab.nseg = 0;
+    memset(&tab, 0, sizeof(tab));
     const uint64_t b = bucket < n ? bucket : n;          // a single bucket is n long
     tab.uniform_bucket = b;
     tab.n_total = n;
@@ -188,10 +363,15 @@ cudaError_t launch_quantize_big_buckets(const void* grad, uint64_t n, int bits, 
     const uint64_t nb = (n + b - 1) / b;
     const uint64_t full = n / b;                          // full buckets have tpb tiles each
     uint64_t ntiles = full * tpb;
-    if (nb > full) ntiles += ((n - full * b) + tile_elems - 1) / tile_elems;
     // the grid enumerates tiles_per_bucket tiles for every bucket; the last (shorter) bucket
     // has fewer real tiles, so its tail tiles are simply not launched
-    return two_pass(a, tab, ntiles, nb, bits, dtype, stream);
+    if (nb > full) ntiles += ((n - full * b) + tile_elems - 1) / tile_elems;
+    if (ntiles > 0x3FFFFFFFull) return cudaErrorInvalidValue;
+    tab.tile_start[0] = (uint32_t)ntiles;                 // nseg = 0: the grid's tiles
+    cudaError_t err = cudaMemsetAsync(scales, 0, nb * sizeof(float), stream);
+    if (err == cudaSuccess) err = launch_absmax_table(a, tab, dtype, stream);
+    if (err == cudaSuccess) err = launch_encode_table(a, tab, bits, dtype, stream);
+    return err;
 }
 
 }  // namespace mqg

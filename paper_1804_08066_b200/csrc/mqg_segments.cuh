@@ -7,18 +7,38 @@
 
 namespace mqg {
 
-struct SegQuantArgs {
-    const void* grad;
-    uint32_t* codes;
-    float* scales;          // scale of segment j at scales[j]
+// The gradients of the workers that share a table, and the keys of their draws.
+struct TableArgs {
+    const void* grad[kMaxWorkers];
+    uint32_t* codes[kMaxWorkers];
+    float* scales[kMaxWorkers];     // scale of the table's segment j at scales[w][j]
     uint64_t elem_offset;
-    DrawKey key;
+    uint32_t first_worker;
+    int W;
+    RoundKeys rk;
 };
+TableArgs make_table_args(const void* const* grads, int W, uint32_t* const* codes, float* const* scales, uint64_t seed,
+                          uint32_t first_worker, uint32_t step, uint64_t elem_offset);
 
-// The encode pass of the segment quantizers: one CTA per tile, scale of the tile's segment read
-// from a.scales (already final, or the raw maximum that the first tile then flushes).
-cudaError_t launch_encode_segments(const SegQuantArgs& a, const SegmentTable& tab, int bits, int dtype,
-                                   unsigned grid, cudaStream_t stream);
+// The two passes over the tiles a table lists, for every worker (scales zeroed before the first).
+inline uint32_t tab_tiles(const SegmentTable& tab) { return tab.tile_start[tab.nseg]; }
+cudaError_t launch_absmax_table(const TableArgs& a, const SegmentTable& tab, int dtype, cudaStream_t stream);
+cudaError_t launch_encode_table(const TableArgs& a, const SegmentTable& tab, int bits, int dtype, cudaStream_t stream);
+
+// Spans: what one CTA quantizes as a whole.  bucket != 0: span j is bucket j of a gradient of n elements;
+// otherwise the lists, and the launch also clears the scales first + i for which bit i of clear[] is set.
+constexpr int kMaxSpanRows = 1536;      // 192 KB of shared memory
+enum : int { kSpanMaxAbs = 0, kSpanRange = 1, kSpanNorm = 2 };
+struct SpanTable {
+    uint64_t bucket, n;
+    int nspan, first;
+    uint32_t clear[kMaxSegmentsPerLaunch / 32];
+    uint32_t scale_idx[kMaxSegmentsPerLaunch];
+    uint64_t elem0[kMaxSegmentsPerLaunch], len[kMaxSegmentsPerLaunch], code0[kMaxSegmentsPerLaunch];
+};
+// `nspan` CTAs per worker; `most` = elements of the longest span.
+cudaError_t launch_spans(const TableArgs& a, const SpanTable& tab, unsigned nspan, uint64_t most, int mode, int bits,
+                         int dtype, cudaStream_t stream);
 
 struct TileGeom {
     uint64_t elem0;       // flat index of the tile's first element

@@ -148,6 +148,24 @@ cudaError_t launch_pdl_smem(void (*kernel)(KArgs...), unsigned grid, unsigned bl
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// The same with a grid of more than one dimension.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_grid(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t dynamic_smem,
+                            cudaStream_t stream, Args&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = dynamic_smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // Ordinary stream-ordered launch with dynamic shared memory.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_with_smem(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t dynamic_smem,
