@@ -28,38 +28,59 @@ __device__ __forceinline__ float tree8(const float* v, uint32_t first, uint32_t 
                      __fadd_rn(__fadd_rn(x[4], x[5]), __fadd_rn(x[6], x[7])));
 }
 
-// The bucket's sum from the per-row values of a 256-thread tile that holds whole buckets of `rpb` rows
-// (thread t owns row t of the tile; threads without a row pass 0).  Every thread of the CTA must
-// call it.  s_part: kMaxTileRows floats of shared memory, free for reuse after the call's last
+// The buckets' sums of N values per row, from the per-row values of a tile of THREADS (at most 256) rows that
+// holds whole buckets of `rpb` rows (thread t owns row t of the tile; threads without a row pass 0).  Every
+// thread of the CTA must call it.  s_part: N * THREADS floats of shared memory, free for reuse after the next
 // barrier only.
-__device__ __forceinline__ float bucket_tree_sum(float a, uint32_t rpb, float* s_part)
+template <int THREADS, int N>
+__device__ __forceinline__ void bucket_tree_sums(float (&a)[N], uint32_t rpb, float* s_part)
 {
     const uint32_t t = threadIdx.x;
-    if ((rpb & (rpb - 1)) == 0 && rpb <= 32) return warp_tree(a, rpb);
+    if ((rpb & (rpb - 1)) == 0 && rpb <= 32) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) a[i] = warp_tree(a[i], rpb);
+        return;
+    }
     if (rpb % 32 == 0) {
-        a = warp_tree(a, 32);
-        if ((t & 31) == 0) s_part[t >> 5] = a;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            a[i] = warp_tree(a[i], 32);
+            if ((t & 31) == 0) s_part[i * THREADS + (t >> 5)] = a[i];
+        }
         __syncthreads();
         const uint32_t wpb = rpb / 32;
         const uint32_t first = (t / rpb) * wpb;
-        return first + wpb <= kMaxTileRows / 32 ? tree8(s_part, first, wpb) : 0.0f;
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            a[i] = first + wpb <= THREADS / 32 ? tree8(s_part + i * THREADS, first, wpb) : 0.0f;
+        return;
     }
-    // any other shape: one tree level per barrier pair, in place
-    s_part[t] = a;
+    // any other shape: a bucket's tree is a warp's work, lane l on rows 8l .. 8l + 7 of it, zeros beyond
+#pragma unroll
+    for (int i = 0; i < N; ++i) s_part[i * THREADS + t] = a[i];
     __syncthreads();
-    const uint32_t b0 = (t / rpb) * rpb, j = t - b0;
-    for (uint32_t d = 1; d < rpb; d <<= 1) {
-        const bool node = (j & (2 * d - 1)) == 0;
-        float v = 0.0f;
-        if (node) {
-            v = s_part[t];
-            if (j + d < rpb && t + d < (uint32_t)kMaxTileRows) v = __fadd_rn(v, s_part[t + d]);
+    const uint32_t lane = t & 31u, buckets = THREADS / rpb;
+    for (uint32_t b = t >> 5; b < buckets; b += THREADS / 32) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            float* p = s_part + i * THREADS + b * rpb;
+            const uint32_t left = 8 * lane < rpb ? min(8u, rpb - 8 * lane) : 0u;
+            const float s = warp_tree(tree8(p, 8 * lane, left), 32);
+            __syncwarp();                          // every lane has read the bucket's values
+            if (lane == 0) p[0] = s;
         }
-        __syncthreads();
-        if (node) s_part[t] = v;
-        __syncthreads();
     }
-    return b0 < (uint32_t)kMaxTileRows ? s_part[b0] : 0.0f;
+    __syncthreads();
+    const uint32_t mine = t / rpb;
+#pragma unroll
+    for (int i = 0; i < N; ++i) a[i] = mine < buckets ? s_part[i * THREADS + mine * rpb] : 0.0f;
+}
+
+__device__ __forceinline__ float bucket_tree_sum(float a, uint32_t rpb, float* s_part)
+{
+    float v[1] = {a};
+    bucket_tree_sums<kMaxTileRows, 1>(v, rpb, s_part);
+    return v[0];
 }
 
 }  // namespace mqg
