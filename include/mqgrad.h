@@ -90,8 +90,9 @@ mqg_status mqg_quantize(const void* grad, uint64_t n, int bits, uint64_t bucket,
  *   grads, codes, scales  HOST arrays of W device pointers (read during the call only); each
  *                         buffer as in mqg_quantize; the outputs are what mqg_server_step and
  *                         mqg_dequant_accumulate take as codes[] / scales[]
- * Shapes outside the one-launch kernel (buckets above 4096 elements, fewer than 2048 elements,
- * elem_offset not a multiple of 8, W = 1) run as W launches inside the call.
+ * Shapes outside the one-launch kernels (fewer than 2048 elements, elem_offset not a multiple of 8, buckets
+ * of 129 .. 255 rows of 32 that are not whole multiples of 32 rows, buckets above 49152 elements) run as W
+ * launches inside the call.
  * Errors: as mqg_quantize, per worker; MQG_ERR_TOO_MANY_WORKERS for W outside 1..MQG_MAX_WORKERS.
  */
 mqg_status mqg_quantize_workers(const void* const* grads, int W, uint64_t n, int bits, uint64_t bucket,
@@ -153,7 +154,7 @@ mqg_status mqg_server_requantize(const uint32_t* const* codes, const float* cons
  *   ranges  [out] 2 * mqg_num_buckets(n, bucket) floats, 8-byte aligned: ranges[2b] = lo,
  *                 ranges[2b + 1] = hi of bucket b
  *   codes   [out] as mqg_quantize
- * Buckets of at most 4096 elements take one pass over the gradient; larger ones two.
+ * Buckets of at most 49152 elements take one pass over the gradient; larger ones two.
  * Errors as mqg_quantize; MQG_ERR_ALIGN for a ranges pointer that is not 8-byte aligned.
  */
 mqg_status mqg_quantize_minmax(const void* grad, uint64_t n, int bits, uint64_t bucket, uint32_t* codes,
@@ -299,11 +300,11 @@ mqg_status mqg_quantize_segments_l2_static(const void* grad, int nseg, const uin
  *   codes     [out] code_off[nseg] words;  scales [out] nseg floats
  * Element i of segment j draws with position elem_offset + seg_off[j] + i.  Empty segments get
  * scale 0.  The gradient is read twice (max pass, encode pass).
- * Performance note: a segment of 2^20 elements or more (2^15 or more in mqg_quantize_segments_workers
- * and mqg_server_step_segments, where such segments share a launch) is encoded (and, in
- * mqg_server_step_segments, applied) by the bulk-copy kernels when grad + seg_off[j], codes + code_off[j] (every worker's, on
- * the server) and params + seg_off[j] are 16-byte aligned and elem_offset + seg_off[j] is a multiple
- * of 8; otherwise by the table-driven kernels.  The results do not depend on which kernel ran.
+ * Performance note: a segment of at most 16384 elements is read once, a longer one twice; the longer ones are
+ * encoded by the bulk-copy kernel when grad + seg_off[j] is 16-byte aligned and elem_offset + seg_off[j] is a
+ * multiple of 8 (and, from 2^15 elements on, applied by mqg_server_step_segments' bulk-copy kernel when
+ * params + seg_off[j] and every worker's codes + code_off[j] are 16-byte aligned); otherwise by the table-driven
+ * kernels.  The results do not depend on which kernel ran.
  */
 mqg_status mqg_quantize_segments(const void* grad, int nseg, const uint64_t* seg_off,
                                  const uint64_t* code_off, int bits, uint64_t seed,
@@ -311,8 +312,8 @@ mqg_status mqg_quantize_segments(const void* grad, int nseg, const uint64_t* seg
                                  uint32_t step, uint64_t elem_offset, void* cuda_stream);
 
 /*
- * mqg_quantize_segments for W workers' gradients that share one segment table, in three launches for
- * all of them (zero the scales, max pass, encode pass) instead of five per worker - the per-layer
+ * mqg_quantize_segments for W workers' gradients that share one segment table, in up to three launches for
+ * all of them (short segments whole, max pass and encode pass of the longer ones) - the per-layer
  * counterpart of mqg_quantize_workers, for a host that plays several workers on one device (all
  * workers run Quantize(g, K) with the same K in an iteration; Algorithm 1, WorkerIterate line 3).
  *   grads/codes/scales [in] HOST arrays of W device pointers; worker w draws with worker id

@@ -80,8 +80,8 @@ cudaError_t launch_segments_l2_scales(const void* grad, const SegmentTable& tab,
 cudaError_t launch_quantize_onebit_ef(const void* grad, float* residual, uint64_t n, uint64_t bucket,
                                       uint32_t* codes, float* ranges, int dtype, cudaStream_t stream);
 
-// Whether a segment's buffers are aligned for the bulk-copy encode of the per-layer quantizer.
-bool quantize_given_scale_applies(const void* grad, uint64_t n, const uint32_t* codes, uint64_t elem_offset);
+// Whether a segment starts where the bulk-copy encode of the per-layer quantizer can.
+bool quantize_given_scale_applies(const void* grad, uint64_t n, uint64_t elem_offset);
 
 // Per-layer quantization of W >= 1 workers that share a (checked) segment table: mqg_segments_workers.cu.
 // workspace != nullptr: L2-norm scales (one worker), the partial sums of its long segments go there.

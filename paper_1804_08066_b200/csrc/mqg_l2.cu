@@ -36,7 +36,7 @@ struct L2Args {
 // norm and the encode share one pass over the gradient.
 template <int BITS, int DTYPE>
 __global__ void __launch_bounds__(kMaxTileRows)
-l2_quantize_kernel(const L2Args a)
+l2_quantize_kernel(const __grid_constant__ L2Args a)
 {
     __shared__ __align__(1024) float4 tile[kMaxTileRows * 8];
     __shared__ float s_part[kMaxTileRows];
@@ -46,6 +46,8 @@ l2_quantize_kernel(const L2Args a)
     const uint64_t rows_left = a.nrows - row0;
     const int rows = (int)(rows_left < a.tile_rows ? rows_left : a.tile_rows);
 
+    grid_dependency_release();
+    grid_dependency_wait();
     if constexpr (DTYPE == 0)
         load_tile_f32<kMaxTileRows>(tile, static_cast<const float*>(a.grad) + row0 * 32,
                                     a.n - row0 * 32, rows);
@@ -159,9 +161,8 @@ l2_finish_kernel(const __grid_constant__ SegmentTable tab, float* __restrict__ p
 template <int BITS>
 cudaError_t launch_l2_bits(const L2Args& a, int dtype, unsigned grid, cudaStream_t stream)
 {
-    if (dtype == 0) l2_quantize_kernel<BITS, 0><<<grid, kMaxTileRows, 0, stream>>>(a);
-    else l2_quantize_kernel<BITS, 1><<<grid, kMaxTileRows, 0, stream>>>(a);
-    return cudaGetLastError();
+    return dtype == 0 ? launch_pdl(l2_quantize_kernel<BITS, 0>, grid, kMaxTileRows, stream, a)
+                      : launch_pdl(l2_quantize_kernel<BITS, 1>, grid, kMaxTileRows, stream, a);
 }
 
 }  // namespace

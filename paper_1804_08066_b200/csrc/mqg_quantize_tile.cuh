@@ -75,6 +75,12 @@ __device__ __noinline__ void stage_ragged_row(uint8_t* stage, int row, const voi
     }
 }
 
+// How the rows of a bucket are reduced: a bucket is an aligned power-of-two group of at most 32 rows (lane
+// shuffles), a whole number of warps (one shared-memory atomic per warp), or any other number of rows (one
+// shared-memory atomic per row; at least three rows, so at most 42 buckets per tile of 128).
+enum : int { kByShuffle = 0, kByWarps = 1, kByRows = 2 };
+constexpr int kSlots = 44;
+
 template <int DTYPE, int THREADS>
 struct TmaQuantizeShared {
     static constexpr int kRowBytes = DTYPE == 0 ? 128 : 64;
@@ -82,8 +88,9 @@ struct TmaQuantizeShared {
     // of a single stage still hides behind the tile's arithmetic)
     static constexpr int kStages = 2 * THREADS * kRowBytes <= 32768 ? 2 : 1;
     alignas(1024) uint8_t stage[kStages][THREADS * kRowBytes];
-    uint32_t slots[3][THREADS / 32];       // bucket maxima, rotating so no reset races a use
-    uint32_t slots_lo[3][THREADS / 32];    // bucket minima of the (min, max) variant, as ordered bits
+    uint32_t slots[3][kSlots];             // bucket maxima, rotating so no reset races a use
+    uint32_t slots_lo[3][kSlots];          // bucket minima of the (min, max) variant, as ordered bits
+    float row_sums[THREADS];               // L2 norm, reduction by rows
     alignas(8) uint64_t bar[kStages];
 };
 
@@ -107,17 +114,16 @@ struct WorkerView {
     float* scales;
     PhiloxHead head;             // launch-wide part of this worker's Philox blocks
     uint32_t blk0_lo;            // low half of the Philox block index of the gradient's element 0
+    bool scalar_store;           // GIVEN: the codes start off a 16-byte boundary (mqg_quantize's never do)
 };
 
 // One tile, the k-th of this CTA, tile `tile` of worker `wv`.  FULL: every thread owns a complete
-// row (no bounds checks).  SHUFFLE: a bucket is an aligned power-of-two group of at most 32 rows
-// (lane shuffles); otherwise a whole number of warps (one shared-memory atomic per warp).  After
-// the tile's rows are in registers thread 0 calls `refill(stage, bar)` to start the copy that
+// row (no bounds checks).  RED: how a bucket's rows are reduced.  After the tile's rows are in registers thread 0 calls `refill(stage, bar)` to start the copy that
 // uses the stage next.  Returns false if the tile's copy never landed.
 // GIVEN: the scale is not computed here: every tile belongs to one bucket whose scale already stands
 // at wv.scales[0] (per-layer quantization after its max or norm pass, which also applies the flush);
 // no reduction, no scale written.
-template <int BITS, int DTYPE, int THREADS, bool FULL, bool SHUFFLE, bool NORM = false, bool GIVEN = false,
+template <int BITS, int DTYPE, int THREADS, bool FULL, int RED, bool NORM = false, bool GIVEN = false,
           typename Refill>
 __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>& sh, const WorkerView wv,
                                               const QuantizeArgs& a, const TmaQuantizeConsts& c,
@@ -125,6 +131,7 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
                                               uint32_t local_bucket, bool scale_writer)
 {
     constexpr int kQuantStages = TmaQuantizeShared<DTYPE, THREADS>::kStages;
+    constexpr bool SHUFFLE = RED == kByShuffle;
     const uint32_t t = threadIdx.x;
     const uint32_t row = tile * a.tile_rows + t;
     const bool active = FULL || (t < a.tile_rows && row < (uint32_t)a.nrows);
@@ -168,15 +175,21 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
         // (one launch per worker at n = 25 M: 22.3 / 22.5 / 23.0 us at K = 1 / 4 / 8 against 22.6 / 22.6 / 24.9 us)
         if (active) draw_row_blocks_head(wv.blk0_lo + 4u * row, wv.head, c.rk, h);
         float ss = row_sum_squares(x);
-        const uint32_t lanes = SHUFFLE ? a.rows_per_bucket : 32u;
-        for (uint32_t d = 1; d < lanes; d <<= 1) ss = __fadd_rn(ss, __shfl_xor_sync(0xFFFFFFFFu, ss, d));
-        if (!SHUFFLE && (t & 31) == 0) slot[t >> 5] = __float_as_uint(ss);
+        if constexpr (RED == kByRows) {
+            sh.row_sums[t] = ss;
+        } else {
+            const uint32_t lanes = SHUFFLE ? a.rows_per_bucket : 32u;
+            for (uint32_t d = 1; d < lanes; d <<= 1) ss = __fadd_rn(ss, __shfl_xor_sync(0xFFFFFFFFu, ss, d));
+            if (!SHUFFLE && (t & 31) == 0) slot[t >> 5] = __float_as_uint(ss);
+        }
         m = __float_as_uint(ss);
     } else {
         m = __float_as_uint(row_abs_max(x));
         if (SHUFFLE) {
             for (uint32_t d = a.rows_per_bucket >> 1; d > 0; d >>= 1)
                 m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
+        } else if (RED == kByRows) {
+            if (active) atomicMax(&slot[local_bucket], m);
         } else {
             m = __reduce_max_sync(0xFFFFFFFFu, m);
             if ((t & 31) == 0) atomicMax(&slot[local_bucket], m);
@@ -185,19 +198,38 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     if (__syncthreads_or(!ok)) return false;
     if (t == 0) refill(smem_u32(stage), bar);                    // every thread has read the stage
     if (!SHUFFLE && !GIVEN) {
-        if constexpr (NORM) {
-            // tree over the bucket's warp sums, zero leaves up to four (plain stores: nothing to reset;
-            // the slot array is written again two barriers from here)
-            static_assert(THREADS / 32 == 4, "the warp-sum tree is written for four warps");
-            const uint32_t wpb = a.rows_per_bucket >> 5, first = local_bucket * wpb;
-            float v[4];
+        if constexpr (NORM && RED == kByRows) {
+            // a bucket's tree is a warp's work: lane l on rows 4l .. 4l + 3 of it (at most 128), zeros beyond
+            const uint32_t lane = t & 31u, rpb = a.rows_per_bucket;
+            for (uint32_t b = t >> 5; b < a.buckets_per_tile; b += THREADS / 32) {
+                float v[4];
 #pragma unroll
-            for (uint32_t i = 0; i < 4; ++i)
-                v[i] = (i < wpb && first + i < 4u) ? __uint_as_float(slot[first + i]) : 0.0f;
-            m = __float_as_uint(__fadd_rn(__fadd_rn(v[0], v[1]), __fadd_rn(v[2], v[3])));
+                for (uint32_t i = 0; i < 4; ++i) v[i] = 4 * lane + i < rpb ? sh.row_sums[b * rpb + 4 * lane + i] : 0.0f;
+                float s = __fadd_rn(__fadd_rn(v[0], v[1]), __fadd_rn(v[2], v[3]));
+#pragma unroll
+                for (uint32_t d = 1; d < 32; d <<= 1) s = __fadd_rn(s, __shfl_xor_sync(0xFFFFFFFFu, s, d));
+                if (lane == 0) slot[b] = __float_as_uint(s);
+            }
+            __syncthreads();
+            m = slot[local_bucket];
+        } else if constexpr (NORM) {
+            // tree over the bucket's warp sums, zero leaves up to four or eight (plain stores: nothing to reset;
+            // the slot array is written again two barriers from here)
+            constexpr uint32_t kWarps = THREADS / 32;
+            static_assert(kWarps == 4 || kWarps == 8, "the tree is written for four or eight warps");
+            const uint32_t wpb = a.rows_per_bucket >> 5, first = local_bucket * wpb;
+            float v[kWarps];
+#pragma unroll
+            for (uint32_t i = 0; i < kWarps; ++i)
+                v[i] = (i < wpb && first + i < kWarps) ? __uint_as_float(slot[first + i]) : 0.0f;
+            float root = __fadd_rn(__fadd_rn(v[0], v[1]), __fadd_rn(v[2], v[3]));
+            if constexpr (kWarps == 8)
+                root = __fadd_rn(root, __fadd_rn(__fadd_rn(v[4], v[5]), __fadd_rn(v[6], v[7])));
+            m = __float_as_uint(root);
         } else {
             m = slot[local_bucket];
-            if (t < THREADS / 32) sh.slots[rot == 0 ? 2 : rot - 1][t] = 0u; // next used by this CTA's tile k + 2
+            constexpr uint32_t kUsed = RED == kByRows ? kSlots : THREADS / 32;
+            if (t < kUsed) sh.slots[rot == 0 ? 2 : rot - 1][t] = 0u;        // next used by this CTA's tile k + 2
         }
     }
     if (!active) return true;
@@ -226,6 +258,93 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     // K = 5, 20.6 against 21.6 us at K = 8 (batched launch, 0.3 s of launches back to back, 1650 - 1720 MHz).
     encode_pack_row_packed<BITS>(x, es, h, w);
     const uint64_t word0 = (uint64_t)row * BITS;
+    if (GIVEN && wv.scalar_store && (FULL || (uint64_t)row * 32 + 32 <= a.n)) {
+#pragma unroll
+        for (int j = 0; j < BITS; ++j) wv.codes[word0 + j] = w[j];
+    } else if (FULL || (uint64_t)row * 32 + 32 <= a.n) {
+        store_row_words<BITS>(wv.codes, word0, w);
+    } else {
+        mask_row_words<BITS>(w, (int)(a.n - (uint64_t)row * 32) * BITS);
+#pragma unroll
+        for (int j = 0; j < BITS; ++j)
+            if (word0 + j < a.ncode_words) wv.codes[word0 + j] = w[j];
+    }
+    return true;
+}
+
+// The same tile for the (min, max) nearest-rounding variant: two reductions instead of one, two
+// floats per bucket (ranges[2b] = lo, ranges[2b + 1] = hi), no random draws.  Padding must not
+// take part in the range: the elements a ragged row lacks repeat its first element, and threads
+// without a row contribute the identities.  sh.slots holds maxima, sh.slots_lo minima, both as
+// ordered bits; the kernel initialises them to the identities.
+template <int BITS, int DTYPE, int THREADS, bool FULL, int RED, typename Refill>
+__device__ __forceinline__ bool range_quantize_tile(TmaQuantizeShared<DTYPE, THREADS>& sh, const WorkerView wv,
+                                                    const QuantizeArgs& a, uint32_t k, uint32_t rot, uint32_t tile,
+                                                    Refill&& refill, uint32_t local_bucket, bool scale_writer)
+{
+    constexpr int kQuantStages = TmaQuantizeShared<DTYPE, THREADS>::kStages;
+    constexpr bool SHUFFLE = RED == kByShuffle;
+    const uint32_t t = threadIdx.x;
+    const uint32_t row = tile * a.tile_rows + t;
+    const bool active = FULL || (t < a.tile_rows && row < (uint32_t)a.nrows);
+    const uint32_t stg = k % kQuantStages, parity = (k / kQuantStages) & 1;
+    const uint32_t bar = smem_u32(&sh.bar[stg]);
+    uint8_t* stage = sh.stage[stg];
+
+    bool ok = mbar_try_wait(bar, parity);
+    if (!ok) ok = mbar_wait(bar, parity, a.poll_limit);
+
+    float x[32];
+    uint32_t mlo = kOrderedMinIdentity, mhi = kOrderedMaxIdentity;
+    if (active) {
+        const bool ragged = !FULL && row >= (uint32_t)a.nrows_full;
+        if (ragged) stage_ragged_row<DTYPE>(stage, (int)t, wv.grad, (uint64_t)row * 32, a.n);
+        read_row_swizzled<DTYPE>(stage, (int)t, x);
+        if (ragged) fence_proxy_async();     // orders those stores before the bulk copy that refills the stage
+        if (!FULL) {
+            const uint64_t left = a.n - (uint64_t)row * 32;      // >= 1
+#pragma unroll
+            for (int j = 1; j < 32; ++j) x[j] = ((uint64_t)j < left) ? x[j] : x[0];
+        }
+        float lo, hi;
+        row_min_max(x, lo, hi);
+        mlo = ordered_bits(lo); mhi = ordered_bits(hi);
+    }
+    uint32_t* slot_hi = sh.slots[rot];       // rot = k % 3
+    uint32_t* slot_lo = sh.slots_lo[rot];
+    if (SHUFFLE) {
+        for (uint32_t d = a.rows_per_bucket >> 1; d > 0; d >>= 1) {
+            mlo = min(mlo, __shfl_xor_sync(0xFFFFFFFFu, mlo, d));
+            mhi = max(mhi, __shfl_xor_sync(0xFFFFFFFFu, mhi, d));
+        }
+    } else if (RED == kByRows) {
+        if (active) { atomicMin(&slot_lo[local_bucket], mlo); atomicMax(&slot_hi[local_bucket], mhi); }
+    } else {
+        mlo = __reduce_min_sync(0xFFFFFFFFu, mlo);
+        mhi = __reduce_max_sync(0xFFFFFFFFu, mhi);
+        if ((t & 31) == 0) { atomicMin(&slot_lo[local_bucket], mlo); atomicMax(&slot_hi[local_bucket], mhi); }
+    }
+    if (__syncthreads_or(!ok)) return false;
+    if (t == 0) refill(smem_u32(stage), bar);                    // every thread has read the stage
+    if (!SHUFFLE) {
+        mlo = slot_lo[local_bucket]; mhi = slot_hi[local_bucket];
+        if (t < (RED == kByRows ? kSlots : THREADS / 32)) {      // next used by this CTA's tile k + 2
+            sh.slots[rot == 0 ? 2 : rot - 1][t] = kOrderedMaxIdentity;
+            sh.slots_lo[rot == 0 ? 2 : rot - 1][t] = kOrderedMinIdentity;
+        }
+    }
+    if (!active) return true;
+
+    // a zero of either sign is stored as +0
+    const float lo = __fadd_rn(from_ordered_bits(mlo), 0.0f), hi = __fadd_rn(from_ordered_bits(mhi), 0.0f);
+    const uint32_t bucket = tile * a.buckets_per_tile + local_bucket;
+    if (scale_writer && (FULL || bucket < a.nbuckets))
+        reinterpret_cast<float2*>(wv.scales)[bucket] = make_float2(lo, hi);
+
+    const RangeEncodeScale es = range_encode_scale<BITS>(lo, hi);
+    uint32_t w[BITS];
+    range_encode_pack_row<BITS>(x, es, w);
+    const uint64_t word0 = (uint64_t)row * BITS;
     if (FULL || (uint64_t)row * 32 + 32 <= a.n) {
         store_row_words<BITS>(wv.codes, word0, w);
     } else {
@@ -235,6 +354,43 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
             if (word0 + j < a.ncode_words) wv.codes[word0 + j] = w[j];
     }
     return true;
+}
+
+// MODE: kMaxAbs = the main codec, kRange = the (min, max) variant, kNorm = the L2-norm scale variant.
+enum : int { kMaxAbs = 0, kRange = 1, kNorm = 2 };
+
+// One tile in the given mode.
+template <int BITS, int DTYPE, int THREADS, bool FULL, int RED, int MODE, typename Refill>
+__device__ __forceinline__ bool mode_tile(TmaQuantizeShared<DTYPE, THREADS>& sh, const WorkerView& wv, const QuantizeArgs& a,
+                                          const TmaQuantizeConsts& c, uint32_t k, uint32_t rot, uint32_t tile,
+                                          Refill&& refill, uint32_t local_bucket, bool scale_writer)
+{
+    if constexpr (MODE == kRange)
+        return range_quantize_tile<BITS, DTYPE, THREADS, FULL, RED>(sh, wv, a, k, rot, tile, refill, local_bucket,
+                                                                    scale_writer);
+    else
+        return quantize_tile<BITS, DTYPE, THREADS, FULL, RED, MODE == kNorm>(sh, wv, a, c, k, rot, tile, refill,
+                                                                             local_bucket, scale_writer);
+}
+
+// First contents of a CTA's slots: the identities of the reductions.
+template <int DTYPE, int THREADS>
+__device__ __forceinline__ void init_slots(TmaQuantizeShared<DTYPE, THREADS>& sh)
+{
+    for (uint32_t i = threadIdx.x; i < 3u * kSlots; i += THREADS) {
+        (&sh.slots[0][0])[i] = 0u;         // = kOrderedMaxIdentity
+        (&sh.slots_lo[0][0])[i] = kOrderedMinIdentity;
+    }
+}
+
+// Host side, shared by the launchers of mqg_quantize.cu and mqg_quantize_workers.cu.
+bool tma_path_applies(uint64_t n, uint64_t rpb, uint64_t elem_offset);
+uint64_t fill_args(QuantizeArgs& a, const void* grad, uint64_t n, int bits, uint64_t bucket, uint64_t seed,
+                   uint32_t* codes, float* scales, uint32_t worker, uint32_t step, uint64_t elem_offset);
+int fill_tma_args(QuantizeArgs& a, TmaQuantizeConsts& c, uint64_t rpb);
+inline int reduction_of(uint64_t rpb)
+{
+    return (rpb & (rpb - 1)) == 0 && rpb <= 32 ? kByShuffle : rpb % 32 == 0 ? kByWarps : kByRows;
 }
 
 }  // namespace mqg

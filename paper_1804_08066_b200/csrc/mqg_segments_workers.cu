@@ -93,12 +93,13 @@ encode_entries_kernel(const __grid_constant__ SegEntryTable<CAP> ent, const __gr
     for (; ok && v < total_tiles; v += stride, ++k, rot = (rot == 2 ? 0 : rot + 1)) {
         const SegEntry& e = ent.e[cur.e];
         const uint32_t tile = cur.tile;
-        const WorkerView wv = {&ent.map[cur.e], e.grad, e.codes, e.scale, e.head, e.blk0_lo};
+        const WorkerView wv = {&ent.map[cur.e], e.grad, e.codes, e.scale, e.head, e.blk0_lo,
+                               (reinterpret_cast<uintptr_t>(e.codes) & 15u) != 0};
         auto refill = [&](uint32_t stage, uint32_t bar) {
             if (vfill < total_tiles) load_tile(fill, stage, bar);
         };
         if (tile < e.full_tiles) {
-            ok = quantize_tile<BITS, DTYPE, THREADS, true, false, false, true>(sh, wv, a, c, k, rot, tile, refill,
+            ok = quantize_tile<BITS, DTYPE, THREADS, true, kByWarps, false, true>(sh, wv, a, c, k, rot, tile, refill,
                                                                                 0u, false);
         } else {
             QuantizeArgs ae = a;           // the bounds of this entry, needed by its last tile only
@@ -106,7 +107,7 @@ encode_entries_kernel(const __grid_constant__ SegEntryTable<CAP> ent, const __gr
             ae.nrows = (e.n + 31) / 32;
             ae.nrows_full = e.n / 32;
             ae.ncode_words = (e.n * BITS + 31) / 32;
-            ok = quantize_tile<BITS, DTYPE, THREADS, false, false, false, true>(sh, wv, ae, c, k, rot, tile, refill,
+            ok = quantize_tile<BITS, DTYPE, THREADS, false, kByWarps, false, true>(sh, wv, ae, c, k, rot, tile, refill,
                                                                                  0u, false);
         }
         if (v + stride < total_tiles) advance(cur, stride);
@@ -214,11 +215,10 @@ cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, 
 {
     const size_t esz = dtype == 0 ? 4 : 2;
     const TableArgs a = make_table_args(grads, W, codes, scales, seed, first_worker, step, elem_offset);
-    auto bulk = [&](int j) {                          // every worker's buffers are aligned for bulk copies
+    auto bulk = [&](int j) {                          // every worker's gradient is aligned for bulk copies
         for (int w = 0; w < W; ++w)
             if (!quantize_given_scale_applies(static_cast<const char*>(grads[w]) + seg_off[j] * esz,
-                                              seg_off[j + 1] - seg_off[j], codes[w] + code_off[j],
-                                              elem_offset + seg_off[j]))
+                                              seg_off[j + 1] - seg_off[j], elem_offset + seg_off[j]))
                 return false;
         return true;
     };
