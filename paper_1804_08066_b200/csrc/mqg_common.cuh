@@ -304,6 +304,94 @@ __device__ __forceinline__ void encode_pack_row_packed(const float (&x)[32], con
     }
 }
 
+// ---- the encode through integers, for at most seven bits -----------------------------------------
+// With T = 2^16 t rounded as above and h the draw, code = ceil((T - h - 1/2) / 2^16).  For any p >= 1 and
+// J = ceil(2^p T) this is (J - 2^p h + 2^(16 + p) - 2^(p - 1) - 1) >> (16 + p), because 2^p (h + 1/2) is an integer.
+//   * J and the constant come from ONE packed fma: multiplied by 2^(p - 149), 2^p T lies among the subnormal floats
+//     (and the first normal ones), whose bit patterns are the integers 0 .. 2^24 - 1 in units of 2^-149; rounding up
+//     there is the ceiling, and there is no bias to remove.  16 + p + BITS <= 24 keeps the sum below 2^24; it is never
+//     negative, because T > -1/2 and the constant is larger.
+//   * - 2^p h is a two-way dot product (dp2a) of the Philox word with (-2^p, 0) or (0, -2^p), so that neither half of
+//     the word has to be extracted.
+// Against the form in floats this saves two of four packed instructions per pair of elements and the two byte
+// permutes; the codes then lie in byte 2 of J's words, at a bit of the byte that p chooses.
+__device__ __forceinline__ uint32_t minus_draw(uint32_t j, uint32_t word, uint32_t coef)
+{
+    uint32_t d;
+    asm("dp2a.lo.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(word), "r"(coef), "r"(j));
+    return d;
+}
+
+// Byte 2 of four words.
+__device__ __forceinline__ uint32_t gather_byte2(uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    return __byte_perm(__byte_perm(a, b, 0x0062), __byte_perm(c, d, 0x0062), 0x5410);
+}
+
+template <int BITS>
+__device__ __forceinline__ void encode_pack_row_int(const float (&x)[32], const EncodeScale& e,
+                                                    const uint32_t (&h)[16], uint32_t (&w)[BITS])
+{
+    static_assert(BITS <= 7, "2^24 integers");
+    constexpr bool kBytes = BITS == 1 || BITS == 2 || BITS == 4;        // codes tile the bytes
+    // bit of byte 2 at which element j's code lies: its place in the output byte (place 0 does not exist: p >= 1),
+    // or the top of the byte
+    auto place = [](int j) constexpr { return kBytes && (j * BITS) % 8 != 0 ? (j * BITS) % 8 : 8 - BITS; };
+    const float2 inv = make_float2(e.inv16, e.inv16), half = make_float2(e.half_l16, e.half_l16);
+    uint32_t s[32];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+        const int pa = place(2 * q), pb = place(2 * q + 1);
+        const float2 mul = make_float2(__uint_as_float(1u << pa), __uint_as_float(1u << pb));
+        const float2 add = make_float2(__uint_as_float((1u << (16 + pa)) - (1u << (pa - 1)) - 1u),
+                                       __uint_as_float((1u << (16 + pb)) - (1u << (pb - 1)) - 1u));
+        const float2 T = __ffma2_rn(make_float2(x[2 * q], x[2 * q + 1]), inv, half);
+        const float2 J = __ffma2_ru(T, mul, add);
+        s[2 * q] = minus_draw(__float_as_uint(J.x), h[q], (0u - (1u << pa)) & 0xFFu);
+        s[2 * q + 1] = minus_draw(__float_as_uint(J.y), h[q], ((0u - (1u << pb)) & 0xFFu) << 8);
+    }
+    if constexpr (kBytes) {
+        constexpr int kPer = 8 / BITS;                                  // codes per output byte
+        constexpr uint32_t kOnes = 0x01010101u;
+#pragma unroll
+        for (int k = 0; k < BITS; ++k) {
+            const int j0 = k * (32 / BITS);
+            // elements j0 + kPer * byte + i for i = 0 .. kPer - 1
+            uint32_t v = gather_byte2(s[j0], s[j0 + kPer], s[j0 + 2 * kPer], s[j0 + 3 * kPer]) >> (8 - BITS);
+#pragma unroll
+            for (int i = 1; i < kPer; ++i) {
+                const uint32_t below = ((1u << (i * BITS)) - 1u) * kOnes;
+                v = (v & below) |
+                    (gather_byte2(s[j0 + i], s[j0 + kPer + i], s[j0 + 2 * kPer + i], s[j0 + 3 * kPer + i]) & ~below);
+            }
+            w[k] = v;
+        }
+    } else {
+        constexpr int kAt = 24 - BITS;                                  // the code's lowest bit; nothing lies above it
+        constexpr uint32_t kMask = (1u << BITS) - 1u;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+            const int o = j * BITS, wi = o >> 5, sh = o & 31;
+            const uint32_t at = sh <= kAt ? s[j] >> (kAt - sh) : s[j] << (sh - kAt);
+            if (sh == 0) w[wi] = at;
+            else w[wi] = (w[wi] & ((1u << sh) - 1u)) | (at & (kMask << sh));
+            if (sh + BITS > 32) w[wi + 1] = s[j] >> (kAt + 32 - sh);
+        }
+    }
+}
+
+// The encode of the kernels that are bound by it.  Batched launch held at the power limit, per 10^8 bytes of gradient,
+// against the packed float form: fp32 K = 1 / 4 / 6 18.3 / 19.0 / 20.0 us against 18.8 / 19.7 / 20.3 us, K = 7 no
+// difference; bf16 K = 1 / 4 / 6 30.4 / 30.5 / 32.7 against 31.9 / 32.2 / 33.3 us.  (436 instead of 463 executed
+// instructions per row at K = 4; the multiply-add pipe that takes the Philox products is 70 % instead of 74 % busy.)
+template <int BITS>
+__device__ __forceinline__ void encode_pack_row_best(const float (&x)[32], const EncodeScale& e,
+                                                     const uint32_t (&h)[16], uint32_t (&w)[BITS])
+{
+    if constexpr (BITS <= 7) encode_pack_row_int<BITS>(x, e, h, w);
+    else encode_pack_row_packed<BITS>(x, e, h, w);
+}
+
 // ---------------------------------------------------------------------------------
 // Codec variant: (min, max) range with nearest rounding.  Per bucket lo = min x, hi = max x
 // (a zero of either sign stored as +0), r = fl(hi - lo); code = min(L, floor(fma(fl(x - lo),

@@ -55,6 +55,42 @@ __device__ __forceinline__ void read_row_swizzled(const uint8_t* stage, int row,
     }
 }
 
+// A bf16 row as it lies in the stage: element pairs, two to a word.
+__device__ __forceinline__ void read_row_words(const uint8_t* stage, int row, uint32_t (&u)[16])
+{
+    const uint4* t = reinterpret_cast<const uint4*>(stage);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const uint4 v = t[row * 4 + (c ^ ((row >> 1) & 3))];
+        u[4 * c] = v.x; u[4 * c + 1] = v.y; u[4 * c + 2] = v.z; u[4 * c + 3] = v.w;
+    }
+}
+
+__device__ __forceinline__ void widen_row(const uint32_t (&u)[16], float (&x)[32])
+{
+#pragma unroll
+    for (int k = 0; k < 16; ++k) { x[2 * k] = bf16_lo(u[k]); x[2 * k + 1] = bf16_hi(u[k]); }
+}
+
+// Largest magnitude of a bf16 row: two elements per instruction (the sign of the running maximum is an exclusive or
+// and means nothing; the magnitude is the maximum).
+__device__ __forceinline__ float row_abs_max_bf16(const uint32_t (&u)[16])
+{
+    auto max2 = [](uint32_t a, uint32_t b) {
+        uint32_t r;
+        asm("max.xorsign.abs.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+        return r;
+    };
+    uint32_t m[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) m[k] = max2(u[2 * k], u[2 * k + 1]);
+#pragma unroll
+    for (int d = 4; d > 0; d >>= 1)
+#pragma unroll
+        for (int k = 0; k < d; ++k) m[k] = max2(m[k], m[k + d]);
+    return fmaxf(fabsf(bf16_lo(m[0])), fabsf(bf16_hi(m[0])));
+}
+
 // The one row of the gradient that is shorter than 32 elements is not covered by the tensor
 // map: its owner copies it (zero-padded) into its own row of the stage with plain loads and
 // then reads it back like any other row.
@@ -153,15 +189,22 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     bool ok = mbar_try_wait(bar, parity);
     if (!ok) ok = mbar_wait(bar, parity, a.poll_limit);
 
+    // bf16 rows whose maximum is wanted stay packed until the encode: half the registers across the barrier, and the
+    // maximum takes two elements per instruction (30.0 against 30.5 us per 50 M elements at K = 4)
+    constexpr bool kPackedRow = DTYPE == 1 && !NORM && !GIVEN;
     float x[32];
+    uint32_t raw[16];
     if (active) {
         const bool ragged = !FULL && row >= (uint32_t)a.nrows_full;
         if (ragged) stage_ragged_row<DTYPE>(stage, (int)t, wv.grad, (uint64_t)row * 32, a.n);
-        read_row_swizzled<DTYPE>(stage, (int)t, x);
+        if (kPackedRow) read_row_words(stage, (int)t, raw);
+        else read_row_swizzled<DTYPE>(stage, (int)t, x);
         if (ragged) fence_proxy_async();     // orders those stores before the bulk copy that refills the stage
     } else {
 #pragma unroll
         for (int j = 0; j < 32; ++j) x[j] = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) raw[j] = 0u;
     }
     uint32_t m;
     uint32_t* slot = sh.slots[rot];          // rot = k % 3
@@ -184,7 +227,7 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
         }
         m = __float_as_uint(ss);
     } else {
-        m = __float_as_uint(row_abs_max(x));
+        m = __float_as_uint(kPackedRow ? row_abs_max_bf16(raw) : row_abs_max(x));
         if (SHUFFLE) {
             for (uint32_t d = a.rows_per_bucket >> 1; d > 0; d >>= 1)
                 m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
@@ -248,15 +291,16 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     // Philox blocks of the row: elem_offset / 8 + 4 * row + 0 .. 3, all in the launch's high half
     if constexpr (!NORM && !kEarlyDraw)
         draw_row_blocks_head(wv.blk0_lo + 4u * row, wv.head, c.rk, h);
+    if (kPackedRow) widen_row(raw, x);
     uint32_t w[BITS];
     // The encode's arithmetic runs in packed fp32x2 instructions at every width: 14.3 instead of 17.0 - 17.6
-    // executed instructions per element.  With the SM clock at its maximum this gains only at one and two bits
+    // executed instructions per element (13.6 with the integer form up to seven bits).  With the SM clock at its maximum this gains only at one and two bits
     // (16.6 against 17.2 us per 100 MB gradient at K = 1; from K = 4 on the constant pairs compete with the
     // early draws for registers), but a launch that runs for more than a few tens of milliseconds is held at
     // the board's power limit, where the clock falls until the power fits and fewer instructions per element
     // mean less time: 19.6 against 20.5 us at K = 3, 19.4 against 20.4 us at K = 4, 20.5 against 21.2 us at
     // K = 5, 20.6 against 21.6 us at K = 8 (batched launch, 0.3 s of launches back to back, 1650 - 1720 MHz).
-    encode_pack_row_packed<BITS>(x, es, h, w);
+    encode_pack_row_best<BITS>(x, es, h, w);
     const uint64_t word0 = (uint64_t)row * BITS;
     if (GIVEN && wv.scalar_store && (FULL || (uint64_t)row * 32 + 32 <= a.n)) {
 #pragma unroll

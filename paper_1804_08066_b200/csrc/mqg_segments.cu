@@ -35,7 +35,7 @@ __device__ __forceinline__ void encode_store_row(const float (&x)[32], const Sca
             const DrawKey key = {a.rk.k0[0], a.rk.k1[0], a.first_worker + w, a.rk.step};
             draw_row_unaligned(g0, key, h);
         }
-        encode_pack_row_packed<BITS>(x, es, h, cw);
+        encode_pack_row_best<BITS>(x, es, h, cw);
     }
     if (vec && left >= 32) {
         store_row_words<BITS>(a.codes[w], word0, cw);

@@ -945,7 +945,7 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
             // (the encode's arithmetic in packed fp32x2 instructions: 0.5 to 1 us per launch at every width;
             // a fifth resident CTA, which 95 registers would allow, changes nothing: the kernel waits on
             // its arithmetic pipes, not on latency)
-            encode_pack_row_packed<BITS>(x, es, h, w);
+            encode_pack_row_best<BITS>(x, es, h, w);
             store_row_words<BITS>(ra.codes_out, (uint64_t)row * BITS, w);
         }
         if (have_next) store_tile_scales<BITS, false>(a, table, lane, wide, s_next);
