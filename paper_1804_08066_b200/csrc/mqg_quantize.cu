@@ -105,7 +105,7 @@ quantize_pack_kernel(const __grid_constant__ QuantizeArgs a)
 
 
 template <int BITS, int DTYPE, int THREADS, int RED, int MODE>
-__global__ void __launch_bounds__(THREADS, 512 / THREADS)
+__global__ void __launch_bounds__(THREADS, DTYPE == kBf16Wide ? 5 : 512 / THREADS)
 quantize_tma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ QuantizeArgs a,
                     const __grid_constant__ TmaQuantizeConsts c, unsigned int* __restrict__ timeouts)
 {
@@ -212,7 +212,8 @@ static cudaError_t launch_tma_shape(const CUtensorMap& map, const QuantizeArgs& 
                                     unsigned int* timeouts, cudaStream_t stream)
 {
     const int red = reduction_of(a.rows_per_bucket);
-    if (threads == 256) return launch_tma_inst<BITS, DTYPE, 256, kByWarps, MODE>(map, a, c, timeouts, stream);
+    if constexpr (DTYPE != kBf16Wide)        // 128 rows of 64 hold every bucket
+        if (threads == 256) return launch_tma_inst<BITS, DTYPE, 256, kByWarps, MODE>(map, a, c, timeouts, stream);
     if (red == kByShuffle) return launch_tma_inst<BITS, DTYPE, 128, kByShuffle, MODE>(map, a, c, timeouts, stream);
     if (red == kByRows) return launch_tma_inst<BITS, DTYPE, 128, kByRows, MODE>(map, a, c, timeouts, stream);
     return launch_tma_inst<BITS, DTYPE, 128, kByWarps, MODE>(map, a, c, timeouts, stream);
@@ -229,12 +230,15 @@ static cudaError_t launch_tma(QuantizeArgs& a, uint64_t rpb, int bits, int dtype
     if (timeouts == nullptr) return cudaErrorNotSupported;
     CUtensorMap map;
     const char* why = nullptr;
-    if (!encode_rows_map(&map, a.grad, a.nrows_full, dtype == 0 ? 4 : 2, 32, a.tile_rows, &why))
+    if (!encode_rows_map(&map, a.grad, a.nrows_full, dtype == 0 ? 4 : 2, a.row_elems, a.tile_rows, &why))
         return cudaErrorNotSupported;        // the driver cannot encode a tensor map: no silent detour
     switch (bits) {
 #define MQG_TMA_CASE(B) \
-        case B: return dtype == 0 ? launch_tma_shape<B, 0, MODE>(map, a, c, threads, timeouts, stream) \
-                                  : launch_tma_shape<B, 1, MODE>(map, a, c, threads, timeouts, stream)
+        case B: \
+            if constexpr (MODE == kMaxAbs) \
+                if (a.row_elems == 64) return launch_tma_shape<B, kBf16Wide, MODE>(map, a, c, threads, timeouts, stream); \
+            return dtype == 0 ? launch_tma_shape<B, 0, MODE>(map, a, c, threads, timeouts, stream) \
+                              : launch_tma_shape<B, 1, MODE>(map, a, c, threads, timeouts, stream)
         MQG_TMA_CASE(1); MQG_TMA_CASE(2); MQG_TMA_CASE(3); MQG_TMA_CASE(4);
         MQG_TMA_CASE(5); MQG_TMA_CASE(6); MQG_TMA_CASE(7); MQG_TMA_CASE(8);
 #undef MQG_TMA_CASE
@@ -262,25 +266,35 @@ bool tma_path_applies(uint64_t n, uint64_t rpb, uint64_t elem_offset)
     return reduction_of(rpb) != kByRows || rpb <= 128;
 }
 
+// Rows of 64 halve the number of tiles, so a short launch is longer with them: us narrow / wide at one worker, K = 4,
+// n = 2^21 / 2^23 / 2^24 / 2^25: 3.2 / 4.4, 7.1 / 7.6, 11.6 / 11.3, 22.0 / 20.0 (four workers of a quarter of
+// that the same).  Long launches, held at the power limit: 30.6 -> 27.2 us per 50 M elements at K = 1, 29.8 -> 27.8 at
+// K = 4, 33.4 -> 32.6 at K = 8.
+bool bf16_wide_applies(uint64_t n, uint64_t total, uint64_t bucket, int dtype)
+{
+    return dtype == 1 && total >= (20ull << 20) && n >= 64 * 64 && (bucket >= n || bucket % 64 == 0);
+}
+
 // Fills the arguments every fused kernel shares.  Returns rows per bucket.
 uint64_t fill_args(QuantizeArgs& a, const void* grad, uint64_t n, int bits, uint64_t bucket,
                           uint64_t seed, uint32_t* codes, float* scales, uint32_t worker, uint32_t step,
-                          uint64_t elem_offset)
+                          uint64_t elem_offset, uint32_t row_elems)
 {
     a.grad = grad; a.codes = codes; a.scales = scales;
     a.n = n;
-    a.nrows = (n + 31) / 32;
+    a.row_elems = row_elems;
+    a.nrows = (n + row_elems - 1) / row_elems;
     a.nbuckets = (n + bucket - 1) / bucket;
     a.ncode_words = (n * (uint64_t)bits + 31) / 32;
     a.elem_offset = elem_offset;
     // bucket % 32 == 0 and bucket <= 8192, or a single bucket of at most 8192 elements
-    const uint64_t rpb = (bucket >= n) ? a.nrows : bucket / 32;
+    const uint64_t rpb = (bucket >= n) ? a.nrows : bucket / row_elems;
     a.rows_per_bucket = (uint32_t)rpb;
     a.buckets_per_tile = (uint32_t)(kMaxTileRows / rpb);
     a.tile_rows = a.buckets_per_tile * a.rows_per_bucket;
     a.key.seed_lo = (uint32_t)seed; a.key.seed_hi = (uint32_t)(seed >> 32);
     a.key.worker = worker; a.key.step = step;
-    a.nrows_full = n / 32;
+    a.nrows_full = n / row_elems;
     const WaitPolicy policy = wait_policy();
     a.poll_limit = policy.poll_limit;
     a.arm_only = policy.arm_only;
@@ -316,7 +330,11 @@ cudaError_t launch_quantize_fused(const void* grad, uint64_t n, int bits, uint64
 {
     QuantizeArgs a;
     const uint64_t rpb = fill_args(a, grad, n, bits, bucket, seed, codes, scales, worker, step, elem_offset);
-    if (tma_path_applies(n, rpb, elem_offset)) return launch_tma<kMaxAbs>(a, rpb, bits, dtype, stream);
+    if (tma_path_applies(n, rpb, elem_offset)) {
+        if (!bf16_wide_applies(n, n, bucket, dtype)) return launch_tma<kMaxAbs>(a, rpb, bits, dtype, stream);
+        const uint64_t wide = fill_args(a, grad, n, bits, bucket, seed, codes, scales, worker, step, elem_offset, 64);
+        return launch_tma<kMaxAbs>(a, wide, bits, dtype, stream);
+    }
     a.buckets_per_tile = (uint32_t)(kMaxTileRows / rpb);
     a.tile_rows = a.buckets_per_tile * a.rows_per_bucket;
     const uint64_t ntiles = (a.nrows + a.tile_rows - 1) / a.tile_rows;

@@ -24,7 +24,7 @@ struct WorkerTable {
 };
 
 template <int BITS, int DTYPE, int THREADS, int RED, int MODE>
-__global__ void __launch_bounds__(THREADS, 512 / THREADS)
+__global__ void __launch_bounds__(THREADS, DTYPE == kBf16Wide ? 5 : 512 / THREADS)
 quantize_workers_kernel(const __grid_constant__ WorkerTable tab, const __grid_constant__ QuantizeArgs a,
                         const __grid_constant__ TmaQuantizeConsts c, uint32_t total_tiles,
                         unsigned int* __restrict__ timeouts)
@@ -135,7 +135,9 @@ static cudaError_t launch_workers_shape(const WorkerTable& tab, const QuantizeAr
                                         uint32_t total_tiles, int threads, unsigned int* timeouts, cudaStream_t stream)
 {
     const int red = reduction_of(a.rows_per_bucket);
-    if (threads == 256) return launch_workers_inst<BITS, DTYPE, 256, kByWarps, MODE>(tab, a, c, total_tiles, timeouts, stream);
+    if constexpr (DTYPE != kBf16Wide)        // 128 rows of 64 hold every bucket
+        if (threads == 256)
+            return launch_workers_inst<BITS, DTYPE, 256, kByWarps, MODE>(tab, a, c, total_tiles, timeouts, stream);
     if (red == kByShuffle) return launch_workers_inst<BITS, DTYPE, 128, kByShuffle, MODE>(tab, a, c, total_tiles, timeouts, stream);
     if (red == kByRows) return launch_workers_inst<BITS, DTYPE, 128, kByRows, MODE>(tab, a, c, total_tiles, timeouts, stream);
     return launch_workers_inst<BITS, DTYPE, 128, kByWarps, MODE>(tab, a, c, total_tiles, timeouts, stream);
@@ -151,6 +153,7 @@ static cudaError_t launch_workers_bits(const WorkerTable& tab, const QuantizeArg
                       : launch_workers_shape<BITS, 1, M>(tab, a, c, total_tiles, threads, timeouts, stream)
     if (mode == kNorm) MQG_WORKERS_MODE(kNorm);
     if (mode == kRange) MQG_WORKERS_MODE(kRange);
+    if (a.row_elems == 64) return launch_workers_shape<BITS, kBf16Wide, kMaxAbs>(tab, a, c, total_tiles, threads, timeouts, stream);
     MQG_WORKERS_MODE(kMaxAbs);
 #undef MQG_WORKERS_MODE
 }
@@ -173,8 +176,9 @@ cudaError_t launch_quantize_workers(const void* const* grads, int W, uint64_t n,
                                     uint32_t step, uint64_t elem_offset, int mode, cudaStream_t stream)
 {
     QuantizeArgs a;
+    const bool wide = mode == kMaxAbs && bf16_wide_applies(n, n * (uint64_t)W, bucket, dtype);
     const uint64_t rpb = fill_args(a, grads[0], n, bits, bucket, seed, codes[0], scales[0], first_worker,
-                                   step, elem_offset);
+                                   step, elem_offset, wide ? 64 : 32);
     TmaQuantizeConsts c;
     const int threads = fill_tma_args(a, c, rpb);
     if (threads == 0) return cudaErrorInvalidValue;
@@ -184,7 +188,7 @@ cudaError_t launch_quantize_workers(const void* const* grads, int W, uint64_t n,
     memset(&tab, 0, sizeof(tab));
     for (int w = 0; w < W; ++w) {
         const char* why = nullptr;
-        if (!encode_rows_map(&tab.map[w], grads[w], a.nrows_full, dtype == 0 ? 4 : 2, 32, a.tile_rows, &why))
+        if (!encode_rows_map(&tab.map[w], grads[w], a.nrows_full, dtype == 0 ? 4 : 2, a.row_elems, a.tile_rows, &why))
             return cudaErrorNotSupported;
         tab.grad[w] = grads[w]; tab.codes[w] = codes[w]; tab.scales[w] = scales[w];
         tab.head[w] = philox_head(c.blk0_hi, first_worker + (uint32_t)w, c.rk.k0[0]);

@@ -49,3 +49,35 @@ def test_bucket_reductions(n, bucket, mode, bits, bf16):
             assert bits_equal(scales[w].numpy(np.float32), np.asarray(ref[w][1]).reshape(-1)) == 0
             assert np.array_equal(codes[w].numpy(np.uint32), ref[w][0])
     assert mqg.mqg_device_timeouts() == 0
+
+
+@pytest.mark.parametrize("n,bucket,W,bits", [
+    ((20 << 20) // 3 + 64 + 1, 2048, 3, 4),          # rows of 64 bf16 elements; a last row of one element
+    ((20 << 20) // 3 + 64 + 63, 768, 3, 3),          # 12 rows per bucket, a last row of 63
+    ((20 << 20) // 2 + 4096 + 33, 8192, 2, 7),       # 128 rows per bucket
+    ((20 << 20) // 2 + 32, 256, 2, 1), ((20 << 20) // 2, 64, 2, 8), ((20 << 20) // 2 + 96, 32, 2, 2),   # 4, 1 rows; narrow
+    ((20 << 20) + 5, 4096, 1, 6),
+])
+def test_long_bf16_gradients(n, bucket, W, bits):
+    """Every bucket near the ends and a sample of the others, each encoded by the checker on its own."""
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    grads = [(torch.randn(n, generator=gen, device="cuda") * 1e-3).to(torch.bfloat16) for _ in range(W)]
+    nb = mqg.mqg_num_buckets(n, bucket)
+    codes = [Guarded(mqg.mqg_code_words(n, bits), torch.int32) for _ in range(W)]
+    scales = [Guarded(nb, torch.float32) for _ in range(W)]
+    mqg.mqg_quantize_workers(grads, W, n, bits, bucket, 7, [c.view for c in codes], [s.view for s in scales],
+                             first_worker=4, step=3, elem_offset=64)
+    torch.cuda.synchronize()
+    rng = np.random.default_rng(n)
+    some = np.unique(np.concatenate([np.arange(3), np.arange(max(0, nb - 70), nb), rng.integers(0, nb, 200)]))
+    for w in range(W):
+        codes[w].check_guards(), scales[w].check_guards()
+        got_c, got_s = codes[w].numpy(np.uint32), scales[w].numpy(np.float32)
+        x = grads[w].view(torch.int16).cpu().numpy().view(np.uint16)
+        for b in some.tolist():
+            lo, hi = b * bucket, min(n, (b + 1) * bucket)
+            c_ref, s_ref = O.quantize(x[lo:hi], bits, bucket, 7, worker=4 + w, step=3, elem_offset=64 + lo, dtype="bf16")
+            assert got_s[b] == s_ref[0]
+            at = lo * bits // 32
+            assert np.array_equal(got_c[at:at + c_ref.size], c_ref), (w, b)
+    assert mqg.mqg_device_timeouts() == 0
