@@ -137,7 +137,7 @@ quantize_tma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
     const uint32_t local_bucket = t / a.rows_per_bucket;
     const bool scale_writer = (t % a.rows_per_bucket) == 0;
     const uint32_t ahead = kQuantStages * stride;       // distance to the tile that refills a stage
-    const WorkerView wv = {&tmap, a.grad, a.codes, a.scales, c.head, c.blk0_lo, false};
+    const WorkerView wv = {&tmap, a.grad, a.codes, a.scales, c.head, c.blk0_lo};
 
     uint32_t k = 0, rot = 0;
     bool ok = true;

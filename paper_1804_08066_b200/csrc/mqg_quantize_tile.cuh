@@ -151,16 +151,12 @@ struct WorkerView {
     float* scales;
     PhiloxHead head;             // launch-wide part of this worker's Philox blocks
     uint32_t blk0_lo;            // low half of the Philox block index of the gradient's element 0
-    bool scalar_store;           // GIVEN: the codes start off a 16-byte boundary (mqg_quantize's never do)
 };
 
 // One tile, the k-th of this CTA, tile `tile` of worker `wv`.  FULL: every thread owns a complete
 // row (no bounds checks).  RED: how a bucket's rows are reduced.  After the tile's rows are in registers thread 0 calls `refill(stage, bar)` to start the copy that
 // uses the stage next.  Returns false if the tile's copy never landed.
-// GIVEN: the scale is not computed here: every tile belongs to one bucket whose scale already stands
-// at wv.scales[0] (per-layer quantization after its max or norm pass, which also applies the flush);
-// no reduction, no scale written.
-template <int BITS, int DTYPE, int THREADS, bool FULL, int RED, bool NORM = false, bool GIVEN = false,
+template <int BITS, int DTYPE, int THREADS, bool FULL, int RED, bool NORM = false,
           typename Refill>
 __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>& sh, const WorkerView wv,
                                               const QuantizeArgs& a, const TmaQuantizeConsts& c,
@@ -184,7 +180,7 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     // limit sets the clock and both forms take the same time: the instruction count decides there.)
     // bf16 input (half the bytes per tile, no wait to cover) keeps the draws after the wait at every width:
     // 32.3 / 32.1 / 32.7 / 32.4 us per 50 M elements at K = 3 / 4 / 6 / 8 against 33.2 / 32.8 / 33.6 / 32.8 us.
-    constexpr bool kEarlyDraw = !NORM && !GIVEN && DTYPE == 0 && BITS >= 3;
+    constexpr bool kEarlyDraw = !NORM && DTYPE == 0 && BITS >= 3;
     uint32_t h[16];
     if (kEarlyDraw && active) draw_row_blocks_head(wv.blk0_lo + 4u * row, wv.head, c.rk, h);
     bool ok = mbar_try_wait(bar, parity);
@@ -192,7 +188,7 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
 
     // bf16 rows whose maximum is wanted stay packed until the encode: half the registers across the barrier, and the
     // maximum takes two elements per instruction (30.0 against 30.5 us per 50 M elements at K = 4)
-    constexpr bool kPackedRow = DTYPE == 1 && !NORM && !GIVEN;
+    constexpr bool kPackedRow = DTYPE == 1 && !NORM;
     float x[32];
     uint32_t raw[16];
     if (active) {
@@ -209,9 +205,7 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     }
     uint32_t m;
     uint32_t* slot = sh.slots[rot];          // rot = k % 3
-    if constexpr (GIVEN) {
-        m = 0u;
-    } else if constexpr (NORM) {
+    if constexpr (NORM) {
         // L2-norm scale: the fixed tree over the rows' sums of squares - partner distance 1, 2, 4, ...
         // inside the warp, then (buckets of whole warps) the warp sums, one slot per warp.
         // The row's draws depend on nothing but its number: they are computed here, before the chain of
@@ -241,7 +235,7 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     }
     if (__syncthreads_or(!ok)) return false;
     if (t == 0) refill(smem_u32(stage), bar);                    // every thread has read the stage
-    if (!SHUFFLE && !GIVEN) {
+    if (!SHUFFLE) {
         if constexpr (NORM && RED == kByRows) {
             // a bucket's tree is a warp's work: lane l on rows 4l .. 4l + 3 of it (at most 128), zeros beyond
             const uint32_t lane = t & 31u, rpb = a.rows_per_bucket;
@@ -279,14 +273,10 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     if (!active) return true;
 
     float sc = __uint_as_float(m);
-    if constexpr (GIVEN) {
-        sc = __ldg(wv.scales);           // final: the scale pass has applied the flush
-    } else {
-        if constexpr (NORM) sc = sc < flush_limit() ? 0.0f : __fsqrt_rn(sc);     // flush decided on the sum
-        else if (sc < flush_limit()) sc = 0.0f;
-        const uint32_t bucket = tile * a.buckets_per_tile + local_bucket;
-        if (scale_writer && (FULL || bucket < a.nbuckets)) wv.scales[bucket] = sc;
-    }
+    if constexpr (NORM) sc = sc < flush_limit() ? 0.0f : __fsqrt_rn(sc);         // flush decided on the sum
+    else if (sc < flush_limit()) sc = 0.0f;
+    const uint32_t bucket = tile * a.buckets_per_tile + local_bucket;
+    if (scale_writer && (FULL || bucket < a.nbuckets)) wv.scales[bucket] = sc;
 
     const EncodeScale es = encode_scale<BITS>(sc);
     // Philox blocks of the row: elem_offset / 8 + 4 * row + 0 .. 3, all in the launch's high half
@@ -303,10 +293,7 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     // K = 5, 20.6 against 21.6 us at K = 8 (batched launch, 0.3 s of launches back to back, 1650 - 1720 MHz).
     encode_pack_row_best<BITS>(x, es, h, w);
     const uint64_t word0 = (uint64_t)row * BITS;
-    if (GIVEN && wv.scalar_store && (FULL || (uint64_t)row * 32 + 32 <= a.n)) {
-#pragma unroll
-        for (int j = 0; j < BITS; ++j) wv.codes[word0 + j] = w[j];
-    } else if (FULL || (uint64_t)row * 32 + 32 <= a.n) {
+    if (FULL || (uint64_t)row * 32 + 32 <= a.n) {
         store_row_words<BITS>(wv.codes, word0, w);
     } else {
         mask_row_words<BITS>(w, (int)(a.n - (uint64_t)row * 32) * BITS);

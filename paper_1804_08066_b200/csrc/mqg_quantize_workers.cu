@@ -77,7 +77,7 @@ quantize_workers_kernel(const __grid_constant__ WorkerTable tab, const __grid_co
     // indexed loads from the kernel's parameter block are long-latency loads the tile would wait for.
 #pragma unroll 1
     while (ok && v < total_tiles) {
-        const WorkerView wv = {&tab.map[w], tab.grad[w], tab.codes[w], tab.scales[w], tab.head[w], c.blk0_lo, false};
+        const WorkerView wv = {&tab.map[w], tab.grad[w], tab.codes[w], tab.scales[w], tab.head[w], c.blk0_lo};
 #pragma unroll 1
         for (; ok && tile < a.ntiles && v < total_tiles;
              tile += stride, v += stride, ++k, rot = (rot == 2 ? 0 : rot + 1)) {

@@ -5,9 +5,7 @@
 //      the launch also clears the scales of the longer ones;
 //   2. absmax_table_kernel - the max pass over the longer segments;
 //   3. encode_entries_kernel - their encode.  Every (worker, segment) pair is an entry with a tensor map of its
-//      own; the persistent CTAs walk the 128-row tiles of all entries as one sequence, fed by tiled bulk copies
-//      exactly like quantize_workers_kernel (tile code of mqg_quantize_tile.cuh, given-scale mode).  Segments
-//      that start where bulk copies cannot go through encode_table_kernel instead.
+//      own; the persistent CTAs walk the 128-row tiles of all entries as one sequence, fed by tiled bulk copies.  Segments that start where bulk copies cannot go through encode_table_kernel instead.
 // Worker w's outputs are the same whichever way a segment goes and however many workers there are.
 #include <string.h>
 
@@ -31,8 +29,7 @@ struct SegEntry {
     uint32_t* codes;         // the segment's first code word
     float* scale;            // its scale, final when the encode pass starts
     uint64_t n;              // elements
-    uint32_t ntiles;         // tiles of 128 rows
-    uint32_t full_tiles;     // leading tiles whose 128 rows are all complete
+    uint32_t tile0;          // its first tile's number in the launch's sequence
     uint32_t blk0_lo;        // low half of the Philox block index of the segment's first element
     PhiloxHead head;         // launch-wide part of its blocks (worker, high half of the block index)
 };
@@ -41,87 +38,143 @@ template <int CAP>
 struct SegEntryTable {
     CUtensorMap map[CAP];
     SegEntry e[CAP];
-    int nent;
+    uint32_t tile_end[CAP];              // one past each entry's last tile; 2^32 - 1 beyond the last entry
+    uint32_t tiles;
+    uint32_t poll_limit, arm_only;       // as in QuantizeArgs
+    RoundKeys rk;
 };
 
-// total_tiles = tiles of all entries.
+// The scale is given, so no warp needs another: the four warps of a CTA share the tiles' copies (16 KB: 128 rows of
+// 32 fp32 or 64 bf16 elements; a copy per warp's 4 KB took 635 against 622 us for eight AlexNet-shaped gradients) and
+// nothing else.  There is no CTA barrier: the last warp to have read a stage refills it.  What an entry's tiles share -
+// pointers, Philox head, the encode's constants with their division - is fetched when the entry changes.  The draws
+// come before the wait for the data, at the price of the fifth CTA per SM: 604 against 620 us for that call, 413
+// against 440 us in bf16 (622 and 437 us with a CTA barrier per tile and the tile code of the one-pass kernels).
 template <int BITS, int DTYPE, int CAP>
-__global__ void __launch_bounds__(128, 5)
-encode_entries_kernel(const __grid_constant__ SegEntryTable<CAP> ent, const __grid_constant__ QuantizeArgs a,
-                      const __grid_constant__ TmaQuantizeConsts c, uint32_t total_tiles,
-                      unsigned int* __restrict__ timeouts)
+__global__ void __launch_bounds__(128, 4)
+encode_entries_kernel(const __grid_constant__ SegEntryTable<CAP> T, unsigned int* __restrict__ timeouts)
 {
-    constexpr int THREADS = 128;
-    using Shared = TmaQuantizeShared<DTYPE, THREADS>;
-    constexpr int kQuantStages = Shared::kStages;
+    constexpr uint32_t kWarps = 4, kStages = 2, kRows = 32 * kWarps, kTileBytes = kRows * 128;
+    constexpr int kHalves = DTYPE == 0 ? 1 : 2, kElems = 32 * kHalves, kWords = BITS * kHalves;
+    struct Shared {
+        alignas(1024) uint8_t stage[kStages][kTileBytes];
+        alignas(8) uint64_t bar[kStages];
+        uint32_t read[kStages];        // warps that have read the stage, over all its uses
+    };
     __shared__ Shared sh;
-
-    const uint32_t t = threadIdx.x;
-    const uint32_t stride = gridDim.x;
-    const uint32_t box_bytes = THREADS * Shared::kRowBytes;
+    const uint32_t t = threadIdx.x, lane = t & 31u;
+    const uint32_t step = gridDim.x;
     if (t == 0) {
-        for (int s = 0; s < kQuantStages; ++s) mbar_init(smem_u32(&sh.bar[s]), 1);
+        for (uint32_t s = 0; s < kStages; ++s) { mbar_init(smem_u32(&sh.bar[s]), 1); sh.read[s] = 0u; }
         fence_barrier_init();
     }
     grid_dependency_release();
     __syncthreads();
     grid_dependency_wait();            // nothing above touches global memory
 
-    // ---- the tiles of the entries, one sequence walked like quantize_workers_kernel walks its workers
-    struct Pos { uint32_t e, tile; };
-    auto advance = [&](Pos& p, uint32_t by) {
-        p.tile += by;
-        while (p.tile >= ent.e[p.e].ntiles) { p.tile -= ent.e[p.e].ntiles; ++p.e; }
+    uint32_t u = blockIdx.x, fill = u;             // the tile in work, the next one to fetch
+    uint32_t fe = 0;                               // the entry of `fill`: searched once, then only moved forward
+#pragma unroll
+    for (uint32_t half = CAP / 2; half > 0; half >>= 1)
+        if (u >= T.tile_end[fe + half - 1]) fe += half;
+    if (u >= T.tiles) fe = 0;
+    uint32_t e = fe;
+    auto fetch = [&](uint32_t s, bool mine) {
+        if (fill < T.tiles) {
+            while (fill >= T.tile_end[fe]) ++fe;
+            if (mine) {
+                const uint32_t bar = smem_u32(&sh.bar[s]);
+                mbar_expect_tx(bar, kTileBytes);
+                if (!T.arm_only)
+                    tma_load_2d(smem_u32(sh.stage[s]), &T.map[fe], 0, (int)((fill - T.e[fe].tile0) * kRows), bar);
+            }
+        }
+        fill += step;
     };
-    auto load_tile = [&](const Pos& p, uint32_t stage, uint32_t bar) {     // thread 0 only
-        mbar_expect_tx(bar, box_bytes);
-        if (!a.arm_only) tma_load_2d(stage, &ent.map[p.e], 0, (int)(p.tile * THREADS), bar);
-    };
-    uint32_t v = blockIdx.x;
-    Pos cur = {0u, 0u}, fill = {0u, 0u};
-    if (v < total_tiles) { advance(cur, v); advance(fill, v); }
-    uint32_t vfill = v;
-    for (uint32_t s = 0; s < (uint32_t)kQuantStages; ++s) {
-        if (t == 0 && vfill < total_tiles) load_tile(fill, smem_u32(sh.stage[s]), smem_u32(&sh.bar[s]));
-        vfill += stride;
-        if (vfill < total_tiles) advance(fill, stride);
-    }
+    for (uint32_t s = 0; s < kStages; ++s) fetch(s, t == 0);
 
-    uint32_t k = 0, rot = 0;
-    bool ok = true;
+    uint32_t k = 0, end = 0, tile0 = 0, blk0 = 0, rows = 0, rows_full = 0;
+    uint32_t* codes = nullptr;
+    bool vec = false, ok = true;
+    PhiloxHead head = {};
+    EncodeScale es = {0.0f, 0.0f};
 #pragma unroll 1
-    for (; ok && v < total_tiles; v += stride, ++k, rot = (rot == 2 ? 0 : rot + 1)) {
-        const SegEntry& e = ent.e[cur.e];
-        const uint32_t tile = cur.tile;
-        const WorkerView wv = {&ent.map[cur.e], e.grad, e.codes, e.scale, e.head, e.blk0_lo,
-                               (reinterpret_cast<uintptr_t>(e.codes) & 15u) != 0};
-        auto refill = [&](uint32_t stage, uint32_t bar) {
-            if (vfill < total_tiles) load_tile(fill, stage, bar);
-        };
-        if (tile < e.full_tiles) {
-            ok = quantize_tile<BITS, DTYPE, THREADS, true, kByWarps, false, true>(sh, wv, a, c, k, rot, tile, refill,
-                                                                                0u, false);
-        } else {
-            QuantizeArgs ae = a;           // the bounds of this entry, needed by its last tile only
-            ae.n = e.n;
-            ae.nrows = (e.n + 31) / 32;
-            ae.nrows_full = e.n / 32;
-            ae.ncode_words = (e.n * BITS + 31) / 32;
-            ok = quantize_tile<BITS, DTYPE, THREADS, false, kByWarps, false, true>(sh, wv, ae, c, k, rot, tile, refill,
-                                                                                 0u, false);
+    for (; u < T.tiles; u += step, ++k) {
+        if (u >= end) {
+            while (u >= T.tile_end[e]) ++e;
+            const SegEntry& x = T.e[e];
+            end = T.tile_end[e]; tile0 = x.tile0; blk0 = x.blk0_lo; head = x.head; codes = x.codes;
+            rows = (uint32_t)((x.n + kElems - 1) / kElems); rows_full = (uint32_t)(x.n / kElems);
+            vec = (reinterpret_cast<uintptr_t>(codes) & 15u) == 0;
+            es = encode_scale<BITS>(__ldcg(x.scale));
         }
-        if (v + stride < total_tiles) advance(cur, stride);
-        vfill += stride;
-        if (vfill < total_tiles) advance(fill, stride);
+        const uint32_t s = k % kStages, row = (u - tile0) * kRows + t;
+        uint8_t* stage = sh.stage[s];
+        const uint32_t bar = smem_u32(&sh.bar[s]);
+        uint32_t h[16];
+        draw_row_blocks_head(blk0 + 4u * kHalves * row, head, T.rk, h);
+        ok = mbar_try_wait(bar, (k / kStages) & 1);
+        if (!ok) ok = mbar_wait(bar, (k / kStages) & 1, T.poll_limit);
+        if (!__all_sync(0xFFFFFFFFu, ok)) { ok = false; break; }
+
+        uint4 v[8];
+        const bool active = row < rows, ragged = active && row >= rows_full;
+        if (ragged) {
+            if constexpr (DTYPE == 0) stage_ragged_row<0>(stage, (int)t, T.e[e].grad, (uint64_t)row * 32, T.e[e].n);
+            else stage_ragged_wide_row(stage, (int)t, static_cast<const uint16_t*>(T.e[e].grad), (uint64_t)row * 64, T.e[e].n);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = reinterpret_cast<const uint4*>(stage)[swz((int)t, i)];
+        if (ragged) fence_proxy_async();   // orders those stores before the bulk copy that refills the stage
+        __syncwarp();                      // every lane has read the stage
+        bool last = false;
+        if (lane == 0) {
+            __threadfence_block();
+            last = (atomicAdd(&sh.read[s], 1u) & (kWarps - 1)) == kWarps - 1;
+            if (last) __threadfence_block();
+        }
+        fetch(s, last);
+
+        const uint32_t* raw = reinterpret_cast<const uint32_t*>(v);
+        uint32_t w[kWords];
+#pragma unroll
+        for (int half = 0; half < kHalves; ++half) {
+            float x[32];
+            if constexpr (DTYPE == 0) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) x[j] = __uint_as_float(raw[j]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) { x[2 * j] = bf16_lo(raw[16 * half + j]); x[2 * j + 1] = bf16_hi(raw[16 * half + j]); }
+            }
+            if (half != 0) draw_row_blocks_head(blk0 + 4u * (kHalves * row + half), head, T.rk, h);
+            uint32_t wh[BITS];
+            encode_pack_row_best<BITS>(x, es, h, wh);
+#pragma unroll
+            for (int j = 0; j < BITS; ++j) w[half * BITS + j] = wh[j];
+        }
+        const uint64_t word0 = (uint64_t)row * kWords;
+        if (row < rows_full) {
+            if (vec) {
+                store_row_words<kWords>(codes, word0, w);
+            } else {
+#pragma unroll
+                for (int j = 0; j < kWords; ++j) codes[word0 + j] = w[j];
+            }
+        } else if (active) {
+            const uint64_t n = T.e[e].n, words = (n * BITS + 31) / 32;
+            mask_row_words<kWords>(w, (int)(n - (uint64_t)row * kElems) * BITS);
+#pragma unroll
+            for (int j = 0; j < kWords; ++j)
+                if (word0 + j < words) codes[word0 + j] = w[j];
+        }
     }
-    if (!ok) {                         // as in quantize_workers_kernel
-        if (t == 0) {
-            atomicAdd(timeouts, 1u);
-            uint32_t j = k - 1, vl = v - stride;
-            for (int s = 0; s < kQuantStages && vl < total_tiles; ++s, ++j, vl += stride)
-                mbar_wait(smem_u32(&sh.bar[j % kQuantStages]), (j / kQuantStages) & 1, a.poll_limit);
-        }
-        __syncthreads();
+    if (!ok && lane == 0) {
+        // A copy never landed: record it, then give the copies still in flight (the one that was being waited for and
+        // the one after it) a last bounded chance before the shared memory can be handed to another CTA.
+        atomicAdd(timeouts, 1u);
+        for (uint32_t j = k; j < k + kStages && u < T.tiles; ++j, u += step)
+            mbar_wait(smem_u32(&sh.bar[j % kStages]), (j / kStages) & 1, T.poll_limit);
     }
 }
 
@@ -137,8 +190,7 @@ struct EntryHost {
 };
 
 template <int BITS, int DTYPE, int CAP>
-cudaError_t launch_entries_inst(const SegEntryTable<CAP>& ent, const QuantizeArgs& a, const TmaQuantizeConsts& c,
-                                uint32_t total_tiles, unsigned int* timeouts, cudaStream_t stream)
+cudaError_t launch_entries_inst(const SegEntryTable<CAP>& tab, unsigned int* timeouts, cudaStream_t stream)
 {
     auto kernel = encode_entries_kernel<BITS, DTYPE, CAP>;
     static std::atomic<int> grid_cap[64];          // per device; 0 = not yet queried (zero-initialised)
@@ -157,8 +209,8 @@ cudaError_t launch_entries_inst(const SegEntryTable<CAP>& ent, const QuantizeArg
         grid_cap[dev].store(cap, std::memory_order_relaxed);   // every thread computes the same value
     }
     unsigned grid = (unsigned)cap;
-    if (grid > total_tiles) grid = total_tiles;
-    return launch_pdl(kernel, grid, 128, stream, ent, a, c, total_tiles, timeouts);
+    if (grid > tab.tiles) grid = tab.tiles;
+    return launch_pdl(kernel, grid, 128, stream, tab, timeouts);
 }
 
 template <int CAP>
@@ -167,38 +219,34 @@ cudaError_t launch_entries(const EntryHost* entries, int nent, int bits, const R
 {
     unsigned int* timeouts = wait_timeout_counter();
     if (timeouts == nullptr) return cudaErrorNotSupported;
-    QuantizeArgs a;
-    memset(&a, 0, sizeof(a));
-    a.tile_rows = 128; a.rows_per_bucket = 128; a.buckets_per_tile = 1; a.nbuckets = 1;
+    SegEntryTable<CAP> tab;
     const WaitPolicy policy = wait_policy();
-    a.poll_limit = policy.poll_limit;
-    a.arm_only = policy.arm_only;
-    TmaQuantizeConsts c;
-    memset(&c, 0, sizeof(c));
-    c.rk = rk;
-    SegEntryTable<CAP> ent;
-    ent.nent = nent;
-    uint64_t total = 0;
+    tab.poll_limit = policy.poll_limit;
+    tab.arm_only = policy.arm_only;
+    tab.rk = rk;
+    const uint32_t row_elems = dtype == 0 ? 32 : 64;
+    uint64_t tiles = 0;
     for (int i = 0; i < nent; ++i) {
         const EntryHost& h = entries[i];
-        SegEntry& e = ent.e[i];
-        const uint64_t nrows = (h.n + 31) / 32, nrows_full = h.n / 32;
+        SegEntry& e = tab.e[i];
         const char* why = nullptr;
-        if (!encode_rows_map(&ent.map[i], h.grad, nrows_full, dtype == 0 ? 4 : 2, 32, 128, &why))
+        if (!encode_rows_map(&tab.map[i], h.grad, h.n / row_elems, dtype == 0 ? 4 : 2, row_elems, 128, &why))
             return cudaErrorNotSupported;
         e.grad = h.grad; e.codes = h.codes; e.scale = h.scale; e.n = h.n;
-        e.ntiles = (uint32_t)((nrows + 127) / 128);
-        e.full_tiles = (uint32_t)(nrows_full / 128);
+        e.tile0 = (uint32_t)tiles;
+        tiles += (h.n + 128 * row_elems - 1) / (128 * row_elems);
+        if (tiles > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+        tab.tile_end[i] = (uint32_t)tiles;
         const uint64_t blk0 = h.elem_offset >> 3;
         e.blk0_lo = (uint32_t)blk0;
         e.head = philox_head((uint32_t)(blk0 >> 32), h.worker, rk.k0[0]);
-        total += e.ntiles;
     }
-    if (total > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+    for (int i = nent; i < CAP; ++i) tab.tile_end[i] = 0xFFFFFFFFu;
+    tab.tiles = (uint32_t)tiles;
     switch (bits) {
 #define MQG_ENT_CASE(B) \
-        case B: return dtype == 0 ? launch_entries_inst<B, 0, CAP>(ent, a, c, (uint32_t)total, timeouts, stream) \
-                                  : launch_entries_inst<B, 1, CAP>(ent, a, c, (uint32_t)total, timeouts, stream)
+        case B: return dtype == 0 ? launch_entries_inst<B, 0, CAP>(tab, timeouts, stream) \
+                                  : launch_entries_inst<B, kBf16Wide, CAP>(tab, timeouts, stream)
         MQG_ENT_CASE(1); MQG_ENT_CASE(2); MQG_ENT_CASE(3); MQG_ENT_CASE(4);
         MQG_ENT_CASE(5); MQG_ENT_CASE(6); MQG_ENT_CASE(7); MQG_ENT_CASE(8);
 #undef MQG_ENT_CASE
