@@ -69,12 +69,15 @@ mqg_status check_workers(const uint32_t* const* codes, const float* const* scale
 
 uint64_t eff_bucket(uint64_t n, uint64_t bucket) { return bucket < n ? bucket : n; }
 
-// (min, max) shapes outside the one-pass kernel: a bucket per CTA where it fills the CTA's warps, or where the
-// gradient is so short that one launch instead of four decides.
-bool range_spans_preferred(uint64_t n, uint64_t bucket)
+// Shapes outside the one-pass kernel, for several workers (few elements, a bucket of an odd number of rows above 128, draws
+// off a block boundary): a bucket per CTA, all workers in one launch, where a bucket fills the CTA's warps or there are
+// so few of them that one launch instead of W decides (n = 6581, one bucket, W = 8: 25 us in eight launches); the
+// (min, max) variant also for one worker, which takes four launches otherwise.
+bool worker_spans_preferred(uint64_t n, uint64_t bucket)
 {
     return mqg::bucket_spans_apply(n, bucket) && (eff_bucket(n, bucket) > 4096 || n < 65536);
 }
+
 
 mqg_status check_segments(int nseg, const uint64_t* seg_off, const uint64_t* code_off, int bits)
 {
@@ -252,7 +255,7 @@ mqg_status mqg_quantize_workers(const void* const* grads, int W, uint64_t n, int
         if (err != cudaSuccess) return cuda_fail("mqg_quantize_workers", err);
         return MQG_OK;
     }
-    if (W > 1 && eff_bucket(n, bucket) > (uint64_t)mqg::kMaxFusedBucket && mqg::bucket_spans_apply(n, bucket)) {
+    if (W > 1 && worker_spans_preferred(n, bucket)) {
         const cudaError_t err = mqg::launch_bucket_spans(grads, W, n, bits, bucket, seed, codes, scales, 0, (int)dtype,
                                                          first_worker, step, elem_offset, stream);
         if (err != cudaSuccess) return cuda_fail("mqg_quantize_workers", err);
@@ -281,7 +284,7 @@ mqg_status mqg_quantize_minmax(const void* grad, uint64_t n, int bits, uint64_t 
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const cudaError_t err = mqg::quantize_range_fused_applies(n, bucket)
         ? mqg::launch_quantize_range_fused(grad, n, bits, bucket, codes, ranges, (int)dtype, stream)
-        : range_spans_preferred(n, bucket)
+        : worker_spans_preferred(n, bucket)
         ? mqg::launch_bucket_spans(&grad, 1, n, bits, bucket, 0, &codes, &ranges, 1, (int)dtype, 0, 0, 0, stream)
         : mqg::launch_quantize_range_general(grad, n, bits, bucket, codes, ranges, (int)dtype, stream);
     if (err != cudaSuccess) return cuda_fail("mqg_quantize_minmax", err);
@@ -313,7 +316,7 @@ mqg_status mqg_quantize_workers_minmax(const void* const* grads, int W, uint64_t
         if (err != cudaSuccess) return cuda_fail("mqg_quantize_workers_minmax", err);
         return MQG_OK;
     }
-    if (range_spans_preferred(n, bucket)) {
+    if (worker_spans_preferred(n, bucket)) {
         const cudaError_t err = mqg::launch_bucket_spans(grads, W, n, bits, bucket, 0, codes, ranges, 1, (int)dtype, 0, 0, 0,
                                                          stream);
         if (err != cudaSuccess) return cuda_fail("mqg_quantize_workers_minmax", err);
@@ -539,7 +542,13 @@ mqg_status mqg_quantize_workers_l2(const void* const* grads, int W, uint64_t n, 
         if (err != cudaSuccess) return cuda_fail("mqg_quantize_workers_l2", err);
         return MQG_OK;
     }
-    // shapes the batched kernel does not take: one launch per worker, same results
+    if (W > 1 && worker_spans_preferred(n, bucket)) {
+        const cudaError_t err = mqg::launch_bucket_spans(grads, W, n, bits, bucket, seed, codes, scales, 2, (int)dtype,
+                                                         first_worker, step, elem_offset, stream);
+        if (err != cudaSuccess) return cuda_fail("mqg_quantize_workers_l2", err);
+        return MQG_OK;
+    }
+    // shapes the batched kernels do not take: one launch per worker, same results
     for (int w = 0; w < W; ++w) {
         const mqg_status st = mqg_quantize_l2(grads[w], n, bits, bucket, seed, codes[w], scales[w], dtype,
                                               first_worker + (uint32_t)w, step, elem_offset, cuda_stream);

@@ -3,8 +3,11 @@
 // again with the same bit width for the broadcast -- in one pass, so the fp32 global gradient
 // never touches HBM.  A thread owns a row of 32 elements; a CTA owns whole buckets: the row sums
 // stay in registers while the bucket maximum is found, then are encoded and packed.
+#include <atomic>
+
 #include "mqg_common.cuh"
 #include "mqg_internal.h"
+#include "mqg_tma.cuh"
 
 namespace mqg {
 
@@ -14,7 +17,7 @@ struct RequantArgs {
     float* scales_out;
     uint64_t n, nrows, nbuckets, ncode_words;
     uint32_t rows_per_bucket, tile_rows, buckets_per_tile;
-    uint32_t full_tiles;         // leading tiles whose 256 rows are all complete
+    uint32_t full_tiles;         // leading tiles whose tile_rows rows are all complete
     int W;
     float mean_scale;
     uint32_t bias_bits;          // 0x4B000000 (2^23), a run-time constant for the byte permutes
@@ -47,7 +50,7 @@ __device__ __forceinline__ void staged_row_words(const uint32_t* __restrict__ p,
     }
 }
 
-// One tile.  FULL: every thread owns a complete row (vector loads, no bounds checks).  TABLE: the
+// One tile.  FULL: every row of the tile is complete (vector loads, no bounds checks).  TABLE: the
 // de-quantization constants come from the shared table.  STAGE (full tiles only): all workers' code
 // words of the tile are copied into shared memory by 16-byte asynchronous copies at the start, so
 // that no worker's decode waits for a global load.
@@ -59,16 +62,16 @@ __device__ __forceinline__ void requantize_tile(const RequantArgs& a, uint32_t* 
     const uint64_t row0 = (uint64_t)blockIdx.x * a.tile_rows;
     const uint64_t rows_left = a.nrows - row0;
     const uint32_t rows = FULL ? a.tile_rows : (uint32_t)(rows_left < a.tile_rows ? rows_left : a.tile_rows);
-    const bool active = FULL || t < rows;
+    const bool active = t < rows;
     const uint64_t row = row0 + t;
     const uint32_t local_bucket = t / a.rows_per_bucket;
     const uint64_t bucket = (uint64_t)blockIdx.x * a.buckets_per_tile + local_bucket;
 
     constexpr uint32_t kWorkerWords = kMaxTileRows * BITS;      // one worker's words of a full tile
     if constexpr (FULL && STAGE) {
-        const uint32_t chunks = (uint32_t)a.W * (kWorkerWords / 4);
+        const uint32_t per = a.tile_rows * BITS / 4, chunks = (uint32_t)a.W * per;
         for (uint32_t idx = t; idx < chunks; idx += kMaxTileRows) {
-            const uint32_t w = idx / (kWorkerWords / 4), c = idx - w * (kWorkerWords / 4);
+            const uint32_t w = idx / per, c = idx - w * per;
             cp_async16(s_codes + w * kWorkerWords + 4 * c, a.ptrs.codes[w] + row0 * BITS + 4 * c);
         }
     }
@@ -130,7 +133,12 @@ __device__ __forceinline__ void requantize_tile(const RequantArgs& a, uint32_t* 
     if ((rpb & (rpb - 1)) == 0 && rpb <= 32) {
         for (uint32_t d = rpb >> 1; d > 0; d >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
     } else {
-        if (active) atomicMax(&s_bucket[local_bucket], m);
+        if (rpb % 32 == 0) {                       // whole warps: one atomic per warp
+            m = __reduce_max_sync(0xFFFFFFFFu, m);
+            if ((t & 31) == 0 && active) atomicMax(&s_bucket[local_bucket], m);
+        } else if (active) {
+            atomicMax(&s_bucket[local_bucket], m);
+        }
         __syncthreads();
         m = active ? s_bucket[local_bucket] : 0u;
     }
@@ -145,7 +153,7 @@ __device__ __forceinline__ void requantize_tile(const RequantArgs& a, uint32_t* 
     // Philox block of the row's first element: 4 * row (64-bit; the downlink draws from position 0)
     draw_row_blocks((uint32_t)(row << 2), (uint32_t)(row >> 30), a.rk, h);
     uint32_t w[BITS];
-    encode_pack_row<BITS>(x, es, h, w);
+    encode_pack_row_best<BITS>(x, es, h, w);
     const uint64_t word0 = row * BITS;
     if (FULL || row * 32 + 32 <= a.n) {
         store_row_words<BITS>(a.codes_out, word0, w);
@@ -164,6 +172,8 @@ requantize_kernel(const __grid_constant__ RequantArgs a)
     extern __shared__ __align__(16) uint32_t s_codes[];        // STAGE: W x 256 x BITS words
     __shared__ uint32_t s_bucket[kMaxTileRows];
     __shared__ float2 s_table[TABLE ? kMaxWorkers : 1][kTableBuckets];
+    grid_dependency_release();
+    grid_dependency_wait();
     if (blockIdx.x < a.full_tiles) requantize_tile<BITS, true, TABLE, STAGE>(a, s_bucket, s_table, s_codes);
     else requantize_tile<BITS, false, TABLE, STAGE>(a, s_bucket, s_table, s_codes);
 }
@@ -176,19 +186,16 @@ template <int BITS>
 static cudaError_t launch_requantize_bits(const RequantArgs& a, unsigned grid, cudaStream_t stream)
 {
     if (a.buckets_per_tile > (uint32_t)kTableBuckets) {
-        requantize_kernel<BITS, false, false><<<grid, kMaxTileRows, 0, stream>>>(a);
-        return cudaGetLastError();
+        return launch_pdl(requantize_kernel<BITS, false, false>, grid, kMaxTileRows, stream, a);
     }
     // Measured per width at n = 25 M, W = 8 (us per launch, register loads -> staged): 2: 60.6 -> 51.9,
     // 3: 58.4 -> 54.5, 4: 58.6 -> 57.0, 8: 67.9 -> 57.5; 1 unchanged; 5, 6, 7 two microseconds slower
     // (their rows are not 8- or 16-byte multiples, so the staged words are read back one by one).
     constexpr bool kStagePays = BITS == 2 || BITS == 3 || BITS == 4 || BITS == 8;
     const size_t staged = (size_t)a.W * kMaxTileRows * BITS * sizeof(uint32_t);
-    if (!kStagePays || a.full_tiles == 0 || staged > kMaxStagedCodeBytes) {
-        requantize_kernel<BITS, true, false><<<grid, kMaxTileRows, 0, stream>>>(a);
-        return cudaGetLastError();
-    }
-    static bool configured[64] = {};                           // per device
+    if (!kStagePays || a.full_tiles == 0 || staged > kMaxStagedCodeBytes || a.tile_rows * BITS % 4 != 0)
+        return launch_pdl(requantize_kernel<BITS, true, false>, grid, kMaxTileRows, stream, a);
+    static std::atomic<bool> configured[64];                   // per device (zero-initialised)
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
@@ -199,8 +206,7 @@ static cudaError_t launch_requantize_bits(const RequantArgs& a, unsigned grid, c
         if (err != cudaSuccess) return err;
         configured[dev] = true;
     }
-    requantize_kernel<BITS, true, true><<<grid, kMaxTileRows, staged, stream>>>(a);
-    return cudaGetLastError();
+    return launch_pdl_smem(requantize_kernel<BITS, true, true>, grid, kMaxTileRows, staged, stream, a);
 }
 
 cudaError_t launch_requantize(const WorkerPtrs& ptrs, int W, int bits, uint64_t n, uint64_t bucket,
@@ -230,7 +236,7 @@ cudaError_t launch_requantize(const WorkerPtrs& ptrs, int W, int bits, uint64_t 
     a.rk.worker = worker; a.rk.step = step;
     const uint64_t ntiles = (a.nrows + a.tile_rows - 1) / a.tile_rows;
     if (ntiles > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    a.full_tiles = a.tile_rows == (uint32_t)kMaxTileRows ? (uint32_t)((n / 32) / a.tile_rows) : 0u;
+    a.full_tiles = (uint32_t)((n / 32) / a.tile_rows);
     const unsigned grid = (unsigned)ntiles;
     switch (bits) {
         case 1: return launch_requantize_bits<1>(a, grid, stream);
