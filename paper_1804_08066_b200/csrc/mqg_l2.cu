@@ -46,7 +46,6 @@ l2_quantize_kernel(const __grid_constant__ L2Args a)
     const uint64_t rows_left = a.nrows - row0;
     const int rows = (int)(rows_left < a.tile_rows ? rows_left : a.tile_rows);
 
-    grid_dependency_release();
     grid_dependency_wait();
     if constexpr (DTYPE == 0)
         load_tile_f32<kMaxTileRows>(tile, static_cast<const float*>(a.grad) + row0 * 32,
@@ -103,7 +102,6 @@ l2_partials_kernel(const void* __restrict__ grad, const __grid_constant__ Segmen
     __shared__ float s_part[kMaxTileRows / 32];
     const uint32_t t = threadIdx.x;
     const TileGeom g = locate_tile<1>(tab, blockIdx.x);
-    grid_dependency_release();
     grid_dependency_wait();
     if constexpr (DTYPE == 0)
         load_tile_f32<kMaxTileRows>(tile, static_cast<const float*>(grad) + g.elem0, g.valid, g.rows);
@@ -133,7 +131,6 @@ l2_finish_kernel(const __grid_constant__ SegmentTable tab, float* __restrict__ p
     const uint32_t seg = blockIdx.x, t = threadIdx.x;
     const uint64_t first = tab.tile_start[seg];
     uint64_t count = tab.tile_start[seg + 1] - first;
-    grid_dependency_release();
     grid_dependency_wait();
     if (count == 0) return;                        // a segment that another kernel has taken
     float* p = partial + first;

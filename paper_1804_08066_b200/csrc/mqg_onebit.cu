@@ -84,7 +84,6 @@ onebit_ef_kernel(const __grid_constant__ OneBitArgs a)
     const uint64_t row0 = (uint64_t)blockIdx.x * a.tile_rows;
     const uint64_t rows_left = a.nrows - row0;
     const int rows = (int)(rows_left < a.tile_rows ? rows_left : a.tile_rows);
-    grid_dependency_release();
     grid_dependency_wait();
     stage_tiles<DTYPE, THREADS>(tile_g, tile, a, row0 * 32, rows);
     __syncthreads();

@@ -50,7 +50,6 @@ quantize_pack_kernel(const __grid_constant__ QuantizeArgs a)
     const int rows = (int)(rows_left < a.tile_rows ? rows_left : a.tile_rows);
 
     if (t < a.buckets_per_tile) s_bucket[t] = 0u;
-    grid_dependency_release();
     grid_dependency_wait();
     if constexpr (DTYPE == 0)
         load_tile_f32<kMaxTileRows>(tile, static_cast<const float*>(a.grad) + row0 * 32,
@@ -122,7 +121,6 @@ quantize_tma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
     }
     init_slots<DTYPE, THREADS>(sh);
     if (t == 0) prefetch_tensormap(&tmap);
-    grid_dependency_release();
     __syncthreads();
     grid_dependency_wait();            // nothing above touches global memory
     uint32_t tile = blockIdx.x;

@@ -41,7 +41,6 @@ quantize_workers_kernel(const __grid_constant__ WorkerTable tab, const __grid_co
         fence_barrier_init();
     }
     init_slots<DTYPE, THREADS>(sh);
-    grid_dependency_release();
     __syncthreads();
     grid_dependency_wait();            // nothing above touches global memory
 

@@ -172,7 +172,6 @@ requantize_kernel(const __grid_constant__ RequantArgs a)
     extern __shared__ __align__(16) uint32_t s_codes[];        // STAGE: W x 256 x BITS words
     __shared__ uint32_t s_bucket[kMaxTileRows];
     __shared__ float2 s_table[TABLE ? kMaxWorkers : 1][kTableBuckets];
-    grid_dependency_release();
     grid_dependency_wait();
     if (blockIdx.x < a.full_tiles) requantize_tile<BITS, true, TABLE, STAGE>(a, s_bucket, s_table, s_codes);
     else requantize_tile<BITS, false, TABLE, STAGE>(a, s_bucket, s_table, s_codes);

@@ -61,7 +61,6 @@ span_kernel(const __grid_constant__ TableArgs a, const __grid_constant__ SpanTab
     constexpr int kWarps = THREADS / 32;
     __shared__ uint32_t s_a[kMaxSpanRows / 32], s_b[kWarps];   // kSpanNorm: a sum per 32 rows, else a word per warp
     const uint32_t t = threadIdx.x, lane = t & 31u, wid = t >> 5, w = blockIdx.y;
-    grid_dependency_release();
     grid_dependency_wait();
 
     uint64_t elem0, len, code0, scale_idx;
@@ -157,7 +156,6 @@ absmax_table_kernel(const __grid_constant__ TableArgs a, const __grid_constant__
     __shared__ uint32_t s_warp[THREADS / 32];
     const TileGeom g = locate_tile<1>(tab, blockIdx.x);
     const uint64_t count = g.valid < (uint64_t)(kMaxTileRows * 32) ? g.valid : (uint64_t)(kMaxTileRows * 32);
-    grid_dependency_release();
     grid_dependency_wait();
 
     using T = typename std::conditional<DTYPE == 0, float, uint16_t>::type;
@@ -217,7 +215,6 @@ encode_table_kernel(const __grid_constant__ TableArgs a, const __grid_constant__
     const TileGeom g = locate_tile<BITS>(tab, blockIdx.x >> 1);
     const int r0 = (int)(blockIdx.x & 1u) * kEncodeThreads, t = (int)threadIdx.x;
     const uint32_t w = blockIdx.y;
-    grid_dependency_release();
     grid_dependency_wait();
     if (r0 >= g.rows) return;
     const uint64_t elem0 = g.elem0 + 32ull * r0, valid = g.valid - 32ull * r0;

@@ -68,7 +68,6 @@ encode_entries_kernel(const __grid_constant__ SegEntryTable<CAP> T, unsigned int
         for (uint32_t s = 0; s < kStages; ++s) { mbar_init(smem_u32(&sh.bar[s]), 1); sh.read[s] = 0u; }
         fence_barrier_init();
     }
-    grid_dependency_release();
     __syncthreads();
     grid_dependency_wait();            // nothing above touches global memory
 

@@ -93,7 +93,6 @@ server_direct_kernel(const __grid_constant__ DirectArgs a, const __grid_constant
     // words that hold K bytes which start at any byte of the first one (K = 1, 2, 4, 8: inside one / two words)
     constexpr int kWords = BITS == 1 || BITS == 2 || BITS == 4 ? 1 : BITS == 7 ? 3 : 2;
     constexpr int kBatch = 8;
-    grid_dependency_release();
     grid_dependency_wait();
 
     // threads beyond the end keep going with clamped addresses: the warp's shuffles need them
@@ -289,7 +288,6 @@ apply_kernel(float* __restrict__ params, const float* __restrict__ acc, float lr
     const float nlr = -lr;
     const uint64_t n4 = n / 4;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    grid_dependency_release();
     grid_dependency_wait();
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
         float4 p = __ldcg(reinterpret_cast<const float4*>(params) + i);

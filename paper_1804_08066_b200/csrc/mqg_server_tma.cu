@@ -673,12 +673,8 @@ static cudaError_t launch_server_tma_inst(const void* params, ServerTmaArgs& a, 
     CUtensorMap map_full;
     const char* why = nullptr;
     if (!encode_rows_map(&map_full, params, a.nrows_full, 4, 32, kSrvTileRows, &why)) return cudaErrorNotSupported;
-    // Launched as a programmatic dependent of the kernel before it, WITHOUT releasing its own dependents
-    // early: the launch is set up while that kernel still runs and starts the moment its last CTA has
-    // gone (2.2 us per launch at every bit width, eight launches back to back).  Releasing the
-    // dependents at the top of the kernel, as the quantize kernels do, loses that again: the next
-    // launch's CTAs then take the SMs in the order in which this launch's CTAs retire, and the even
-    // split of the tiles over the SMs is gone.
+    // Launched as a programmatic dependent of the kernel before it (2.2 us per launch at every bit width, eight
+    // launches back to back).
     return launch_pdl_smem(kernel, (unsigned)grid, kSrvThreads, kSmemBytes, stream, map_full, a, timeouts);
 }
 

@@ -103,14 +103,15 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map)
     asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
 
-// Programmatic dependent launch.  A kernel launched with launch_pdl() may begin while the
-// previous kernel of the stream is still draining: its CTAs become resident as the earlier
-// kernel's CTAs retire and run their set-up, then block in grid_dependency_wait() until the
-// earlier kernel has completed and its writes are visible.  Every access to global memory must
-// come after that wait.  grid_dependency_release() lets the NEXT kernel be scheduled early in
-// the same way.
+// Programmatic dependent launch.  A kernel launched with launch_pdl() is set up while the previous kernel of
+// the stream is still running, starts the moment that kernel's last CTA has gone, and blocks in
+// grid_dependency_wait() until its writes are visible.  Every access to global memory must come after
+// that wait.  No kernel releases its dependents early (griddepcontrol.launch_dependents): the next launch's
+// CTAs then take the SMs in the order in which this launch's CTAs retire and crowd on those that come free
+// first.  Without it a step on 300,000 elements, W = 8, takes 6.9 against 9.1 us (batched quantize, server), on
+// 2^20, W = 4, 8.3 against 9.2 us, the per-layer quantizer of 11 M elements, W = 2, 74 against 79 us; long
+// launches are the same.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dependency_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---- host side ------------------------------------------------------------------------
 template <typename... KArgs, typename... Args>
