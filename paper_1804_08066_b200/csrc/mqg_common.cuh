@@ -659,6 +659,7 @@ __device__ __forceinline__ void store_tile_f32(const float4* tile, float* __rest
 // De-quantization.  Constants of one (worker, bucket): x^ = fma(q - (L-1)/2, 2h, -h) with
 // h = fl(s / L).  The product (q - (L-1)/2) * 2h and the subtraction of h are exact inside
 // the fma, so its single rounding is the rounding of (2q - L) * h.  A zero scale gives +0.
+// With one bit x^ = +-s, and 2h is no finite float when s > 2^127: one_bit_value sets the sign of s instead.
 // ---------------------------------------------------------------------------------
 struct DecodeScale {
     float two_h, minus_h;
@@ -690,6 +691,16 @@ __device__ __forceinline__ DecodeScale decode_scale(float s)
     return d;
 }
 
+// One bit: the value of the code in bit 31 of `code31`.  A zero scale gives -0, which adds nothing to a sum that is
+// not -0 itself: sums start from +0, or from sum_start of what they continue.  (A mask that gave +0 instead, in the
+// register that is free here, cost the server step of 60 M parameters and 16 workers 131 against 122 us.)
+__device__ __forceinline__ float one_bit_value(float minus_h, uint32_t code31)
+{
+    return __uint_as_float(__float_as_uint(-minus_h) | (~code31 & 0x80000000u));
+}
+template <int BITS, bool RANGE = false>
+__device__ __forceinline__ float sum_start(float x) { return BITS == 1 && !RANGE ? __fadd_rn(x, 0.0f) : x; }   // -0 -> +0
+
 // (min, max) variant: (two_h, minus_h) := (step, lo), step = fl(r / L), 0 for a constant bucket.
 template <int BITS>
 __device__ __forceinline__ DecodeScale range_decode_scale(float lo, float hi)
@@ -715,6 +726,7 @@ __device__ __forceinline__ DecodeScale range_decode_scale(float lo, float hi)
 template <int BITS, bool RANGE = false>
 __device__ __forceinline__ float2 accumulate2(float2 v, float2 m, float2 two_h, float2 minus_h)
 {
+    static_assert(RANGE || BITS > 1, "one_bit_value");
     constexpr float kNegOff = RANGE ? -8388608.0f
                                     : -(8388608.0f + (float)(((1 << BITS) - 2) / 2));   // -(2^23 + (L - 1) / 2)
     const float2 qi = __fadd2_rn(m, make_float2(kNegOff, kNegOff));             // q - (L - 1) / 2, exact
@@ -729,21 +741,17 @@ __device__ __forceinline__ float byte_to_biased(uint32_t v, int byte, uint32_t b
     return __uint_as_float(__byte_perm(v, bias, 0x7650 + byte));
 }
 
-// v2[] <- v2[] + de-quantized row; v2[p] holds the running sums of elements 2p and 2p+1 (+0
-// before the first worker: 0 + x^ is exact, and turns the -0 of a zero-scale bucket into +0).
+// v2[] <- v2[] + de-quantized row; v2[p] holds the running sums of elements 2p and 2p+1 (+0, or
+// sum_start of the sum to continue, before the first worker).
 template <int BITS, bool RANGE = false>
 __device__ __forceinline__ void add_decoded_row(const uint32_t (&w)[BITS], const DecodeScale2& d,
                                                 float2 (&v2)[16], uint32_t bias = 0x4B000000u)
 {
     if constexpr (BITS == 1 && !RANGE) {
-        // x^ = +-s (s = h for one bit): set the sign where the code bit is 0
-        const uint32_t sbits = __float_as_uint(-d.minus_h.x);
 #pragma unroll
-        for (int p = 0; p < 16; ++p) {
-            const uint32_t s0 = (~(w[0] << (31 - 2 * p))) & 0x80000000u;
-            const uint32_t s1 = (~(w[0] << (30 - 2 * p))) & 0x80000000u;
-            v2[p] = __fadd2_rn(v2[p], make_float2(__uint_as_float(sbits | s0), __uint_as_float(sbits | s1)));
-        }
+        for (int p = 0; p < 16; ++p)
+            v2[p] = __fadd2_rn(v2[p], make_float2(one_bit_value(d.minus_h.x, w[0] << (31 - 2 * p)),
+                                                  one_bit_value(d.minus_h.x, w[0] << (30 - 2 * p))));
     } else {
         const float2 th = d.two_h, mh = d.minus_h;
         if constexpr (BITS == 8) {

@@ -71,16 +71,23 @@ __device__ __forceinline__ void add_decoded8(const uint32_t (&words)[WORDS], uin
     win[0] = WORDS > 1 ? __funnelshift_r(words[0], words[WORDS > 1 ? 1 : 0], shift) : words[0] >> shift;
     win[1] = WORDS > 2 ? __funnelshift_r(words[1], words[WORDS > 2 ? 2 : 0], shift)
                        : WORDS > 1 ? words[WORDS > 1 ? 1 : 0] >> shift : 0u;
-    const float2 th = make_float2(d.two_h, d.two_h), mh = make_float2(d.minus_h, d.minus_h);
-    auto code = [&](int j) -> float {                             // the float 2^23 + q of code j
-        const int o = j * BITS;
-        const uint32_t q = o + BITS <= 32 ? win[0] >> o : o >= 32 ? win[1] >> (o - 32)
-                                                                  : __funnelshift_r(win[0], win[1], o);
-        return __uint_as_float((q & kMask) | kTwo23);
-    };
+    if constexpr (BITS == 1 && !RANGE) {
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
-        v[p] = accumulate2<BITS, RANGE>(v[p], make_float2(code(2 * p), code(2 * p + 1)), th, mh);
+        for (int p = 0; p < 4; ++p)
+            v[p] = __fadd2_rn(v[p], make_float2(one_bit_value(d.minus_h, win[0] << (31 - 2 * p)),
+                                                one_bit_value(d.minus_h, win[0] << (30 - 2 * p))));
+    } else {
+        const float2 th = make_float2(d.two_h, d.two_h), mh = make_float2(d.minus_h, d.minus_h);
+        auto code = [&](int j) -> float {                             // the float 2^23 + q of code j
+            const int o = j * BITS;
+            const uint32_t q = o + BITS <= 32 ? win[0] >> o : o >= 32 ? win[1] >> (o - 32)
+                                                                      : __funnelshift_r(win[0], win[1], o);
+            return __uint_as_float((q & kMask) | kTwo23);
+        };
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+            v[p] = accumulate2<BITS, RANGE>(v[p], make_float2(code(2 * p), code(2 * p + 1)), th, mh);
+    }
 }
 
 // SEG: tiles come from a segment table (one scale per segment) instead of uniform buckets.
@@ -124,7 +131,11 @@ server_direct_kernel(const __grid_constant__ DirectArgs a, const __grid_constant
     if (a.params != nullptr) load8(a.params + elem0, left, p);
 #pragma unroll
     for (int j = 0; j < 4; ++j) v[j] = make_float2(0.0f, 0.0f);
-    if (a.add_into) load8(a.acc + elem0, left, v);
+    if (a.add_into) {
+        load8(a.acc + elem0, left, v);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = make_float2(sum_start<BITS, RANGE>(v[j].x), sum_start<BITS, RANGE>(v[j].y));
+    }
 
     auto load_scale = [&](int w) -> float2 {
         if (RANGE) return __ldcg(reinterpret_cast<const float2*>(a.ptrs.scales[w]) + scale_idx);
@@ -250,6 +261,8 @@ server_row_kernel(const __grid_constant__ ServerArgs a)
             load_tile_f32<kMaxTileRows>(tile, acc, valid, rows);
             __syncthreads();
             if (active) read_row(tile, (int)t, v);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = sum_start<BITS>(v[j]);
         }
         if (active) {
             accumulate_row<BITS>(a, scale_idx, word0, words_end, full_row, v, a.add_into != 0);

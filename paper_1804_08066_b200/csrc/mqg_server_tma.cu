@@ -268,7 +268,7 @@ __device__ __noinline__ void server_ragged_row(const ServerTmaArgs& a, float* pa
     const uint64_t word = code_word0 + (uint64_t)row * BITS + (bit >> 5);
     const bool two = shift + BITS > 32 && word + 1 < words_end;
     const float old = MODE != 0 ? params[e] : 0.0f;
-    float2 v = make_float2(MODE == 2 ? old : 0.0f, 0.0f);
+    float2 v = make_float2(MODE == 2 ? sum_start<BITS, RANGE>(old) : 0.0f, 0.0f);
     constexpr int kBatch = 8;
 #pragma unroll 1
     for (int w0 = 0; w0 < a.W; w0 += kBatch) {
@@ -287,8 +287,11 @@ __device__ __noinline__ void server_ragged_row(const ServerTmaArgs& a, float* pa
             if (w0 + i >= a.W) break;
             const DecodeScale d = RANGE ? range_decode_scale<BITS>(sc[i].x, sc[i].y) : decode_scale<BITS>(sc[i].x);
             const uint32_t q = __funnelshift_r(lo[i], hi[i], shift) & ((1u << BITS) - 1u);
-            v = accumulate2<BITS, RANGE>(v, make_float2(__uint_as_float(q | 0x4B000000u), 8388608.0f),
-                                         make_float2(d.two_h, d.two_h), make_float2(d.minus_h, d.minus_h));
+            if constexpr (BITS == 1 && !RANGE)
+                v.x = __fadd_rn(v.x, one_bit_value(d.minus_h, q << 31));
+            else
+                v = accumulate2<BITS, RANGE>(v, make_float2(__uint_as_float(q | 0x4B000000u), 8388608.0f),
+                                             make_float2(d.two_h, d.two_h), make_float2(d.minus_h, d.minus_h));
         }
     }
     params[e] = MODE == 1 ? __fmaf_rn(a.neg_lr, v.x, old) : v.x;
@@ -413,8 +416,8 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 const float4 p = tl[swz((int)lane, c)];
-                v2[2 * c] = make_float2(p.x, p.y);
-                v2[2 * c + 1] = make_float2(p.z, p.w);
+                v2[2 * c] = make_float2(sum_start<BITS, RANGE>(p.x), sum_start<BITS, RANGE>(p.y));
+                v2[2 * c + 1] = make_float2(sum_start<BITS, RANGE>(p.z), sum_start<BITS, RANGE>(p.w));
             }
         } else {
 #pragma unroll
