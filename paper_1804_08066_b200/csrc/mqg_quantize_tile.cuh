@@ -89,7 +89,7 @@ __device__ __forceinline__ float row_abs_max_bf16(const uint32_t (&u)[16])
     for (int d = 4; d > 0; d >>= 1)
 #pragma unroll
         for (int k = 0; k < d; ++k) m[k] = max2(m[k], m[k + d]);
-    return fmaxf(fabsf(bf16_lo(m[0])), fabsf(bf16_hi(m[0])));
+    return max3_abs(0.0f, bf16_lo(m[0]), bf16_hi(m[0]));      // from 0: a row that is NaN throughout does not count
 }
 
 // The one row of the gradient that is shorter than 32 elements is not covered by the tensor
