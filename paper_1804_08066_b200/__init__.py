@@ -117,21 +117,34 @@ _NATIVE = frozenset((
     "mqg_quantize_1bit_ef"))
 
 
+def _native(name):
+    """The native function `name`; the first call loads them all."""
+    if name not in globals():
+        for path in (LIB_PATH, os.path.join(_HERE, "_binding.so")):
+            if not os.path.exists(path):
+                raise ImportError(_NOT_BUILT % (os.path.basename(path), path))
+        import importlib
+
+        import torch  # noqa: F401  (its libraries have to be loaded before the native module's)
+        native = importlib.import_module(__name__ + "._binding")
+        native._set_error_class(MqgError)
+        for fn in _NATIVE:
+            getattr(native, fn).__module__ = __name__      # found here when a pickle names it
+            globals()[fn] = getattr(native, fn)
+    return globals()[name]
+
+
 def __getattr__(name):
     """Loads the native functions when the first of them is asked for, not at import (as _LazyLibrary)."""
     if name not in _NATIVE:
         raise AttributeError("module %r has no attribute %r" % (__name__, name))
-    for path in (LIB_PATH, os.path.join(_HERE, "_binding.so")):
-        if not os.path.exists(path):
-            raise ImportError(_NOT_BUILT % (os.path.basename(path), path))
-    import importlib
-
-    import torch  # noqa: F401  (its libraries have to be loaded before the native module's)
-    native = importlib.import_module(__name__ + "._binding")
-    native._set_error_class(MqgError)
-    for fn in _NATIVE:
-        globals()[fn] = getattr(native, fn)
-    return globals()[name]
+    try:
+        return _native(name)
+    except ImportError:
+        def not_built(*args, **kwargs):                    # the name is there all the same; a call says what is missing
+            return _native(name)(*args, **kwargs)
+        not_built.__name__ = not_built.__qualname__ = name
+        return not_built
 
 
 def __dir__():
@@ -190,3 +203,6 @@ def raw_library() -> C.CDLL:
     """The ctypes handle, for callers that pass raw device pointers themselves."""
     _lib.mqg_version                       # loads the library if this is its first use
     return _lib._lib
+
+
+__all__ = [_name for _name in __dir__() if not _name.startswith("_")]     # the native functions among them
