@@ -230,13 +230,19 @@ PyObject* finish(mqg_status st)
     return nullptr;
 }
 
-// The call itself runs without the interpreter lock: a full launch queue blocks it.
+// The call itself runs without the interpreter lock: a full launch queue blocks it.  The lock is back whichever way
+// the call ends.
+struct WithoutLock {
+    PyThreadState* state = PyEval_SaveThread();
+    ~WithoutLock() { PyEval_RestoreThread(state); }
+};
 template <typename Fn> PyObject* enqueue(Fn&& fn)
 {
     mqg_status st;
-    Py_BEGIN_ALLOW_THREADS
-    st = fn();
-    Py_END_ALLOW_THREADS
+    {
+        const WithoutLock unlocked;
+        st = fn();
+    }
     return finish(st);
 }
 

@@ -10,7 +10,6 @@
 #include <string.h>
 
 #include <atomic>
-#include <vector>
 
 #include "mqg_quantize_tile.cuh"
 #include "mqg_segments.cuh"
@@ -269,8 +268,8 @@ cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, 
                 return false;
         return true;
     };
-    std::vector<EntryHost> entries;
     cudaError_t err = cudaSuccess;
+    bool any_entries = false;
     uint64_t sums = 0;                                // partial sums of the tables already launched
     for (int first = 0; first < nseg; first += kMaxSegmentsPerLaunch) {
         const int count = nseg - first < kMaxSegmentsPerLaunch ? nseg - first : kMaxSegmentsPerLaunch;
@@ -298,13 +297,8 @@ cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, 
                 if (!workspace) spans.clear[i >> 5] |= 1u << (i & 31);
                 const uint64_t nt = (len + kMaxTileRows * 32 - 1) / (kMaxTileRows * 32);
                 tiles += nt;
-                if (bulk(j)) {
-                    for (int w = 0; w < W; ++w)
-                        entries.push_back({static_cast<const char*>(grads[w]) + seg_off[j] * esz, codes[w] + code_off[j],
-                                           scales[w] + j, len, elem_offset + seg_off[j], first_worker + (uint32_t)w});
-                } else {
-                    plain_tiles += nt;
-                }
+                if (bulk(j)) any_entries = true;
+                else plain_tiles += nt;
             }
             if (tiles > 0x3FFFFFFFull) return cudaErrorInvalidValue;
         }
@@ -325,12 +319,25 @@ cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, 
         if (err == cudaSuccess) err = launch_encode_table(t, plain, bits, dtype, stream);
         if (err != cudaSuccess) return err;
     }
-    const size_t total = entries.size();
-    for (size_t from = 0; from < total && err == cudaSuccess; from += (size_t)kMaxEntries) {
-        const int n = (int)(total - from < (size_t)kMaxEntries ? total - from : (size_t)kMaxEntries);
-        err = n <= kFewEntries ? launch_entries<kFewEntries>(entries.data() + from, n, bits, a.rk, dtype, stream)
-                               : launch_entries<kMaxEntries>(entries.data() + from, n, bits, a.rk, dtype, stream);
+    if (!any_entries) return cudaSuccess;
+    // no heap here: the C ABI throws nothing
+    EntryHost batch[kMaxEntries];
+    int n = 0;
+    auto launch = [&] {
+        err = n <= kFewEntries ? launch_entries<kFewEntries>(batch, n, bits, a.rk, dtype, stream)
+                               : launch_entries<kMaxEntries>(batch, n, bits, a.rk, dtype, stream);
+        n = 0;
+    };
+    for (int j = 0; j < nseg && err == cudaSuccess; ++j) {
+        const uint64_t len = seg_off[j + 1] - seg_off[j];
+        if (len <= kSegmentSpanElems || !bulk(j)) continue;
+        for (int w = 0; w < W && err == cudaSuccess; ++w) {
+            batch[n++] = {static_cast<const char*>(grads[w]) + seg_off[j] * esz, codes[w] + code_off[j], scales[w] + j, len,
+                          elem_offset + seg_off[j], first_worker + (uint32_t)w};
+            if (n == kMaxEntries) launch();
+        }
     }
+    if (n != 0 && err == cudaSuccess) launch();
     return err;
 }
 

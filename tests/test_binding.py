@@ -44,3 +44,42 @@ def test_names_exist_where_nothing_is_built(tmp_path):
                   "except ImportError as e:\n"
                   "    print(e)", cwd=tmp_path)
     assert "is not built" in out
+
+
+NO_HEAP = r"""
+#include <cstdlib>
+#include <new>
+extern "C" { int no_heap = 0; }
+void* operator new(std::size_t n)
+{
+    void* p = no_heap ? nullptr : std::malloc(n ? n : 1);
+    if (!p) throw std::bad_alloc();
+    return p;
+}
+void operator delete(void* p) noexcept { std::free(p); }
+void operator delete(void* p, std::size_t) noexcept { std::free(p); }
+"""
+
+
+def test_no_exception_leaves_the_c_abi(tmp_path):
+    """The calls that take segment tables need no memory of the host's heap, however many segments there are."""
+    (tmp_path / "no_heap.cpp").write_text(NO_HEAP)
+    lib = str(tmp_path / "no_heap.so")
+    subprocess.run(["g++", "-O1", "-shared", "-fPIC", str(tmp_path / "no_heap.cpp"), "-o", lib], check=True)
+    out = _python("""
+import ctypes as C
+import paper_1804_08066_b200 as mqg
+lib, no_heap = mqg.raw_library(), C.c_int.in_dll(C.CDLL(%r), "no_heap")
+nseg = 300
+off = (C.c_uint64 * (nseg + 1))(*[65536 * j for j in range(nseg + 1)])       # long segments, all aligned
+p = C.c_void_p(0x10000)                                                      # never dereferenced on the host
+tab = (C.c_void_p * 2)(0x10000, 0x20000)
+quantize = lambda: lib.mqg_quantize_segments_workers(tab, 2, nseg, off, off, 4, 0, tab, tab, 0, 0, 0, 0, None)
+server = lambda: lib.mqg_server_step_segments(tab, tab, 2, 4, nseg, off, off, p, 0.1, None, None)
+st = [quantize(), server()]                                                  # what the first call sets up is done
+no_heap.value = 1
+st += [quantize(), server()]
+no_heap.value = 0
+print(st)
+""" % lib, LD_PRELOAD=lib, CUDA_VISIBLE_DEVICES="")                              # no device: no launch, on any machine
+    assert out.strip() == str([mqg.MQG_ERR_CUDA] * 4)
