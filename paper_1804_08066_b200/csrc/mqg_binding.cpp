@@ -88,6 +88,9 @@ bool to_bool(PyObject* o)
     return v != 0;
 }
 
+// THPVariable_Check asks isinstance(), which an object can answer without being a tensor.
+bool is_tensor(PyObject* o) { return PyObject_TypeCheck(o, reinterpret_cast<PyTypeObject*>(THPVariableClass)); }
+
 // Device pointer of a contiguous CUDA tensor.  `index` >= 0: the tensor is that item of a list.
 void* device_ptr(PyObject* o, const char* what, Py_ssize_t index = -1)
 {
@@ -97,7 +100,7 @@ void* device_ptr(PyObject* o, const char* what, Py_ssize_t index = -1)
         snprintf(name, sizeof(name), "%s[%zd]", what, index);
         return name;
     };
-    if (!THPVariable_Check(o) || !THPVariable_Unpack(o).is_cuda()) {
+    if (!is_tensor(o) || !THPVariable_Unpack(o).is_cuda()) {
         PyErr_Format(PyExc_TypeError, "%s must be a CUDA tensor (libmqgrad has no CPU path)", called());
         throw PythonError();
     }
@@ -111,7 +114,7 @@ void* device_ptr(PyObject* o, const char* what, Py_ssize_t index = -1)
 
 mqg_dtype grad_dtype(PyObject* o)
 {
-    if (THPVariable_Check(o)) {
+    if (is_tensor(o)) {
         const at::ScalarType s = THPVariable_Unpack(o).scalar_type();
         if (s == at::kFloat) return MQG_F32;
         if (s == at::kBFloat16) return MQG_BF16;

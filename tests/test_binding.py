@@ -5,6 +5,10 @@ import pickle
 import shutil
 import subprocess
 import sys
+from unittest.mock import Mock
+
+import pytest
+import torch
 
 import paper_1804_08066_b200 as mqg
 
@@ -83,3 +87,13 @@ no_heap.value = 0
 print(st)
 """ % lib, LD_PRELOAD=lib, CUDA_VISIBLE_DEVICES="")                              # no device: no launch, on any machine
     assert out.strip() == str([mqg.MQG_ERR_CUDA] * 4)
+
+
+def test_objects_that_only_look_like_tensors_are_refused():
+    like = Mock(spec=torch.Tensor)
+    assert isinstance(like, torch.Tensor)
+    for call in (lambda: mqg.mqg_apply(like, like, 0.1, 4),
+                 lambda: mqg.mqg_quantize(like, 0, 4, 32, 0, None, None),
+                 lambda: mqg.mqg_server_step([like], [like], 1, 4, 32, 32, like, 0.1)):
+        with pytest.raises(TypeError, match="tensor"):
+            call()
