@@ -125,7 +125,8 @@ mqg_dtype grad_dtype(PyObject* o)
     throw PythonError();
 }
 
-// A list (or tuple, or any iterable) of W tensors as a table of device pointers.
+// A list (or tuple, or any iterable) of W tensors as a table of device pointers.  Everything that is wanted of the
+// items is read at once: later arguments may run Python code that changes the list.
 struct PointerTable {
     void* ptr[MQG_MAX_WORKERS];
     PyObject* items = nullptr;
@@ -146,65 +147,76 @@ struct PointerTable {
         const Py_ssize_t n = count < MQG_MAX_WORKERS ? count : MQG_MAX_WORKERS;
         for (Py_ssize_t i = 0; i < n; ++i) ptr[i] = device_ptr(PySequence_Fast_GET_ITEM(items, i), what, i);
     }
-    mqg_dtype dtype(bool all_alike) const
+    template <typename T> T* const* as() const { return reinterpret_cast<T* const*>(ptr); }
+};
+
+struct GradientTable : PointerTable {
+    mqg_dtype dtype;
+
+    // `all_alike`: every gradient must have the first one's type.
+    void read(PyObject* o, int W, bool exact, bool all_alike)
     {
+        PointerTable::read(o, "grads", W, exact);
         if (count == 0) {
             PyErr_SetString(PyExc_ValueError, "grads is empty");
             throw PythonError();
         }
-        const mqg_dtype d = grad_dtype(PySequence_Fast_GET_ITEM(items, 0));
+        dtype = grad_dtype(PySequence_Fast_GET_ITEM(items, 0));
         for (Py_ssize_t i = 1; all_alike && i < count; ++i)
-            if (grad_dtype(PySequence_Fast_GET_ITEM(items, i)) != d) {
+            if (grad_dtype(PySequence_Fast_GET_ITEM(items, i)) != dtype) {
                 PyErr_SetString(PyExc_TypeError, "all gradients must have the same dtype");
                 throw PythonError();
             }
-        return d;
     }
-    template <typename T> T* const* as() const { return reinterpret_cast<T* const*>(ptr); }
 };
 
-// A segment table: 64-bit integers from an array that exposes them, or from any sequence of numbers.
+struct Reference {
+    PyObject* object;
+    ~Reference() { Py_XDECREF(object); }
+};
+
+// A segment table: 64-bit integers from an array that exposes them, or from any sequence of numbers.  Copied: the
+// library checks the table and then uses it, without the interpreter lock.
 struct OffsetTable {
     uint64_t inline_store[65];
     std::vector<uint64_t> store;
-    Py_buffer view;
-    bool have_view = false;
     const uint64_t* data = nullptr;
     Py_ssize_t count = 0;
-    ~OffsetTable() { if (have_view) PyBuffer_Release(&view); }
 
     void read(PyObject* o)
     {
-        if (!PyList_Check(o) && !PyTuple_Check(o) && PyObject_CheckBuffer(o)) {
-            if (PyObject_GetBuffer(o, &view, PyBUF_FORMAT | PyBUF_C_CONTIGUOUS) == 0) {
-                have_view = true;
-                if (view.ndim == 1 && view.itemsize == 8 && view.format && view.format[1] == '\0' &&
-                    std::strchr("lLqQ", view.format[0])) {
-                    data = static_cast<const uint64_t*>(view.buf);
-                    count = view.shape ? view.shape[0] : view.len / 8;
-                    return;
-                }
-            } else {
-                PyErr_Clear();
-            }
-        }
-        PyObject* items = PySequence_Fast(o, "a sequence of offsets is expected");
-        if (!items) throw PythonError();
-        count = PySequence_Fast_GET_SIZE(items);
-        uint64_t* to = inline_store;
-        if (count > 65) { store.resize((size_t)count); to = store.data(); }
-        data = to;
+        if (!PyList_Check(o) && !PyTuple_Check(o) && PyObject_CheckBuffer(o) && read_buffer(o)) return;
+        const Reference items = {PySequence_Tuple(o)};  // a list could change while its items are converted
+        if (!items.object) throw PythonError();
+        uint64_t* to = room(PyTuple_GET_SIZE(items.object));
         for (Py_ssize_t i = 0; i < count; ++i) {
-            PyObject* v = PySequence_Fast_GET_ITEM(items, i);
-            PyObject* whole = PyLong_CheckExact(v) ? Py_NewRef(v) : PyNumber_Long(v);
-            if (whole) to[i] = PyLong_AsUnsignedLongLongMask(whole);
-            Py_XDECREF(whole);
-            if (!whole || (to[i] == (uint64_t)-1 && PyErr_Occurred())) {
-                Py_DECREF(items);
-                throw PythonError();
-            }
+            PyObject* v = PyTuple_GET_ITEM(items.object, i);
+            const Reference whole = {PyLong_CheckExact(v) ? Py_NewRef(v) : PyNumber_Long(v)};
+            if (!whole.object) throw PythonError();
+            to[i] = to_u64(whole.object);
         }
-        Py_DECREF(items);
+    }
+
+private:
+    uint64_t* room(Py_ssize_t n)
+    {
+        uint64_t* to = inline_store;
+        if (n > 65) { store.resize((size_t)n); to = store.data(); }
+        data = to;
+        count = n;
+        return to;
+    }
+    bool read_buffer(PyObject* o)
+    {
+        struct View : Py_buffer { ~View() { PyBuffer_Release(this); } } view;       // (releasing an empty one does nothing)
+        if (PyObject_GetBuffer(o, &view, PyBUF_FORMAT | PyBUF_C_CONTIGUOUS) != 0) {
+            PyErr_Clear();
+            return false;
+        }
+        const bool offsets = view.ndim == 1 && view.itemsize == 8 && view.format && view.format[0] != '\0' &&
+                             view.format[1] == '\0' && std::strchr("lLqQ", view.format[0]);
+        if (offsets) std::memcpy(room(view.len / 8), view.buf, (size_t)view.len);
+        return offsets;
     }
 };
 
@@ -298,13 +310,13 @@ template <typename Fn> PyObject* quantize_workers(PyObject** v, Fn fn)
     const int W = to_int(v[1]), bits = to_int(v[3]);
     const uint64_t n = to_u64(v[2]), bucket = to_u64(v[4]), seed = to_u64(v[5]), off = to_u64(v[10]);
     const uint32_t first = to_u32(v[8]), step = to_u32(v[9]);
-    PointerTable g, c, sc;
-    g.read(v[0], "grads", W, true);
+    GradientTable g;
+    PointerTable c, sc;
+    g.read(v[0], W, true, true);
     c.read(v[6], "codes", W, true);
     sc.read(v[7], "scales", W, true);
-    const mqg_dtype dt = g.dtype(true);
     void* s = stream();
-    return enqueue([&] { return fn(g.as<const void>(), W, n, bits, bucket, seed, c.as<uint32_t>(), sc.as<float>(), dt,
+    return enqueue([&] { return fn(g.as<const void>(), W, n, bits, bucket, seed, c.as<uint32_t>(), sc.as<float>(), g.dtype,
                                    first, step, off, s); });
 }
 
@@ -324,14 +336,14 @@ MQG_ENTRY(mqg_quantize_workers_minmax, 0, 7, "grads", "W", "n", "bits", "bucket"
 {
     const int W = to_int(v[1]), bits = to_int(v[3]);
     const uint64_t n = to_u64(v[2]), bucket = to_u64(v[4]);
-    PointerTable g, c, r;
-    g.read(v[0], "grads", W, true);
+    GradientTable g;
+    PointerTable c, r;
+    g.read(v[0], W, true, true);
     c.read(v[5], "codes", W, true);
     r.read(v[6], "ranges", W, true);
-    const mqg_dtype dt = g.dtype(true);
     void* s = stream();
     return enqueue([&] { return ::mqg_quantize_workers_minmax(g.as<const void>(), W, n, bits, bucket, c.as<uint32_t>(),
-                                                              r.as<float>(), dt, s); });
+                                                              r.as<float>(), g.dtype, s); });
 }
 
 MQG_ENTRY(mqg_quantize_minmax, 0, 6, "grad", "n", "bits", "bucket", "codes", "ranges")
@@ -494,14 +506,14 @@ MQG_ENTRY(mqg_quantize_segments_workers, 3, 11, "grads", "W", "seg_off", "code_o
     const int W = to_int(v[1]), nseg = read_segments(v[2], v[3], seg, code), bits = to_int(v[4]);
     const uint64_t seed = to_u64(v[5]), off = to_u64(v[10]);
     const uint32_t first = to_u32(v[8]), step = to_u32(v[9]);
-    PointerTable g, c, sc;
-    g.read(v[0], "grads", W, false);
+    GradientTable g;
+    PointerTable c, sc;
+    g.read(v[0], W, false, false);
     c.read(v[6], "codes", W, false);
     sc.read(v[7], "scales", W, false);
-    const mqg_dtype dt = g.dtype(false);
     void* s = stream();
     return enqueue([&] { return ::mqg_quantize_segments_workers(g.as<const void>(), W, nseg, seg.data, code.data, bits,
-                                                                seed, c.as<uint32_t>(), sc.as<float>(), dt, first, step,
+                                                                seed, c.as<uint32_t>(), sc.as<float>(), g.dtype, first, step,
                                                                 off, s); });
 }
 

@@ -97,3 +97,24 @@ def test_objects_that_only_look_like_tensors_are_refused():
                  lambda: mqg.mqg_server_step([like], [like], 1, 4, 32, 32, like, 0.1)):
         with pytest.raises(TypeError, match="tensor"):
             call()
+
+
+class Shrinking:
+    """A number whose conversion empties the list it stands in."""
+
+    def __init__(self, home):
+        self.home = home
+
+    def __int__(self):
+        self.home.clear()
+        return 0
+
+    __index__ = __int__
+
+
+def test_a_list_that_changes_while_it_is_read():
+    offsets = []
+    offsets += [Shrinking(offsets)] + [10**6 * j for j in range(1, 60)]
+    with pytest.raises(TypeError, match="grad must be a CUDA tensor"):
+        mqg.mqg_quantize_segments(None, offsets, list(range(60)), 4, 0, None, None)
+    assert not offsets
