@@ -139,11 +139,11 @@ struct PointerTable {
         items = PySequence_Fast(o, "a list of tensors is expected");
         if (!items) throw PythonError();
         count = PySequence_Fast_GET_SIZE(items);
-        if (exact ? count != W : count < W) {
+        // a worker count outside the library's range is the C ABI's to reject: it reads no table then
+        if (exact ? count != W : count < W && W <= MQG_MAX_WORKERS) {
             PyErr_Format(PyExc_ValueError, "%s must hold %s%d tensors, got %zd", what, exact ? "" : "at least ", W, count);
             throw PythonError();
         }
-        // a worker count outside the library's range is the C ABI's to reject: it reads no table then
         const Py_ssize_t n = count < MQG_MAX_WORKERS ? count : MQG_MAX_WORKERS;
         for (Py_ssize_t i = 0; i < n; ++i) ptr[i] = device_ptr(PySequence_Fast_GET_ITEM(items, i), what, i);
     }
@@ -158,7 +158,8 @@ struct GradientTable : PointerTable {
     {
         PointerTable::read(o, "grads", W, exact);
         if (count == 0) {
-            PyErr_SetString(PyExc_ValueError, "grads is empty");
+            if (all_alike) PyErr_SetString(PyExc_TypeError, "all gradients must have the same dtype: there are none");
+            else PyErr_SetString(PyExc_IndexError, "grads is empty");
             throw PythonError();
         }
         dtype = grad_dtype(PySequence_Fast_GET_ITEM(items, 0));

@@ -118,3 +118,12 @@ def test_a_list_that_changes_while_it_is_read():
     with pytest.raises(TypeError, match="grad must be a CUDA tensor"):
         mqg.mqg_quantize_segments(None, offsets, list(range(60)), 4, 0, None, None)
     assert not offsets
+
+
+def test_what_empty_lists_of_workers_raise():
+    with pytest.raises(TypeError, match="same dtype"):
+        mqg.mqg_quantize_workers([], 0, 0, 4, 32, 0, [], [])
+    with pytest.raises(TypeError, match="same dtype"):
+        mqg.mqg_quantize_workers_minmax([], 0, 0, 4, 32, [], [])
+    with pytest.raises(IndexError):
+        mqg.mqg_quantize_segments_workers([], 0, [0], [0], 4, 0, [], [])

@@ -40,3 +40,9 @@ def test_offset_arrays_are_copied():
     codes.check_guards(), scales.check_guards()
     assert np.array_equal(scales.numpy(np.float32), s_ref)
     assert np.array_equal(codes.numpy(np.uint32), c_ref)
+
+
+def test_worker_counts_outside_the_range_are_the_library_s_to_reject():
+    with pytest.raises(mqg.MqgError) as err:
+        mqg.mqg_server_step([], [], 40, 4, 0, 32, None, 0.1)
+    assert err.value.status == mqg.MQG_ERR_TOO_MANY_WORKERS
