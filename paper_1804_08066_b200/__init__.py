@@ -107,7 +107,7 @@ def _u64_table(values):
     return (C.c_uint64 * len(vals))(*vals)
 
 
-# The calls that enqueue work are native functions (csrc/mqg_binding.cpp, built as _binding.so): the device is
+# The calls that enqueue work are native functions (csrc/mqg_binding.cpp; its file: build.binding_path): the device is
 # done with a small gradient in less time than Python and ctypes need to marshal a call's arguments.
 _NATIVE = frozenset((
     "mqg_quantize", "mqg_quantize_workers", "mqg_dequant_accumulate", "mqg_apply", "mqg_server_step",
@@ -120,13 +120,16 @@ _NATIVE = frozenset((
 def _native(name):
     """The native function `name`; the first call loads them all."""
     if name not in globals():
-        for path in (LIB_PATH, os.path.join(_HERE, "_binding.so")):
-            if not os.path.exists(path):
-                raise ImportError(_NOT_BUILT % (os.path.basename(path), path))
-        import importlib
+        import importlib.util
 
-        import torch  # noqa: F401  (its libraries have to be loaded before the native module's)
-        native = importlib.import_module(__name__ + "._binding")
+        from .build import binding_path
+        path = binding_path()              # imports torch: its libraries have to be loaded before the native module's
+        for file in (LIB_PATH, path):
+            if not os.path.exists(file):
+                raise ImportError(_NOT_BUILT % (os.path.basename(file), file))
+        spec = importlib.util.spec_from_file_location(__name__ + "._binding", path)
+        native = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(native)
         native._set_error_class(MqgError)
         for fn in _NATIVE:
             getattr(native, fn).__module__ = __name__      # found here when a pickle names it

@@ -1,4 +1,4 @@
-"""Build libmqgrad.so (sm_100a) with nvcc and the Python binding _binding.so with the host compiler, in-tree.
+"""Build libmqgrad.so (sm_100a) with nvcc and the Python binding (binding_path) with the host compiler, in-tree.
 
 Usage: python paper_1804_08066_b200/build.py [--force] [--verbose]
 The shared objects land next to this file; nvcc cross-compiles without a GPU.
@@ -13,13 +13,21 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libmqgrad.so")
-BINDING = os.path.join(HERE, "_binding.so")
 BINDING_SRC = os.path.join(CSRC, "mqg_binding.cpp")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "-shared", "-Xcompiler", "-fPIC", "-I", INCLUDE, "--threads", "4",
 ]
+
+
+def binding_path() -> str:
+    """The binding's file.  It fits one interpreter and one torch, so both are part of its name: after an upgrade of
+    either, the file is not there and is built, instead of a stale one being loaded."""
+    import sysconfig
+
+    import torch
+    return os.path.join(HERE, "_binding.torch-%s%s" % (torch.__version__, sysconfig.get_config_var("EXT_SUFFIX")))
 
 
 def sources():
@@ -42,8 +50,9 @@ def _compile(cmd, target):
 
 def build_binding(force: bool = False) -> str:
     """The native functions of the Python package: torch tensors in, C ABI calls out."""
-    if not force and not _stale(BINDING, [BINDING_SRC, *_headers()]):
-        return BINDING
+    binding = binding_path()
+    if not force and not _stale(binding, [BINDING_SRC, *_headers()]):
+        return binding
     import sysconfig
 
     import torch
@@ -55,8 +64,8 @@ def build_binding(force: bool = False) -> str:
     _compile([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
               "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), *("-I" + d for d in include), BINDING_SRC,
               "-L" + HERE, "-l:libmqgrad.so", "-Wl,-rpath,$ORIGIN",
-              "-L" + torch_lib, "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"], BINDING)
-    return BINDING
+              "-L" + torch_lib, "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"], binding)
+    return binding
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

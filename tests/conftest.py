@@ -9,16 +9,16 @@ if ROOT not in sys.path:
 
 
 def _ensure_library_is_built():
-    """The binding refuses to import without libmqgrad.so (there is no fallback path), so a fresh
-    checkout builds it here once; nvcc cross-compiles without a GPU."""
-    lib = os.path.join(ROOT, "paper_1804_08066_b200", "libmqgrad.so")
-    if os.path.exists(lib):
-        return
+    """The package refuses its calls without libmqgrad.so and the binding for this interpreter and
+    torch (there is no fallback path), so a checkout that lacks either builds it here once; nvcc
+    cross-compiles without a GPU.  (Files that are older than their sources are left alone: a copy
+    of a built tree need not keep the times.)"""
     import importlib.util
     spec = importlib.util.spec_from_file_location("_mqg_build", os.path.join(ROOT, "paper_1804_08066_b200", "build.py"))
     mod = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(mod)
-    mod.build()
+    if not os.path.exists(mod.LIB) or not os.path.exists(mod.binding_path()):
+        mod.build()
 
 
 _ensure_library_is_built()

@@ -5,6 +5,7 @@ import pickle
 import shutil
 import subprocess
 import sys
+import sysconfig
 from unittest.mock import Mock
 
 import pytest
@@ -127,3 +128,20 @@ def test_what_empty_lists_of_workers_raise():
         mqg.mqg_quantize_workers_minmax([], 0, 0, 4, 32, [], [])
     with pytest.raises(IndexError):
         mqg.mqg_quantize_segments_workers([], 0, [0], [0], 4, 0, [], [])
+
+
+def test_the_binding_fits_one_interpreter_and_one_torch(monkeypatch):
+    from paper_1804_08066_b200 import build
+    here = build.binding_path()
+    assert os.path.exists(here) and here.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    assert mqg.mqg_quantize.__self__.__file__ == here
+    monkeypatch.setattr(torch, "__version__", "9.8.7")
+    assert "9.8.7" in build.binding_path() and not os.path.exists(build.binding_path())
+    out = _python("import torch\n"
+                  "torch.__version__ = '9.8.7'\n"
+                  "import paper_1804_08066_b200 as m\n"
+                  "try:\n"
+                  "    m.mqg_quantize(None, 0, 4, 32, 0, None, None)\n"
+                  "except ImportError as e:\n"
+                  "    print(e)")
+    assert "9.8.7" in out and "is not built" in out
