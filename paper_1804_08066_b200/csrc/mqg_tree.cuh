@@ -55,20 +55,22 @@ __device__ __forceinline__ void bucket_tree_sums(float (&a)[N], uint32_t rpb, fl
             a[i] = first + wpb <= THREADS / 32 ? tree8(s_part + i * THREADS, first, wpb) : 0.0f;
         return;
     }
-    // any other shape: a bucket's tree is a warp's work, lane l on rows 8l .. 8l + 7 of it, zeros beyond
+    // any other shape: a bucket's tree is the work of an aligned group of 2^k lanes, 8 rows of it per lane, zeros
+    // beyond; there are more groups than buckets
 #pragma unroll
     for (int i = 0; i < N; ++i) s_part[i * THREADS + t] = a[i];
     __syncthreads();
-    const uint32_t lane = t & 31u, buckets = THREADS / rpb;
-    for (uint32_t b = t >> 5; b < buckets; b += THREADS / 32) {
+    const uint32_t buckets = THREADS / rpb;
+    uint32_t lanes = 1;
+    while (8 * lanes < rpb) lanes <<= 1;
+    const uint32_t b = t / lanes, row = 8 * (t & (lanes - 1));
+    const uint32_t left = b < buckets && row < rpb ? min(8u, rpb - row) : 0u;
+    float* p = s_part + (left != 0 ? b * rpb : 0u);
 #pragma unroll
-        for (int i = 0; i < N; ++i) {
-            float* p = s_part + i * THREADS + b * rpb;
-            const uint32_t left = 8 * lane < rpb ? min(8u, rpb - 8 * lane) : 0u;
-            const float s = warp_tree(tree8(p, 8 * lane, left), 32);
-            __syncwarp();                          // every lane has read the bucket's values
-            if (lane == 0) p[0] = s;
-        }
+    for (int i = 0; i < N; ++i, p += THREADS) {
+        const float s = warp_tree(tree8(p, row, left), lanes);
+        __syncwarp();                              // every lane has read the bucket's values
+        if (row == 0 && left != 0) p[0] = s;
     }
     __syncthreads();
     const uint32_t mine = t / rpb;

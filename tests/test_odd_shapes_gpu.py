@@ -1,0 +1,36 @@
+"""Shapes outside the bulk-copy kernels: the (min, max) server step on the row kernel, several workers on a CTA per bucket
+or a launch per worker, and buckets of an odd number of rows in the variants whose scale is a sum.  Against the CPU
+checker bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import paper_1804_08066_b200 as mqg
+from oracle import mqg_oracle as O
+from paper_1804_08066_b200 import workloads as wl
+from tests.gpu_util import Guarded, bits_equal, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("rows", [3, 7, 9, 17, 31, 33, 65, 127, 129, 255])
+def test_sums_over_an_odd_number_of_rows(rows):
+    """1, 2, 4 .. 32 lanes on a bucket's tree; the last bucket is short."""
+    bucket = 32 * rows
+    n = 9 * bucket + bucket // 2 + 5
+    rng = np.random.default_rng(rows)
+    x = (rng.standard_normal(n, dtype=np.float32) * np.exp2(rng.integers(-12, 12, n))).astype(np.float32)
+    c, s = Guarded(O.code_words(n, 4), torch.int32), Guarded(O.num_buckets(n, bucket), torch.float32)
+    mqg.mqg_quantize_l2(to_dev(x), n, 4, bucket, 5, c.view, s.view, elem_offset=3)
+    e0 = rng.standard_normal(n, dtype=np.float32)
+    e, c1, r = Guarded(n, torch.float32, fill=e0), Guarded(O.code_words(n, 1), torch.int32), \
+        Guarded(2 * O.num_buckets(n, bucket), torch.float32)
+    mqg.mqg_quantize_1bit_ef(to_dev(x), e.view, n, bucket, c1.view, r.view)
+    torch.cuda.synchronize()
+    c_ref, s_ref = O.quantize_l2(x, 4, bucket, 5, elem_offset=3)
+    assert bits_equal(s.numpy(np.float32), s_ref) == 0 and np.array_equal(c.numpy(np.uint32), c_ref)
+    want = O.quantize_1bit_ef(x, e0.copy(), bucket)
+    for got, ref in zip((c1.numpy(np.uint32), r.numpy(np.float32), e.numpy(np.float32)), want):
+        assert bits_equal(got, np.asarray(ref).ravel()) == 0
+    for b in (c, s, e, c1, r):
+        b.check_guards()
