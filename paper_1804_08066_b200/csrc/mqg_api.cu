@@ -69,11 +69,14 @@ uint64_t eff_bucket(uint64_t n, uint64_t bucket) { return bucket < n ? bucket : 
 
 // Shapes outside the one-pass kernel, for several workers (few elements, a bucket of an odd number of rows above 128, draws
 // off a block boundary): a bucket per CTA, all workers in one launch, where a bucket fills the CTA's warps or there are
-// so few of them that one launch instead of W decides (n = 6581, one bucket, W = 8: 25 us in eight launches); the
-// (min, max) variant also for one worker, which takes four launches otherwise.
+// so few of them that one launch instead of W decides.  A launch takes about 3.3 us, a CTA per bucket 5 ns, whatever it
+// holds: spans / launches 4.2 / 8.8 us for one bucket of 6581 elements, 7.6 / 8.4 us for 508 buckets of 128, 8.5 / 6.8 us
+// for 625 and 22 / 6.8 us for 2032 of 32, all at W = 2; the same ratios at W = 8 and 32.  The (min, max) variant also for
+// one worker, which takes four launches otherwise.
 bool worker_spans_preferred(uint64_t n, uint64_t bucket)
 {
-    return mqg::bucket_spans_apply(n, bucket) && (eff_bucket(n, bucket) > 4096 || n < 65536);
+    const uint64_t b = eff_bucket(n, bucket);
+    return mqg::bucket_spans_apply(n, bucket) && (b > 4096 || (n < 65536 && n <= 512 * b));
 }
 
 

@@ -13,6 +13,27 @@ from tests.gpu_util import Guarded, bits_equal, to_dev
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("n,bucket", [
+    (512 * 32, 32), (512 * 32 + 1, 32),            # as many spans as one launch takes, one more
+    (65_535, 128), (65_536, 128),
+])
+@pytest.mark.parametrize("norm", [False, True])
+def test_several_workers_with_draws_off_a_block_boundary(n, bucket, norm):
+    W, bits, off = 3, 5, 3
+    xs = [wl.normal(n, 1e-3, config=1, worker=w) for w in range(W)]
+    codes = [Guarded(O.code_words(n, bits), torch.int32) for _ in range(W)]
+    scales = [Guarded(O.num_buckets(n, bucket), torch.float32) for _ in range(W)]
+    call, ref = (mqg.mqg_quantize_workers_l2, O.quantize_l2) if norm else (mqg.mqg_quantize_workers, O.quantize)
+    call([to_dev(x) for x in xs], W, n, bits, bucket, 7, [c.view for c in codes], [s.view for s in scales],
+         first_worker=2, step=1, elem_offset=off)
+    torch.cuda.synchronize()
+    for w in range(W):
+        codes[w].check_guards(), scales[w].check_guards()
+        c_ref, s_ref = ref(xs[w], bits, bucket, 7, worker=2 + w, step=1, elem_offset=off)
+        assert bits_equal(scales[w].numpy(np.float32), s_ref) == 0
+        assert np.array_equal(codes[w].numpy(np.uint32), c_ref)
+
+
 @pytest.mark.parametrize("rows", [3, 7, 9, 17, 31, 33, 65, 127, 129, 255])
 def test_sums_over_an_odd_number_of_rows(rows):
     """1, 2, 4 .. 32 lanes on a bucket's tree; the last bucket is short."""
