@@ -194,7 +194,7 @@ struct ServerArgs {
 };
 
 // Sum of the W de-quantized rows in worker order, continuing from v[] when have_init.
-template <int BITS>
+template <int BITS, bool RANGE>
 __device__ __forceinline__ void accumulate_row(const ServerArgs& a, uint64_t scale_idx,
                                                uint64_t word0, uint64_t words_end, bool full_row,
                                                float (&v)[32], bool have_init)
@@ -210,7 +210,7 @@ __device__ __forceinline__ void accumulate_row(const ServerArgs& a, uint64_t sca
     constexpr int kBatch = 4;
     for (int w0 = 0; w0 < a.W; w0 += kBatch) {
         uint32_t w[kBatch][BITS];
-        float sc[kBatch];
+        float2 sc[kBatch];
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) {
             const int wk = min(w0 + i, a.W - 1);            // a worker past the last one repeats it (not summed)
@@ -220,13 +220,14 @@ __device__ __forceinline__ void accumulate_row(const ServerArgs& a, uint64_t sca
                 for (int k = 0; k < BITS; ++k)
                     w[i][k] = (word0 + k < words_end) ? __ldg(a.ptrs.codes[wk] + word0 + k) : 0u;
             }
-            sc[i] = __ldg(a.ptrs.scales[wk] + scale_idx);
+            if (RANGE) sc[i] = __ldg(reinterpret_cast<const float2*>(a.ptrs.scales[wk]) + scale_idx);
+            else sc[i] = make_float2(__ldg(a.ptrs.scales[wk] + scale_idx), 0.0f);
         }
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) {
             if (w0 + i < a.W) {
-                const DecodeScale2 d = widen(decode_scale<BITS>(sc[i]));
-                add_decoded_row<BITS>(w[i], d, v2);
+                const DecodeScale d = RANGE ? range_decode_scale<BITS>(sc[i].x, sc[i].y) : decode_scale<BITS>(sc[i].x);
+                add_decoded_row<BITS, RANGE>(w[i], widen(d), v2);
             }
         }
     }
@@ -237,7 +238,7 @@ __device__ __forceinline__ void accumulate_row(const ServerArgs& a, uint64_t sca
 // elements, whose parameters move through a swizzled shared-memory tile.  Fewer instructions per element than
 // the direct kernel, a longer chain per thread.
 // MODE 0: acc = sum (optionally continuing from acc).  MODE 1: params update, acc optional.
-template <int BITS, int MODE>
+template <int BITS, int MODE, bool RANGE>
 __global__ void __launch_bounds__(kMaxTileRows)
 server_row_kernel(const __grid_constant__ ServerArgs a)
 {
@@ -262,10 +263,10 @@ server_row_kernel(const __grid_constant__ ServerArgs a)
             __syncthreads();
             if (active) read_row(tile, (int)t, v);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = sum_start<BITS>(v[j]);
+            for (int j = 0; j < 32; ++j) v[j] = sum_start<BITS, RANGE>(v[j]);
         }
         if (active) {
-            accumulate_row<BITS>(a, scale_idx, word0, words_end, full_row, v, a.add_into != 0);
+            accumulate_row<BITS, RANGE>(a, scale_idx, word0, words_end, full_row, v, a.add_into != 0);
             write_row(tile, (int)t, v);
         }
         __syncthreads();
@@ -273,7 +274,7 @@ server_row_kernel(const __grid_constant__ ServerArgs a)
     } else {
         float* params = a.params + elem0;
         load_tile_f32<kMaxTileRows, false>(tile, params, valid, rows);    // in flight during the decode
-        if (active) accumulate_row<BITS>(a, scale_idx, word0, words_end, full_row, v, false);
+        if (active) accumulate_row<BITS, RANGE>(a, scale_idx, word0, words_end, full_row, v, false);
         cp_async_wait_all();
         __syncthreads();
         if (active) {
@@ -363,6 +364,7 @@ static cudaError_t server_direct(const WorkerPtrs& ptrs, int W, int bits, uint64
 // Direct below: 8.1 against 10.6 us at n = 2^22, W = 1.
 static bool row_kernel_preferred(uint64_t n, int W) { return n * (uint64_t)(W + 4) >= (1ull << 25); }
 
+template <bool RANGE>
 static cudaError_t server_rows(const WorkerPtrs& ptrs, int W, int bits, uint64_t n, uint64_t bucket, float* params,
                                float lr, float* acc, int add_into, cudaStream_t stream)
 {
@@ -380,8 +382,8 @@ static cudaError_t server_rows(const WorkerPtrs& ptrs, int W, int bits, uint64_t
     const unsigned grid = (unsigned)tiles;
     switch (bits) {
 #define MQG_ROW_CASE(B) \
-        case B: return params == nullptr ? launch_pdl(server_row_kernel<B, 0>, grid, kMaxTileRows, stream, a) \
-                                         : launch_pdl(server_row_kernel<B, 1>, grid, kMaxTileRows, stream, a)
+        case B: return params == nullptr ? launch_pdl(server_row_kernel<B, 0, RANGE>, grid, kMaxTileRows, stream, a) \
+                                         : launch_pdl(server_row_kernel<B, 1, RANGE>, grid, kMaxTileRows, stream, a)
         MQG_ROW_CASE(1); MQG_ROW_CASE(2); MQG_ROW_CASE(3); MQG_ROW_CASE(4);
         MQG_ROW_CASE(5); MQG_ROW_CASE(6); MQG_ROW_CASE(7); MQG_ROW_CASE(8);
 #undef MQG_ROW_CASE
@@ -409,8 +411,8 @@ static cudaError_t server_any(const WorkerPtrs& ptrs, int W, int bits, uint64_t 
                                       : launch_server_tma(ptrs, W, bits, n, bucket, dst, lr, mode, stream);
         return err == cudaSuccess && split ? launch_apply(params, acc, lr, n, stream) : err;
     }
-    if (!RANGE && row_kernel_preferred(n, W))
-        return server_rows(ptrs, W, bits, n, bucket, params, lr, acc, add_into, stream);
+    if (row_kernel_preferred(n, W))
+        return server_rows<RANGE>(ptrs, W, bits, n, bucket, params, lr, acc, add_into, stream);
     return server_direct<RANGE>(ptrs, W, bits, n, bucket, params, lr, acc, add_into, stream);
 }
 

@@ -13,6 +13,34 @@ from tests.gpu_util import Guarded, bits_equal, to_dev
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("n,W,bits", [
+    ((1 << 25) // 12 + 37, 8, 3), ((1 << 25) // 12 + 32, 8, 7), ((1 << 25) // 5 + 1, 1, 1), ((1 << 25) // 36 + 31, 32, 8),
+])
+def test_range_server_rows(n, W, bits):
+    bucket = 96
+    rng = np.random.default_rng(n)
+    codes = [rng.integers(0, 1 << 32, O.code_words(n, bits), dtype=np.uint32) for _ in range(W)]
+    ranges = [np.sort(rng.standard_normal((O.num_buckets(n, bucket), 2), dtype=np.float32) * np.float32(1e-3), axis=1).ravel()
+              for _ in range(W)]
+    ranges[0][-2:] = 1e-3                                                  # a constant bucket, the ragged one
+    dc, dr = [to_dev(c.view(np.int32)) for c in codes], [to_dev(r) for r in ranges]
+    p0 = wl.params(n, 0.05, config=21)
+    p_ref, acc_ref = O.server_step_minmax(codes, ranges, bits, n, bucket, p0.copy(), 0.1, want_acc=True)
+    for with_acc in (False, True):
+        p, acc = Guarded(n, torch.float32, fill=p0), Guarded(n, torch.float32) if with_acc else None
+        mqg.mqg_server_step_minmax(dc, dr, W, bits, n, bucket, p.view, 0.1, acc.view if with_acc else None)
+        torch.cuda.synchronize()
+        p.check_guards()
+        assert bits_equal(p.numpy(np.float32), p_ref) == 0
+        if with_acc:
+            acc.check_guards()
+            assert bits_equal(acc.numpy(np.float32), acc_ref) == 0
+    acc = Guarded(n, torch.float32, fill=p0)
+    mqg.mqg_dequant_accumulate_minmax(dc, dr, W, bits, n, acc.view, bucket, add_into_acc=True)
+    torch.cuda.synchronize()
+    assert bits_equal(acc.numpy(np.float32), O.dequant_accumulate_minmax(codes, ranges, bits, n, bucket, p0)) == 0
+
+
 @pytest.mark.parametrize("n,bucket", [
     (512 * 32, 32), (512 * 32 + 1, 32),            # as many spans as one launch takes, one more
     (65_535, 128), (65_536, 128),
