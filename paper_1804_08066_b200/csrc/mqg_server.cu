@@ -335,6 +335,9 @@ static cudaError_t launch_direct(int bits, const DirectArgs& a, const SegmentTab
     return cudaErrorInvalidValue;
 }
 
+// Whether every warp of the direct kernel works inside one bucket.
+static bool warp_in_one_bucket(uint64_t n, uint64_t bucket) { return bucket >= n || bucket % (32 * kDirectElems) == 0; }
+
 template <bool RANGE>
 static cudaError_t server_direct(const WorkerPtrs& ptrs, int W, int bits, uint64_t n, uint64_t bucket, float* params,
                                  float lr, float* acc, int add_into, cudaStream_t stream)
@@ -352,17 +355,24 @@ static cudaError_t server_direct(const WorkerPtrs& ptrs, int W, int bits, uint64
         if ((1ull << s) == rpb) a.rpb_shift = s;
     a.scale_base = 0;
     a.W = W; a.add_into = add_into; a.neg_lr = -lr;
-    a.warp_in_bucket = bucket >= n || rpb % (32 * kDirectElems / 32) == 0;
+    a.warp_in_bucket = warp_in_one_bucket(n, bucket);
     SegmentTable tab;
     tab.nseg = 0; tab.uniform_bucket = 0; tab.n_total = n; tab.tiles_per_bucket = 0;
     const uint64_t per_block = (uint64_t)kDirectThreads * kDirectElems;
     return launch_direct<RANGE, false>(bits, a, tab, (n + per_block - 1) / per_block, stream);
 }
 
-// Where the row kernel takes over from the direct one: 91 against 177 us at n = 25 M, bucket 96, W = 8, seven
-// bits, 42 against 54 us at n = 25 M, bucket 640, W = 1, but 18 against 20 us at n = 2^22, W = 8 and 10.6 against
-// Direct below: 8.1 against 10.6 us at n = 2^22, W = 1.
-static bool row_kernel_preferred(uint64_t n, int W) { return n * (uint64_t)(W + 4) >= (1ull << 25); }
+// Where the row kernel takes over from the direct one.  Direct / row in us, four bits.  Several buckets among a warp's 256
+// elements (bucket 96; direct divides for every worker and thread): W = 1 4.5 / 4.7, 5.0 / 4.8 for n = 1.5 and 2 * 2^20,
+// W = 8 5.8 / 6.1, 8.6 / 7.9 for n = 1 and 1.5 * 2^20, W = 32 12.7 / 14.4, 14.4 / 14.5 for n = 0.5 and 0.75 * 2^20; the
+// (min, max) variant within 4 % of that, and at n = 25 M 53 / 41 us with W = 1, 134 / 69 us with W = 8.  One bucket to a
+// warp, the sum as an extra output (bucket 2048): W = 1 4.8 / 4.8, 7.2 / 6.2, 12.1 / 10.6 for n = 1, 2 and 4 * 2^20,
+// W = 4 11.5 / 12.8 for n = 4 * 2^20, W = 8 4.9 / 7.0, 7.9 / 9.2 for n = 1 and 2 * 2^20.
+static bool row_kernel_preferred(uint64_t n, int W, bool warp_in_bucket, bool sum_out)
+{
+    if (!warp_in_bucket) return n * (uint64_t)(W + 16) >= (27ull << 20);
+    return W <= 2 ? n >= (1ull << 21) : !sum_out && n * (uint64_t)(W + 4) >= (1ull << 25);
+}
 
 template <bool RANGE>
 static cudaError_t server_rows(const WorkerPtrs& ptrs, int W, int bits, uint64_t n, uint64_t bucket, float* params,
@@ -411,7 +421,7 @@ static cudaError_t server_any(const WorkerPtrs& ptrs, int W, int bits, uint64_t 
                                       : launch_server_tma(ptrs, W, bits, n, bucket, dst, lr, mode, stream);
         return err == cudaSuccess && split ? launch_apply(params, acc, lr, n, stream) : err;
     }
-    if (row_kernel_preferred(n, W))
+    if (row_kernel_preferred(n, W, warp_in_one_bucket(n, bucket), params != nullptr && acc != nullptr))
         return server_rows<RANGE>(ptrs, W, bits, n, bucket, params, lr, acc, add_into, stream);
     return server_direct<RANGE>(ptrs, W, bits, n, bucket, params, lr, acc, add_into, stream);
 }

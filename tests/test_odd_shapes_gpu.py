@@ -9,12 +9,14 @@ import paper_1804_08066_b200 as mqg
 from oracle import mqg_oracle as O
 from paper_1804_08066_b200 import workloads as wl
 from tests.gpu_util import Guarded, bits_equal, to_dev
+from tests.test_server_dispatch_gpu import test_server_step_at_the_dispatch_lines as _step_at_the_lines
 
 pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n,W,bits", [
     ((1 << 25) // 12 + 37, 8, 3), ((1 << 25) // 12 + 32, 8, 7), ((1 << 25) // 5 + 1, 1, 1), ((1 << 25) // 36 + 31, 32, 8),
+    ((27 << 20) // 24, 8, 4), ((27 << 20) // 24 - 1, 8, 4), ((27 << 20) // 17 + 1, 1, 6),      # at the line of the rule
 ])
 def test_range_server_rows(n, W, bits):
     bucket = 96
@@ -39,6 +41,14 @@ def test_range_server_rows(n, W, bits):
     mqg.mqg_dequant_accumulate_minmax(dc, dr, W, bits, n, acc.view, bucket, add_into_acc=True)
     torch.cuda.synchronize()
     assert bits_equal(acc.numpy(np.float32), O.dequant_accumulate_minmax(codes, ranges, bits, n, bucket, p0)) == 0
+
+
+@pytest.mark.parametrize("n,bucket,W,bits,with_acc", [
+    ((27 << 20) // 24, 96, 8, 3, False), ((27 << 20) // 24 - 1, 96, 8, 5, False),              # row kernel, direct kernel
+    ((1 << 21), 2048, 2, 4, True), ((1 << 21) - 1, 2048, 2, 4, True), ((1 << 21) + 9, 2048, 3, 4, True),
+])
+def test_server_rows_at_the_line(n, bucket, W, bits, with_acc):
+    _step_at_the_lines(n, bucket, W, bits, with_acc)
 
 
 @pytest.mark.parametrize("n,bucket", [
