@@ -2,7 +2,7 @@
 // one-pass kernels.  Two ways:
 //   * span_kernel - a span is a segment or a bucket that fits one CTA's shared memory: the CTA stages all of it,
 //     finds the scale and encodes from there, so the gradient is read once and every span of every worker
-//     is one launch's work;
+//     is one launch's work (spans_absmax_kernel: the same beside a max pass);
 //   * absmax_table_kernel, encode_table_kernel - longer ones: a max pass that folds every tile's maximum into
 //     scales[] with an atomic max on the float's bit pattern, then an encode pass.
 // Worker w of W is blockIdx.y in all of them; its results do not depend on W or on the way taken.
@@ -53,8 +53,7 @@ __device__ __forceinline__ void encode_store_row(const float (&x)[32], const Sca
 // Up to 512 rows: 256 threads (one or two rows each) and the registers of three CTAs per SM; longer spans: 512
 // threads, one CTA per SM.
 template <int BITS, int DTYPE, int MODE, int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 3 : 1)
-span_kernel(const __grid_constant__ TableArgs a, const __grid_constant__ SpanTable tab)
+__device__ __forceinline__ void quantize_span(const TableArgs& a, const SpanTable& tab)
 {
     extern __shared__ uint8_t smem_raw[];
     float4* tile = reinterpret_cast<float4*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
@@ -147,14 +146,21 @@ span_kernel(const __grid_constant__ TableArgs a, const __grid_constant__ SpanTab
     }
 }
 
+template <int BITS, int DTYPE, int MODE, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 3 : 1)
+span_kernel(const __grid_constant__ TableArgs a, const __grid_constant__ SpanTable tab)
+{
+    quantize_span<BITS, DTYPE, MODE, THREADS>(a, tab);
+}
+
 // ---- two passes over tiles of 256 rows ---------------------------------------------------------------
+// Tile `tile` of the table, whose first segment has the scale a.scales[w][first].
 template <int DTYPE>
-__global__ void __launch_bounds__(kMaxTileRows)
-absmax_table_kernel(const __grid_constant__ TableArgs a, const __grid_constant__ SegmentTable tab)
+__device__ __forceinline__ void absmax_tile(const TableArgs& a, const SegmentTable& tab, uint32_t tile, uint32_t first)
 {
     constexpr int THREADS = kMaxTileRows;
     __shared__ uint32_t s_warp[THREADS / 32];
-    const TileGeom g = locate_tile<1>(tab, blockIdx.x);
+    const TileGeom g = locate_tile<1>(tab, tile);
     const uint64_t count = g.valid < (uint64_t)(kMaxTileRows * 32) ? g.valid : (uint64_t)(kMaxTileRows * 32);
     grid_dependency_wait();
 
@@ -201,8 +207,33 @@ absmax_table_kernel(const __grid_constant__ TableArgs a, const __grid_constant__
         // a tile's maximum below the flush limit does not count: a segment whose every tile stays below it
         // keeps the scale 0 the pass started from, so the scale that stands after the pass is final
         if (r >= __float_as_uint(flush_limit()))
-            atomicMax(reinterpret_cast<unsigned int*>(a.scales[blockIdx.y]) + g.seg, r);
+            atomicMax(reinterpret_cast<unsigned int*>(a.scales[blockIdx.y]) + first + g.seg, r);
     }
+}
+
+template <int DTYPE>
+__global__ void __launch_bounds__(kMaxTileRows)
+absmax_table_kernel(const __grid_constant__ TableArgs a, const __grid_constant__ SegmentTable tab)
+{
+    absmax_tile<DTYPE>(a, tab, blockIdx.x, 0);
+}
+
+// The spans of a table and the max pass over its longer segments, whose scales are clear, in one launch: a span is a
+// chain of a staging copy, a reduction and an encode, 3 us beside which the max pass reads.
+template <int BITS, int DTYPE>
+__global__ void __launch_bounds__(kMaxTileRows, 3)
+spans_absmax_kernel(const __grid_constant__ TableArgs a, const __grid_constant__ SpanTable spans,
+                    const __grid_constant__ SegmentTable longs)
+{
+    if (blockIdx.x < (uint32_t)spans.nspan) quantize_span<BITS, DTYPE, kSpanMaxAbs, kMaxTileRows>(a, spans);
+    else absmax_tile<DTYPE>(a, longs, blockIdx.x - (uint32_t)spans.nspan, (uint32_t)spans.first);
+}
+
+__global__ void __launch_bounds__(kMaxTileRows)
+clear_scales_kernel(const __grid_constant__ TableArgs a, int nseg)
+{
+    grid_dependency_wait();
+    for (int j = (int)threadIdx.x; j < nseg; j += kMaxTileRows) a.scales[blockIdx.x][j] = 0.0f;
 }
 
 // A 256-row tile of the table is two CTAs' work.
@@ -250,24 +281,33 @@ TableArgs make_table_args(const void* const* grads, int W, uint32_t* const* code
     return a;
 }
 
-template <int BITS, int DTYPE, int MODE, int THREADS>
-static cudaError_t launch_span_inst(const TableArgs& a, const SpanTable& tab, unsigned nspan, uint64_t most,
-                                    cudaStream_t stream)
+// Shared memory of a launch whose longest span has `most` elements (with slack to round the base up), and the attribute
+// that allows a kernel the most of it.
+static size_t span_smem(uint64_t most) { return (size_t)((most + 31) / 32) * 128 + 1024; }
+template <typename Kernel>
+static cudaError_t allow_span_smem(Kernel kernel, std::atomic<bool> (&ready)[64], int threads)
 {
-    auto kernel = span_kernel<BITS, DTYPE, MODE, THREADS>;
-    const size_t smem = (size_t)((most + 31) / 32) * 128 + 1024;       // + slack to round the base up
-    static std::atomic<bool> ready[64];                                // per device (zero-initialised)
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!ready[dev].load(std::memory_order_relaxed)) {
-        constexpr int kMost = (THREADS == 256 ? 512 : kMaxSpanRows) * 128 + 1024;
-        err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
-        if (err != cudaSuccess) return err;
-        ready[dev].store(true, std::memory_order_relaxed);
+        const int most = (threads == 256 ? 512 : kMaxSpanRows) * 128 + 1024;
+        err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (err == cudaSuccess) ready[dev].store(true, std::memory_order_relaxed);
     }
-    return launch_pdl_grid(kernel, dim3(nspan, (unsigned)a.W), THREADS, smem, stream, a, tab);
+    return err;
+}
+
+template <int BITS, int DTYPE, int MODE, int THREADS>
+static cudaError_t launch_span_inst(const TableArgs& a, const SpanTable& tab, unsigned nspan, uint64_t most,
+                                    cudaStream_t stream)
+{
+    static std::atomic<bool> ready[64];                                // per device (zero-initialised)
+    const cudaError_t err = allow_span_smem(span_kernel<BITS, DTYPE, MODE, THREADS>, ready, THREADS);
+    if (err != cudaSuccess) return err;
+    return launch_pdl_grid(span_kernel<BITS, DTYPE, MODE, THREADS>, dim3(nspan, (unsigned)a.W), THREADS, span_smem(most),
+                           stream, a, tab);
 }
 
 template <int MODE>
@@ -322,6 +362,36 @@ cudaError_t launch_absmax_table(const TableArgs& a, const SegmentTable& tab, int
     const dim3 grid(tiles, (unsigned)a.W);
     return dtype == 0 ? launch_pdl_grid(absmax_table_kernel<0>, grid, kMaxTileRows, 0, stream, a, tab)
                       : launch_pdl_grid(absmax_table_kernel<1>, grid, kMaxTileRows, 0, stream, a, tab);
+}
+
+cudaError_t launch_clear_scales(const TableArgs& a, int nseg, cudaStream_t stream)
+{
+    return launch_pdl(clear_scales_kernel, (unsigned)a.W, kMaxTileRows, stream, a, nseg);
+}
+
+template <int BITS, int DTYPE>
+static cudaError_t launch_spans_absmax_inst(const TableArgs& a, const SpanTable& spans, uint64_t most,
+                                            const SegmentTable& longs, cudaStream_t stream)
+{
+    static std::atomic<bool> ready[64];                                // per device (zero-initialised)
+    const cudaError_t err = allow_span_smem(spans_absmax_kernel<BITS, DTYPE>, ready, kMaxTileRows);
+    if (err != cudaSuccess) return err;
+    return launch_pdl_grid(spans_absmax_kernel<BITS, DTYPE>, dim3((unsigned)spans.nspan + tab_tiles(longs), (unsigned)a.W),
+                           kMaxTileRows, span_smem(most), stream, a, spans, longs);
+}
+
+cudaError_t launch_spans_absmax(const TableArgs& a, const SpanTable& spans, uint64_t most, const SegmentTable& longs,
+                                int bits, int dtype, cudaStream_t stream)
+{
+    switch (bits) {
+#define MQG_FUSED_CASE(B) \
+        case B: return dtype == 0 ? launch_spans_absmax_inst<B, 0>(a, spans, most, longs, stream) \
+                                  : launch_spans_absmax_inst<B, 1>(a, spans, most, longs, stream)
+        MQG_FUSED_CASE(1); MQG_FUSED_CASE(2); MQG_FUSED_CASE(3); MQG_FUSED_CASE(4);
+        MQG_FUSED_CASE(5); MQG_FUSED_CASE(6); MQG_FUSED_CASE(7); MQG_FUSED_CASE(8);
+#undef MQG_FUSED_CASE
+    }
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_encode_table(const TableArgs& a, const SegmentTable& tab, int bits, int dtype, cudaStream_t stream)

@@ -40,6 +40,11 @@ struct SpanTable {
 cudaError_t launch_spans(const TableArgs& a, const SpanTable& tab, unsigned nspan, uint64_t most, int mode, int bits,
                          int dtype, cudaStream_t stream);
 
+// The same in the main codec together with the max pass over `longs`, whose scales launch_clear_scales has cleared.
+cudaError_t launch_clear_scales(const TableArgs& a, int nseg, cudaStream_t stream);
+cudaError_t launch_spans_absmax(const TableArgs& a, const SpanTable& spans, uint64_t most, const SegmentTable& longs,
+                                int bits, int dtype, cudaStream_t stream);
+
 struct TileGeom {
     uint64_t elem0;       // flat index of the tile's first element
     uint64_t valid;       // elements from elem0 to the end of the segment

@@ -1,11 +1,14 @@
 // Per-layer quantization (one scale per segment; Section 4.1 quantizes whole layers) of one or several
 // workers' gradients that share a segment table (Algorithm 1, WorkerIterate line 3, for every worker of the
-// simulation), in up to three launches whatever the number of workers and segments:
-//   1. span_kernel (mqg_segments.cu) - every segment of at most kSegmentSpanElems elements, scale and codes;
-//      the launch also clears the scales of the longer ones;
-//   2. absmax_table_kernel - the max pass over the longer segments;
-//   3. encode_entries_kernel - their encode.  Every (worker, segment) pair is an entry with a tensor map of its
-//      own; the persistent CTAs walk the 128-row tiles of all entries as one sequence, fed by tiled bulk copies.  Segments that start where bulk copies cannot go through encode_table_kernel instead.
+// simulation), in three launches for up to 64 segments and 64 (worker, long segment) pairs:
+//   1. clear_scales_kernel (mqg_segments.cu);
+//   2. spans_absmax_kernel - every segment of at most kSegmentSpanElems elements, scale and codes by one CTA, and beside
+//      them the max pass over the longer segments; a launch for every 64 segments;
+//   3. encode_entries_kernel - the longer ones' encode.  Every (worker, segment) pair is an entry with a tensor map of its
+//      own; the persistent CTAs walk the 128-row tiles of all entries as one sequence, fed by tiled bulk copies; a launch
+//      for every 64 entries.  Segments that start where bulk copies cannot go through encode_table_kernel instead.
+// Where the first two do not go together (spans_join_max_pass), span_kernel also clears the scales and absmax_table_kernel
+// follows it.
 // Worker w's outputs are the same whichever way a segment goes and however many workers there are.
 #include <string.h>
 
@@ -22,6 +25,18 @@ constexpr int kFewEntries = 16, kMaxEntries = 64;
 
 // Longest segment that one CTA handles alone: two rows per thread, 2 to 3 us.
 constexpr uint64_t kSegmentSpanElems = 512 * 32;
+
+// Whether the spans and the max pass share a launch (`tiles` of 256 rows in the max pass).  Spans on their own are 3 us
+// during which a few CTAs are at work; the launch before then only clears the scales, 1.2 us.  The other side is the spans'
+// registers and shared memory, with which three CTAs share an SM: the max pass reads no slower in fp32 (16 KB requested by
+// every CTA: 592 against 598 us for the quantizer's whole call on eight AlexNet-shaped gradients, 4 bits), but in bf16 (8 KB:
+// 463 against 409 us) or where segments start off a 16-byte boundary (shorter chains of loads: 100 against 93 us for 31 M
+// elements in 16 tensors).  bf16 gradients of 41 M elements in 100 tensors 65 against 70 us, fp32 74 against 81 us; 10 M off
+// the boundary in 20 tensors 28 against 30 us.
+static bool spans_join_max_pass(uint64_t tiles, int dtype, bool aligned)
+{
+    return aligned ? dtype == 0 || tiles <= 8192 : tiles <= 2048;
+}
 
 struct SegEntry {
     const void* grad;        // the segment's first element (for its ragged last row)
@@ -268,7 +283,18 @@ cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, 
                 return false;
         return true;
     };
-    cudaError_t err = cudaSuccess;
+    uint64_t long_tiles = 0;                          // of 256 rows
+    bool any_span = false, aligned = true;            // aligned: the long segments, as the gradients are
+    for (int j = 0; j < nseg; ++j) {
+        const uint64_t len = seg_off[j + 1] - seg_off[j];
+        if (len <= kSegmentSpanElems) { any_span = true; continue; }
+        long_tiles += (len + kMaxTileRows * 32 - 1) / (kMaxTileRows * 32);
+        aligned = aligned && (seg_off[j] * esz) % 16 == 0;
+    }
+    const bool together = !workspace && any_span && long_tiles != 0 &&
+                          spans_join_max_pass(long_tiles * (uint64_t)W, dtype, aligned);
+    cudaError_t err = together ? launch_clear_scales(a, nseg, stream) : cudaSuccess;
+    if (err != cudaSuccess) return err;
     bool any_entries = false;
     uint64_t sums = 0;                                // partial sums of the tables already launched
     for (int first = 0; first < nseg; first += kMaxSegmentsPerLaunch) {
@@ -294,7 +320,7 @@ cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, 
                 spans.scale_idx[k] = (uint32_t)j;
                 if (len > most) most = len;
             } else {
-                if (!workspace) spans.clear[i >> 5] |= 1u << (i & 31);
+                if (!workspace && !together) spans.clear[i >> 5] |= 1u << (i & 31);
                 const uint64_t nt = (len + kMaxTileRows * 32 - 1) / (kMaxTileRows * 32);
                 tiles += nt;
                 if (bulk(j)) any_entries = true;
@@ -305,7 +331,11 @@ cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, 
         longs.tile_start[count] = (uint32_t)tiles;
         plain.tile_start[count] = (uint32_t)plain_tiles;
         longs.seg_off[count] = plain.seg_off[count] = seg_off[first + count];
-        if (spans.nspan != 0 || (tiles != 0 && !workspace)) {
+        const bool one_launch = together && spans.nspan != 0 && tiles != 0;
+        if (one_launch) {
+            err = launch_spans_absmax(a, spans, most, longs, bits, dtype, stream);
+            if (err != cudaSuccess) return err;
+        } else if (spans.nspan != 0 || (tiles != 0 && !workspace && !together)) {
             err = launch_spans(a, spans, spans.nspan != 0 ? (unsigned)spans.nspan : 1u, most,
                                workspace ? kSpanNorm : kSpanMaxAbs, bits, dtype, stream);
             if (err != cudaSuccess) return err;
@@ -314,7 +344,7 @@ cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, 
         TableArgs t = a;                              // a table numbers its segments from 0
         for (int w = 0; w < W; ++w) t.scales[w] += first;
         err = workspace ? launch_segments_l2_scales(grads[0], longs, t.scales[0], dtype, workspace + sums, stream)
-                        : launch_absmax_table(t, longs, dtype, stream);
+            : one_launch ? cudaSuccess : launch_absmax_table(t, longs, dtype, stream);
         sums += tiles;
         if (err == cudaSuccess) err = launch_encode_table(t, plain, bits, dtype, stream);
         if (err != cudaSuccess) return err;
