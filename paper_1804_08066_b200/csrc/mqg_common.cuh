@@ -154,25 +154,26 @@ __device__ __forceinline__ void draw_row_aligned(uint64_t g0, const RoundKeys& r
     draw_row_blocks((uint32_t)blk0, (uint32_t)(blk0 >> 32), rk, h);
 }
 
-// Same for any g0 (slow path: up to five blocks, run-time selection).
-static __device__ __noinline__ void draw_row_unaligned(uint64_t g0, const DrawKey& key, uint32_t (&h)[16])
+// Same for any g0: five blocks, whose 40 draws are moved down by g0 % 8 - by two words, by one, by a half - without an
+// index that would take them through local memory.
+__device__ __forceinline__ void draw_row_any(uint64_t g0, uint32_t worker, const RoundKeys& rk, uint32_t (&h)[16])
 {
-    const RoundKeys rk = make_round_keys(key);
+    const uint32_t blk_lo = (uint32_t)(g0 >> 3), blk_hi = (uint32_t)(g0 >> 35), shift = (uint32_t)g0 & 7u;
     uint32_t y[20];
-    const uint64_t blk0 = g0 >> 3;
+#pragma unroll
     for (int b = 0; b < 5; ++b) {
-        const uint64_t blk = blk0 + b;
         uint32_t t[4];
-        philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), rk.worker, rk.step, rk, t);
+        const uint32_t lo = blk_lo + b;
+        philox4x32_10(lo, blk_hi + (lo < blk_lo ? 1u : 0u), worker, rk.step, rk, t);
+#pragma unroll
         for (int k = 0; k < 4; ++k) y[4 * b + k] = t[k];
     }
-    const unsigned shift = (unsigned)(g0 & 7u);       // first element's field in the 40-field run
-    for (int j = 0; j < 16; ++j) {
-        const unsigned f0 = shift + 2u * j, f1 = f0 + 1u;
-        const uint32_t lo = (y[f0 >> 1] >> (16u * (f0 & 1u))) & 0xFFFFu;
-        const uint32_t hi = (y[f1 >> 1] >> (16u * (f1 & 1u))) & 0xFFFFu;
-        h[j] = lo | (hi << 16);
-    }
+#pragma unroll
+    for (int j = 0; j < 18; ++j) y[j] = (shift & 4u) ? y[j + 2] : y[j];
+#pragma unroll
+    for (int j = 0; j < 17; ++j) y[j] = (shift & 2u) ? y[j + 1] : y[j];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) h[j] = __funnelshift_r(y[j], y[j + 1], 16u * (shift & 1u));
 }
 
 // max(m, |a|, |b|) in one three-input instruction.

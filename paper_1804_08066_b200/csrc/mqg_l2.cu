@@ -75,7 +75,7 @@ l2_quantize_kernel(const __grid_constant__ L2Args a)
     const uint64_t g0 = a.elem_offset + row * 32;
     uint32_t h[16];
     if ((g0 & 7u) == 0) draw_row_aligned(g0, make_round_keys(a.key), h);
-    else draw_row_unaligned(g0, a.key, h);
+    else draw_row_any(g0, a.key.worker, make_round_keys(a.key), h);
 
     uint32_t w[BITS];
     encode_pack_row<BITS>(x, es, h, w);

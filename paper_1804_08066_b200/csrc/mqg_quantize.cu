@@ -83,7 +83,7 @@ quantize_pack_kernel(const __grid_constant__ QuantizeArgs a)
     const uint64_t row = row0 + t;
     uint32_t h[16];
     if constexpr (ALIGNED_DRAWS) draw_row_aligned(a.elem_offset + row * 32, make_round_keys(a.key), h);
-    else draw_row_unaligned(a.elem_offset + row * 32, a.key, h);
+    else draw_row_any(a.elem_offset + row * 32, a.key.worker, make_round_keys(a.key), h);
 
     uint32_t w[BITS];
     encode_pack_row<BITS>(x, es, h, w);

@@ -32,8 +32,7 @@ __device__ __forceinline__ void encode_store_row(const float (&x)[32], const Sca
             const uint64_t blk = g0 >> 3;
             draw_row_blocks((uint32_t)blk, (uint32_t)(blk >> 32), a.first_worker + w, a.rk, h);
         } else {
-            const DrawKey key = {a.rk.k0[0], a.rk.k1[0], a.first_worker + w, a.rk.step};
-            draw_row_unaligned(g0, key, h);
+            draw_row_any(g0, a.first_worker + w, a.rk, h);
         }
         encode_pack_row_best<BITS>(x, es, h, cw);
     }
