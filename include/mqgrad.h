@@ -90,9 +90,11 @@ mqg_status mqg_quantize(const void* grad, uint64_t n, int bits, uint64_t bucket,
  *   grads, codes, scales  HOST arrays of W device pointers (read during the call only); each
  *                         buffer as in mqg_quantize; the outputs are what mqg_server_step and
  *                         mqg_dequant_accumulate take as codes[] / scales[]
- * Shapes outside the one-launch kernels (fewer than 2048 elements, elem_offset not a multiple of 8, buckets
- * of 129 .. 255 rows of 32 that are not whole multiples of 32 rows, buckets above 49152 elements) run as W
- * launches inside the call.
+ * Two kernels take all workers in one launch.  The first wants at least 2048 elements, elem_offset a multiple of 8 and
+ * buckets of at most 8192 elements, those above 4096 a multiple of 1024.  The second takes buckets of up to 49152
+ * elements (or one such gradient) with any elem_offset, a CTA to a bucket: used where the first does not apply for
+ * buckets above 4096 elements, and below 65536 elements for up to 512 buckets.  Other shapes run as W launches (or more)
+ * inside the call.
  * Errors: as mqg_quantize, per worker; MQG_ERR_TOO_MANY_WORKERS for W outside 1..MQG_MAX_WORKERS.
  */
 mqg_status mqg_quantize_workers(const void* const* grads, int W, uint64_t n, int bits, uint64_t bucket,
@@ -299,7 +301,7 @@ mqg_status mqg_quantize_segments_l2_static(const void* grad, int nseg, const uin
  *   grad      [in] the whole flat gradient (element 0 of the array is flat index 0)
  *   codes     [out] code_off[nseg] words;  scales [out] nseg floats
  * Element i of segment j draws with position elem_offset + seg_off[j] + i.  Empty segments get
- * scale 0.  The gradient is read twice (max pass, encode pass).
+ * scale 0.
  * Performance note: a segment of at most 16384 elements is read once, a longer one twice; the longer ones are
  * encoded by the bulk-copy kernel when grad + seg_off[j] is 16-byte aligned and elem_offset + seg_off[j] is a
  * multiple of 8 (and, from 2^15 elements on, applied by mqg_server_step_segments' bulk-copy kernel when
@@ -312,8 +314,8 @@ mqg_status mqg_quantize_segments(const void* grad, int nseg, const uint64_t* seg
                                  uint32_t step, uint64_t elem_offset, void* cuda_stream);
 
 /*
- * mqg_quantize_segments for W workers' gradients that share one segment table, in up to three launches for
- * all of them (short segments whole, max pass and encode pass of the longer ones) - the per-layer
+ * mqg_quantize_segments for W workers' gradients that share one segment table, in three launches for up to 64 segments
+ * and 64 (worker, long segment) pairs (short segments whole, max pass and encode pass of the longer ones) - the per-layer
  * counterpart of mqg_quantize_workers, for a host that plays several workers on one device (all
  * workers run Quantize(g, K) with the same K in an iteration; Algorithm 1, WorkerIterate line 3).
  *   grads/codes/scales [in] HOST arrays of W device pointers; worker w draws with worker id

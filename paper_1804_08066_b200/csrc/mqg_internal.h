@@ -49,8 +49,9 @@ cudaError_t launch_quantize_workers(const void* const* grads, int W, uint64_t n,
                                     uint32_t step, uint64_t elem_offset, int mode, cudaStream_t stream);
 
 // (min, max) nearest-rounding variant.  ranges[2b] = lo, ranges[2b + 1] = hi of bucket b.
-// Fused one-pass kernel for buckets of at most 4096 elements; otherwise the general launches
-// (ranges by atomics on ordered bits, then encode).
+// One-pass kernel for buckets of at most kMaxFusedBucket elements (mqg_quantize.cu), a CTA per bucket for those it does not
+// take and up to 49152 elements (launch_bucket_spans), the general launches for longer ones (ranges by atomics on ordered
+// bits, then encode).
 bool quantize_range_fused_applies(uint64_t n, uint64_t bucket);
 cudaError_t launch_quantize_range_fused(const void* grad, uint64_t n, int bits, uint64_t bucket,
                                         uint32_t* codes, float* ranges, int dtype, cudaStream_t stream);
@@ -95,7 +96,7 @@ cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, 
 constexpr uint64_t kEntrySegmentElems = 1ull << 15;
 
 // Buckets (or a single bucket n) that one CTA quantizes as a whole, for W >= 1 workers; mode: 0 = main codec,
-// 1 = (min, max) variant (`scales` are ranges).
+// 1 = (min, max) variant (`scales` are ranges), 2 = L2-norm scale variant.
 bool bucket_spans_apply(uint64_t n, uint64_t bucket);
 cudaError_t launch_bucket_spans(const void* const* grads, int W, uint64_t n, int bits, uint64_t bucket, uint64_t seed,
                                 uint32_t* const* codes, float* const* scales, int mode, int dtype, uint32_t first_worker,
@@ -122,7 +123,7 @@ cudaError_t launch_server_tma(const WorkerPtrs& ptrs, int W, int bits, uint64_t 
 
 // The fused update of up to kMaxServerSegsPerLaunch long segments of a per-layer step in ONE launch of
 // the TMA-fed server kernel (a segment is a gradient with a single bucket).  Every segment must
-// satisfy server_tma_segment_applies(n), and params + elem0 and every worker's codes + code_word0
+// satisfy server_tma_applies(n, n), and params + elem0 and every worker's codes + code_word0
 // must be 16-byte aligned.
 struct ServerSegHost {
     uint64_t n;              // elements of the segment
@@ -131,7 +132,6 @@ struct ServerSegHost {
     uint32_t scale_idx;      // index of its scale in every worker's scale array
 };
 constexpr int kMaxServerSegsPerLaunch = 16;
-bool server_tma_segment_applies(uint64_t len);
 // short_tab (may be null): the table of the step's other segments, updated by the same launch with plain
 // loads; short_first = index of the table's first segment in the scale arrays.
 cudaError_t launch_server_tma_segments(const WorkerPtrs& ptrs, int W, int bits, const ServerSegHost* segs, int nseg,

@@ -1,5 +1,5 @@
 // The tile code of the TMA-fed quantize kernels (one tile of whole buckets per CTA turn: scale,
-// draws, encode, pack), shared by the kernels of mqg_quantize.cu and mqg_segments_workers.cu.
+// draws, encode, pack), shared by the kernels of mqg_quantize.cu, mqg_quantize_workers.cu and mqg_segments_workers.cu.
 #pragma once
 
 #include "mqg_common.cuh"
@@ -154,8 +154,8 @@ struct WorkerView {
 };
 
 // One tile, the k-th of this CTA, tile `tile` of worker `wv`.  FULL: every thread owns a complete
-// row (no bounds checks).  RED: how a bucket's rows are reduced.  After the tile's rows are in registers thread 0 calls `refill(stage, bar)` to start the copy that
-// uses the stage next.  Returns false if the tile's copy never landed.
+// row (no bounds checks).  RED: how a bucket's rows are reduced.  After the tile's rows are in registers thread 0 calls
+// `refill(stage, bar)` to start the copy that uses the stage next.  Returns false if the tile's copy never landed.
 template <int BITS, int DTYPE, int THREADS, bool FULL, int RED, bool NORM = false,
           typename Refill>
 __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>& sh, const WorkerView wv,
@@ -388,7 +388,8 @@ __device__ __forceinline__ bool range_quantize_tile(TmaQuantizeShared<DTYPE, THR
     return true;
 }
 
-// MODE: kMaxAbs = the main codec, kRange = the (min, max) variant, kNorm = the L2-norm scale variant.
+// MODE: kMaxAbs = the main codec, kRange = the (min, max) variant, kNorm = the L2-norm scale variant.  (Rows of 64 bf16
+// elements below exist for the main codec only: the variants' long bf16 launches were not tried with them.)
 enum : int { kMaxAbs = 0, kRange = 1, kNorm = 2 };
 
 // ---------------------------------------------------------------------------------------

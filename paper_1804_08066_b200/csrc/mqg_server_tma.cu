@@ -1066,8 +1066,6 @@ static cudaError_t launch_server_segs_inst(const ServerSegTable& tab, const Serv
     return launch_pdl_smem(kernel, (unsigned)grid, kSrvThreads, kSmemBytes, stream, tab, ss, a, timeouts);
 }
 
-bool server_tma_segment_applies(uint64_t len) { return server_tma_applies(len, len); }
-
 cudaError_t launch_server_tma_segments(const WorkerPtrs& ptrs, int W, int bits, const ServerSegHost* segs, int nseg,
                                        const SegmentTable* short_tab, int short_first, float* params, float lr,
                                        cudaStream_t stream)

@@ -40,12 +40,6 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
-// Plain arrival (no bytes expected): completes a phase whose data was written with ordinary stores.
-__device__ __forceinline__ void mbar_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
@@ -81,14 +75,6 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int 
                  ::"l"(map), "r"(x), "r"(y), "r"(src) : "memory");
 }
 
-// 1-D bulk load global -> shared: both addresses 16-byte aligned, bytes a multiple of 16.
-__device__ __forceinline__ void bulk_load_1d(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-        ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 
 // Wait until at most N of this thread's bulk groups still READ their shared-memory source.
@@ -115,42 +101,6 @@ __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepco
 
 // ---- host side ------------------------------------------------------------------------
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, cudaStream_t stream,
-                       Args&&... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-
-// The same with dynamic shared memory.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl_smem(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t dynamic_smem,
-                            cudaStream_t stream, Args&&... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = dynamic_smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-
-// The same with a grid of more than one dimension.
-template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl_grid(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t dynamic_smem,
                             cudaStream_t stream, Args&&... args)
 {
@@ -167,17 +117,17 @@ cudaError_t launch_pdl_grid(void (*kernel)(KArgs...), dim3 grid, unsigned block,
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// Ordinary stream-ordered launch with dynamic shared memory.
+// The same on a grid of one dimension, without and with dynamic shared memory.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_with_smem(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t dynamic_smem,
-                             cudaStream_t stream, Args&&... args)
+cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, cudaStream_t stream, Args&&... args)
 {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = dynamic_smem;
-    cfg.stream = stream;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    return launch_pdl_grid(kernel, dim3(grid), block, 0, stream, args...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_smem(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t dynamic_smem,
+                            cudaStream_t stream, Args&&... args)
+{
+    return launch_pdl_grid(kernel, dim3(grid), block, dynamic_smem, stream, args...);
 }
 
 // Encodes a 2-D row-major tensor map: `rows` rows of `row_elems` elements (row_bytes =
