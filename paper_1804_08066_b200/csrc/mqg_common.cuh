@@ -556,14 +556,19 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
                  ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gmem_src) : "memory");
 }
+__device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;"
+                 ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gmem_src) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Cooperative, coalesced copy of a tile of `rows` rows into / out of a swizzled tile.  `src`
 // points at the tile's first element and `valid` is the number of elements that exist from
 // there on (elements at or beyond it read as zero and are never written).  128-bit accesses
 // when the tile's first element is 16-byte aligned, 32-bit (16-bit for bf16) otherwise.
-// The aligned fp32 path copies asynchronously; with WAIT = false the caller overlaps other work
-// with the copies and calls cp_async_wait_all() itself before the barrier that precedes the reads.
+// fp32 tiles are copied asynchronously, so a thread has all its pieces in flight; with WAIT = false the caller overlaps
+// other work with the copies and calls cp_async_wait_all() itself before the barrier that precedes the reads.
 template <int THREADS, bool WAIT = true>
 __device__ __forceinline__ void load_tile_f32(float4* tile, const float* __restrict__ src,
                                               uint64_t valid, int rows)
@@ -588,9 +593,11 @@ __device__ __forceinline__ void load_tile_f32(float4* tile, const float* __restr
         float* tf = reinterpret_cast<float*>(tile);
         const int elems = rows * 32;
         for (int k = threadIdx.x; k < elems; k += THREADS) {
-            const float v = ((uint64_t)k < valid) ? __ldcs(src + k) : 0.0f;
-            tf[swz(k >> 5, (k >> 2) & 7) * 4 + (k & 3)] = v;
+            float* dst = &tf[swz(k >> 5, (k >> 2) & 7) * 4 + (k & 3)];
+            if ((uint64_t)k < valid) cp_async4(dst, src + k);
+            else *dst = 0.0f;
         }
+        if (WAIT) cp_async_wait_all();
     }
 }
 
@@ -624,9 +631,19 @@ __device__ __forceinline__ void load_tile_bf16(float4* tile, const uint16_t* __r
     } else {
         float* tf = reinterpret_cast<float*>(tile);
         const int elems = rows * 32;
-        for (int k = threadIdx.x; k < elems; k += THREADS) {
-            const uint32_t b = ((uint64_t)k < valid) ? (uint32_t)src[k] : 0u;
-            tf[swz(k >> 5, (k >> 2) & 7) * 4 + (k & 3)] = bf16_lo(b);
+        constexpr int kBatch = 8;                       // loads in flight per thread
+        for (int k0 = threadIdx.x; k0 < elems; k0 += kBatch * THREADS) {
+            uint32_t b[kBatch];
+#pragma unroll
+            for (int i = 0; i < kBatch; ++i) {
+                const int k = k0 + i * THREADS;
+                b[i] = k < elems && (uint64_t)k < valid ? (uint32_t)src[k] : 0u;
+            }
+#pragma unroll
+            for (int i = 0; i < kBatch; ++i) {
+                const int k = k0 + i * THREADS;
+                if (k < elems) tf[swz(k >> 5, (k >> 2) & 7) * 4 + (k & 3)] = bf16_lo(b[i]);
+            }
         }
     }
 }
