@@ -177,7 +177,7 @@ def stress_case(torch, mqg, lib, check, peak):
         row = {"bits": b, "quantize_all_workers": _entry(q[0], q[1], qb, peak),
                "quantize_us_per_worker": q[0] / W, "server_step": _entry(s[0], s[1], sb, peak)}
         row["quantize_all_workers"]["fp32_equivalent_grad_gbs"] = W * 4 * n / q[0] / 1e3
-        # the ceiling this kernel actually runs against: warp instructions issued per second (14.3 executed
+        # the ceiling this kernel actually runs against: warp instructions issued per second (12.4 executed
         # instructions per element, from the ncu counters of the bf16 instantiation) against one instruction
         # per cycle and scheduler at the maximum SM clock
         row["quantize_all_workers"]["issue_rate"] = {

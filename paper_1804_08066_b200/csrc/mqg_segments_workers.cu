@@ -7,7 +7,7 @@
 //   3. encode_entries_kernel - the longer ones' encode.  Every (worker, segment) pair is an entry with a tensor map of its
 //      own; the persistent CTAs walk the 128-row tiles of all entries as one sequence, fed by tiled bulk copies; a launch
 //      for every 64 entries.  Segments that start where bulk copies cannot go through encode_table_kernel instead.
-// Where the first two do not go together (spans_join_max_pass), span_kernel also clears the scales and absmax_table_kernel
+// Where these two do not go together (spans_join_max_pass), span_kernel also clears the scales and absmax_table_kernel
 // follows it.
 // Worker w's outputs are the same whichever way a segment goes and however many workers there are.
 #include <string.h>
@@ -28,14 +28,14 @@ constexpr uint64_t kSegmentSpanElems = 512 * 32;
 
 // Whether the spans and the max pass share a launch (`tiles` of 256 rows in the max pass).  Spans on their own are 3 us
 // during which a few CTAs are at work; the launch before then only clears the scales, 1.2 us.  The other side is the spans'
-// registers and shared memory, with which three CTAs share an SM: the max pass reads no slower in fp32 (16 KB requested by
-// every CTA: 592 against 598 us for the quantizer's whole call on eight AlexNet-shaped gradients, 4 bits), but in bf16 (8 KB:
-// 463 against 409 us) or where segments start off a 16-byte boundary (shorter chains of loads: 100 against 93 us for 31 M
-// elements in 16 tensors).  bf16 gradients of 41 M elements in 100 tensors 65 against 70 us, fp32 74 against 81 us; 10 M off
+// registers and shared memory, with which three CTAs share an SM: the max pass reads hardly slower in fp32 (32 KB requested
+// by every CTA: an AlexNet-shaped gradient 80.4 against 83.0 us, four 303 against 305 us, eight with the server's step 763
+// against 759 us), but in bf16 (16 KB: eight 463 against 409 us) or where segments start off a 16-byte boundary (100 against
+// 93 us for 31 M elements in 16 tensors).  bf16 gradients of 41 M elements in 100 tensors 65 against 70 us, fp32 74 against 81 us; 10 M off
 // the boundary in 20 tensors 28 against 30 us.
 static bool spans_join_max_pass(uint64_t tiles, int dtype, bool aligned)
 {
-    return aligned ? dtype == 0 || tiles <= 8192 : tiles <= 2048;
+    return tiles <= (!aligned ? 2048u : dtype == 0 ? 32768u : 8192u);
 }
 
 struct SegEntry {

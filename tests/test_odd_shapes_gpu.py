@@ -95,14 +95,15 @@ def test_sums_over_an_odd_number_of_rows(rows):
         b.check_guards()
 
 
-@pytest.mark.parametrize("longest", [512 * 8192, 512 * 8192 + 1])
-def test_bf16_spans_beside_the_max_pass_and_before_it(longest):
-    """16 workers: 8192 tiles in the max pass, with which the short segment shares a launch, and more."""
+@pytest.mark.parametrize("bf16,longest", [(True, 512 * 8192), (True, 512 * 8192 + 1), (False, 2048 * 8192 + 1)])
+def test_spans_beside_the_max_pass_and_before_it(bf16, longest):
+    """16 workers: 8192 tiles (bf16) or 32,768 in the max pass, with which the short segment shares a launch, and more."""
     W, bits = 16, 3
     seg = np.cumsum([0, 504, longest]).astype(np.uint64)
     code = np.cumsum([0] + [O.code_words(int(b - a), bits) for a, b in zip(seg, seg[1:])]).astype(np.uint64)
-    x = wl.f32_to_bf16_bits(wl.normal(int(seg[-1]), 1e-3, config=3, worker=0))
-    g = to_dev(x.view(np.int16)).view(torch.bfloat16)
+    x = wl.normal(int(seg[-1]), 1e-3, config=3, worker=0)
+    x = wl.f32_to_bf16_bits(x) if bf16 else x
+    g = to_dev(x.view(np.int16)).view(torch.bfloat16) if bf16 else to_dev(x)
     codes = [Guarded(int(code[-1]), torch.int32) for _ in range(W)]
     scales = [Guarded(2, torch.float32) for _ in range(W)]
     mqg.mqg_quantize_segments_workers([g] * W, W, seg, code, bits, 7, [c.view for c in codes], [s.view for s in scales])
@@ -110,6 +111,6 @@ def test_bf16_spans_beside_the_max_pass_and_before_it(longest):
     for w in range(W):
         codes[w].check_guards(), scales[w].check_guards()
         if w in (0, W - 1):
-            c_ref, s_ref = O.quantize_segments(x, seg, code, bits, seed=7, worker=w, dtype="bf16")
+            c_ref, s_ref = O.quantize_segments(x, seg, code, bits, seed=7, worker=w, dtype="bf16" if bf16 else "f32")
             assert np.array_equal(codes[w].numpy(np.uint32), c_ref)
         assert bits_equal(scales[w].numpy(np.float32), s_ref) == 0
