@@ -830,6 +830,127 @@ __device__ __forceinline__ void add_decoded_row(const uint32_t (&w)[BITS], const
     }
 }
 
+// ---- the same sum in units of 2^40, two packed instructions to a pair of codes instead of three --------------------
+// The bit pattern of a float below 2^24 is the float's value in units of 2^-149 (the subnormal floats and the first normal
+// ones), so a code masked in place, q 2^s with s + K <= 24, IS a float.  With the bit below the field set it is
+// (2q + 1) 2^(s - 1), and x^ = (2q - L) h = (2q + 1) h - 2^K h: one fma whose addend is exact, where the sum above first has
+// to bring the code to q - (L - 1) / 2.  (The variant: x^ = q step + lo, no bit below.)
+// The factor is h 2^(150 - s), which has to be finite, so the sum is kept in units of 2^40: every factor, addend and x^ is
+// 2^-40 times what it would be, and what the sum is multiplied with afterwards (-lr, the mean's 1/W, or 1) carries the 2^40.
+// For |h| (step, lo) in [2^-86, 2^18] or 0 that changes no rounding: all x^ and all sums are multiples of 2^-109, in units
+// of 2^40 multiples of 2^-149, so a result that is subnormal there is exact there, and exact in 24 bits here; the largest
+// is below 2^32.  A tile with any other scale is summed by add_decoded_row.
+// What it gives (against the three instructions): 16 workers of 250 M elements at four bits, encode and update 2987 against
+// 3035 us, eight of 25 M re-quantized and applied 75.2 against 77.4 us, the update at two bits 43.6 against 44.5 us.
+constexpr float kSumUnit = 1099511627776.0f, kPerSumUnit = 1.0f / kSumUnit;     // 2^40
+__host__ __device__ inline bool fits_sum_unit(float factor) { return factor > -0x1p80f && factor < 0x1p80f; }
+
+template <int BITS, bool RANGE>
+struct UnitDecode {
+    static constexpr bool kExists = RANGE || BITS >= 2;       // one bit sets a sign instead (one_bit_value)
+    // Fields of a window: code i of its group at bit kBase + i BITS.  kBase >= 1 leaves the bit below the first field,
+    // kBase + kGroup BITS <= 24 keeps the pattern an integer, and with kBase a multiple of the group's offsets in a word
+    // one window of a word (of the row, for widths that do not divide 32) needs no shift.
+    static constexpr bool kCyclic = 32 % BITS == 0;
+    static constexpr int kGroup = BITS <= 5 ? 4 : 2;
+    static constexpr int kBase = kCyclic ? 8 : BITS == 3 ? 8 : BITS == 5 ? 4 : BITS == 6 ? 12 : 8;
+    static_assert(kBase >= 1 && kBase + kGroup * BITS <= 24, "not an integer");
+    // Order of the factors in a table entry (K = 8: its pairs are fields 1, 0).
+    static constexpr int kFirst = kCyclic && kGroup == 2 ? 1 : 0;
+};
+
+// Whether a (worker, bucket) may be summed in units of 2^40.
+__device__ __forceinline__ bool unit_decode_applies(const DecodeScale& d, bool range)
+{
+    auto fits = [](float x) { return x == 0.0f || (x >= 0x1p-86f && x <= 0x1p18f); };
+    // main codec: two_h = 2h, minus_h = -h
+    return range ? fits(d.two_h) && fits(fabsf(d.minus_h)) : fits(-d.minus_h);
+}
+
+// (factor of the pair's first code, of its second, addend, addend); with four codes to a group the second pair's
+// factors are 2^(-2 BITS) times these.
+template <int BITS, bool RANGE>
+__device__ __forceinline__ float4 unit_decode_entry(const DecodeScale& d)
+{
+    using P = UnitDecode<BITS, RANGE>;
+    // 2^(149 - 40 - s), and one more with the field's odd integer (2q + 1) 2^(s - 1)
+    auto power = [](int i) { return __uint_as_float((uint32_t)(127 + 109 + (RANGE ? 0 : 1) - (P::kBase + i * BITS)) << 23); };
+    const float f = RANGE ? d.two_h : -d.minus_h;
+    const float add = RANGE ? __fmul_rn(d.minus_h, kPerSumUnit) : __fmul_rn(d.minus_h, (float)(1 << BITS) * kPerSumUnit);
+    return make_float4(__fmul_rn(f, power(P::kFirst)), __fmul_rn(f, power(1 - P::kFirst)), add, add);
+}
+
+// The bits below the fields of a window, in registers: a logic operation takes one constant, which is the field's mask.
+// `one` = 1 from a kernel argument, so that they are not constants that are materialised again for every use.
+template <int BITS, bool RANGE>
+struct UnitBits {
+    uint32_t below[UnitDecode<BITS, RANGE>::kGroup];
+    __device__ __forceinline__ explicit UnitBits(uint32_t one)
+    {
+        using P = UnitDecode<BITS, RANGE>;
+#pragma unroll
+        for (int i = 0; i < P::kGroup; ++i) below[i] = RANGE ? 0u : one << (P::kBase + i * BITS - 1);
+    }
+};
+
+// v2[] <- v2[] + de-quantized row, all in units of 2^40; `e` = unit_decode_entry.
+template <int BITS, bool RANGE>
+__device__ __forceinline__ void add_decoded_row_unit(const uint32_t (&w)[BITS], const float4& e,
+                                                     const UnitBits<BITS, RANGE>& bits, float2 (&v2)[16])
+{
+    using P = UnitDecode<BITS, RANGE>;
+    constexpr int G = P::kGroup;
+    constexpr float kStep = 1.0f / (float)(1 << (2 * BITS));
+    const float2 first = make_float2(e.x, e.y), add = make_float2(e.z, e.w);
+    const float2 second = G == 4 ? __fmul2_rn(first, make_float2(kStep, kStep)) : first;
+    auto field = [&](uint32_t win, int i) {
+        const uint32_t mask = ((1u << BITS) - 1u) << (P::kBase + i * BITS);
+        return __uint_as_float(RANGE ? win & mask : (win & mask) | bits.below[i]);
+    };
+    if constexpr (P::kCyclic) {
+        constexpr int kWindows = 32 / (G * BITS), kCodes = 32 / BITS;
+#pragma unroll
+        for (int k = 0; k < BITS; ++k) {
+            uint32_t win[kWindows];                         // the word, and the word rotated by whole groups
+#pragma unroll
+            for (int g = 0; g < kWindows; ++g) win[g] = g == 0 ? w[k] : __funnelshift_r(w[k], w[k], g * G * BITS);
+#pragma unroll
+            for (int c = 0; c < kCodes; c += 2) {
+                float2 m;
+                int i0 = 0;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int from_base = ((c + h) * BITS + 32 - P::kBase) % 32;
+                    const int g = from_base / (G * BITS), i = from_base % (G * BITS) / BITS;
+                    (h == 0 ? m.x : m.y) = field(win[g], i);
+                    if (h == 0) i0 = i;
+                }
+                const int p = (k * kCodes + c) / 2;
+                v2[p] = __fadd2_rn(v2[p], __ffma2_rn(m, G == 4 && i0 == 2 ? second : first, add));
+            }
+        }
+    } else {
+#pragma unroll
+        for (int grp = 0; grp < 32 / G; ++grp) {
+            const int o = grp * G * BITS, wi = o >> 5, sh = o & 31;
+            uint32_t win;
+            if (sh + G * BITS > 32) {
+                static_assert(P::kBase + G * BITS <= 32, "");
+                const int r = sh - P::kBase;                // > 0: a straddling group starts above the base
+                win = __funnelshift_r(w[wi], w[wi + 1 < BITS ? wi + 1 : wi], r);
+            } else {
+                win = sh >= P::kBase ? w[wi] >> (sh - P::kBase) : w[wi] << (P::kBase - sh);
+            }
+#pragma unroll
+            for (int h = 0; h < G / 2; ++h) {
+                const int p = grp * (G / 2) + h;
+                const float2 m = make_float2(field(win, 2 * h), field(win, 2 * h + 1));
+                v2[p] = __fadd2_rn(v2[p], __ffma2_rn(m, h == 1 ? second : first, add));
+            }
+        }
+    }
+}
+
 // v[] (32 floats) <-> v2[] (16 pairs)
 __device__ __forceinline__ void pairs_from_floats(const float (&v)[32], float2 (&v2)[16])
 {

@@ -18,6 +18,7 @@
 #include <string.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "mqg_segments.cuh"
 #include "mqg_tma.cuh"
@@ -58,6 +59,9 @@ struct ServerTmaArgs {
                                  // buckets of 8, 4, 2, 1 rows; W << nbt_shift <= 2 * kMaxWorkers
     int W;
     float neg_lr;
+    float unit_factor;           // what a sum in units of 2^40 is multiplied with: 2^40 times -lr (MODE 1), 1 or the mean's factor
+    uint32_t unit;               // 1: tiles whose scales allow it are summed in units of 2^40
+    uint32_t one;                // 1, as a run-time constant
     uint32_t bias_bits;          // 0x4B000000 (2^23), a run-time constant for the byte permutes
     uint32_t poll_limit;         // polls of one barrier wait before the warp gives up
     uint32_t arm_only;           // test hook: 1 = arm the barriers but issue no parameter copy
@@ -149,19 +153,30 @@ __device__ __forceinline__ void load_tile_scales(const ServerTmaArgs& a, const T
     }
 }
 
-template <int BITS, bool RANGE>
-__device__ __forceinline__ void store_tile_scales(const ServerTmaArgs& a, float4* table, uint32_t lane,
+// Returns (for the whole warp) whether the entries are those of a sum in units of 2^40 (UNIT: where such a sum may be).
+template <int BITS, bool RANGE, bool UNIT>
+__device__ __forceinline__ bool store_tile_scales(const ServerTmaArgs& a, float4* table, uint32_t lane,
                                                   bool wide, const float2 (&s)[2])
 {
+    DecodeScale d[2];
+    bool fits = UNIT && a.unit != 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if (h == 1 && !wide) break;
+        // a pair beyond the last worker has the scale 0 and is not stored
+        d[h] = RANGE ? range_decode_scale<BITS>(s[h].x, s[h].y) : decode_scale<BITS>(s[h].x);
+        if (UNIT) fits = fits && unit_decode_applies(d[h], RANGE);
+    }
+    if (UNIT) fits = __all_sync(0xFFFFFFFFu, fits);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         if (h == 1 && !wide) break;
         const uint32_t pair = lane + 32u * h, w = pair >> a.nbt_shift;
-        if (w < (uint32_t)a.W) {
-            const DecodeScale d = RANGE ? range_decode_scale<BITS>(s[h].x, s[h].y) : decode_scale<BITS>(s[h].x);
-            table[pair] = make_float4(d.two_h, d.two_h, d.minus_h, d.minus_h);
-        }
+        if (w < (uint32_t)a.W)
+            table[pair] = UNIT && fits ? unit_decode_entry<BITS, RANGE>(d[h])
+                                       : make_float4(d[h].two_h, d[h].two_h, d[h].minus_h, d[h].minus_h);
     }
+    return fits;
 }
 
 // A lane's K words of one worker from a code stage, with the widest shared-memory access the
@@ -356,6 +371,11 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
     // of all warps then stand in front of the codes of all warps)
     const bool params_first = ntiles < 4;
 
+    // A sum that continues from an accumulator is not kept in other units: the accumulator need not fit them.
+    constexpr bool kUnit = UnitDecode<BITS, RANGE>::kExists && MODE != 2;
+    const UnitBits<BITS, RANGE> unit_bits(a.one);
+    bool unit = false;                             // the tile in work is summed in units of 2^40
+
     bool failed = false;
     uint32_t k = 0, u = 0;                         // tile and code stage in use
     if (ntiles > 0) {
@@ -377,7 +397,7 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
                                       (int)(u2 % groups) * kGroup, lane_off);
             cp_async_commit();
         }
-        store_tile_scales<BITS, RANGE>(a, table, lane, wide, s0);
+        unit = store_tile_scales<BITS, RANGE, kUnit>(a, table, lane, wide, s0);
         __syncwarp();
     }
     // position of the code stage kCodeDepth ahead of the one in use, kept incrementally
@@ -432,13 +452,21 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
             cp_async_wait_group<kCodeDepth - 1>();     // this lane's pieces of the stage have landed
             __syncwarp();                              // ... and so have the other lanes'
             const int g0 = (int)g * kGroup;
-            auto decode_worker = [&](int i) {
+            auto decode_worker = [&](int i, auto in_units) {
                 uint32_t w[BITS];
                 read_stage_words<BITS>(cstage + i * kWorkerWords, w);
                 const float4 e = my_table[(uint32_t)(g0 + i) << a.nbt_shift];
-                DecodeScale2 d;
-                d.two_h = make_float2(e.x, e.y); d.minus_h = make_float2(e.z, e.w);
-                add_decoded_row<BITS, RANGE>(w, d, v2, a.bias_bits);
+                if constexpr (decltype(in_units)::value) {
+                    add_decoded_row_unit<BITS, RANGE>(w, e, unit_bits, v2);
+                } else {
+                    DecodeScale2 d;
+                    d.two_h = make_float2(e.x, e.y); d.minus_h = make_float2(e.z, e.w);
+                    add_decoded_row<BITS, RANGE>(w, d, v2, a.bias_bits);
+                }
+            };
+            auto decode_any = [&](int i) {
+                if (kUnit && unit) decode_worker(i, std::integral_constant<bool, kUnit>());
+                else decode_worker(i, std::false_type());
             };
             // MODE 1: the parameter stage held tile k-1, whose store was committed at the end of the last
             // iteration: once that store has read its source the stage takes tile k, which is not
@@ -460,17 +488,26 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
                     // (the positions a whole stage can hold issue_at at: worker 4 when W >= 5, else the
                     // stage's last worker when W == group size)
                     if (MODE == 1 && g0 + i0 == issue_at) load_params();
+                    const bool at_last = MODE == 1 && i0 + 3 == kGroup - 1 && g0 + i0 + 3 == issue_at;
+                    if (!kUnit || unit) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        if (MODE == 1 && i == 3 && i0 + i == kGroup - 1 && g0 + i0 + i == issue_at) load_params();
-                        decode_worker(i0 + i);
+                        for (int i = 0; i < 4; ++i) {
+                            if (MODE == 1 && i == 3 && at_last) load_params();
+                            decode_worker(i0 + i, std::integral_constant<bool, kUnit>());
+                        }
+                    } else {
+#pragma unroll 1
+                        for (int i = 0; i < 4; ++i) {
+                            if (MODE == 1 && i == 3 && at_last) load_params();
+                            decode_worker(i0 + i, std::false_type());
+                        }
                     }
                 }
             } else {
 #pragma unroll 1
                 for (int i = 0; g0 + i < a.W; ++i) {
                     if (MODE == 1 && g0 + i == issue_at) load_params();
-                    decode_worker(i);
+                    decode_any(i);
                 }
             }
             __syncwarp();                          // every lane has read the stage: refill it
@@ -496,11 +533,16 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
 
         {
             float4* tl = reinterpret_cast<float4*>(stage);
-            const float2 nlr = make_float2(a.neg_lr, a.neg_lr);
+            const float factor = kUnit && unit ? a.unit_factor : MODE == 1 ? a.neg_lr : 1.0f;
+            const float2 nlr = make_float2(factor, factor);
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 const int idx = swz((int)lane, c);
                 float2 lo = v2[2 * c], hi = v2[2 * c + 1];
+                if constexpr (MODE == 0 && kUnit) {
+                    lo = __fmul2_rn(nlr, lo);
+                    hi = __fmul2_rn(nlr, hi);
+                }
                 if constexpr (MODE == 1) {          // params <- fma(-lr, sum, params), in place
                     const float4 p = tl[idx];
                     lo = __ffma2_rn(nlr, lo, make_float2(p.x, p.y));
@@ -513,7 +555,7 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
         if (have_next) {
             // constants of the next tile; the table was last read before the group loop's last
             // __syncwarp
-            store_tile_scales<BITS, RANGE>(a, table, lane, wide, s_next);
+            unit = store_tile_scales<BITS, RANGE, kUnit>(a, table, lane, wide, s_next);
         }
         __syncwarp();
         if (lane == 0) {
@@ -722,6 +764,14 @@ static int server_tma_nbt_shift(uint64_t n, uint64_t bucket, int W)
 
 bool server_tma_applies(uint64_t n, uint64_t bucket, int W) { return server_tma_nbt_shift(n, bucket, W) >= 0; }
 
+// `factor`: what the sum is multiplied with.
+static void set_sum_unit(ServerTmaArgs& a, float factor)
+{
+    a.unit = fits_sum_unit(factor) ? 1u : 0u;
+    a.unit_factor = factor * kSumUnit;
+    a.one = 1u;
+}
+
 // mode 1: dst = params (update with lr); mode 0: dst = acc (overwrite); mode 2: dst = acc (add into)
 template <bool RANGE>
 static cudaError_t launch_server_tma_codec(const WorkerPtrs& ptrs, int W, int bits, uint64_t n, uint64_t bucket,
@@ -745,6 +795,7 @@ static cudaError_t launch_server_tma_codec(const WorkerPtrs& ptrs, int W, int bi
     if (a.nbt_shift < 0) return cudaErrorInvalidValue;
     a.W = W;
     a.neg_lr = -lr;
+    set_sum_unit(a, mode == 1 ? -lr : 1.0f);
     a.bias_bits = 0x4B000000u;
     const WaitPolicy policy = wait_policy();
     a.poll_limit = policy.poll_limit;
@@ -843,11 +894,14 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
         if (t.row0 < a.nrows_full) fill_code_stage<BITS>(a, stage, t, g0, lane_off);
     };
 
+    constexpr bool kUnit = UnitDecode<BITS, false>::kExists;
+    const UnitBits<BITS, false> unit_bits(a.one);
+    bool unit = false;                             // as in the server kernel
     uint32_t u = 0;
     if (nct > 0) {
         float2 s0[2];
         load_tile_scales<false, false>(a, tile_loc(0), lane, wide, s0);
-        store_tile_scales<BITS, false>(a, table, lane, wide, s0);
+        unit = store_tile_scales<BITS, false, kUnit>(a, table, lane, wide, s0);
 #pragma unroll
         for (uint32_t u2 = 0; u2 < (uint32_t)kCodeDepth; ++u2) {
             if (u2 < nunits) fill(code_base + u2 * kCodeStageBytes, u2 / groups, (int)(u2 % groups) * kGroup);
@@ -878,20 +932,28 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
             cp_async_wait_group<kCodeDepth - 1>();
             __syncwarp();
             const int g0 = (int)g * kGroup;
-            auto decode_worker = [&](int i) {
+            auto decode_worker = [&](int i, auto in_units) {
                 uint32_t w[BITS];
                 read_stage_words<BITS>(cstage + i * kWorkerWords, w);
                 const float4 e = my_table[(uint32_t)(g0 + i) << a.nbt_shift];
-                DecodeScale2 d;
-                d.two_h = make_float2(e.x, e.y); d.minus_h = make_float2(e.z, e.w);
-                add_decoded_row<BITS, false>(w, d, v2, a.bias_bits);
+                if constexpr (decltype(in_units)::value) {
+                    add_decoded_row_unit<BITS, false>(w, e, unit_bits, v2);
+                } else {
+                    DecodeScale2 d;
+                    d.two_h = make_float2(e.x, e.y); d.minus_h = make_float2(e.z, e.w);
+                    add_decoded_row<BITS, false>(w, d, v2, a.bias_bits);
+                }
             };
-            if (g0 + kGroup <= a.W) {
+            const int here = min(kGroup, a.W - g0);
+            if (kUnit && !unit) {
+#pragma unroll 1
+                for (int i = 0; i < here; ++i) decode_worker(i, std::false_type());
+            } else if (here == kGroup) {
 #pragma unroll
-                for (int i = 0; i < kGroup; ++i) decode_worker(i);
+                for (int i = 0; i < kGroup; ++i) decode_worker(i, std::integral_constant<bool, kUnit>());
             } else {
 #pragma unroll 1
-                for (int i = 0; g0 + i < a.W; ++i) decode_worker(i);
+                for (int i = 0; i < here; ++i) decode_worker(i, std::integral_constant<bool, kUnit>());
             }
             __syncwarp();                          // every lane has read the stage: refill it
             if (u + kCodeDepth < nunits) fill(code_base + cs * kCodeStageBytes, fill_tile, (int)fill_group * kGroup);
@@ -904,7 +966,8 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
         const bool active = row < a.nrows_full;
         float x[32];
         {
-            const float2 ms = make_float2(ra.mean_scale, ra.mean_scale);
+            const float factor = kUnit && unit ? a.unit_factor : ra.mean_scale;
+            const float2 ms = make_float2(factor, factor);
 #pragma unroll
             for (int p = 0; p < 16; ++p) {
                 const float2 y = __fmul2_rn(v2[p], ms);
@@ -947,7 +1010,7 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
             encode_pack_row_best<BITS>(x, es, h, w);
             store_row_words<BITS>(ra.codes_out, (uint64_t)row * BITS, w);
         }
-        if (have_next) store_tile_scales<BITS, false>(a, table, lane, wide, s_next);
+        if (have_next) unit = store_tile_scales<BITS, false, kUnit>(a, table, lane, wide, s_next);
         __syncwarp();
     }
     cp_async_wait_group<0>();                                  // no code copy outlives the warp
@@ -1011,6 +1074,7 @@ cudaError_t launch_requantize_warp(const WorkerPtrs& ptrs, int W, int bits, uint
     a.nbt_shift = 0;                                     // buckets a tile of 32 rows touches: 32 / rpb
     while (rpb < 32 && (rpb << a.nbt_shift) < 32) ++a.nbt_shift;
     a.W = W;
+    set_sum_unit(a, mean_scale);
     a.bias_bits = 0x4B000000u;
     ra.codes_out = codes_out; ra.scales_out = scales_out;
     ra.mean_scale = mean_scale;
@@ -1113,6 +1177,7 @@ cudaError_t launch_server_tma_segments(const WorkerPtrs& ptrs, int W, int bits, 
     a.nbt_shift = 0;                     // a tile lies in one bucket: table entry = worker
     a.W = W;
     a.neg_lr = -lr;
+    set_sum_unit(a, -lr);
     a.bias_bits = 0x4B000000u;
     const WaitPolicy policy = wait_policy();
     a.poll_limit = policy.poll_limit;
