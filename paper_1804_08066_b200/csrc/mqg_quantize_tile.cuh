@@ -92,25 +92,43 @@ __device__ __forceinline__ float row_abs_max_bf16(const uint32_t (&u)[16])
     return max3_abs(0.0f, bf16_lo(m[0]), bf16_hi(m[0]));      // from 0: a row that is NaN throughout does not count
 }
 
-// The one row of the gradient that is shorter than 32 elements is not covered by the tensor
-// map: its owner copies it (zero-padded) into its own row of the stage with plain loads and
-// then reads it back like any other row.
-template <int DTYPE>
-__device__ __noinline__ void stage_ragged_row(uint8_t* stage, int row, const void* grad, uint64_t e0,
-                                              uint64_t n)
+constexpr int kBf16Wide = 2;                 // as DTYPE of the tile, the shared memory and the kernels: rows of 64 elements
+
+// The one row of a gradient that is shorter than the others is not covered by the tensor map.  Before the tile's copy is
+// waited for, the warp that holds it requests it, zeros behind its end, by asynchronous copies of four bytes a lane into a
+// row of the warp's beside the stages.  (Into the stage by its owner after the wait is one round trip more: 131,073 elements
+// 2.09 against 2.28 us, eight workers 2.86 against 3.15, the range 1.95 against 2.14.)  `row` is the gradient's, of row_bytes
+// bytes.
+__device__ __forceinline__ void fetch_ragged_row(uint32_t to, const uint8_t* grad, uint64_t row, uint64_t total_bytes,
+                                                 uint32_t row_bytes)
 {
-    for (int j = 0; j < 32; ++j) {
-        const bool in = e0 + j < n;
-        if constexpr (DTYPE == 0) {
-            float* tf = reinterpret_cast<float*>(stage);
-            tf[swz(row, j >> 2) * 4 + (j & 3)] = in ? static_cast<const float*>(grad)[e0 + j] : 0.0f;
-        } else {
-            uint16_t* th = reinterpret_cast<uint16_t*>(stage);
-            const int chunk = (j >> 3) ^ ((row >> 1) & 3);
-            th[(row * 4 + chunk) * 8 + (j & 7)] = in ? static_cast<const uint16_t*>(grad)[e0 + j] : (uint16_t)0;
-        }
-    }
+    const uint32_t b = 4u * (threadIdx.x & 31u);
+    if (b >= row_bytes) return;
+    const uint64_t at = row * row_bytes + b;
+    const uint32_t left = at < total_bytes ? (uint32_t)min(total_bytes - at, (uint64_t)4) : 0u;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
+                 ::"r"(to + b), "l"(grad + (left != 0 ? at : 0)), "r"(left) : "memory");
 }
+
+// For rows of 64, whose launches are long: in a function of its own, so that the code of the tiles without such a row stays
+// as it is (inlined, those took 2 % longer).
+static __device__ __noinline__ void fetch_ragged_wide_row(uint32_t to, const uint8_t* grad, uint64_t row, uint64_t total_bytes)
+{
+    fetch_ragged_row(to, grad, row, total_bytes, 128);
+}
+
+// Whether this thread's warp holds that row: `first` is the row of the warp's lane 0, `rows` the tile's rows from there on.
+__device__ __forceinline__ bool warp_has_row(uint64_t row, uint32_t first, int rows)
+{
+    return row >= first && row - first < (uint64_t)max(min(rows, 32), 0);
+}
+
+// The stage and the row in it from which a thread reads its row: the ragged one is row 0 of a stage of its own (whose
+// swizzle leaves row 0 as it is).
+struct RowSource {
+    const uint8_t* stage;
+    int row;
+};
 
 // How the rows of a bucket are reduced: a bucket is an aligned power-of-two group of at most 32 rows (lane
 // shuffles), a whole number of warps (one shared-memory atomic per warp), or any other number of rows (one
@@ -128,6 +146,7 @@ struct TmaQuantizeShared {
     uint32_t slots[3][kSlots];             // bucket maxima, rotating so no reset races a use
     uint32_t slots_lo[3][kSlots];          // bucket minima of the (min, max) variant, as ordered bits
     float row_sums[THREADS];               // L2 norm, reduction by rows
+    alignas(16) uint8_t ragged[THREADS / 32][128];      // fetch_ragged_row
     alignas(8) uint64_t bar[kStages];
 };
 
@@ -168,6 +187,8 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     const uint32_t t = threadIdx.x;
     const uint32_t row = tile * a.tile_rows + t;
     const bool active = FULL || (t < a.tile_rows && row < (uint32_t)a.nrows);
+    const bool ragged_warp = !FULL && a.nrows > a.nrows_full &&
+                             warp_has_row(a.nrows_full, row - (t & 31u), (int)(a.tile_rows - (t & ~31u)));
     const uint32_t stg = k % kQuantStages, parity = (k / kQuantStages) & 1;
     const uint32_t bar = smem_u32(&sh.bar[stg]);
     uint8_t* stage = sh.stage[stg];
@@ -183,8 +204,11 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     constexpr bool kEarlyDraw = !NORM && DTYPE == 0 && BITS >= 3;
     uint32_t h[16];
     if (kEarlyDraw && active) draw_row_blocks_head(wv.blk0_lo + 4u * row, wv.head, c.rk, h);
+    if (ragged_warp) fetch_ragged_row(smem_u32(sh.ragged[t >> 5]), static_cast<const uint8_t*>(wv.grad), a.nrows_full,
+                                      a.n * (DTYPE == 0 ? 4 : 2), DTYPE == 0 ? 128 : 64);
     bool ok = mbar_try_wait(bar, parity);
     if (!ok) ok = mbar_wait(bar, parity, a.poll_limit);
+    if (ragged_warp) { cp_async_wait_all(); __syncwarp(); }
 
     // bf16 rows whose maximum is wanted stay packed until the encode: half the registers across the barrier, and the
     // maximum takes two elements per instruction (30.0 against 30.5 us per 50 M elements at K = 4)
@@ -192,11 +216,10 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     float x[32];
     uint32_t raw[16];
     if (active) {
-        const bool ragged = !FULL && row >= (uint32_t)a.nrows_full;
-        if (ragged) stage_ragged_row<DTYPE>(stage, (int)t, wv.grad, (uint64_t)row * 32, a.n);
-        if (kPackedRow) read_row_words(stage, (int)t, raw);
-        else read_row_swizzled<DTYPE>(stage, (int)t, x);
-        if (ragged) fence_proxy_async();     // orders those stores before the bulk copy that refills the stage
+        const RowSource src = ragged_warp && row >= (uint32_t)a.nrows_full ? RowSource{sh.ragged[t >> 5], 0}
+                                                                           : RowSource{stage, (int)t};
+        if (kPackedRow) read_row_words(src.stage, src.row, raw);
+        else read_row_swizzled<DTYPE>(src.stage, src.row, x);
     } else {
 #pragma unroll
         for (int j = 0; j < 32; ++j) x[j] = 0.0f;
@@ -319,20 +342,24 @@ __device__ __forceinline__ bool range_quantize_tile(TmaQuantizeShared<DTYPE, THR
     const uint32_t t = threadIdx.x;
     const uint32_t row = tile * a.tile_rows + t;
     const bool active = FULL || (t < a.tile_rows && row < (uint32_t)a.nrows);
+    const bool ragged_warp = !FULL && a.nrows > a.nrows_full &&
+                             warp_has_row(a.nrows_full, row - (t & 31u), (int)(a.tile_rows - (t & ~31u)));
     const uint32_t stg = k % kQuantStages, parity = (k / kQuantStages) & 1;
     const uint32_t bar = smem_u32(&sh.bar[stg]);
     uint8_t* stage = sh.stage[stg];
 
+    if (ragged_warp) fetch_ragged_row(smem_u32(sh.ragged[t >> 5]), static_cast<const uint8_t*>(wv.grad), a.nrows_full,
+                                      a.n * (DTYPE == 0 ? 4 : 2), DTYPE == 0 ? 128 : 64);
     bool ok = mbar_try_wait(bar, parity);
     if (!ok) ok = mbar_wait(bar, parity, a.poll_limit);
+    if (ragged_warp) { cp_async_wait_all(); __syncwarp(); }
 
     float x[32];
     uint32_t mlo = kOrderedMinIdentity, mhi = kOrderedMaxIdentity;
     if (active) {
-        const bool ragged = !FULL && row >= (uint32_t)a.nrows_full;
-        if (ragged) stage_ragged_row<DTYPE>(stage, (int)t, wv.grad, (uint64_t)row * 32, a.n);
-        read_row_swizzled<DTYPE>(stage, (int)t, x);
-        if (ragged) fence_proxy_async();     // orders those stores before the bulk copy that refills the stage
+        const RowSource src = ragged_warp && row >= (uint32_t)a.nrows_full ? RowSource{sh.ragged[t >> 5], 0}
+                                                                           : RowSource{stage, (int)t};
+        read_row_swizzled<DTYPE>(src.stage, src.row, x);
         if (!FULL) {
             const uint64_t left = a.n - (uint64_t)row * 32;      // >= 1
 #pragma unroll
@@ -399,16 +426,6 @@ enum : int { kMaxAbs = 0, kRange = 1, kNorm = 2 };
 // here instead of once per 32.  (122 to 128 registers left to itself: four CTAs per SM, 28.3 us per 50 M elements at
 // K = 4; held to 102, five CTAs, 27.8 us; to 85, six CTAs, 29.5 us; rows of 32 29.8 us.)
 // ---------------------------------------------------------------------------------------
-constexpr int kBf16Wide = 2;                 // as DTYPE of the tile, the shared memory and the kernels
-
-static __device__ __noinline__ void stage_ragged_wide_row(uint8_t* stage, int row, const uint16_t* grad, uint64_t e0,
-                                                          uint64_t n)
-{
-    uint16_t* th = reinterpret_cast<uint16_t*>(stage);
-    for (int j = 0; j < 64; ++j)
-        th[(row * 8 + ((j >> 3) ^ (row & 7))) * 8 + (j & 7)] = e0 + j < n ? grad[e0 + j] : (uint16_t)0;
-}
-
 template <int BITS, int THREADS, bool FULL, int RED, typename Refill>
 __device__ __forceinline__ bool quantize_wide_tile(TmaQuantizeShared<kBf16Wide, THREADS>& sh, const WorkerView wv,
                                                    const QuantizeArgs& a, const TmaQuantizeConsts& c, uint32_t k,
@@ -419,25 +436,29 @@ __device__ __forceinline__ bool quantize_wide_tile(TmaQuantizeShared<kBf16Wide, 
     const uint32_t t = threadIdx.x;
     const uint32_t row = tile * a.tile_rows + t;
     const bool active = FULL || (t < a.tile_rows && row < (uint32_t)a.nrows);
+    const bool ragged_warp = !FULL && a.nrows > a.nrows_full &&
+                             warp_has_row(a.nrows_full, row - (t & 31u), (int)(a.tile_rows - (t & ~31u)));
     const uint32_t stg = k % kQuantStages, parity = (k / kQuantStages) & 1;
     const uint32_t bar = smem_u32(&sh.bar[stg]);
     uint8_t* stage = sh.stage[stg];
 
+    if (ragged_warp)
+        fetch_ragged_wide_row(smem_u32(sh.ragged[t >> 5]), static_cast<const uint8_t*>(wv.grad), a.nrows_full, a.n * 2);
     bool ok = mbar_try_wait(bar, parity);
     if (!ok) ok = mbar_wait(bar, parity, a.poll_limit);
+    if (ragged_warp) { cp_async_wait_all(); __syncwarp(); }
 
     uint32_t raw[2][16];
     if (active) {
-        const bool ragged = !FULL && row >= (uint32_t)a.nrows_full;
-        if (ragged) stage_ragged_wide_row(stage, (int)t, static_cast<const uint16_t*>(wv.grad), (uint64_t)row * 64, a.n);
-        const uint4* s = reinterpret_cast<const uint4*>(stage);
+        const RowSource src = ragged_warp && row >= (uint32_t)a.nrows_full ? RowSource{sh.ragged[t >> 5], 0}
+                                                                           : RowSource{stage, (int)t};
+        const uint4* s = reinterpret_cast<const uint4*>(src.stage);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const uint4 v = s[swz((int)t, i)];
+            const uint4 v = s[swz(src.row, i)];
             uint32_t* to = &raw[i >> 2][(i & 3) * 4];
             to[0] = v.x; to[1] = v.y; to[2] = v.z; to[3] = v.w;
         }
-        if (ragged) fence_proxy_async();     // orders those stores before the bulk copy that refills the stage
     } else {
 #pragma unroll
         for (int j = 0; j < 16; ++j) raw[0][j] = raw[1][j] = 0u;

@@ -72,6 +72,7 @@ encode_entries_kernel(const __grid_constant__ SegEntryTable<CAP> T, unsigned int
     constexpr int kHalves = DTYPE == 0 ? 1 : 2, kElems = 32 * kHalves, kWords = BITS * kHalves;
     struct Shared {
         alignas(1024) uint8_t stage[kStages][kTileBytes];
+        alignas(16) uint8_t ragged[kWarps][128];
         alignas(8) uint64_t bar[kStages];
         uint32_t read[kStages];        // warps that have read the stage, over all its uses
     };
@@ -126,19 +127,22 @@ encode_entries_kernel(const __grid_constant__ SegEntryTable<CAP> T, unsigned int
         const uint32_t bar = smem_u32(&sh.bar[s]);
         uint32_t h[16];
         draw_row_blocks_head(blk0 + 4u * kHalves * row, head, T.rk, h);
+        const bool active = row < rows, ragged_warp = rows > rows_full && warp_has_row(rows_full, row - lane, 32);
+        if (ragged_warp) {
+            const uint32_t to = smem_u32(sh.ragged[t >> 5]);
+            const uint8_t* grad = static_cast<const uint8_t*>(T.e[e].grad);
+            if constexpr (DTYPE == 0) fetch_ragged_row(to, grad, rows_full, T.e[e].n * 4, 128);
+            else fetch_ragged_wide_row(to, grad, rows_full, T.e[e].n * 2);
+        }
         ok = mbar_try_wait(bar, (k / kStages) & 1);
         if (!ok) ok = mbar_wait(bar, (k / kStages) & 1, T.poll_limit);
         if (!__all_sync(0xFFFFFFFFu, ok)) { ok = false; break; }
 
         uint4 v[8];
-        const bool active = row < rows, ragged = active && row >= rows_full;
-        if (ragged) {
-            if constexpr (DTYPE == 0) stage_ragged_row<0>(stage, (int)t, T.e[e].grad, (uint64_t)row * 32, T.e[e].n);
-            else stage_ragged_wide_row(stage, (int)t, static_cast<const uint16_t*>(T.e[e].grad), (uint64_t)row * 64, T.e[e].n);
-        }
+        if (ragged_warp) { cp_async_wait_all(); __syncwarp(); }
+        const RowSource src = ragged_warp && row >= rows_full ? RowSource{sh.ragged[t >> 5], 0} : RowSource{stage, (int)t};
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = reinterpret_cast<const uint4*>(stage)[swz((int)t, i)];
-        if (ragged) fence_proxy_async();   // orders those stores before the bulk copy that refills the stage
+        for (int i = 0; i < 8; ++i) v[i] = reinterpret_cast<const uint4*>(src.stage)[swz(src.row, i)];
         __syncwarp();                      // every lane has read the stage
         bool last = false;
         if (lane == 0) {

@@ -60,7 +60,6 @@ struct ServerTmaArgs {
     int W;
     float neg_lr;
     float unit_factor;           // what a sum in units of 2^40 is multiplied with: 2^40 times -lr (MODE 1), 1 or the mean's factor
-    uint32_t unit;               // 1: tiles whose scales allow it are summed in units of 2^40
     uint32_t one;                // 1, as a run-time constant
     uint32_t bias_bits;          // 0x4B000000 (2^23), a run-time constant for the byte permutes
     uint32_t poll_limit;         // polls of one barrier wait before the warp gives up
@@ -159,7 +158,7 @@ __device__ __forceinline__ bool store_tile_scales(const ServerTmaArgs& a, float4
                                                   bool wide, const float2 (&s)[2])
 {
     DecodeScale d[2];
-    bool fits = UNIT && a.unit != 0;
+    bool fits = UNIT;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         if (h == 1 && !wide) break;
@@ -269,38 +268,55 @@ constexpr int server_min_ctas() { return 4; }
 // MODE 2: dst = acc, the sum continues from the value already there.
 // RANGE: the (min, max) nearest-rounding variant (x^ = fma(q, step, lo)).
 // The one row of a gradient that has fewer than 32 elements (row `row`, the last one): a warp, lane j on
-// element j, with plain loads and stores; the code words and scales of eight workers are requested at a
-// time.  (One thread on the whole row, worker after worker, took about 1 us per worker at the end of the
-// launch.)  `params` is the gradient's first parameter, n its length, its bit stream the words
+// element j, with plain loads and stores.  What bounds it is one round trip to memory and the chain of the sum: the code
+// words of eight workers are requested at a time, and lane w divides for worker w (at most 32).  131,073 parameters, 1 / 8 / 16
+// workers: 2.4 / 3.2 / 4.2 us, against 3.1 / 4.7 / 7.0 us with a division per worker and element, after the warp's tile.
+// `params` is the gradient's first parameter, n its length, its bit stream the words
 // [code_word0, words_end) of every worker's buffer, `bucket` the index of the row's scale.
-template <int BITS, int MODE, bool RANGE>
+// SEGS: every lane divides for every worker.  (With the shuffles in a function that a grid over segments calls, its main loop
+// is compiled to something 2.5 % slower at four bits and eight workers.)
+template <int BITS, int MODE, bool RANGE, bool SEGS>
 __device__ __noinline__ void server_ragged_row(const ServerTmaArgs& a, float* params, uint32_t row, uint64_t n,
                                                uint64_t code_word0, uint64_t words_end, uint32_t bucket, uint32_t lane)
 {
+    static_assert(kMaxWorkers <= 32, "a lane per worker");
     const uint64_t e = (uint64_t)row * 32 + lane;
-    if (e >= n) return;
+    const bool in = e < n;                       // the others keep going: the shuffles need them
+    if (SEGS && !in) return;
     const uint32_t bit = lane * BITS, shift = bit & 31u;
-    const uint64_t word = code_word0 + (uint64_t)row * BITS + (bit >> 5);
+    const uint64_t at = code_word0 + (uint64_t)row * BITS + (bit >> 5), word = at < words_end ? at : words_end - 1;
     const bool two = shift + BITS > 32 && word + 1 < words_end;
-    const float old = MODE != 0 ? params[e] : 0.0f;
+    const float old = MODE != 0 && in ? params[e] : 0.0f;
+    auto load_scale = [&](int w) {
+        return RANGE ? __ldg(reinterpret_cast<const float2*>(a.ptrs.scales[w]) + bucket)
+                     : make_float2(__ldg(a.ptrs.scales[w] + bucket), 0.0f);
+    };
+    auto constants = [](float2 s) { return RANGE ? range_decode_scale<BITS>(s.x, s.y) : decode_scale<BITS>(s.x); };
+    DecodeScale mine = {0.0f, 0.0f};
     float2 v = make_float2(MODE == 2 ? sum_start<BITS, RANGE>(old) : 0.0f, 0.0f);
     constexpr int kBatch = 8;
 #pragma unroll 1
     for (int w0 = 0; w0 < a.W; w0 += kBatch) {
         uint32_t lo[kBatch], hi[kBatch];
-        float2 sc[kBatch];
+        float2 sc[SEGS ? kBatch : 1];
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) {
             if (w0 + i >= a.W) break;
             lo[i] = __ldg(a.ptrs.codes[w0 + i] + word);
             hi[i] = two ? __ldg(a.ptrs.codes[w0 + i] + word + 1) : 0u;
-            if (RANGE) sc[i] = __ldg(reinterpret_cast<const float2*>(a.ptrs.scales[w0 + i]) + bucket);
-            else sc[i] = make_float2(__ldg(a.ptrs.scales[w0 + i] + bucket), 0.0f);
+            if (SEGS) sc[SEGS ? i : 0] = load_scale(w0 + i);
         }
+        if (!SEGS && w0 == 0) mine = constants(load_scale(min((int)lane, a.W - 1)));
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) {
             if (w0 + i >= a.W) break;
-            const DecodeScale d = RANGE ? range_decode_scale<BITS>(sc[i].x, sc[i].y) : decode_scale<BITS>(sc[i].x);
+            DecodeScale d;
+            if (SEGS) {
+                d = constants(sc[SEGS ? i : 0]);
+            } else {
+                d.two_h = __shfl_sync(0xFFFFFFFFu, mine.two_h, w0 + i);
+                d.minus_h = __shfl_sync(0xFFFFFFFFu, mine.minus_h, w0 + i);
+            }
             const uint32_t q = __funnelshift_r(lo[i], hi[i], shift) & ((1u << BITS) - 1u);
             if constexpr (BITS == 1 && !RANGE)
                 v.x = __fadd_rn(v.x, one_bit_value(d.minus_h, q << 31));
@@ -309,10 +325,10 @@ __device__ __noinline__ void server_ragged_row(const ServerTmaArgs& a, float* pa
                                              make_float2(d.two_h, d.two_h), make_float2(d.minus_h, d.minus_h));
         }
     }
-    params[e] = MODE == 1 ? __fmaf_rn(a.neg_lr, v.x, old) : v.x;
+    if (in) params[e] = MODE == 1 ? __fmaf_rn(a.neg_lr, v.x, old) : v.x;
 }
 
-template <int BITS, int MODE, bool RANGE, bool SEGS>
+template <int BITS, int MODE, bool RANGE, bool SEGS, bool kUnit>
 __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, const ServerTmaArgs& a,
                                                 const ServerSegTable* segs, unsigned int* __restrict__ timeouts)
 {
@@ -371,8 +387,6 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
     // of all warps then stand in front of the codes of all warps)
     const bool params_first = ntiles < 4;
 
-    // A sum that continues from an accumulator is not kept in other units: the accumulator need not fit them.
-    constexpr bool kUnit = UnitDecode<BITS, RANGE>::kExists && MODE != 2;
     const UnitBits<BITS, RANGE> unit_bits(a.one);
     bool unit = false;                             // the tile in work is summed in units of 2^40
 
@@ -464,10 +478,7 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
                     add_decoded_row<BITS, RANGE>(w, d, v2, a.bias_bits);
                 }
             };
-            auto decode_any = [&](int i) {
-                if (kUnit && unit) decode_worker(i, std::integral_constant<bool, kUnit>());
-                else decode_worker(i, std::false_type());
-            };
+            const std::integral_constant<bool, kUnit> units;
             // MODE 1: the parameter stage held tile k-1, whose store was committed at the end of the last
             // iteration: once that store has read its source the stage takes tile k, which is not
             // needed before the last worker is summed.  The load starts when half of eight workers are
@@ -482,32 +493,30 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
                 }
             };
             static_assert(kIssueAt == 4 && kGroup % 4 == 0, "the parameter load is issued between blocks of four workers");
-            if (g0 + kGroup <= a.W) {              // a whole stage: blocks of four workers in straight-line code
+            const bool in_units = !kUnit || __builtin_expect(unit, 1);
+            if (in_units && g0 + kGroup <= a.W) {  // a whole stage: blocks of four workers in straight-line code
 #pragma unroll 1
                 for (int i0 = 0; i0 < kGroup; i0 += 4) {
                     // (the positions a whole stage can hold issue_at at: worker 4 when W >= 5, else the
                     // stage's last worker when W == group size)
                     if (MODE == 1 && g0 + i0 == issue_at) load_params();
-                    const bool at_last = MODE == 1 && i0 + 3 == kGroup - 1 && g0 + i0 + 3 == issue_at;
-                    if (!kUnit || unit) {
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            if (MODE == 1 && i == 3 && at_last) load_params();
-                            decode_worker(i0 + i, std::integral_constant<bool, kUnit>());
-                        }
-                    } else {
-#pragma unroll 1
-                        for (int i = 0; i < 4; ++i) {
-                            if (MODE == 1 && i == 3 && at_last) load_params();
-                            decode_worker(i0 + i, std::false_type());
-                        }
+                    for (int i = 0; i < 4; ++i) {
+                        if (MODE == 1 && i == 3 && i0 + i == kGroup - 1 && g0 + i0 + i == issue_at) load_params();
+                        decode_worker(i0 + i, units);
                     }
                 }
-            } else {
+            } else if (in_units) {
 #pragma unroll 1
                 for (int i = 0; g0 + i < a.W; ++i) {
                     if (MODE == 1 && g0 + i == issue_at) load_params();
-                    decode_any(i);
+                    decode_worker(i, units);
+                }
+            } else {                               // a tile with a scale outside the range: one worker after another
+#pragma unroll 1
+                for (int i = 0; i < kGroup && g0 + i < a.W; ++i) {
+                    if (MODE == 1 && g0 + i == issue_at) load_params();
+                    decode_worker(i, std::false_type());
                 }
             }
             __syncwarp();                          // every lane has read the stage: refill it
@@ -584,31 +593,31 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
         bulk_wait_all<0>();                                    // stores done before the stage goes away
     }
 
-    // A last row of fewer than 32 elements is not covered by the tensor map: the grid's last warp takes it
-    // (SEGS: the segments that have such a row go to the grid's last warps in turn; those have a tile less than
-    // the first ones, unless all have the same number).
+    // A last row of fewer than 32 elements is not covered by the tensor map: the grid's last warp takes it, which has no
+    // tile unless the grid is as large as it may be.  (SEGS: the segments that have such a row go to the grid's last warps
+    // in turn.)
     const uint32_t from_end = nwarps - 1 - gwarp;
     if constexpr (SEGS) {
         for (uint32_t j = from_end; j < (uint32_t)segs->nseg; j += nwarps) {
             const ServerSegEntry& e = segs->e[j];
             if (e.ragged == 0) continue;
             const uint64_t n = (uint64_t)e.nrows_full * 32 + e.ragged;
-            server_ragged_row<BITS, MODE, RANGE>(a, a.params + e.elem0, e.nrows_full, n, e.code_word0,
+            server_ragged_row<BITS, MODE, RANGE, SEGS>(a, a.params + e.elem0, e.nrows_full, n, e.code_word0,
                                                  e.code_word0 + (n * BITS + 31) / 32, e.scale_idx, lane);
         }
     } else if (a.nrows > a.nrows_full && from_end == 0) {
-        server_ragged_row<BITS, MODE, RANGE>(a, a.params, a.nrows_full, a.n, 0, a.ncode_words,
+        server_ragged_row<BITS, MODE, RANGE, SEGS>(a, a.params, a.nrows_full, a.n, 0, a.ncode_words,
                                              bucket_of_row(a, a.nrows_full), lane);
     }
 }
 
-// One gradient with uniform buckets.
-template <int BITS, int MODE, bool RANGE>
+// One gradient with uniform buckets.  UNIT: tiles whose scales allow it are summed in units of 2^40.
+template <int BITS, int MODE, bool RANGE, bool UNIT>
 __global__ void __launch_bounds__(kSrvThreads, server_min_ctas<BITS>())
 server_tma_kernel(const __grid_constant__ CUtensorMap map_full, const __grid_constant__ ServerTmaArgs a,
                   unsigned int* __restrict__ timeouts)
 {
-    server_tma_body<BITS, MODE, RANGE, false>(&map_full, a, nullptr, timeouts);
+    server_tma_body<BITS, MODE, RANGE, false, UNIT>(&map_full, a, nullptr, timeouts);
 }
 
 // The short segments of a per-layer step (those that are not entries of the segment table): their
@@ -672,24 +681,37 @@ __device__ __noinline__ void server_short_piece(const ServerTmaArgs& a, const Se
 }
 
 // Several long segments of a per-layer step (fused update only), then the step's short segments.
-template <int BITS>
+template <int BITS, bool UNIT>
 __global__ void __launch_bounds__(kSrvThreads, server_min_ctas<BITS>())
 server_tma_segments_kernel(const __grid_constant__ ServerSegTable segs, const __grid_constant__ ServerShortSegs ss,
                            const __grid_constant__ ServerTmaArgs a, unsigned int* __restrict__ timeouts)
 {
-    server_tma_body<BITS, 1, false, true>(nullptr, a, &segs, timeouts);
+    server_tma_body<BITS, 1, false, true, UNIT>(nullptr, a, &segs, timeouts);
     const uint32_t wid = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0);
-    const uint32_t nwarps = gridDim.x * kSrvWarps;
-    // the warps that finished their share of the long segments first are the last ones of the grid
-    for (uint32_t piece = nwarps - 1 - (blockIdx.x * kSrvWarps + wid); piece < ss.pieces; piece += nwarps)
+    const uint32_t nwarps = gridDim.x * kSrvWarps, from_end = nwarps - 1 - (blockIdx.x * kSrvWarps + wid);
+    // the warps that finished their share of the long segments first are the last ones of the grid; the very last ones may
+    // have a segment's last row
+    const uint32_t skip = (uint32_t)segs.nseg % nwarps;
+    for (uint32_t piece = from_end >= skip ? from_end - skip : from_end + nwarps - skip; piece < ss.pieces; piece += nwarps)
         server_short_piece<BITS>(a, ss, piece, threadIdx.x & 31u);
 }
 
-template <int BITS, int MODE, bool RANGE>
+// Whether a launch sums in units of 2^40, and its arguments for that; `factor`: what the sum is multiplied with.  From a
+// whole code stage of workers on: with fewer, what it saves is less than what the second form of the decode costs a launch
+// (three workers, four bits: 7.9 against 7.5 us for 5 M parameters, 2.85 against 2.7 us for 131,072).
+template <int BITS>
+static bool sum_in_units(ServerTmaArgs& a, float factor)
+{
+    a.unit_factor = factor * kSumUnit;
+    a.one = 1u;
+    return a.W >= ServerGroup<BITS>::value && fits_sum_unit(factor);
+}
+
+template <int BITS, int MODE, bool RANGE, bool UNIT>
 static cudaError_t launch_server_tma_inst(const void* params, ServerTmaArgs& a, unsigned int* timeouts,
                                           cudaStream_t stream)
 {
-    auto kernel = server_tma_kernel<BITS, MODE, RANGE>;
+    auto kernel = server_tma_kernel<BITS, MODE, RANGE, UNIT>;
     constexpr size_t kSmemBytes = sizeof(ServerSmem<BITS>) + 1024;   // + slack to round the base up
     static std::atomic<int> grid_cap[64];                 // per device; 0 = not yet set up (zero-initialised)
     int dev = 0;
@@ -713,8 +735,10 @@ static cudaError_t launch_server_tma_inst(const void* params, ServerTmaArgs& a, 
     // against at least four tiles per warp (and the parameter tile, the scales and the codes of a warp's first
     // tile requested in turn): 3.4 against 7.4 us at n = 2^20, W = 4, 5.4 against 12.5 us at W = 16, 6.7 against
     // 8.8 us at n = 2^22, W = 4.
+    // A last row of fewer than 32 elements is a warp's of its own.
+    const uint64_t warps = (uint64_t)a.ntiles + (a.nrows > a.nrows_full ? 1 : 0);
     uint64_t grid = (uint64_t)cap;
-    if (grid * kSrvWarps > a.ntiles) grid = (a.ntiles + kSrvWarps - 1) / kSrvWarps;
+    if (grid * kSrvWarps > warps) grid = (warps + kSrvWarps - 1) / kSrvWarps;
     CUtensorMap map_full;
     const char* why = nullptr;
     if (!encode_rows_map(&map_full, params, a.nrows_full, 4, 32, kSrvTileRows, &why)) return cudaErrorNotSupported;
@@ -727,9 +751,15 @@ template <int BITS, bool RANGE>
 static cudaError_t launch_server_tma_bits(const void* dst, ServerTmaArgs& a, int mode, unsigned int* timeouts,
                                           cudaStream_t stream)
 {
-    if (mode == 1) return launch_server_tma_inst<BITS, 1, RANGE>(dst, a, timeouts, stream);
-    if (mode == 2) return launch_server_tma_inst<BITS, 2, RANGE>(dst, a, timeouts, stream);
-    return launch_server_tma_inst<BITS, 0, RANGE>(dst, a, timeouts, stream);
+    // a sum that continues from an accumulator is not kept in other units: the accumulator need not fit them
+    if (mode == 2) return launch_server_tma_inst<BITS, 2, RANGE, false>(dst, a, timeouts, stream);
+    if constexpr (UnitDecode<BITS, RANGE>::kExists) {
+        if (sum_in_units<BITS>(a, mode == 1 ? a.neg_lr : 1.0f))
+            return mode == 1 ? launch_server_tma_inst<BITS, 1, RANGE, true>(dst, a, timeouts, stream)
+                             : launch_server_tma_inst<BITS, 0, RANGE, true>(dst, a, timeouts, stream);
+    }
+    return mode == 1 ? launch_server_tma_inst<BITS, 1, RANGE, false>(dst, a, timeouts, stream)
+                     : launch_server_tma_inst<BITS, 0, RANGE, false>(dst, a, timeouts, stream);
 }
 
 bool server_tma_applies(uint64_t n, uint64_t bucket)
@@ -764,14 +794,6 @@ static int server_tma_nbt_shift(uint64_t n, uint64_t bucket, int W)
 
 bool server_tma_applies(uint64_t n, uint64_t bucket, int W) { return server_tma_nbt_shift(n, bucket, W) >= 0; }
 
-// `factor`: what the sum is multiplied with.
-static void set_sum_unit(ServerTmaArgs& a, float factor)
-{
-    a.unit = fits_sum_unit(factor) ? 1u : 0u;
-    a.unit_factor = factor * kSumUnit;
-    a.one = 1u;
-}
-
 // mode 1: dst = params (update with lr); mode 0: dst = acc (overwrite); mode 2: dst = acc (add into)
 template <bool RANGE>
 static cudaError_t launch_server_tma_codec(const WorkerPtrs& ptrs, int W, int bits, uint64_t n, uint64_t bucket,
@@ -795,7 +817,6 @@ static cudaError_t launch_server_tma_codec(const WorkerPtrs& ptrs, int W, int bi
     if (a.nbt_shift < 0) return cudaErrorInvalidValue;
     a.W = W;
     a.neg_lr = -lr;
-    set_sum_unit(a, mode == 1 ? -lr : 1.0f);
     a.bias_bits = 0x4B000000u;
     const WaitPolicy policy = wait_policy();
     a.poll_limit = policy.poll_limit;
@@ -853,7 +874,7 @@ struct RequantSmem {
     uint32_t bmax[2][kSrvWarps];                  // tile maxima, double-buffered by the parity of the turn
 };
 
-template <int BITS>
+template <int BITS, bool kUnit>
 __global__ void __launch_bounds__(kSrvThreads, 4)
 requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
 {
@@ -894,7 +915,6 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
         if (t.row0 < a.nrows_full) fill_code_stage<BITS>(a, stage, t, g0, lane_off);
     };
 
-    constexpr bool kUnit = UnitDecode<BITS, false>::kExists;
     const UnitBits<BITS, false> unit_bits(a.one);
     bool unit = false;                             // as in the server kernel
     uint32_t u = 0;
@@ -1016,10 +1036,10 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
     cp_async_wait_group<0>();                                  // no code copy outlives the warp
 }
 
-template <int BITS>
+template <int BITS, bool UNIT>
 static cudaError_t launch_requantize_warp_inst(const RequantWarpArgs& ra, cudaStream_t stream)
 {
-    auto kernel = requantize_warp_kernel<BITS>;
+    auto kernel = requantize_warp_kernel<BITS, UNIT>;
     constexpr size_t kSmemBytes = sizeof(RequantSmem<BITS>) + 16;
     static std::atomic<int> grid_cap[64];                 // per device; 0 = not yet set up (zero-initialised)
     int dev = 0;
@@ -1074,7 +1094,6 @@ cudaError_t launch_requantize_warp(const WorkerPtrs& ptrs, int W, int bits, uint
     a.nbt_shift = 0;                                     // buckets a tile of 32 rows touches: 32 / rpb
     while (rpb < 32 && (rpb << a.nbt_shift) < 32) ++a.nbt_shift;
     a.W = W;
-    set_sum_unit(a, mean_scale);
     a.bias_bits = 0x4B000000u;
     ra.codes_out = codes_out; ra.scales_out = scales_out;
     ra.mean_scale = mean_scale;
@@ -1088,24 +1107,24 @@ cudaError_t launch_requantize_warp(const WorkerPtrs& ptrs, int W, int bits, uint
     ra.rk.worker = worker; ra.rk.step = step;
     ra.head = philox_head(0u, worker, ra.rk.k0[0]);
     switch (bits) {
-        case 1: return launch_requantize_warp_inst<1>(ra, stream);
-        case 2: return launch_requantize_warp_inst<2>(ra, stream);
-        case 3: return launch_requantize_warp_inst<3>(ra, stream);
-        case 4: return launch_requantize_warp_inst<4>(ra, stream);
-        case 5: return launch_requantize_warp_inst<5>(ra, stream);
-        case 6: return launch_requantize_warp_inst<6>(ra, stream);
-        case 7: return launch_requantize_warp_inst<7>(ra, stream);
-        case 8: return launch_requantize_warp_inst<8>(ra, stream);
+#define MQG_REQUANT_CASE(B) \
+        case B: \
+            if constexpr (UnitDecode<B, false>::kExists) \
+                if (sum_in_units<B>(a, mean_scale)) return launch_requantize_warp_inst<B, true>(ra, stream); \
+            return launch_requantize_warp_inst<B, false>(ra, stream)
+        MQG_REQUANT_CASE(1); MQG_REQUANT_CASE(2); MQG_REQUANT_CASE(3); MQG_REQUANT_CASE(4);
+        MQG_REQUANT_CASE(5); MQG_REQUANT_CASE(6); MQG_REQUANT_CASE(7); MQG_REQUANT_CASE(8);
+#undef MQG_REQUANT_CASE
     }
     return cudaErrorInvalidValue;
 }
 
 // ---- several long segments of a per-layer step in one launch --------------------------------------
-template <int BITS>
+template <int BITS, bool UNIT>
 static cudaError_t launch_server_segs_inst(const ServerSegTable& tab, const ServerShortSegs& ss, const ServerTmaArgs& a,
                                            unsigned int* timeouts, cudaStream_t stream)
 {
-    auto kernel = server_tma_segments_kernel<BITS>;
+    auto kernel = server_tma_segments_kernel<BITS, UNIT>;
     constexpr size_t kSmemBytes = sizeof(ServerSmem<BITS>) + 1024;   // + slack to round the base up
     static std::atomic<int> grid_cap[64];                 // per device; 0 = not yet set up (zero-initialised)
     int dev = 0;
@@ -1125,7 +1144,7 @@ static cudaError_t launch_server_segs_inst(const ServerSegTable& tab, const Serv
         grid_cap[dev].store(cap, std::memory_order_relaxed);   // every thread computes the same value
     }
     uint64_t grid = (uint64_t)cap;
-    const uint64_t warps = (uint64_t)a.ntiles + ss.pieces;          // at least one tile or short piece per warp
+    const uint64_t warps = (uint64_t)a.ntiles + (uint64_t)tab.nseg + ss.pieces;   // at least one tile, last row or short piece per warp
     if (grid * kSrvWarps > warps) grid = (warps + kSrvWarps - 1) / kSrvWarps;
     return launch_pdl_smem(kernel, (unsigned)grid, kSrvThreads, kSmemBytes, stream, tab, ss, a, timeouts);
 }
@@ -1177,7 +1196,6 @@ cudaError_t launch_server_tma_segments(const WorkerPtrs& ptrs, int W, int bits, 
     a.nbt_shift = 0;                     // a tile lies in one bucket: table entry = worker
     a.W = W;
     a.neg_lr = -lr;
-    set_sum_unit(a, -lr);
     a.bias_bits = 0x4B000000u;
     const WaitPolicy policy = wait_policy();
     a.poll_limit = policy.poll_limit;
@@ -1185,14 +1203,14 @@ cudaError_t launch_server_tma_segments(const WorkerPtrs& ptrs, int W, int bits, 
     unsigned int* timeouts = wait_timeout_counter();
     if (timeouts == nullptr) return cudaErrorNotSupported;
     switch (bits) {
-        case 1: return launch_server_segs_inst<1>(tab, ss, a, timeouts, stream);
-        case 2: return launch_server_segs_inst<2>(tab, ss, a, timeouts, stream);
-        case 3: return launch_server_segs_inst<3>(tab, ss, a, timeouts, stream);
-        case 4: return launch_server_segs_inst<4>(tab, ss, a, timeouts, stream);
-        case 5: return launch_server_segs_inst<5>(tab, ss, a, timeouts, stream);
-        case 6: return launch_server_segs_inst<6>(tab, ss, a, timeouts, stream);
-        case 7: return launch_server_segs_inst<7>(tab, ss, a, timeouts, stream);
-        case 8: return launch_server_segs_inst<8>(tab, ss, a, timeouts, stream);
+#define MQG_SEGS_CASE(B) \
+        case B: \
+            if constexpr (UnitDecode<B, false>::kExists) \
+                if (sum_in_units<B>(a, -lr)) return launch_server_segs_inst<B, true>(tab, ss, a, timeouts, stream); \
+            return launch_server_segs_inst<B, false>(tab, ss, a, timeouts, stream)
+        MQG_SEGS_CASE(1); MQG_SEGS_CASE(2); MQG_SEGS_CASE(3); MQG_SEGS_CASE(4);
+        MQG_SEGS_CASE(5); MQG_SEGS_CASE(6); MQG_SEGS_CASE(7); MQG_SEGS_CASE(8);
+#undef MQG_SEGS_CASE
     }
     return cudaErrorInvalidValue;
 }
