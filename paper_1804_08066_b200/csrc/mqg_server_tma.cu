@@ -157,14 +157,26 @@ template <int BITS, bool RANGE, bool UNIT>
 __device__ __forceinline__ bool store_tile_scales(const ServerTmaArgs& a, float4* table, uint32_t lane,
                                                   bool wide, const float2 (&s)[2])
 {
+    if constexpr (!UNIT) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (h == 1 && !wide) break;
+            const uint32_t pair = lane + 32u * h, w = pair >> a.nbt_shift;
+            if (w < (uint32_t)a.W) {
+                const DecodeScale d = RANGE ? range_decode_scale<BITS>(s[h].x, s[h].y) : decode_scale<BITS>(s[h].x);
+                table[pair] = make_float4(d.two_h, d.two_h, d.minus_h, d.minus_h);
+            }
+        }
+        return false;
+    }
     DecodeScale d[2];
-    bool fits = UNIT;
+    bool fits = true;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         if (h == 1 && !wide) break;
         // a pair beyond the last worker has the scale 0 and is not stored
         d[h] = RANGE ? range_decode_scale<BITS>(s[h].x, s[h].y) : decode_scale<BITS>(s[h].x);
-        if (UNIT) fits = fits && unit_decode_applies(d[h], RANGE);
+        fits = fits && unit_decode_applies(d[h], RANGE);
     }
     if (UNIT) fits = __all_sync(0xFFFFFFFFu, fits);
 #pragma unroll
@@ -172,7 +184,7 @@ __device__ __forceinline__ bool store_tile_scales(const ServerTmaArgs& a, float4
         if (h == 1 && !wide) break;
         const uint32_t pair = lane + 32u * h, w = pair >> a.nbt_shift;
         if (w < (uint32_t)a.W)
-            table[pair] = UNIT && fits ? unit_decode_entry<BITS, RANGE>(d[h])
+            table[pair] = fits ? unit_decode_entry<BITS, RANGE>(d[h])
                                        : make_float4(d[h].two_h, d[h].two_h, d[h].minus_h, d[h].minus_h);
     }
     return fits;
