@@ -51,18 +51,59 @@ __device__ __forceinline__ void encode_store_row(const float (&x)[32], const Sca
 // encode's instructions; CTAs on an SM are in different phases, which overlaps the copies with the encode.
 // Up to 512 rows: 256 threads (one or two rows each) and the registers of three CTAs per SM; longer spans: 512
 // threads, one CTA per SM.
-template <int BITS, int DTYPE, int MODE, int THREADS>
-__device__ __forceinline__ void quantize_span(const TableArgs& a, const SpanTable& tab)
+//
+// JOINED: a span longer than kJoinedChunk elements is a cluster's work, a CTA for every kJoinedChunk of them, one row to a
+// thread; the CTAs' maxima (sums: aligned subtrees of the span's tree) meet through distributed shared memory.  The
+// first `njoined` spans of the table are of that kind, the others go to the CTAs of the clusters that follow, one each.
+struct ClusterPlace {
+    uint32_t size, rank;
+};
+__device__ __forceinline__ ClusterPlace cluster_place()
 {
+    ClusterPlace p;
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(p.size));
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(p.rank));
+    return p;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// The word of CTA `rank` of the cluster that lies where `word` lies in this one.
+__device__ __forceinline__ uint32_t cluster_load(const uint32_t* word, uint32_t rank)
+{
+    uint32_t at, v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(word)), "r"(rank));
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+    return v;
+}
+
+template <int BITS, int DTYPE, int MODE, int THREADS, bool JOINED = false>
+__device__ __forceinline__ void quantize_span(const TableArgs& a, const SpanTable& tab, uint32_t njoined = 0)
+{
+    static_assert(!JOINED || MODE != kSpanRange, "one word per CTA meets");
     extern __shared__ uint8_t smem_raw[];
     float4* tile = reinterpret_cast<float4*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
     constexpr int kWarps = THREADS / 32;
     __shared__ uint32_t s_a[kMaxSpanRows / 32], s_b[kWarps];   // kSpanNorm: a sum per 32 rows, else a word per warp
+    __shared__ uint32_t s_cta;                                 // JOINED: this CTA's maximum or sum
     const uint32_t t = threadIdx.x, lane = t & 31u, wid = t >> 5, w = blockIdx.y;
     grid_dependency_wait();
 
-    uint64_t elem0, len, code0, scale_idx;
-    if (tab.bucket != 0) {
+    uint64_t elem0, len, code0, scale_idx, words_end;
+    bool joined = false, scale_writer = true;
+    if constexpr (JOINED) {
+        const ClusterPlace cta = cluster_place();
+        const uint32_t cluster = blockIdx.x / cta.size;
+        joined = cluster < njoined;
+        const uint32_t j = joined ? cluster : njoined + (cluster - njoined) * cta.size + cta.rank;
+        if (j >= (uint32_t)tab.nspan) return;                  // (a CTA that joins no other)
+        const uint64_t all = tab.len[j], done = joined ? cta.rank * kJoinedChunk : 0;
+        elem0 = tab.elem0[j] + done;
+        len = all <= done ? 0 : all - done > kJoinedChunk ? kJoinedChunk : all - done;
+        code0 = tab.code0[j] + done / 32 * BITS;
+        words_end = tab.code0[j] + (all * BITS + 31) / 32;
+        scale_idx = tab.scale_idx[j];
+        scale_writer = done == 0;
+    } else if (tab.bucket != 0) {
         scale_idx = blockIdx.x;
         elem0 = scale_idx * tab.bucket;
         len = tab.n - elem0 < tab.bucket ? tab.n - elem0 : tab.bucket;
@@ -76,6 +117,7 @@ __device__ __forceinline__ void quantize_span(const TableArgs& a, const SpanTabl
         code0 = tab.code0[blockIdx.x];
         scale_idx = tab.scale_idx[blockIdx.x];
     }
+    if constexpr (!JOINED) words_end = code0 + (len * BITS + 31) / 32;
     const int rows = (int)((len + 31) / 32);
     if constexpr (DTYPE == 0) load_tile_f32<THREADS>(tile, static_cast<const float*>(a.grad[w]) + elem0, len, rows);
     else load_tile_bf16<THREADS>(tile, static_cast<const uint16_t*>(a.grad[w]) + elem0, len, rows);
@@ -105,6 +147,15 @@ __device__ __forceinline__ void quantize_span(const TableArgs& a, const SpanTabl
             }
         }
     }
+    // Every CTA's word to lane `rank` of every warp, 0 to the lanes beyond.  The shared memory stays until the second wait.
+    auto meet = [&](uint32_t word) -> uint32_t {
+        if (t == 0) s_cta = word;
+        cluster_arrive();
+        cluster_wait();
+        const uint32_t v = lane < cluster_place().size ? cluster_load(&s_cta, lane) : 0u;
+        cluster_arrive();
+        return v;
+    };
     float scale = 0.0f;
     RangeEncodeScale range = {0.0f, 0.0f};
     if constexpr (MODE == kSpanNorm) {
@@ -113,9 +164,11 @@ __device__ __forceinline__ void quantize_span(const TableArgs& a, const SpanTabl
         const uint32_t n32 = (uint32_t)(turns * kWarps);
         const float p = 2 * lane < n32 ? __uint_as_float(s_a[2 * lane]) : 0.0f;
         const float q = 2 * lane + 1 < n32 ? __uint_as_float(s_a[2 * lane + 1]) : 0.0f;
-        const float S = warp_tree(__fadd_rn(p, q), 32);
+        float S = warp_tree(__fadd_rn(p, q), 32);
+        if (JOINED && joined)                      // eight leaves, on lanes 0 .. 7
+            S = __shfl_sync(0xFFFFFFFFu, warp_tree(__uint_as_float(meet(__float_as_uint(S))), 8), 0);
         scale = S < flush_limit() ? 0.0f : __fsqrt_rn(S);
-        if (t == 0) a.scales[w][scale_idx] = scale;
+        if (t == 0 && scale_writer) a.scales[w][scale_idx] = scale;
     } else {
         hi = __reduce_max_sync(0xFFFFFFFFu, hi);
         if (MODE == kSpanRange) lo = __reduce_min_sync(0xFFFFFFFFu, lo);
@@ -123,6 +176,7 @@ __device__ __forceinline__ void quantize_span(const TableArgs& a, const SpanTabl
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < kWarps; ++i) { hi = max(hi, s_a[i]); lo = min(lo, s_b[i]); }
+        if (JOINED && joined) hi = __reduce_max_sync(0xFFFFFFFFu, meet(hi));
         if constexpr (MODE == kSpanRange) {
             // a zero of either sign is stored as +0
             const float l = __fadd_rn(from_ordered_bits(lo), 0.0f), h = __fadd_rn(from_ordered_bits(hi), 0.0f);
@@ -131,11 +185,10 @@ __device__ __forceinline__ void quantize_span(const TableArgs& a, const SpanTabl
         } else {
             scale = __uint_as_float(hi);
             if (scale < flush_limit()) scale = 0.0f;
-            if (t == 0) a.scales[w][scale_idx] = scale;
+            if (t == 0 && scale_writer) a.scales[w][scale_idx] = scale;
         }
     }
     const EncodeScale es = encode_scale<BITS>(scale);
-    const uint64_t words_end = code0 + (len * BITS + 31) / 32;
     const bool vec = (reinterpret_cast<uintptr_t>(a.codes[w] + code0) & 15u) == 0;
     for (int r = (int)t; r < rows; r += THREADS) {
         read_row(tile, r, x);
@@ -143,6 +196,7 @@ __device__ __forceinline__ void quantize_span(const TableArgs& a, const SpanTabl
         if constexpr (MODE == kSpanRange) encode_store_row<BITS, true>(x, range, a, w, g0, left, word0, words_end, vec);
         else encode_store_row<BITS, false>(x, es, a, w, g0, left, word0, words_end, vec);
     }
+    if (JOINED && joined) cluster_wait();          // no CTA's shared memory goes before the others have read it
 }
 
 template <int BITS, int DTYPE, int MODE, int THREADS>
@@ -150,6 +204,13 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 3 : 1)
 span_kernel(const __grid_constant__ TableArgs a, const __grid_constant__ SpanTable tab)
 {
     quantize_span<BITS, DTYPE, MODE, THREADS>(a, tab);
+}
+
+template <int BITS, int DTYPE, int MODE>
+__global__ void __launch_bounds__(kMaxTileRows, 3)
+joined_span_kernel(const __grid_constant__ TableArgs a, const __grid_constant__ SpanTable tab, uint32_t njoined)
+{
+    quantize_span<BITS, DTYPE, MODE, kMaxTileRows, true>(a, tab, njoined);
 }
 
 // ---- two passes over tiles of 256 rows ---------------------------------------------------------------
@@ -323,6 +384,58 @@ static cudaError_t launch_span_mode(const TableArgs& a, const SpanTable& tab, un
         MQG_SPAN_CASE(1); MQG_SPAN_CASE(2); MQG_SPAN_CASE(3); MQG_SPAN_CASE(4);
         MQG_SPAN_CASE(5); MQG_SPAN_CASE(6); MQG_SPAN_CASE(7); MQG_SPAN_CASE(8);
 #undef MQG_SPAN_CASE
+    }
+    return cudaErrorInvalidValue;
+}
+
+// The first `njoined` spans of the list are longer than kJoinedChunk.
+template <int BITS, int DTYPE, int MODE>
+static cudaError_t launch_joined_inst(const TableArgs& a, const SpanTable& tab, uint32_t njoined, unsigned cluster,
+                                      uint64_t most, cudaStream_t stream)
+{
+    cudaLaunchConfig_t cfg = {};
+    const unsigned alone = (unsigned)tab.nspan - njoined;
+    cfg.gridDim = dim3((njoined + (alone + cluster - 1) / cluster) * cluster, (unsigned)a.W);
+    cfg.blockDim = dim3(kMaxTileRows);
+    cfg.dynamicSmemBytes = span_smem(most < kJoinedChunk ? most : kJoinedChunk);      // at most 33 KB
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, joined_span_kernel<BITS, DTYPE, MODE>, a, tab, njoined);
+}
+
+cudaError_t launch_joined_spans(const TableArgs& a, const SpanTable& tab, uint64_t most, int mode, int bits, int dtype,
+                                cudaStream_t stream)
+{
+    if (most > kMaxJoinedElems) return cudaErrorInvalidValue;
+    unsigned cluster = 1;
+    while (cluster * kJoinedChunk < most) cluster *= 2;
+    SpanTable sorted = tab;
+    uint32_t njoined = 0;
+    int at = 0;
+    for (int pass = 0; pass < 2; ++pass)
+        for (int j = 0; j < tab.nspan; ++j) {
+            if ((tab.len[j] > kJoinedChunk) != (pass == 0)) continue;
+            sorted.elem0[at] = tab.elem0[j]; sorted.len[at] = tab.len[j];
+            sorted.code0[at] = tab.code0[j]; sorted.scale_idx[at] = tab.scale_idx[j];
+            ++at;
+            if (pass == 0) ++njoined;
+        }
+    switch (bits) {
+#define MQG_JOINED(B, D) \
+        (mode == kSpanNorm ? launch_joined_inst<B, D, kSpanNorm>(a, sorted, njoined, cluster, most, stream) \
+                           : launch_joined_inst<B, D, kSpanMaxAbs>(a, sorted, njoined, cluster, most, stream))
+#define MQG_JOINED_CASE(B) case B: return dtype == 0 ? MQG_JOINED(B, 0) : MQG_JOINED(B, 1)
+        MQG_JOINED_CASE(1); MQG_JOINED_CASE(2); MQG_JOINED_CASE(3); MQG_JOINED_CASE(4);
+        MQG_JOINED_CASE(5); MQG_JOINED_CASE(6); MQG_JOINED_CASE(7); MQG_JOINED_CASE(8);
+#undef MQG_JOINED_CASE
+#undef MQG_JOINED
     }
     return cudaErrorInvalidValue;
 }

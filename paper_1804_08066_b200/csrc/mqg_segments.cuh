@@ -40,6 +40,14 @@ struct SpanTable {
 cudaError_t launch_spans(const TableArgs& a, const SpanTable& tab, unsigned nspan, uint64_t most, int mode, int bits,
                          int dtype, cudaStream_t stream);
 
+// Spans of a list (no clears) of up to kMaxJoinedElems elements, kSpanMaxAbs or kSpanNorm: those of more than
+// kJoinedChunk are a cluster's each.
+constexpr unsigned kMaxCluster = 8;                                  // CTAs, the portable limit
+constexpr uint64_t kJoinedChunk = (uint64_t)kMaxTileRows * 32;       // elements per CTA, a power of two of rows
+constexpr uint64_t kMaxJoinedElems = kMaxCluster * kJoinedChunk;
+cudaError_t launch_joined_spans(const TableArgs& a, const SpanTable& tab, uint64_t most, int mode, int bits, int dtype,
+                                cudaStream_t stream);
+
 // The same in the main codec together with the max pass over `longs`, whose scales launch_clear_scales has cleared.
 cudaError_t launch_clear_scales(const TableArgs& a, int nseg, cudaStream_t stream);
 cudaError_t launch_spans_absmax(const TableArgs& a, const SpanTable& spans, uint64_t most, const SegmentTable& longs,
