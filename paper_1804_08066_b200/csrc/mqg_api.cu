@@ -216,7 +216,7 @@ mqg_status mqg_quantize(const void* grad, uint64_t n, int bits, uint64_t bucket,
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const uint64_t eff = bucket < n ? bucket : n;
     cudaError_t err;
-    if (eff <= (uint64_t)mqg::kMaxFusedBucket)
+    if (eff <= (uint64_t)mqg::kMaxFusedBucket || mqg::quantize_long_fused_applies(n, bucket, elem_offset))
         err = mqg::launch_quantize_fused(grad, n, bits, bucket, seed, codes, scales, (int)dtype,
                                          worker, step, elem_offset, stream);
     else if (mqg::bucket_spans_apply(n, bucket))

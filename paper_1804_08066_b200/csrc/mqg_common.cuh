@@ -11,7 +11,8 @@ namespace mqg {
 // straddles a thread boundary.
 constexpr int kRowElems = 32;
 constexpr int kMaxTileRows = 256;                 // rows per CTA tile = threads per CTA
-constexpr int kMaxFusedBucket = kRowElems * kMaxTileRows;   // largest bucket of the one-pass kernel
+constexpr int kMaxFusedBucket = kRowElems * kMaxTileRows;   // largest bucket of the one-pass kernels
+constexpr int kMaxTmaBucket = 2 * kMaxFusedBucket;          // and of the TMA-fed ones, main codec and range
 
 // Scales below this are flushed to zero (2^-96).
 __device__ __forceinline__ float flush_limit() { return __uint_as_float(0x0F800000u); }

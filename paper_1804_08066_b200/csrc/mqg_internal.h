@@ -53,6 +53,8 @@ cudaError_t launch_quantize_workers(const void* const* grads, int W, uint64_t n,
 // take and up to 49152 elements (launch_bucket_spans), the general launches for longer ones (ranges by atomics on ordered
 // bits, then encode).
 bool quantize_range_fused_applies(uint64_t n, uint64_t bucket);
+// Buckets of up to kMaxTmaBucket elements in the main codec's one-pass kernel (launch_quantize_fused).
+bool quantize_long_fused_applies(uint64_t n, uint64_t bucket, uint64_t elem_offset);
 cudaError_t launch_quantize_range_fused(const void* grad, uint64_t n, int bits, uint64_t bucket,
                                         uint32_t* codes, float* ranges, int dtype, cudaStream_t stream);
 cudaError_t launch_quantize_range_general(const void* grad, uint64_t n, int bits, uint64_t bucket,

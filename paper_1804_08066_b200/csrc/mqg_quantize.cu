@@ -104,13 +104,14 @@ quantize_pack_kernel(const __grid_constant__ QuantizeArgs a)
 
 
 template <int BITS, int DTYPE, int THREADS, int RED, int MODE>
-__global__ void __launch_bounds__(THREADS, DTYPE == kBf16Wide ? 5 : 512 / THREADS)
+__global__ void __launch_bounds__(THREADS, quantize_min_ctas<DTYPE, THREADS>())
 quantize_tma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ QuantizeArgs a,
                     const __grid_constant__ TmaQuantizeConsts c, unsigned int* __restrict__ timeouts)
 {
     using Shared = TmaQuantizeShared<DTYPE, THREADS>;
     constexpr int kQuantStages = Shared::kStages;
-    __shared__ Shared sh;
+    Shared& sh = tile_shared<Shared>();
+    constexpr bool kHalves = THREADS == 512;       // more rows than the box of a copy
 
     const uint32_t t = threadIdx.x;
     const uint32_t stride = gridDim.x;
@@ -128,8 +129,8 @@ quantize_tma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
         for (uint32_t s = 0; s < (uint32_t)kQuantStages && tile + s * stride < a.ntiles; ++s) {
             mbar_expect_tx(smem_u32(&sh.bar[s]), box_bytes);
             if (!a.arm_only)
-                tma_load_2d(smem_u32(sh.stage[s]), &tmap, 0, (int)((tile + s * stride) * a.tile_rows),
-                            smem_u32(&sh.bar[s]));
+                load_tile_rows(smem_u32(sh.stage[s]), &tmap, (tile + s * stride) * a.tile_rows, a.tile_rows, Shared::kRowBytes,
+                               kHalves, smem_u32(&sh.bar[s]));
         }
     }
     const uint32_t local_bucket = t / a.rows_per_bucket;
@@ -145,7 +146,8 @@ quantize_tma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
             const uint32_t next_tile = tile + ahead;
             if (next_tile < a.ntiles) {
                 mbar_expect_tx(bar, box_bytes);
-                if (!a.arm_only) tma_load_2d(stage, &tmap, 0, (int)(next_tile * a.tile_rows), bar);
+                if (!a.arm_only)
+                    load_tile_rows(stage, &tmap, next_tile * a.tile_rows, a.tile_rows, Shared::kRowBytes, kHalves, bar);
             }
         };
         ok = tile < c.full_tiles ? mode_tile<BITS, DTYPE, THREADS, true, RED, MODE>(sh, wv, a, c, k, rot, tile, refill,
@@ -185,6 +187,7 @@ static cudaError_t launch_tma_inst(const CUtensorMap& map, const QuantizeArgs& a
                                    cudaStream_t stream)
 {
     auto kernel = quantize_tma_kernel<BITS, DTYPE, THREADS, RED, MODE>;
+    constexpr size_t kSmem = dynamic_bytes<TmaQuantizeShared<DTYPE, THREADS>>();
     static std::atomic<int> grid_cap[64];                  // per device; 0 = not yet queried (zero-initialised)
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
@@ -193,7 +196,9 @@ static cudaError_t launch_tma_inst(const CUtensorMap& map, const QuantizeArgs& a
     int cap = grid_cap[dev].load(std::memory_order_relaxed);
     if (cap == 0) {
         int occ = 0, sms = 0;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, THREADS, 0);
+        if (kSmem != 0) err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        if (err != cudaSuccess) return err;
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, THREADS, kSmem);
         if (err != cudaSuccess) return err;
         err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (err != cudaSuccess) return err;
@@ -202,7 +207,7 @@ static cudaError_t launch_tma_inst(const CUtensorMap& map, const QuantizeArgs& a
     }
     unsigned grid = (unsigned)cap;
     if (grid > a.ntiles) grid = a.ntiles;
-    return launch_pdl(kernel, grid, THREADS, stream, map, a, c, timeouts);
+    return launch_pdl_smem(kernel, grid, THREADS, kSmem, stream, map, a, c, timeouts);
 }
 
 template <int BITS, int DTYPE, int MODE>
@@ -210,8 +215,9 @@ static cudaError_t launch_tma_shape(const CUtensorMap& map, const QuantizeArgs& 
                                     unsigned int* timeouts, cudaStream_t stream)
 {
     const int red = reduction_of(a.rows_per_bucket);
-    if constexpr (DTYPE != kBf16Wide)        // 128 rows of 64 hold every bucket
-        if (threads == 256) return launch_tma_inst<BITS, DTYPE, 256, kByWarps, MODE>(map, a, c, timeouts, stream);
+    if (threads == 256) return launch_tma_inst<BITS, DTYPE, 256, kByWarps, MODE>(map, a, c, timeouts, stream);
+    if constexpr (DTYPE != kBf16Wide && MODE != kNorm)       // 256 rows of 64 hold every bucket; no norm of longer ones
+        if (threads == 512) return launch_tma_inst<BITS, DTYPE, 512, kByWarps, MODE>(map, a, c, timeouts, stream);
     if (red == kByShuffle) return launch_tma_inst<BITS, DTYPE, 128, kByShuffle, MODE>(map, a, c, timeouts, stream);
     if (red == kByRows) return launch_tma_inst<BITS, DTYPE, 128, kByRows, MODE>(map, a, c, timeouts, stream);
     return launch_tma_inst<BITS, DTYPE, 128, kByWarps, MODE>(map, a, c, timeouts, stream);
@@ -228,7 +234,7 @@ static cudaError_t launch_tma(QuantizeArgs& a, uint64_t rpb, int bits, int dtype
     if (timeouts == nullptr) return cudaErrorNotSupported;
     CUtensorMap map;
     const char* why = nullptr;
-    if (!encode_rows_map(&map, a.grad, a.nrows_full, dtype == 0 ? 4 : 2, a.row_elems, a.tile_rows, &why))
+    if (!encode_rows_map(&map, a.grad, a.nrows_full, dtype == 0 ? 4 : 2, a.row_elems, box_rows(a), &why))
         return cudaErrorNotSupported;        // the driver cannot encode a tensor map: no silent detour
     switch (bits) {
 #define MQG_TMA_CASE(B) \
@@ -254,11 +260,11 @@ static bool blocks_share_high_half(uint64_t n, uint64_t elem_offset)
     return (first >> 32) == (last >> 32);
 }
 
-// TMA path: enough rows exist and the draws are block-aligned.  Buckets of more than 128 rows have a CTA of 256
-// threads each and must be whole warps.
+// TMA path: enough rows exist and the draws are block-aligned.  Buckets of more than 128 rows have a CTA of 256 or
+// (above 256 rows, main codec and range) 512 threads each and must be whole warps.
 bool tma_path_applies(uint64_t n, uint64_t rpb, uint64_t elem_offset)
 {
-    if (n < 32 * 64 || (elem_offset & 7u) != 0 || rpb == 0 || rpb > (uint64_t)kMaxTileRows) return false;
+    if (n < 32 * 64 || (elem_offset & 7u) != 0 || rpb == 0 || rpb > (uint64_t)kMaxTmaBucket / 32) return false;
     if (n / 32 > 0x7FFFFFFFull) return false;
     if (!blocks_share_high_half(n, elem_offset)) return false;
     return reduction_of(rpb) != kByRows || rpb <= 128;
@@ -270,7 +276,9 @@ bool tma_path_applies(uint64_t n, uint64_t rpb, uint64_t elem_offset)
 // K = 4, 33.4 -> 32.6 at K = 8.
 bool bf16_wide_applies(uint64_t n, uint64_t total, uint64_t bucket, int dtype)
 {
-    return dtype == 1 && total >= (20ull << 20) && n >= 64 * 64 && (bucket >= n || bucket % 64 == 0);
+    const uint64_t rows = bucket >= n ? (n + 63) / 64 : bucket / 64;          // of a bucket: above 128, whole warps
+    return dtype == 1 && total >= (20ull << 20) && n >= 64 * 64 && (bucket >= n || bucket % 64 == 0) &&
+           (rows <= 128 || rows % 32 == 0);
 }
 
 // Fills the arguments every fused kernel shares.  Returns rows per bucket.
@@ -303,7 +311,7 @@ uint64_t fill_args(QuantizeArgs& a, const void* grad, uint64_t n, int bits, uint
 // or 0 if the tile count does not fit.
 int fill_tma_args(QuantizeArgs& a, TmaQuantizeConsts& c, uint64_t rpb)
 {
-    const int threads = rpb <= 128 ? 128 : 256;
+    const int threads = rpb <= 128 ? 128 : rpb <= 256 ? 256 : 512;
     a.buckets_per_tile = (uint32_t)(threads / rpb);
     a.tile_rows = a.buckets_per_tile * a.rows_per_bucket;
     const uint64_t nt = (a.nrows + a.tile_rows - 1) / a.tile_rows;
@@ -350,6 +358,11 @@ cudaError_t launch_quantize_fused(const void* grad, uint64_t n, int bits, uint64
         case 8: return launch_bits<8>(a, dtype, aligned, (unsigned)ntiles, stream);
     }
     return cudaErrorInvalidValue;
+}
+
+bool quantize_long_fused_applies(uint64_t n, uint64_t bucket, uint64_t elem_offset)
+{
+    return tma_path_applies(n, bucket >= n ? (n + 31) / 32 : bucket / 32, elem_offset);
 }
 
 // ---- (min, max) nearest-rounding variant on the TMA kernel ----

@@ -18,7 +18,7 @@ struct QuantizeArgs {
     uint64_t ncode_words;   // ceil(n * bits / 32)
     uint64_t elem_offset;
     uint32_t rows_per_bucket;   // bucket / 32 (a single ragged bucket counts as "all rows")
-    uint32_t tile_rows;         // rows per tile: a multiple of rows_per_bucket, <= 256
+    uint32_t tile_rows;         // rows per tile: a multiple of rows_per_bucket, <= 512
     uint32_t buckets_per_tile;
     uint64_t nrows_full;    // floor(n / 32): rows the tensor map covers
     uint32_t ntiles;
@@ -141,7 +141,8 @@ struct TmaQuantizeShared {
     static constexpr int kRowBytes = DTYPE == 1 ? 64 : 128;
     // depth of the shared-memory ring: two stages where they fit in 32 KB, else one (the refill
     // of a single stage still hides behind the tile's arithmetic)
-    static constexpr int kStages = 2 * THREADS * kRowBytes <= 32768 ? 2 : 1;
+    // (512 threads: two, and one CTA per SM)
+    static constexpr int kStages = 2 * THREADS * kRowBytes <= 32768 || THREADS == 512 || (DTYPE == kBf16Wide && THREADS == 256) ? 2 : 1;
     alignas(1024) uint8_t stage[kStages][THREADS * kRowBytes];
     uint32_t slots[3][kSlots];             // bucket maxima, rotating so no reset races a use
     uint32_t slots_lo[3][kSlots];          // bucket minima of the (min, max) variant, as ordered bits
@@ -150,11 +151,37 @@ struct TmaQuantizeShared {
     alignas(8) uint64_t bar[kStages];
 };
 
+// Above 48 KB the shared memory is dynamic (with slack to round the base up).
+template <typename Shared>
+__host__ __device__ constexpr size_t dynamic_bytes() { return sizeof(Shared) > 48 * 1024 ? sizeof(Shared) + 1024 : 0; }
+template <typename Shared>
+__device__ __forceinline__ Shared& tile_shared()
+{
+    if constexpr (dynamic_bytes<Shared>() == 0) {
+        __shared__ Shared sh;
+        return sh;
+    } else {
+        extern __shared__ uint8_t tile_smem[];
+        return *reinterpret_cast<Shared*>(tile_smem + ((1024u - (smem_u32(tile_smem) & 1023u)) & 1023u));
+    }
+}
+template <int DTYPE, int THREADS>
+constexpr int quantize_min_ctas() { return DTYPE == kBf16Wide ? (THREADS == 128 ? 5 : 2) : THREADS == 512 ? 1 : 512 / THREADS; }
+
+// The tile's rows from row `row0` on into a stage: a bulk copy, or two where the tile has more than the 256 rows that the
+// box of a copy may have.
+__device__ __forceinline__ void load_tile_rows(uint32_t stage, const CUtensorMap* map, uint32_t row0, uint32_t tile_rows,
+                                               uint32_t row_bytes, bool halves, uint32_t bar)
+{
+    tma_load_2d(stage, map, 0, (int)row0, bar);
+    if (halves) tma_load_2d(stage + (tile_rows >> 1) * row_bytes, map, 0, (int)(row0 + (tile_rows >> 1)), bar);
+}
+
 // Kernel-constant inputs of the TMA kernel beyond QuantizeArgs: the ten Philox round keys are
 // computed on the host so the kernel reads them as constant operands.
 struct TmaQuantizeConsts {
     RoundKeys rk;
-    uint32_t full_tiles;         // leading tiles whose rows are all complete and in range
+    uint32_t full_tiles;         // leading tiles in which every thread has a complete row
     uint32_t blk0_lo, blk0_hi;   // Philox block index of element 0: elem_offset / 8; the launch's blocks
                                  // all have the high half blk0_hi (tma_path_applies)
     PhiloxHead head;             // launch-wide part of the blocks of worker rk.worker
@@ -277,7 +304,7 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
             // tree over the bucket's warp sums, zero leaves up to four or eight (plain stores: nothing to reset;
             // the slot array is written again two barriers from here)
             constexpr uint32_t kWarps = THREADS / 32;
-            static_assert(kWarps == 4 || kWarps == 8, "the tree is written for four or eight warps");
+            static_assert(kWarps == 4 || kWarps == 8, "the tree is written for four or eight warps");     // (no norm of longer buckets)
             const uint32_t wpb = a.rows_per_bucket >> 5, first = local_bucket * wpb;
             float v[kWarps];
 #pragma unroll
@@ -544,6 +571,7 @@ uint64_t fill_args(QuantizeArgs& a, const void* grad, uint64_t n, int bits, uint
 // Whether the launch (all workers' n together: total) takes rows of 64 bf16 elements.
 bool bf16_wide_applies(uint64_t n, uint64_t total, uint64_t bucket, int dtype);
 int fill_tma_args(QuantizeArgs& a, TmaQuantizeConsts& c, uint64_t rpb);
+inline uint32_t box_rows(const QuantizeArgs& a) { return a.tile_rows <= 256 ? a.tile_rows : a.tile_rows / 2; }
 inline int reduction_of(uint64_t rpb)
 {
     return (rpb & (rpb - 1)) == 0 && rpb <= 32 ? kByShuffle : rpb % 32 == 0 ? kByWarps : kByRows;

@@ -24,14 +24,15 @@ struct WorkerTable {
 };
 
 template <int BITS, int DTYPE, int THREADS, int RED, int MODE>
-__global__ void __launch_bounds__(THREADS, DTYPE == kBf16Wide ? 5 : 512 / THREADS)
+__global__ void __launch_bounds__(THREADS, quantize_min_ctas<DTYPE, THREADS>())
 quantize_workers_kernel(const __grid_constant__ WorkerTable tab, const __grid_constant__ QuantizeArgs a,
                         const __grid_constant__ TmaQuantizeConsts c, uint32_t total_tiles,
                         unsigned int* __restrict__ timeouts)
 {
     using Shared = TmaQuantizeShared<DTYPE, THREADS>;
     constexpr int kQuantStages = Shared::kStages;
-    __shared__ Shared sh;
+    Shared& sh = tile_shared<Shared>();
+    constexpr bool kHalves = THREADS == 512;       // more rows than the box of a copy
 
     const uint32_t t = threadIdx.x;
     const uint32_t stride = gridDim.x;
@@ -53,7 +54,8 @@ quantize_workers_kernel(const __grid_constant__ WorkerTable tab, const __grid_co
     };
     auto load_tile = [&](const Pos& p, uint32_t stage, uint32_t bar) {     // thread 0 only
         mbar_expect_tx(bar, box_bytes);
-        if (!a.arm_only) tma_load_2d(stage, &tab.map[p.w], 0, (int)(p.tile * a.tile_rows), bar);
+        if (!a.arm_only)
+            load_tile_rows(stage, &tab.map[p.w], p.tile * a.tile_rows, a.tile_rows, Shared::kRowBytes, kHalves, bar);
     };
     uint32_t v = blockIdx.x;
     Pos cur = {0u, 0u}, fill = {0u, 0u};   // the tile in work and the one kQuantStages turns ahead of it
@@ -109,6 +111,7 @@ static cudaError_t launch_workers_inst(const WorkerTable& tab, const QuantizeArg
                                        unsigned int* timeouts, cudaStream_t stream)
 {
     auto kernel = quantize_workers_kernel<BITS, DTYPE, THREADS, RED, MODE>;
+    constexpr size_t kSmem = dynamic_bytes<TmaQuantizeShared<DTYPE, THREADS>>();
     static std::atomic<int> grid_cap[64];                  // per device; 0 = not yet queried (zero-initialised)
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
@@ -117,7 +120,9 @@ static cudaError_t launch_workers_inst(const WorkerTable& tab, const QuantizeArg
     int cap = grid_cap[dev].load(std::memory_order_relaxed);
     if (cap == 0) {
         int occ = 0, sms = 0;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, THREADS, 0);
+        if (kSmem != 0) err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+        if (err != cudaSuccess) return err;
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, THREADS, kSmem);
         if (err != cudaSuccess) return err;
         err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (err != cudaSuccess) return err;
@@ -126,7 +131,7 @@ static cudaError_t launch_workers_inst(const WorkerTable& tab, const QuantizeArg
     }
     unsigned grid = (unsigned)cap;
     if (grid > total_tiles) grid = total_tiles;
-    return launch_pdl(kernel, grid, THREADS, stream, tab, a, c, total_tiles, timeouts);
+    return launch_pdl_smem(kernel, grid, THREADS, kSmem, stream, tab, a, c, total_tiles, timeouts);
 }
 
 template <int BITS, int DTYPE, int MODE>
@@ -134,9 +139,11 @@ static cudaError_t launch_workers_shape(const WorkerTable& tab, const QuantizeAr
                                         uint32_t total_tiles, int threads, unsigned int* timeouts, cudaStream_t stream)
 {
     const int red = reduction_of(a.rows_per_bucket);
-    if constexpr (DTYPE != kBf16Wide)        // 128 rows of 64 hold every bucket
-        if (threads == 256)
-            return launch_workers_inst<BITS, DTYPE, 256, kByWarps, MODE>(tab, a, c, total_tiles, timeouts, stream);
+    if (threads == 256)
+        return launch_workers_inst<BITS, DTYPE, 256, kByWarps, MODE>(tab, a, c, total_tiles, timeouts, stream);
+    if constexpr (DTYPE != kBf16Wide && MODE != kNorm)       // 256 rows of 64 hold every bucket; no norm of longer ones
+        if (threads == 512)
+            return launch_workers_inst<BITS, DTYPE, 512, kByWarps, MODE>(tab, a, c, total_tiles, timeouts, stream);
     if (red == kByShuffle) return launch_workers_inst<BITS, DTYPE, 128, kByShuffle, MODE>(tab, a, c, total_tiles, timeouts, stream);
     if (red == kByRows) return launch_workers_inst<BITS, DTYPE, 128, kByRows, MODE>(tab, a, c, total_tiles, timeouts, stream);
     return launch_workers_inst<BITS, DTYPE, 128, kByWarps, MODE>(tab, a, c, total_tiles, timeouts, stream);
@@ -162,7 +169,7 @@ bool quantize_workers_applies(int W, uint64_t n, uint64_t bucket, uint64_t elem_
     if (W < 2 || W > kMaxWorkers || n == 0) return false;
     const uint64_t nrows = (n + 31) / 32;
     const uint64_t rpb = (bucket >= n) ? nrows : bucket / 32;
-    if ((bucket < n ? bucket : n) > (uint64_t)kMaxFusedBucket) return false;
+    if ((bucket < n ? bucket : n) > (uint64_t)kMaxTmaBucket) return false;
     if (!tma_path_applies(n, rpb, elem_offset)) return false;
     const uint64_t tile_rows = rpb <= 128 ? (128 / rpb) * rpb : rpb;
     const uint64_t nt = (nrows + tile_rows - 1) / tile_rows;
@@ -187,7 +194,7 @@ cudaError_t launch_quantize_workers(const void* const* grads, int W, uint64_t n,
     memset(&tab, 0, sizeof(tab));
     for (int w = 0; w < W; ++w) {
         const char* why = nullptr;
-        if (!encode_rows_map(&tab.map[w], grads[w], a.nrows_full, dtype == 0 ? 4 : 2, a.row_elems, a.tile_rows, &why))
+        if (!encode_rows_map(&tab.map[w], grads[w], a.nrows_full, dtype == 0 ? 4 : 2, a.row_elems, box_rows(a), &why))
             return cudaErrorNotSupported;
         tab.grad[w] = grads[w]; tab.codes[w] = codes[w]; tab.scales[w] = scales[w];
         tab.head[w] = philox_head(c.blk0_hi, first_worker + (uint32_t)w, c.rk.k0[0]);
