@@ -150,7 +150,7 @@ cudaError_t launch_requantize(const WorkerPtrs& ptrs, int W, int bits, uint64_t 
                               uint32_t worker, uint32_t step, cudaStream_t stream);
 
 // The same on the warp-pipelined kernel of mqg_server_tma.cu (whole rows, buckets of 2^k rows up to 128).
-bool requantize_warp_applies(uint64_t n, uint64_t bucket, int W);
+bool requantize_warp_applies(uint64_t n, uint64_t bucket, int W, int bits);
 cudaError_t launch_requantize_warp(const WorkerPtrs& ptrs, int W, int bits, uint64_t n, uint64_t bucket,
                                    float mean_scale, uint64_t seed, uint32_t* codes_out, float* scales_out,
                                    uint32_t worker, uint32_t step, cudaStream_t stream);

@@ -212,7 +212,7 @@ cudaError_t launch_requantize(const WorkerPtrs& ptrs, int W, int bits, uint64_t 
                               float mean_scale, uint64_t seed, uint32_t* codes_out, float* scales_out,
                               uint32_t worker, uint32_t step, cudaStream_t stream)
 {
-    if (requantize_warp_applies(n, bucket, W))
+    if (requantize_warp_applies(n, bucket, W, bits))
         return launch_requantize_warp(ptrs, W, bits, n, bucket, mean_scale, seed, codes_out, scales_out, worker, step,
                                       stream);
     RequantArgs a;

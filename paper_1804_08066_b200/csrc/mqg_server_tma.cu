@@ -178,7 +178,7 @@ __device__ __forceinline__ bool store_tile_scales(const ServerTmaArgs& a, float4
         d[h] = RANGE ? range_decode_scale<BITS>(s[h].x, s[h].y) : decode_scale<BITS>(s[h].x);
         fits = fits && unit_decode_applies(d[h], RANGE);
     }
-    if (UNIT) fits = __all_sync(0xFFFFFFFFu, fits);
+    fits = __all_sync(0xFFFFFFFFu, fits);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         if (h == 1 && !wide) break;
@@ -236,14 +236,16 @@ __device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.w
 // (and so does the bit stream of a segment that takes part in a SEGS launch): the warp copies them in 16-byte pieces, lane l the l-th piece (and the (l + 32)-th for more than
 // four bits), asynchronously and without passing through registers.  The piece that holds the end
 // of a short last tile is copied up to that end and zero-filled.  `lane_off` = 16 * lane.
-template <int BITS>
+// TO_END: the gradient's last, ragged row takes part too; its words end where the stream does.
+template <int BITS, bool TO_END = false>
 __device__ __forceinline__ void fill_code_stage(const ServerTmaArgs& a, uint32_t stage, const TileLoc& loc, int g0,
                                                 uint32_t lane_off)
 {
     constexpr int kGroup = ServerGroup<BITS>::value;
     constexpr uint32_t kWorkerBytes = kSrvTileRows * BITS * 4;
     constexpr int kPieces = (int)((kWorkerBytes / 16 + 31) / 32);       // pieces per lane: 1 or 2
-    const uint32_t rows_here = min((uint32_t)kSrvTileRows, loc.nrows_full - loc.row0);
+    const uint32_t rows_here = TO_END && loc.row0 >= loc.nrows_full ? 0u
+                                                                    : min((uint32_t)kSrvTileRows, loc.nrows_full - loc.row0);
     const uint64_t byte0 = (loc.code_word0 + (uint64_t)loc.row0 * BITS) * 4 + lane_off;
     if (rows_here == (uint32_t)kSrvTileRows && g0 + kGroup <= a.W) {
 #pragma unroll
@@ -256,7 +258,9 @@ __device__ __forceinline__ void fill_code_stage(const ServerTmaArgs& a, uint32_t
             }
         }
     } else {
-        const uint32_t bytes_here = rows_here * BITS * 4;
+        uint32_t bytes_here = rows_here * BITS * 4;
+        if (TO_END && rows_here < (uint32_t)kSrvTileRows)
+            bytes_here = (uint32_t)(a.ncode_words - (uint64_t)loc.row0 * BITS) * 4;
         const int nwk = min(kGroup, a.W - g0);
 #pragma unroll
         for (int pc = 0; pc < kPieces; ++pc) {
@@ -864,34 +868,37 @@ cudaError_t launch_server_range_tma(const WorkerPtrs& ptrs, int W, int bits, uin
 // (ReceiveQGThenSendQG of Algorithm 1, lines 1-5; steps 6-8 of Fig. 3.)  The decode half is the server
 // kernel's: every warp stages the code words of its 32-row tiles by asynchronous copies, two stages
 // ahead, and sums the W workers in registers.  The encode half is the quantize kernels' row code.  In
-// between stands the bucket maximum: a CTA takes 128 consecutive rows at a time, one 32-row tile per
-// warp, so a bucket of 32 rows or fewer is reduced by lane shuffles and a bucket of 64 or 128 rows by
-// the two or four warps that hold it, through shared memory and a named barrier of just those warps.
-// Persistent CTAs, no CTA-wide barrier, no global load through registers.
+// between stands the bucket maximum: a CTA of WARPS warps takes 32 WARPS consecutive rows at a time, whole buckets, one
+// 32-row tile per warp.  A bucket of 2^k rows is reduced by lane shuffles (at most 32 rows) or by the two, four or eight
+// warps that hold it, through shared memory and a named barrier of just those warps; buckets of 24, 48 or 96 rows (three
+// warps) by an atomic per row and the CTA's barrier.
+// Persistent CTAs, no global load through registers.
 struct RequantWarpArgs {
     ServerTmaArgs s;             // decode side: ptrs, nrows_full (= all rows), buckets, W, bias
     uint32_t* codes_out;
     float* scales_out;
     float mean_scale;
-    uint32_t nct;                // CTA tiles of 128 rows
-    uint32_t warps_per_bucket;   // 1 (buckets of at most 32 rows), 2 or 4
+    uint32_t complete_rows;      // floor(n / 32)
+    uint32_t nct;                // CTA tiles of 32 WARPS rows
+    uint32_t warps_per_bucket;   // 1 (buckets of at most 32 rows), 2, 4 or 8
     RoundKeys rk;                // Philox round keys of the re-quantization's draws
     PhiloxHead head;             // and the launch-wide part of its blocks
 };
 
-template <int BITS>
+template <int BITS, int WARPS>
 struct RequantSmem {
-    alignas(16) uint32_t code[kSrvWarps][kCodeDepth][ServerGroup<BITS>::value][kSrvTileRows * BITS];
-    float4 table[kSrvWarps][2 * kMaxWorkers];
-    uint32_t bmax[2][kSrvWarps];                  // tile maxima, double-buffered by the parity of the turn
+    alignas(16) uint32_t code[WARPS][kCodeDepth][ServerGroup<BITS>::value][kSrvTileRows * BITS];
+    float4 table[WARPS][2 * kMaxWorkers];
+    uint32_t bmax[2][WARPS];                      // tile maxima, double-buffered by the parity of the turn
+    uint32_t slot[3][4];                          // three warps: bucket maxima, rotating so that no reset races a use
 };
 
-template <int BITS, bool kUnit>
-__global__ void __launch_bounds__(kSrvThreads, 4)
+template <int BITS, int WARPS, bool kUnit>
+__global__ void __launch_bounds__(32 * WARPS, WARPS == 8 ? 2 : WARPS == 4 ? 4 : 5)
 requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
 {
     extern __shared__ uint8_t smem_raw[];
-    RequantSmem<BITS>& sm = *reinterpret_cast<RequantSmem<BITS>*>(
+    RequantSmem<BITS, WARPS>& sm = *reinterpret_cast<RequantSmem<BITS, WARPS>*>(
         smem_raw + ((16u - (smem_u32(smem_raw) & 15u)) & 15u));
     const ServerTmaArgs& a = ra.s;
     constexpr int kGroup = ServerGroup<BITS>::value;
@@ -901,9 +908,13 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
     const uint32_t wid = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0);
     float4* table = sm.table[wid];
     const uint32_t code_base = smem_u32(&sm.code[wid][0][0][0]);
+    if constexpr (WARPS == 3) {
+        if (threadIdx.x < 12) (&sm.slot[0][0])[threadIdx.x] = 0u;
+        __syncthreads();
+    }
     grid_dependency_wait();            // nothing above touches global memory
 
-    // this CTA's tiles of 128 rows: blockIdx.x, blockIdx.x + gridDim.x, ... (the grid works on one window of
+    // this CTA's tiles of 32 WARPS rows: blockIdx.x, blockIdx.x + gridDim.x, ... (the grid works on one window of
     // consecutive tiles at a time, as in the server kernel); warp w takes rows 32 w .. 32 w + 31 of each
     const uint32_t base = ra.nct / gridDim.x, extra = ra.nct % gridDim.x;
     const uint32_t nct = base + (blockIdx.x < extra ? 1u : 0u);
@@ -916,43 +927,43 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
     auto tile_loc = [&](uint32_t kk) {
         TileLoc t;
         t.map = nullptr;
-        t.row0 = ((blockIdx.x + kk * gridDim.x) * kSrvWarps + wid) * kSrvTileRows;
-        t.nrows_full = a.nrows_full;
+        t.row0 = ((blockIdx.x + kk * gridDim.x) * WARPS + wid) * kSrvTileRows;
+        t.nrows_full = ra.complete_rows;
         t.scale_idx = 0;
         t.code_word0 = 0;
         return t;
     };
     auto fill = [&](uint32_t stage, uint32_t kk, int g0) {           // a tile beyond the last row has no codes
         const TileLoc t = tile_loc(kk);
-        if (t.row0 < a.nrows_full) fill_code_stage<BITS>(a, stage, t, g0, lane_off);
+        if (t.row0 < a.nrows_full) fill_code_stage<BITS, true>(a, stage, t, g0, lane_off);
     };
 
     const UnitBits<BITS, false> unit_bits(a.one);
     bool unit = false;                             // as in the server kernel
-    uint32_t u = 0;
+    uint32_t u = 0, rot = 0;
     if (nct > 0) {
         float2 s0[2];
         load_tile_scales<false, false>(a, tile_loc(0), lane, wide, s0);
-        unit = store_tile_scales<BITS, false, kUnit>(a, table, lane, wide, s0);
 #pragma unroll
         for (uint32_t u2 = 0; u2 < (uint32_t)kCodeDepth; ++u2) {
             if (u2 < nunits) fill(code_base + u2 * kCodeStageBytes, u2 / groups, (int)(u2 % groups) * kGroup);
             cp_async_commit();
         }
+        unit = store_tile_scales<BITS, false, kUnit>(a, table, lane, wide, s0);
         __syncwarp();
     }
     uint32_t fill_tile = kCodeDepth / groups, fill_group = kCodeDepth % groups;
 
 #pragma unroll 1
-    for (uint32_t k = 0; k < nct; ++k) {
+    for (uint32_t k = 0; k < nct; ++k, rot = rot == 2 ? 0 : rot + 1) {
         const TileLoc loc = tile_loc(k);
         const uint32_t row0 = loc.row0;
         const bool have_next = k + 1 < nct;
         float2 s_next[2];
         if (have_next) load_tile_scales<false, false>(a, tile_loc(k + 1), lane, wide, s_next);
         const uint32_t row_c = min(row0 + lane, last_row);
-        const uint32_t lb = bucket_of_row(a, row_c) - bucket_of_row(a, min(row0, last_row));
-        const float4* my_table = table + lb;
+        const uint32_t bucket = bucket_of_row(a, row_c);
+        const float4* my_table = table + (bucket - bucket_of_row(a, min(row0, last_row)));
         float2 v2[16];
 #pragma unroll
         for (int p = 0; p < 16; ++p) v2[p] = make_float2(0.0f, 0.0f);
@@ -976,16 +987,17 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
                     add_decoded_row<BITS, false>(w, d, v2, a.bias_bits);
                 }
             };
-            const int here = min(kGroup, a.W - g0);
-            if (kUnit && !unit) {
-#pragma unroll 1
-                for (int i = 0; i < here; ++i) decode_worker(i, std::false_type());
-            } else if (here == kGroup) {
+            const std::integral_constant<bool, kUnit> units;
+            const bool in_units = !kUnit || __builtin_expect(unit, 1);
+            if (in_units && g0 + kGroup <= a.W) {
 #pragma unroll
-                for (int i = 0; i < kGroup; ++i) decode_worker(i, std::integral_constant<bool, kUnit>());
+                for (int i = 0; i < kGroup; ++i) decode_worker(i, units);
+            } else if (in_units) {
+#pragma unroll 1
+                for (int i = 0; g0 + i < a.W; ++i) decode_worker(i, units);
             } else {
 #pragma unroll 1
-                for (int i = 0; i < here; ++i) decode_worker(i, std::integral_constant<bool, kUnit>());
+                for (int i = 0; i < kGroup && g0 + i < a.W; ++i) decode_worker(i, std::false_type());
             }
             __syncwarp();                          // every lane has read the stage: refill it
             if (u + kCodeDepth < nunits) fill(code_base + cs * kCodeStageBytes, fill_tile, (int)fill_group * kGroup);
@@ -996,6 +1008,7 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
         // the mean, and the bucket maximum of its magnitudes
         const uint32_t row = row0 + lane;
         const bool active = row < a.nrows_full;
+        const int left = !active ? 0 : row < ra.complete_rows ? 32 : (int)(a.n - (uint64_t)row * 32);   // elements of the row
         float x[32];
         {
             const float factor = kUnit && unit ? a.unit_factor : ra.mean_scale;
@@ -1006,30 +1019,46 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
                 x[2 * p] = y.x;
                 x[2 * p + 1] = y.y;
             }
-            if (row0 + kSrvTileRows > a.nrows_full && !active) {     // only in the gradient's last tiles:
+            if (row0 + kSrvTileRows > ra.complete_rows) {            // only in the gradient's last tiles:
 #pragma unroll
-                for (int j = 0; j < 32; ++j) x[j] = 0.0f;            // lanes past the end decode what their slot holds
+                for (int j = 0; j < 32; ++j) x[j] = j < left ? x[j] : 0.0f;   // what is past the end is what its slot holds
             }
         }
         uint32_t m = __float_as_uint(row_abs_max(x));
-        if (G == 1) {
+        bool writer;
+        if constexpr (WARPS == 3) {
+            const uint32_t lb = bucket - ((blockIdx.x + k * gridDim.x) * (32u * WARPS)) / a.rows_per_bucket;
+            uint32_t* slot = sm.slot[rot];
+            if (a.rows_per_bucket == 32u * WARPS) {
+                m = __reduce_max_sync(0xFFFFFFFFu, m);
+                if (lane == 0) atomicMax(&slot[0], m);
+            } else if (active) {
+                atomicMax(&slot[lb], m);
+            }
+            named_barrier<1>(32 * WARPS);
+            m = active ? slot[lb] : 0u;
+            if (threadIdx.x < 4) sm.slot[rot == 0 ? 2 : rot - 1][threadIdx.x] = 0u;      // next used in two turns
+            writer = row % a.rows_per_bucket == 0;
+        } else if (G == 1) {
             const uint32_t rpb = min(a.rows_per_bucket, (uint32_t)kSrvTileRows);
             for (uint32_t d = rpb >> 1; d > 0; d >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
+            writer = (row & (a.rows_per_bucket - 1)) == 0;
         } else {
             m = __reduce_max_sync(0xFFFFFFFFu, m);
             uint32_t* slot = sm.bmax[k & 1];
             if (lane == 0) slot[wid] = m;
             const uint32_t first = wid & ~(G - 1);
-            if (G == 4 || first == 0) named_barrier<1>(32 * G);   // the warps that hold this bucket
+            if (WARPS == 8 || G == 4 || first == 0) named_barrier<1>(32 * G);   // the warps that hold this bucket
             else named_barrier<2>(32 * G);
             m = max(slot[first], slot[first + 1]);
-            if (G == 4) m = max(m, max(slot[first + 2], slot[first + 3]));
+            if (WARPS == 8 || G == 4) m = max(m, max(slot[first + 2], slot[first + 3]));
+            if constexpr (WARPS == 8) m = max(m, max(max(slot[4], slot[5]), max(slot[6], slot[7])));
+            writer = (wid & (G - 1)) == 0 && lane == 0;
         }
         float sc = __uint_as_float(m);
         if (sc < flush_limit()) sc = 0.0f;
         if (active) {
-            const bool writer = G == 1 ? (row & (a.rows_per_bucket - 1)) == 0 : ((wid & (G - 1)) == 0 && lane == 0);
-            if (writer) ra.scales_out[row >> a.rpb_shift] = sc;
+            if (writer) ra.scales_out[bucket] = sc;
             const EncodeScale es = encode_scale<BITS>(sc);
             // (spreading the four Philox blocks over the decode of the workers, to fill its gaps, measured
             // 3 to 5 us slower per launch: the kernel then needs all 128 registers)
@@ -1040,7 +1069,15 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
             // a fifth resident CTA, which 95 registers would allow, changes nothing: the kernel waits on
             // its arithmetic pipes, not on latency)
             encode_pack_row_best<BITS>(x, es, h, w);
-            store_row_words<BITS>(ra.codes_out, (uint64_t)row * BITS, w);
+            const uint64_t word0 = (uint64_t)row * BITS;
+            if (left == 32) {
+                store_row_words<BITS>(ra.codes_out, word0, w);
+            } else {
+                mask_row_words<BITS>(w, left * BITS);
+#pragma unroll
+                for (int j = 0; j < BITS; ++j)
+                    if (word0 + j < a.ncode_words) ra.codes_out[word0 + j] = w[j];
+            }
         }
         if (have_next) unit = store_tile_scales<BITS, false, kUnit>(a, table, lane, wide, s_next);
         __syncwarp();
@@ -1048,11 +1085,11 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
     cp_async_wait_group<0>();                                  // no code copy outlives the warp
 }
 
-template <int BITS, bool UNIT>
-static cudaError_t launch_requantize_warp_inst(const RequantWarpArgs& ra, cudaStream_t stream)
+template <int BITS, int WARPS, bool UNIT>
+static cudaError_t launch_requantize_warp_inst(RequantWarpArgs& ra, cudaStream_t stream)
 {
-    auto kernel = requantize_warp_kernel<BITS, UNIT>;
-    constexpr size_t kSmemBytes = sizeof(RequantSmem<BITS>) + 16;
+    auto kernel = requantize_warp_kernel<BITS, WARPS, UNIT>;
+    constexpr size_t kSmemBytes = sizeof(RequantSmem<BITS, WARPS>) + 16;
     static std::atomic<int> grid_cap[64];                 // per device; 0 = not yet set up (zero-initialised)
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
@@ -1063,28 +1100,59 @@ static cudaError_t launch_requantize_warp_inst(const RequantWarpArgs& ra, cudaSt
         int occ = 0, sms = 0;
         err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
         if (err != cudaSuccess) return err;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kSrvThreads, kSmemBytes);
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 32 * WARPS, kSmemBytes);
         if (err != cudaSuccess) return err;
         err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (err != cudaSuccess) return err;
         cap = sms * (occ > 0 ? occ : 1);
         grid_cap[dev].store(cap, std::memory_order_relaxed);   // every thread computes the same value
     }
+    ra.nct = (ra.s.nrows_full + 32 * WARPS - 1) / (32 * WARPS);
     unsigned grid = (unsigned)cap;
     if (grid > ra.nct) grid = ra.nct;
-    return launch_pdl_smem(kernel, grid, kSrvThreads, kSmemBytes, stream, ra);
+    return launch_pdl_smem(kernel, grid, 32 * WARPS, kSmemBytes, stream, ra);
 }
 
-// Whole rows, at least 512 of them, fewer than 2^30 (so the draws' block numbers have no high half),
-// and buckets of 2^k rows, k <= 7 (at most 4096 elements), those below 32 rows few enough per tile for
-// the warp's table.
-bool requantize_warp_applies(uint64_t n, uint64_t bucket, int W)
+template <int BITS>
+static cudaError_t launch_requantize_warp_bits(RequantWarpArgs& ra, int warps, cudaStream_t stream)
 {
-    if (n % 32 != 0 || n / 32 < 512 || n / 32 >= (1ull << 30) || bucket >= n || bucket % 32 != 0) return false;
+    if constexpr (UnitDecode<BITS, false>::kExists) {
+        if (sum_in_units<BITS>(ra.s, ra.mean_scale))
+            return warps == 3 ? launch_requantize_warp_inst<BITS, 3, true>(ra, stream)
+                 : warps == 8 ? launch_requantize_warp_inst<BITS, 8, true>(ra, stream)
+                              : launch_requantize_warp_inst<BITS, 4, true>(ra, stream);
+    }
+    return warps == 3 ? launch_requantize_warp_inst<BITS, 3, false>(ra, stream)
+         : warps == 8 ? launch_requantize_warp_inst<BITS, 8, false>(ra, stream)
+                      : launch_requantize_warp_inst<BITS, 4, false>(ra, stream);
+}
+
+// Warps of a CTA for buckets of `rpb` rows, 0 where the kernel does not take them: whole buckets fill the CTA's rows, and a
+// warp's 32 rows touch at most two buckets (or a power of two of them).
+static int requantize_warps(uint64_t rpb)
+{
+    if (rpb == 24 || rpb == 48 || rpb == 96) return 3;
+    if ((rpb & (rpb - 1)) != 0 || rpb > 256) return 0;
+    return rpb == 256 ? 8 : 4;
+}
+
+// At least 512 complete rows, fewer than 2^30 (so the draws' block numbers have no high half), buckets as above, those
+// below 32 rows few enough per tile for the warp's table; and where it is the faster one.  Against a CTA per tile
+// (mqg_requantize.cu) a warp's copies and constants are ahead of their use, which short launches gain from - at two bits 2.7 /
+// 4.3 against 2.9 / 7.5 us for 130,001 elements and 1 / 16 workers, 5.5 against 7.1 us for a million and 16 - and long ones
+// when there is much to sum: 25 M elements, bucket 2048, four bits, 8 / 16 workers 44 / 68 against 52 / 86 us, eight bits, 4
+// workers 35 against 39 us, two bits, 16 workers 69 against 72 us.  Otherwise the other's smaller CTAs with fewer
+// registers win: one bit, 4 / 16 workers 28 / 54 against 32 / 62 us, two bits, 4 / 8 workers 32 / 43.4 against 35 / 44.1 us,
+// eight bits, 2 workers 28 against 30 us; no difference at four bits.  Three warps: bucket 768, four bits, 4 / 8 workers 40 / 50
+// against 36 / 55 us, eight bits, 4 / 8 42 / 56 against 40 / 63 us.
+bool requantize_warp_applies(uint64_t n, uint64_t bucket, int W, int bits)
+{
+    if (n / 32 < 512 || n / 32 >= (1ull << 30) - 1 || bucket >= n || bucket % 32 != 0) return false;
     const uint64_t rpb = bucket / 32;
-    if ((rpb & (rpb - 1)) != 0 || rpb > 128) return false;
-    if (rpb >= 32) return true;
-    return ((uint64_t)W * (32 / rpb)) <= 2 * (uint64_t)kMaxWorkers;
+    const int warps = requantize_warps(rpb);
+    if (warps == 0 || (rpb < 24 && (uint64_t)W * (32 / rpb) > 2 * (uint64_t)kMaxWorkers)) return false;
+    if (n < (1u << 20)) return true;
+    return warps == 3 ? W >= 8 && W * bits >= 32 : bits == 4 || (bits >= 2 && W * bits >= 24);
 }
 
 cudaError_t launch_requantize_warp(const WorkerPtrs& ptrs, int W, int bits, uint64_t n, uint64_t bucket,
@@ -1097,19 +1165,22 @@ cudaError_t launch_requantize_warp(const WorkerPtrs& ptrs, int W, int bits, uint
     a.ptrs = ptrs;
     a.n = n;
     a.ncode_words = (n * (uint64_t)bits + 31) / 32;
-    a.nrows = a.nrows_full = (uint32_t)(n / 32);
+    a.nrows = a.nrows_full = (uint32_t)((n + 31) / 32);
+    ra.complete_rows = (uint32_t)(n / 32);
     a.nbuckets = (uint32_t)((n + bucket - 1) / bucket);
     const uint64_t rpb = bucket / 32;
+    const int warps = requantize_warps(rpb);
     a.rows_per_bucket = (uint32_t)rpb;
-    a.rpb_shift = 0;
-    while (((uint64_t)1 << a.rpb_shift) < rpb) ++a.rpb_shift;
-    a.nbt_shift = 0;                                     // buckets a tile of 32 rows touches: 32 / rpb
-    while (rpb < 32 && (rpb << a.nbt_shift) < 32) ++a.nbt_shift;
+    a.rpb_shift = -1;
+    for (int sft = 0; sft < 32; ++sft)
+        if (((uint64_t)1 << sft) == rpb) a.rpb_shift = sft;
+    // log2 of the buckets a tile of 32 rows touches
+    a.nbt_shift = rpb == 24 || rpb == 48 ? 1 : 0;
+    while (rpb < 24 && (rpb << a.nbt_shift) < 32) ++a.nbt_shift;
     a.W = W;
     a.bias_bits = 0x4B000000u;
     ra.codes_out = codes_out; ra.scales_out = scales_out;
     ra.mean_scale = mean_scale;
-    ra.nct = (uint32_t)((n / 32 + kSrvThreads - 1) / kSrvThreads);
     ra.warps_per_bucket = rpb <= 32 ? 1u : (uint32_t)(rpb / 32);
     uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
     for (int r = 0; r < 10; ++r) {
@@ -1120,10 +1191,7 @@ cudaError_t launch_requantize_warp(const WorkerPtrs& ptrs, int W, int bits, uint
     ra.head = philox_head(0u, worker, ra.rk.k0[0]);
     switch (bits) {
 #define MQG_REQUANT_CASE(B) \
-        case B: \
-            if constexpr (UnitDecode<B, false>::kExists) \
-                if (sum_in_units<B>(a, mean_scale)) return launch_requantize_warp_inst<B, true>(ra, stream); \
-            return launch_requantize_warp_inst<B, false>(ra, stream)
+        case B: return launch_requantize_warp_bits<B>(ra, warps, stream)
         MQG_REQUANT_CASE(1); MQG_REQUANT_CASE(2); MQG_REQUANT_CASE(3); MQG_REQUANT_CASE(4);
         MQG_REQUANT_CASE(5); MQG_REQUANT_CASE(6); MQG_REQUANT_CASE(7); MQG_REQUANT_CASE(8);
 #undef MQG_REQUANT_CASE
