@@ -245,7 +245,11 @@ __device__ __forceinline__ void absmax_tile(const TableArgs& a, const SegmentTab
         }
     };
     constexpr int kFull = kMaxTileRows * 32 / kPer / THREADS;          // accesses per thread of a whole tile
-    if (nvec == (uint64_t)kFull * THREADS) {
+    // A tile off the boundary takes its successor's first elements instead of its own, where the segment goes on that far: a
+    // maximum may see them twice.  (23 M elements off the boundary, two workers, with the encode: 66 against 73 us, bf16 51
+    // against 56 us.)
+    if (g.valid >= to_align + kMaxTileRows * 32) {
+        if (g.tile_local == 0 && threadIdx.x < to_align) m = value(threadIdx.x);
         uint4 v[kFull];
 #pragma unroll
         for (int k = 0; k < kFull; ++k) v[k] = __ldcg(v4 + k * THREADS + threadIdx.x);

@@ -6,7 +6,8 @@
 //      them the max pass over the longer segments; a launch for every 64 segments;
 //   3. encode_entries_kernel - the longer ones' encode.  Every (worker, segment) pair is an entry with a tensor map of its
 //      own; the persistent CTAs walk the 128-row tiles of all entries as one sequence, fed by tiled bulk copies; a launch
-//      for every 64 entries.  Segments that start where bulk copies cannot go through encode_table_kernel instead.
+//      for every 64 entries.  Segments that start where bulk copies cannot: encode_flat_kernel, by rows of the whole gradient
+//      (encode_table_kernel where that cannot either).
 // Where these two do not go together (spans_join_max_pass), span_kernel also clears the scales and absmax_table_kernel
 // follows it.
 // Worker w's outputs are the same whichever way a segment goes and however many workers there are.
@@ -127,7 +128,7 @@ encode_entries_kernel(const __grid_constant__ SegEntryTable<CAP> T, unsigned int
         const uint32_t bar = smem_u32(&sh.bar[s]);
         uint32_t h[16];
         draw_row_blocks_head(blk0 + 4u * kHalves * row, head, T.rk, h);
-        const bool active = row < rows, ragged_warp = rows > rows_full && warp_has_row(rows_full, row - lane, 32);
+        const bool active = row < rows, ragged_warp = u + 1 == end && rows > rows_full && warp_has_row(rows_full, row - lane, 32);
         if (ragged_warp) {
             const uint32_t to = smem_u32(sh.ragged[t >> 5]);
             const uint8_t* grad = static_cast<const uint8_t*>(T.e[e].grad);
@@ -139,10 +140,16 @@ encode_entries_kernel(const __grid_constant__ SegEntryTable<CAP> T, unsigned int
         if (!__all_sync(0xFFFFFFFFu, ok)) { ok = false; break; }
 
         uint4 v[8];
-        if (ragged_warp) { cp_async_wait_all(); __syncwarp(); }
-        const RowSource src = ragged_warp && row >= rows_full ? RowSource{sh.ragged[t >> 5], 0} : RowSource{stage, (int)t};
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = reinterpret_cast<const uint4*>(src.stage)[swz(src.row, i)];
+        for (int i = 0; i < 8; ++i) v[i] = reinterpret_cast<const uint4*>(stage)[swz((int)t, i)];
+        if (ragged_warp) {
+            cp_async_wait_all();
+            __syncwarp();
+            if (row >= rows_full) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = reinterpret_cast<const uint4*>(sh.ragged[t >> 5])[i];
+            }
+        }
         __syncwarp();                      // every lane has read the stage
         bool last = false;
         if (lane == 0) {
@@ -195,6 +202,186 @@ encode_entries_kernel(const __grid_constant__ SegEntryTable<CAP> T, unsigned int
     }
 }
 
+// The encode of segments that start off a 16-byte boundary (a layered gradient whose tensors are not padded).  A row here is
+// a row of the worker's whole gradient, 128 aligned bytes that belong to one or two segments, so that bulk copies fetch the
+// tiles and the draws come in whole blocks; what is shifted is the bit stream.  A row's packed words go to shared memory, where
+// a warp's 32 rows are one stretch of the gradient's stream, and the warp writes the segment's words from there, each
+// from two neighbouring ones by a shift that is the segment's.  A word may need the row after the warp's last, so a warp
+// writes 31 rows' words from the 32 it encodes.  Bound by the encode, like the entries'.  23 M elements off the boundary, two
+// workers, four bits, max pass and encode 66 us (61 on it), bf16 51 (49), against 100 and 97 us with encode_table_kernel, which
+// copies four and two bytes at a time and draws a fifth block per row.
+struct FlatEntry {
+    const void* base;        // the gradient's row in which the segment starts
+    uint32_t* codes;         // the segment's first code word
+    float* scale;            // its scale, final when the encode pass starts
+    uint64_t n;              // elements
+    uint64_t bytes;          // from `base` to the gradient's end
+    uint32_t pad;            // elements of that row before the segment
+    uint32_t rows;           // rows the segment touches
+    uint32_t tile0;          // its first tile's number in the launch's sequence
+    uint32_t blk0_lo;        // low half of the Philox block index of the row's first element
+    PhiloxHead head;         // launch-wide part of its blocks (worker, high half of the block index)
+};
+
+template <int CAP>
+struct FlatTable {
+    CUtensorMap map[CAP];
+    FlatEntry e[CAP];
+    uint32_t tile_end[CAP];              // one past each entry's last tile; 2^32 - 1 beyond the last entry
+    uint32_t tiles;
+    uint32_t poll_limit, arm_only;       // as in QuantizeArgs
+    RoundKeys rk;
+};
+constexpr uint32_t kFlatWarps = 4, kFlatWarpRows = 31, kFlatTileRows = kFlatWarps * kFlatWarpRows;
+
+template <int BITS, int DTYPE, int CAP>
+__global__ void __launch_bounds__(32 * kFlatWarps, 4)
+encode_flat_kernel(const __grid_constant__ FlatTable<CAP> T, unsigned int* __restrict__ timeouts)
+{
+    constexpr uint32_t kStages = 2, kBoxRows = 128, kTileBytes = kBoxRows * 128;
+    constexpr int kHalves = DTYPE == 0 ? 1 : 2, kElems = 32 * kHalves, kWords = BITS * kHalves;
+    struct Shared {
+        alignas(1024) uint8_t stage[kStages][kTileBytes];
+        alignas(16) uint32_t out[kFlatWarps][32 * kWords];
+        alignas(16) uint8_t ragged[kFlatWarps][128];
+        alignas(8) uint64_t bar[kStages];
+        uint32_t read[kStages];        // warps that have read the stage, over all its uses
+    };
+    __shared__ Shared sh;
+    const uint32_t t = threadIdx.x, lane = t & 31u, wid = t >> 5;
+    const uint32_t step = gridDim.x;
+    if (t == 0) {
+        for (uint32_t s = 0; s < kStages; ++s) { mbar_init(smem_u32(&sh.bar[s]), 1); sh.read[s] = 0u; }
+        fence_barrier_init();
+    }
+    __syncthreads();
+    grid_dependency_wait();            // nothing above touches global memory
+
+    uint32_t u = blockIdx.x, fill = u;             // the tile in work, the next one to fetch
+    uint32_t fe = 0;                               // the entry of `fill`: searched once, then only moved forward
+#pragma unroll
+    for (uint32_t half = CAP / 2; half > 0; half >>= 1)
+        if (u >= T.tile_end[fe + half - 1]) fe += half;
+    if (u >= T.tiles) fe = 0;
+    uint32_t e = fe;
+    auto fetch = [&](uint32_t s, bool mine) {
+        if (fill < T.tiles) {
+            while (fill >= T.tile_end[fe]) ++fe;
+            if (mine) {
+                const uint32_t bar = smem_u32(&sh.bar[s]);
+                mbar_expect_tx(bar, kTileBytes);
+                if (!T.arm_only)
+                    tma_load_2d(smem_u32(sh.stage[s]), &T.map[fe], 0, (int)((fill - T.e[fe].tile0) * kFlatTileRows), bar);
+            }
+        }
+        fill += step;
+    };
+    for (uint32_t s = 0; s < kStages; ++s) fetch(s, t == 0);
+
+    uint32_t k = 0, end = 0, tile0 = 0, blk0 = 0, rows = 0, rows_full = 0, pad = 0, off = 0, shift = 0;
+    uint64_t words = 0, last = 0;                  // the segment's words; one past its last element, from `base`
+    uint32_t* codes = nullptr;
+    bool ok = true;
+    PhiloxHead head = {};
+    EncodeScale es = {0.0f, 0.0f};
+#pragma unroll 1
+    for (; u < T.tiles; u += step, ++k) {
+        if (u >= end) {
+            while (u >= T.tile_end[e]) ++e;
+            const FlatEntry& x = T.e[e];
+            end = T.tile_end[e]; tile0 = x.tile0; blk0 = x.blk0_lo; head = x.head; codes = x.codes;
+            rows = x.rows; rows_full = (uint32_t)(x.bytes >> 7 < rows ? x.bytes >> 7 : rows); pad = x.pad;
+            off = (pad * BITS) >> 5; shift = (pad * BITS) & 31u;
+            words = (x.n * BITS + 31) / 32; last = pad + x.n;
+            es = encode_scale<BITS>(__ldcg(x.scale));
+        }
+        const uint32_t s = k % kStages, at = wid * kFlatWarpRows + lane;         // the row's place in the stage
+        const uint32_t row0 = (u - tile0) * kFlatTileRows + wid * kFlatWarpRows, row = row0 + lane;
+        uint8_t* stage = sh.stage[s];
+        const uint32_t bar = smem_u32(&sh.bar[s]);
+        uint32_t h[16];
+        draw_row_blocks_head(blk0 + 4u * kHalves * row, head, T.rk, h);
+        const bool ragged_warp = u + 1 == end && rows > rows_full && warp_has_row(rows_full, row0, 32);
+        if (ragged_warp) {
+            const uint32_t to = smem_u32(sh.ragged[wid]);
+            const uint8_t* grad = static_cast<const uint8_t*>(T.e[e].base);
+            if constexpr (DTYPE == 0) fetch_ragged_row(to, grad, rows_full, T.e[e].bytes, 128);
+            else fetch_ragged_wide_row(to, grad, rows_full, T.e[e].bytes);
+        }
+        ok = mbar_try_wait(bar, (k / kStages) & 1);
+        if (!ok) ok = mbar_wait(bar, (k / kStages) & 1, T.poll_limit);
+        if (!__all_sync(0xFFFFFFFFu, ok)) { ok = false; break; }
+
+        uint4 v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = reinterpret_cast<const uint4*>(stage)[swz((int)at, i)];
+        if (ragged_warp) {
+            cp_async_wait_all();
+            __syncwarp();
+            if (row >= rows_full) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = reinterpret_cast<const uint4*>(sh.ragged[wid])[i];
+            }
+        }
+        __syncwarp();                      // every lane has read the stage
+        bool refill = false;
+        if (lane == 0) {
+            __threadfence_block();
+            refill = (atomicAdd(&sh.read[s], 1u) & (kFlatWarps - 1)) == kFlatWarps - 1;
+            if (refill) __threadfence_block();
+        }
+        fetch(s, refill);
+
+        // what lies beside the segment in its first and last row is another's, and no value of this scale
+        const uint32_t* raw = reinterpret_cast<const uint32_t*>(v);
+        const uint64_t first_elem = (uint64_t)row * kElems;
+        const bool edge = row == 0 || row + 1 >= rows;
+        uint32_t w[kWords];
+#pragma unroll
+        for (int half = 0; half < kHalves; ++half) {
+            float x[32];
+            if constexpr (DTYPE == 0) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) x[j] = __uint_as_float(raw[j]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) { x[2 * j] = bf16_lo(raw[16 * half + j]); x[2 * j + 1] = bf16_hi(raw[16 * half + j]); }
+            }
+            if (edge) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const uint64_t i = first_elem + 32 * half + j;
+                    x[j] = i >= pad && i < last ? x[j] : 0.0f;
+                }
+            }
+            if (half != 0) draw_row_blocks_head(blk0 + 4u * (kHalves * row + half), head, T.rk, h);
+            uint32_t wh[BITS];
+            encode_pack_row_best<BITS>(x, es, h, wh);
+#pragma unroll
+            for (int j = 0; j < BITS; ++j) w[half * BITS + j] = wh[j];
+        }
+        if (row + 1 >= rows) {             // nothing beyond the segment's last code
+            const uint64_t left = last > first_elem ? last - first_elem : 0;
+            mask_row_words<kWords>(w, (int)(left < (uint64_t)kElems ? left : (uint64_t)kElems) * BITS);
+        }
+        uint32_t* out = sh.out[wid];
+        store_row_words<kWords>(out, lane * kWords, w);
+        __syncwarp();
+#pragma unroll
+        for (int i0 = 0; i0 < kWords; ++i0) {
+            const uint32_t i = 32u * i0 + lane;
+            const int64_t m = (int64_t)((uint64_t)row0 * kWords + i) - off;
+            if (i < kFlatWarpRows * kWords && m >= 0 && m < (int64_t)words) codes[m] = __funnelshift_r(out[i], out[i + 1], shift);
+        }
+        __syncwarp();                      // every lane has read the words
+    }
+    if (!ok && lane == 0) {                // as in encode_entries_kernel
+        atomicAdd(timeouts, 1u);
+        for (uint32_t j = k; j < k + kStages && u < T.tiles; ++j, u += step)
+            mbar_wait(smem_u32(&sh.bar[j % kStages]), (j / kStages) & 1, T.poll_limit);
+    }
+}
+
 // ---- host side --------------------------------------------------------------------------------
 namespace {
 
@@ -204,12 +391,19 @@ struct EntryHost {
     float* scale;
     uint64_t n, elem_offset;
     uint32_t worker;
+    uint32_t pad;            // flat entries: elements of `grad`'s row before the segment,
+    uint64_t bytes;          // and bytes from `grad` to the gradient's end
 };
 
 template <int BITS, int DTYPE, int CAP>
-cudaError_t launch_entries_inst(const SegEntryTable<CAP>& tab, unsigned int* timeouts, cudaStream_t stream)
+auto entries_kernel(const SegEntryTable<CAP>&) { return encode_entries_kernel<BITS, DTYPE, CAP>; }
+template <int BITS, int DTYPE, int CAP>
+auto entries_kernel(const FlatTable<CAP>&) { return encode_flat_kernel<BITS, DTYPE, CAP>; }
+
+template <int BITS, int DTYPE, int CAP, template <int> class Table>
+cudaError_t launch_entries_inst(const Table<CAP>& tab, unsigned int* timeouts, cudaStream_t stream)
 {
-    auto kernel = encode_entries_kernel<BITS, DTYPE, CAP>;
+    auto kernel = entries_kernel<BITS, DTYPE, CAP>(tab);
     static std::atomic<int> grid_cap[64];          // per device; 0 = not yet queried (zero-initialised)
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
@@ -230,17 +424,34 @@ cudaError_t launch_entries_inst(const SegEntryTable<CAP>& tab, unsigned int* tim
     return launch_pdl(kernel, grid, 128, stream, tab, timeouts);
 }
 
-template <int CAP>
-cudaError_t launch_entries(const EntryHost* entries, int nent, int bits, const RoundKeys& rk, int dtype,
-                           cudaStream_t stream)
+template <int CAP, template <int> class Table>
+cudaError_t launch_table(Table<CAP>& tab, int nent, uint64_t tiles, int bits, const RoundKeys& rk, int dtype,
+                         cudaStream_t stream)
 {
     unsigned int* timeouts = wait_timeout_counter();
     if (timeouts == nullptr) return cudaErrorNotSupported;
-    SegEntryTable<CAP> tab;
     const WaitPolicy policy = wait_policy();
     tab.poll_limit = policy.poll_limit;
     tab.arm_only = policy.arm_only;
     tab.rk = rk;
+    for (int i = nent; i < CAP; ++i) tab.tile_end[i] = 0xFFFFFFFFu;
+    tab.tiles = (uint32_t)tiles;
+    switch (bits) {
+#define MQG_ENT_CASE(B) \
+        case B: return dtype == 0 ? launch_entries_inst<B, 0>(tab, timeouts, stream) \
+                                  : launch_entries_inst<B, kBf16Wide>(tab, timeouts, stream)
+        MQG_ENT_CASE(1); MQG_ENT_CASE(2); MQG_ENT_CASE(3); MQG_ENT_CASE(4);
+        MQG_ENT_CASE(5); MQG_ENT_CASE(6); MQG_ENT_CASE(7); MQG_ENT_CASE(8);
+#undef MQG_ENT_CASE
+    }
+    return cudaErrorInvalidValue;
+}
+
+template <int CAP>
+cudaError_t launch_entries(const EntryHost* entries, int nent, int bits, const RoundKeys& rk, int dtype,
+                           cudaStream_t stream)
+{
+    SegEntryTable<CAP> tab;
     const uint32_t row_elems = dtype == 0 ? 32 : 64;
     uint64_t tiles = 0;
     for (int i = 0; i < nent; ++i) {
@@ -258,17 +469,43 @@ cudaError_t launch_entries(const EntryHost* entries, int nent, int bits, const R
         e.blk0_lo = (uint32_t)blk0;
         e.head = philox_head((uint32_t)(blk0 >> 32), h.worker, rk.k0[0]);
     }
-    for (int i = nent; i < CAP; ++i) tab.tile_end[i] = 0xFFFFFFFFu;
-    tab.tiles = (uint32_t)tiles;
-    switch (bits) {
-#define MQG_ENT_CASE(B) \
-        case B: return dtype == 0 ? launch_entries_inst<B, 0, CAP>(tab, timeouts, stream) \
-                                  : launch_entries_inst<B, kBf16Wide, CAP>(tab, timeouts, stream)
-        MQG_ENT_CASE(1); MQG_ENT_CASE(2); MQG_ENT_CASE(3); MQG_ENT_CASE(4);
-        MQG_ENT_CASE(5); MQG_ENT_CASE(6); MQG_ENT_CASE(7); MQG_ENT_CASE(8);
-#undef MQG_ENT_CASE
+    return launch_table(tab, nent, tiles, bits, rk, dtype, stream);
+}
+
+template <int CAP>
+cudaError_t launch_flat(const EntryHost* entries, int nent, int bits, const RoundKeys& rk, int dtype, cudaStream_t stream)
+{
+    FlatTable<CAP> tab;
+    const uint32_t row_elems = dtype == 0 ? 32 : 64;
+    uint64_t tiles = 0;
+    for (int i = 0; i < nent; ++i) {
+        const EntryHost& h = entries[i];
+        FlatEntry& e = tab.e[i];
+        const uint64_t rows = (h.pad + h.n + row_elems - 1) / row_elems, whole = h.bytes / 128;
+        const char* why = nullptr;
+        if (!encode_rows_map(&tab.map[i], h.grad, rows < whole ? rows : whole, dtype == 0 ? 4 : 2, row_elems, 128, &why))
+            return cudaErrorNotSupported;
+        e.base = h.grad; e.codes = h.codes; e.scale = h.scale; e.n = h.n; e.bytes = h.bytes; e.pad = h.pad;
+        e.rows = (uint32_t)rows;
+        e.tile0 = (uint32_t)tiles;
+        tiles += (rows + kFlatTileRows - 1) / kFlatTileRows;
+        if (tiles > 0x7FFFFFFFull / kFlatTileRows) return cudaErrorInvalidValue;
+        tab.tile_end[i] = (uint32_t)tiles;
+        const uint64_t blk0 = h.elem_offset >> 3;
+        e.blk0_lo = (uint32_t)blk0;
+        e.head = philox_head((uint32_t)(blk0 >> 32), h.worker, rk.k0[0]);
     }
-    return cudaErrorInvalidValue;
+    return launch_table(tab, nent, tiles, bits, rk, dtype, stream);
+}
+
+// Whether the segments of a call may be encoded by rows of the whole gradient: rows that start on 16-byte boundaries and on
+// blocks of draws, nothing read before the first segment, and one high half of the blocks' indexes.
+bool flat_applies(const void* const* grads, int W, uint64_t begin, uint64_t end, uint64_t elem_offset)
+{
+    for (int w = 0; w < W; ++w)
+        if ((reinterpret_cast<uintptr_t>(grads[w]) & 15u) != 0) return false;
+    const uint64_t first = elem_offset >> 3, last = (elem_offset + end + 63) >> 3;
+    return begin % 64 == 0 && elem_offset % 8 == 0 && first >> 32 == last >> 32 && (end + 31) / 32 <= 0x7FFFFFFFull;
 }
 
 }  // namespace
@@ -325,7 +562,8 @@ cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, 
                           spans_join_max_pass(long_tiles * (uint64_t)W, dtype, aligned);
     cudaError_t err = together ? launch_clear_scales(a, nseg, stream) : cudaSuccess;
     if (err != cudaSuccess) return err;
-    bool any_entries = false;
+    const bool flat = flat_applies(grads, W, seg_off[0], seg_off[nseg], elem_offset);
+    bool any_entries = false, any_flat = false;
     uint64_t sums = 0;                                // partial sums of the tables already launched
     for (int first = 0; first < nseg; first += kMaxSegmentsPerLaunch) {
         const int count = nseg - first < kMaxSegmentsPerLaunch ? nseg - first : kMaxSegmentsPerLaunch;
@@ -354,6 +592,7 @@ cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, 
                 const uint64_t nt = (len + kMaxTileRows * 32 - 1) / (kMaxTileRows * 32);
                 tiles += nt;
                 if (bulk(j)) any_entries = true;
+                else if (flat) any_flat = true;
                 else plain_tiles += nt;
             }
             if (tiles > 0x3FFFFFFFull) return cudaErrorInvalidValue;
@@ -379,25 +618,32 @@ cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, 
         if (err == cudaSuccess) err = launch_encode_table(t, plain, bits, dtype, stream);
         if (err != cudaSuccess) return err;
     }
-    if (!any_entries) return cudaSuccess;
     // no heap here: the C ABI throws nothing
     EntryHost batch[kMaxEntries];
-    int n = 0;
-    auto launch = [&] {
-        err = n <= kFewEntries ? launch_entries<kFewEntries>(batch, n, bits, a.rk, dtype, stream)
-                               : launch_entries<kMaxEntries>(batch, n, bits, a.rk, dtype, stream);
-        n = 0;
-    };
-    for (int j = 0; j < nseg && err == cudaSuccess; ++j) {
-        const uint64_t len = seg_off[j + 1] - seg_off[j];
-        if (len <= kSegmentSpanElems || !bulk(j)) continue;
-        for (int w = 0; w < W && err == cudaSuccess; ++w) {
-            batch[n++] = {static_cast<const char*>(grads[w]) + seg_off[j] * esz, codes[w] + code_off[j], scales[w] + j, len,
-                          elem_offset + seg_off[j], first_worker + (uint32_t)w};
-            if (n == kMaxEntries) launch();
+    for (int pass = any_entries ? 0 : 1; pass < (any_flat ? 2 : 1) && err == cudaSuccess; ++pass) {
+        int n = 0;
+        auto launch = [&] {
+            if (pass == 0)
+                err = n <= kFewEntries ? launch_entries<kFewEntries>(batch, n, bits, a.rk, dtype, stream)
+                                       : launch_entries<kMaxEntries>(batch, n, bits, a.rk, dtype, stream);
+            else
+                err = n <= kFewEntries ? launch_flat<kFewEntries>(batch, n, bits, a.rk, dtype, stream)
+                                       : launch_flat<kMaxEntries>(batch, n, bits, a.rk, dtype, stream);
+            n = 0;
+        };
+        for (int j = 0; j < nseg && err == cudaSuccess; ++j) {
+            const uint64_t len = seg_off[j + 1] - seg_off[j];
+            if (len <= kSegmentSpanElems || bulk(j) != (pass == 0)) continue;
+            const uint32_t pad = pass == 0 ? 0u : (uint32_t)(seg_off[j] % (dtype == 0 ? 32 : 64));
+            const uint64_t from = seg_off[j] - pad;
+            for (int w = 0; w < W && err == cudaSuccess; ++w) {
+                batch[n++] = {static_cast<const char*>(grads[w]) + from * esz, codes[w] + code_off[j], scales[w] + j, len,
+                              elem_offset + from, first_worker + (uint32_t)w, pad, (seg_off[nseg] - from) * esz};
+                if (n == kMaxEntries) launch();
+            }
         }
+        if (n != 0 && err == cudaSuccess) launch();
     }
-    if (n != 0 && err == cudaSuccess) launch();
     return err;
 }
 
