@@ -630,20 +630,35 @@ mqg_status mqg_server_step_segments(const uint32_t* const* codes, const float* c
         if (acc_out && !aligned16(acc_out)) return fail(MQG_ERR_ALIGN, "acc_out not 16-byte aligned");
     }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    // A long segment is a gradient with a single bucket: the long segments whose buffers are aligned for
-    // bulk copies go to the TMA-fed server kernel together, in one launch; all other segments share
+    // A long segment is a gradient with a single bucket: the long segments go to the TMA-fed server kernel together, in one
+    // launch (its form for segments that start anywhere, if one of them is off a 16-byte boundary); all other segments share
     // the table-driven launch.  The results are the same bit for bit either way.
     constexpr uint64_t kOwnLaunchElems = mqg::kEntrySegmentElems;
-    auto own = [&](int j) {
+    auto is_long = [&](int j) {
         const uint64_t len = seg_off[j + 1] - seg_off[j];
-        if (acc_out || len < kOwnLaunchElems || !mqg::server_tma_applies(len, len)) return false;
-        bool aligned = aligned16(params + seg_off[j]);
-        for (int w = 0; w < W && aligned; ++w) aligned = aligned16(codes[w] + code_off[j]);
-        return aligned;
+        return !acc_out && len >= kOwnLaunchElems && mqg::server_tma_applies(len, len);
+    };
+    auto aligned = [&](int j) {
+        bool all = aligned16(params + seg_off[j]);
+        for (int w = 0; w < W && all; ++w) all = aligned16(codes[w] + code_off[j]);
+        return all;
     };
     if (mqg_status st = check_segments(nseg, seg_off, code_off, bits)) return st;
-    bool any_long = false;
-    for (int j = 0; j < nseg && !any_long; ++j) any_long = own(j);
+    // That form takes over from the table-driven launch at half a million elements (more than four workers: a million): one
+    // tensor off the boundary, table / that form, one worker 3.4 / 3.9, 4.7 / 4.0, 9.9 / 4.9 us for 0.2, 0.4 and 1.6 M
+    // elements, eight 3.8 / 5.2, 6.4 / 6.6, 10.5 / 7.6 us for 0.2, 0.8 and 1.6 M, sixteen 8.2 / 9.6, 12.9 / 11.2 us for 0.8 and
+    // 1.6 M; 50 M elements and eight workers 631 / 110 us.
+    uint64_t longs_total = 0;
+    bool any_long = false, any_off = false;
+    for (int j = 0; j < nseg; ++j) {
+        if (!is_long(j)) continue;
+        longs_total += seg_off[j + 1] - seg_off[j];
+        if (aligned(j)) any_long = true;
+        else any_off = true;
+    }
+    const bool flat = any_off && longs_total >= (W <= 4 ? 1ull << 19 : 1ull << 20);
+    any_long = any_long || flat;
+    auto own = [&](int j) { return is_long(j) && (flat || aligned(j)); };
     // The other segments: table-driven launches - except that ONE table of short segments rides along
     // with the (first) launch of the long ones, so that a typical layered step is a single launch.
     mqg::SegmentTable folded;
@@ -668,7 +683,7 @@ mqg_status mqg_server_step_segments(const uint32_t* const* codes, const float* c
             longs[count++] = {seg_off[j + 1] - seg_off[j], seg_off[j], code_off[j], (uint32_t)j};
         if (count == 0 || (count < mqg::kMaxServerSegsPerLaunch && j < nseg)) continue;
         const cudaError_t err = mqg::launch_server_tma_segments(ptrs, W, bits, longs, count, folded_first >= 0 ? &folded : nullptr,
-                                                                folded_first, params, lr, stream);
+                                                                folded_first, params, lr, flat, stream);
         if (err != cudaSuccess) return cuda_fail("mqg_server_step_segments", err);
         folded_first = -1;
         count = 0;

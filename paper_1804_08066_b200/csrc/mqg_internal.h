@@ -126,7 +126,7 @@ cudaError_t launch_server_tma(const WorkerPtrs& ptrs, int W, int bits, uint64_t 
 // The fused update of up to kMaxServerSegsPerLaunch long segments of a per-layer step in ONE launch of
 // the TMA-fed server kernel (a segment is a gradient with a single bucket).  Every segment must
 // satisfy server_tma_applies(n, n), and params + elem0 and every worker's codes + code_word0
-// must be 16-byte aligned.
+// must be 16-byte aligned; with `flat` only `params` itself.
 struct ServerSegHost {
     uint64_t n;              // elements of the segment
     uint64_t elem0;          // offset of its first parameter in `params`
@@ -138,7 +138,7 @@ constexpr int kMaxServerSegsPerLaunch = 16;
 // loads; short_first = index of the table's first segment in the scale arrays.
 cudaError_t launch_server_tma_segments(const WorkerPtrs& ptrs, int W, int bits, const ServerSegHost* segs, int nseg,
                                        const SegmentTable* short_tab, int short_first, float* params, float lr,
-                                       cudaStream_t stream);
+                                       bool flat, cudaStream_t stream);
 
 cudaError_t launch_server_segments(const WorkerPtrs& ptrs, int W, int bits, const SegmentTable& tab,
                                    int scale_base, float* params, float lr, float* acc,

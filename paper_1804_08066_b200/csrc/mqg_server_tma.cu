@@ -75,8 +75,10 @@ struct ServerSegEntry {
     uint32_t tile_start;     // number of the segment's first tile in the launch's sequence
     uint32_t nrows_full;     // floor(n / 32): rows its tensor map and code copies cover
     uint32_t scale_idx;      // index of its scale in every worker's scale array
-    uint32_t ragged;         // n % 32: elements of its last, incomplete row (0 = none)
-    uint64_t code_word0;     // word offset of its bit stream in every worker's code buffer
+    uint32_t ragged;         // elements of its last, incomplete row (0 = none)
+    uint32_t head, shift;    // FLAT: elements before its first row, bit of code_word0 at which that row's codes start
+    uint64_t code_word0;     // word offset of its first row's codes in every worker's code buffer
+    uint64_t words0, words_end;          // its bit stream there
     uint64_t elem0;          // offset of its first element in a.params
 };
 struct ServerSegTable {
@@ -90,7 +92,8 @@ struct ServerSegTable {
 struct TileLoc {
     const CUtensorMap* map;
     uint32_t row0, nrows_full, scale_idx;
-    uint64_t code_word0;
+    uint32_t shift;                              // FLAT, and the end of the bit stream
+    uint64_t code_word0, words_end;
 };
 
 template <bool SEGS>
@@ -105,22 +108,31 @@ __device__ __forceinline__ TileLoc locate_srv_tile(const CUtensorMap* map_full, 
         t.row0 = (tile - e.tile_start) * kSrvTileRows;
         t.nrows_full = e.nrows_full;
         t.scale_idx = e.scale_idx;
+        t.shift = e.shift;
         t.code_word0 = e.code_word0;
+        t.words_end = e.words_end;
     } else {
         t.map = map_full;
         t.row0 = tile * kSrvTileRows;
         t.nrows_full = a.nrows_full;
-        t.scale_idx = 0;
-        t.code_word0 = 0;
+        t.scale_idx = t.shift = 0;
+        t.code_word0 = t.words_end = 0;
     }
     return t;
 }
 
+// FLAT: the segments of the launch may start anywhere.  Their rows are rows of the whole parameter buffer, so the
+// parameters travel as ever; a row's codes then start at any bit, the same one for all rows of a segment.  A tile's
+// words are copied one by one, each worker's and the one behind them, so that they lie in the stage as ever, and a lane shifts
+// its K + 1 words into place.
+template <int BITS, bool FLAT>
+__host__ __device__ constexpr uint32_t stage_words() { return kSrvTileRows * BITS + (FLAT ? 4 : 0); }      // of one worker
+
 // Dynamic shared memory of one CTA (base rounded up to 1024 bytes for the 128-byte swizzle).
-template <int BITS>
+template <int BITS, bool FLAT>
 struct ServerSmem {
     alignas(1024) uint8_t stage[kSrvWarps][kSrvTileBytes];      // one parameter tile per warp
-    alignas(16) uint32_t code[kSrvWarps][kCodeDepth][ServerGroup<BITS>::value][kSrvTileRows * BITS];
+    alignas(16) uint32_t code[kSrvWarps][kCodeDepth][ServerGroup<BITS>::value][stage_words<BITS, FLAT>()];
     float4 table[kSrvWarps][2 * kMaxWorkers];     // (2h, 2h, -h, -h) per (worker, bucket of the tile): entry
                                                   // (worker << nbt_shift) + bucket-of-tile
     uint64_t bar[kSrvWarps];                      // parameter tile landed
@@ -275,6 +287,34 @@ __device__ __forceinline__ void fill_code_stage(const ServerTmaArgs& a, uint32_t
     }
 }
 
+template <int BITS>
+__device__ __forceinline__ void fill_code_stage_flat(const ServerTmaArgs& a, uint32_t stage, const TileLoc& loc, int g0,
+                                                     uint32_t lane)
+{
+    constexpr int kGroup = ServerGroup<BITS>::value;
+    constexpr uint32_t kBytes = stage_words<BITS, true>() * 4, kWords = kSrvTileRows * BITS;
+    const uint64_t word0 = loc.code_word0 + (uint64_t)loc.row0 * BITS;
+    const int nwk = min(kGroup, a.W - g0);
+    auto copy = [&](uint32_t to, const uint32_t* from, bool in) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(to), "l"(from), "r"(in ? 4u : 0u) : "memory");
+    };
+    if (word0 + kWords + 1 <= loc.words_end && nwk == kGroup) {
+#pragma unroll
+        for (int i = 0; i < kGroup; ++i) {
+            const uint32_t* from = a.ptrs.codes[g0 + i] + word0 + lane;
+#pragma unroll
+            for (int k = 0; k < BITS; ++k) copy(stage + i * kBytes + (32 * k + lane) * 4, from + 32 * k, true);
+            if (lane == 0) copy(stage + i * kBytes + kWords * 4, from + kWords, true);
+        }
+    } else {
+        for (int i = 0; i < nwk; ++i)
+            for (uint32_t k = lane; k < kWords + 1; k += 32) {       // words past the stream's end are zeros
+                const bool in = word0 + k < loc.words_end;
+                copy(stage + i * kBytes + k * 4, a.ptrs.codes[g0 + i] + (in ? word0 + k : 0), in);
+            }
+    }
+}
+
 // CTAs per SM the register budget is set for (what the shared memory allows at three bits and more;
 // five CTAs of 96 registers at one and two bits measured 0.3 us slower per launch than four).
 template <int BITS>
@@ -287,22 +327,21 @@ constexpr int server_min_ctas() { return 4; }
 // element j, with plain loads and stores.  What bounds it is one round trip to memory and the chain of the sum: the code
 // words of eight workers are requested at a time, and lane w divides for worker w (at most 32).  131,073 parameters, 1 / 8 / 16
 // workers: 2.4 / 3.2 / 4.2 us, against 3.1 / 4.7 / 7.0 us with a division per worker and element, after the warp's tile.
-// `params` is the gradient's first parameter, n its length, its bit stream the words
-// [code_word0, words_end) of every worker's buffer, `bucket` the index of the row's scale.
+// `params` is the row's first parameter, `count` its length; its codes start at bit `bit0` of word `word0` of every worker's
+// buffer, and their stream ends before word `words_end`; `bucket` is the index of the row's scale.
 // SEGS: every lane divides for every worker.  (With the shuffles in a function that a grid over segments calls, its main loop
 // is compiled to something 2.5 % slower at four bits and eight workers.)
 template <int BITS, int MODE, bool RANGE, bool SEGS>
-__device__ __noinline__ void server_ragged_row(const ServerTmaArgs& a, float* params, uint32_t row, uint64_t n,
-                                               uint64_t code_word0, uint64_t words_end, uint32_t bucket, uint32_t lane)
+__device__ __noinline__ void server_ragged_row(const ServerTmaArgs& a, float* params, uint32_t count, uint64_t word0,
+                                               uint32_t bit0, uint64_t words_end, uint32_t bucket, uint32_t lane)
 {
     static_assert(kMaxWorkers <= 32, "a lane per worker");
-    const uint64_t e = (uint64_t)row * 32 + lane;
-    const bool in = e < n;                       // the others keep going: the shuffles need them
+    const bool in = lane < count;                // the others keep going: the shuffles need them
     if (SEGS && !in) return;
-    const uint32_t bit = lane * BITS, shift = bit & 31u;
-    const uint64_t at = code_word0 + (uint64_t)row * BITS + (bit >> 5), word = at < words_end ? at : words_end - 1;
+    const uint32_t bit = bit0 + lane * BITS, shift = bit & 31u;
+    const uint64_t at = word0 + (bit >> 5), word = at < words_end ? at : words_end - 1;
     const bool two = shift + BITS > 32 && word + 1 < words_end;
-    const float old = MODE != 0 && in ? params[e] : 0.0f;
+    const float old = MODE != 0 && in ? params[lane] : 0.0f;
     auto load_scale = [&](int w) {
         return RANGE ? __ldg(reinterpret_cast<const float2*>(a.ptrs.scales[w]) + bucket)
                      : make_float2(__ldg(a.ptrs.scales[w] + bucket), 0.0f);
@@ -341,18 +380,18 @@ __device__ __noinline__ void server_ragged_row(const ServerTmaArgs& a, float* pa
                                              make_float2(d.two_h, d.two_h), make_float2(d.minus_h, d.minus_h));
         }
     }
-    if (in) params[e] = MODE == 1 ? __fmaf_rn(a.neg_lr, v.x, old) : v.x;
+    if (in) params[lane] = MODE == 1 ? __fmaf_rn(a.neg_lr, v.x, old) : v.x;
 }
 
-template <int BITS, int MODE, bool RANGE, bool SEGS, bool kUnit>
+template <int BITS, int MODE, bool RANGE, bool SEGS, bool kUnit, bool FLAT = false>
 __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, const ServerTmaArgs& a,
                                                 const ServerSegTable* segs, unsigned int* __restrict__ timeouts)
 {
     extern __shared__ uint8_t smem_raw[];
-    ServerSmem<BITS>& sm = *reinterpret_cast<ServerSmem<BITS>*>(
+    ServerSmem<BITS, FLAT>& sm = *reinterpret_cast<ServerSmem<BITS, FLAT>*>(
         smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
     constexpr int kGroup = ServerGroup<BITS>::value;
-    constexpr uint32_t kWorkerWords = kSrvTileRows * BITS;
+    constexpr uint32_t kWorkerWords = stage_words<BITS, FLAT>();
     const uint32_t lane = threadIdx.x & 31u;
     // the warp's number, taken from lane 0 so that the compiler knows it is the same in every lane
     const uint32_t wid = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0);
@@ -406,6 +445,11 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
     const UnitBits<BITS, RANGE> unit_bits(a.one);
     bool unit = false;                             // the tile in work is summed in units of 2^40
 
+    auto fill = [&](uint32_t to, const TileLoc& loc, int g0) {
+        if constexpr (FLAT) fill_code_stage_flat<BITS>(a, to, loc, g0, lane);
+        else fill_code_stage<BITS>(a, to, loc, g0, lane_off);
+    };
+
     bool failed = false;
     uint32_t k = 0, u = 0;                         // tile and code stage in use
     if (ntiles > 0) {
@@ -422,9 +466,9 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
 #pragma unroll
         for (uint32_t u2 = 0; u2 < (uint32_t)kCodeDepth; ++u2) {
             if (u2 < nunits)
-                fill_code_stage<BITS>(a, code_base + u2 * kCodeStageBytes,
-                                      locate_srv_tile<SEGS>(map_full, a, segs, t_begin + (u2 / groups) * t_step, fill_e),
-                                      (int)(u2 % groups) * kGroup, lane_off);
+                fill(code_base + u2 * kCodeStageBytes,
+                     locate_srv_tile<SEGS>(map_full, a, segs, t_begin + (u2 / groups) * t_step, fill_e),
+                     (int)(u2 % groups) * kGroup);
             cp_async_commit();
         }
         unit = store_tile_scales<BITS, RANGE, kUnit>(a, table, lane, wide, s0);
@@ -485,6 +529,11 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
             auto decode_worker = [&](int i, auto in_units) {
                 uint32_t w[BITS];
                 read_stage_words<BITS>(cstage + i * kWorkerWords, w);
+                if constexpr (FLAT) {
+                    const uint32_t behind = cstage[i * kWorkerWords + BITS];
+#pragma unroll
+                    for (int q = 0; q < BITS; ++q) w[q] = __funnelshift_r(w[q], q + 1 < BITS ? w[q + 1 < BITS ? q + 1 : 0] : behind, loc.shift);
+                }
                 const float4 e = my_table[(uint32_t)(g0 + i) << a.nbt_shift];
                 if constexpr (decltype(in_units)::value) {
                     add_decoded_row_unit<BITS, RANGE>(w, e, unit_bits, v2);
@@ -537,9 +586,8 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
             }
             __syncwarp();                          // every lane has read the stage: refill it
             if (u + kCodeDepth < nunits)
-                fill_code_stage<BITS>(a, cstage_addr,
-                                      locate_srv_tile<SEGS>(map_full, a, segs, t_begin + fill_tile * t_step, fill_e),
-                                      (int)fill_group * kGroup, lane_off);
+                fill(cstage_addr, locate_srv_tile<SEGS>(map_full, a, segs, t_begin + fill_tile * t_step, fill_e),
+                     (int)fill_group * kGroup);
             cp_async_commit();
             if (++fill_group == groups) { fill_group = 0; ++fill_tile; }
         }
@@ -614,16 +662,19 @@ __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, con
     // in turn.)
     const uint32_t from_end = nwarps - 1 - gwarp;
     if constexpr (SEGS) {
-        for (uint32_t j = from_end; j < (uint32_t)segs->nseg; j += nwarps) {
-            const ServerSegEntry& e = segs->e[j];
-            if (e.ragged == 0) continue;
-            const uint64_t n = (uint64_t)e.nrows_full * 32 + e.ragged;
-            server_ragged_row<BITS, MODE, RANGE, SEGS>(a, a.params + e.elem0, e.nrows_full, n, e.code_word0,
-                                                 e.code_word0 + (n * BITS + 31) / 32, e.scale_idx, lane);
+        for (uint32_t j = from_end; j < (uint32_t)segs->nseg * (FLAT ? 2u : 1u); j += nwarps) {
+            const bool first = FLAT && j >= (uint32_t)segs->nseg;              // the elements before the first row
+            const ServerSegEntry& e = segs->e[first ? j - (uint32_t)segs->nseg : j];
+            const uint32_t count = first ? e.head : e.ragged;
+            if (count == 0) continue;
+            const uint64_t done = first ? 0 : (uint64_t)(FLAT ? e.head : 0u) + 32ull * e.nrows_full;
+            server_ragged_row<BITS, MODE, RANGE, SEGS>(a, a.params + e.elem0 + done, count, e.words0 + (done * BITS >> 5),
+                                                       (uint32_t)(done * BITS) & 31u, e.words_end, e.scale_idx, lane);
         }
     } else if (a.nrows > a.nrows_full && from_end == 0) {
-        server_ragged_row<BITS, MODE, RANGE, SEGS>(a, a.params, a.nrows_full, a.n, 0, a.ncode_words,
-                                             bucket_of_row(a, a.nrows_full), lane);
+        server_ragged_row<BITS, MODE, RANGE, SEGS>(a, a.params + (uint64_t)a.nrows_full * 32, (uint32_t)(a.n & 31u),
+                                                   (uint64_t)a.nrows_full * BITS, 0u, a.ncode_words,
+                                                   bucket_of_row(a, a.nrows_full), lane);
     }
 }
 
@@ -697,17 +748,17 @@ __device__ __noinline__ void server_short_piece(const ServerTmaArgs& a, const Se
 }
 
 // Several long segments of a per-layer step (fused update only), then the step's short segments.
-template <int BITS, bool UNIT>
+template <int BITS, bool UNIT, bool FLAT>
 __global__ void __launch_bounds__(kSrvThreads, server_min_ctas<BITS>())
 server_tma_segments_kernel(const __grid_constant__ ServerSegTable segs, const __grid_constant__ ServerShortSegs ss,
                            const __grid_constant__ ServerTmaArgs a, unsigned int* __restrict__ timeouts)
 {
-    server_tma_body<BITS, 1, false, true, UNIT>(nullptr, a, &segs, timeouts);
+    server_tma_body<BITS, 1, false, true, UNIT, FLAT>(nullptr, a, &segs, timeouts);
     const uint32_t wid = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0);
     const uint32_t nwarps = gridDim.x * kSrvWarps, from_end = nwarps - 1 - (blockIdx.x * kSrvWarps + wid);
     // the warps that finished their share of the long segments first are the last ones of the grid; the very last ones may
     // have a segment's last row
-    const uint32_t skip = (uint32_t)segs.nseg % nwarps;
+    const uint32_t skip = (uint32_t)segs.nseg * (FLAT ? 2u : 1u) % nwarps;
     for (uint32_t piece = from_end >= skip ? from_end - skip : from_end + nwarps - skip; piece < ss.pieces; piece += nwarps)
         server_short_piece<BITS>(a, ss, piece, threadIdx.x & 31u);
 }
@@ -728,7 +779,7 @@ static cudaError_t launch_server_tma_inst(const void* params, ServerTmaArgs& a, 
                                           cudaStream_t stream)
 {
     auto kernel = server_tma_kernel<BITS, MODE, RANGE, UNIT>;
-    constexpr size_t kSmemBytes = sizeof(ServerSmem<BITS>) + 1024;   // + slack to round the base up
+    constexpr size_t kSmemBytes = sizeof(ServerSmem<BITS, false>) + 1024;   // + slack to round the base up
     static std::atomic<int> grid_cap[64];                 // per device; 0 = not yet set up (zero-initialised)
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
@@ -929,8 +980,8 @@ requantize_warp_kernel(const __grid_constant__ RequantWarpArgs ra)
         t.map = nullptr;
         t.row0 = ((blockIdx.x + kk * gridDim.x) * WARPS + wid) * kSrvTileRows;
         t.nrows_full = ra.complete_rows;
-        t.scale_idx = 0;
-        t.code_word0 = 0;
+        t.scale_idx = t.shift = 0;
+        t.code_word0 = t.words_end = 0;
         return t;
     };
     auto fill = [&](uint32_t stage, uint32_t kk, int g0) {           // a tile beyond the last row has no codes
@@ -1200,12 +1251,12 @@ cudaError_t launch_requantize_warp(const WorkerPtrs& ptrs, int W, int bits, uint
 }
 
 // ---- several long segments of a per-layer step in one launch --------------------------------------
-template <int BITS, bool UNIT>
+template <int BITS, bool UNIT, bool FLAT>
 static cudaError_t launch_server_segs_inst(const ServerSegTable& tab, const ServerShortSegs& ss, const ServerTmaArgs& a,
                                            unsigned int* timeouts, cudaStream_t stream)
 {
-    auto kernel = server_tma_segments_kernel<BITS, UNIT>;
-    constexpr size_t kSmemBytes = sizeof(ServerSmem<BITS>) + 1024;   // + slack to round the base up
+    auto kernel = server_tma_segments_kernel<BITS, UNIT, FLAT>;
+    constexpr size_t kSmemBytes = sizeof(ServerSmem<BITS, FLAT>) + 1024;   // + slack to round the base up
     static std::atomic<int> grid_cap[64];                 // per device; 0 = not yet set up (zero-initialised)
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
@@ -1224,14 +1275,14 @@ static cudaError_t launch_server_segs_inst(const ServerSegTable& tab, const Serv
         grid_cap[dev].store(cap, std::memory_order_relaxed);   // every thread computes the same value
     }
     uint64_t grid = (uint64_t)cap;
-    const uint64_t warps = (uint64_t)a.ntiles + (uint64_t)tab.nseg + ss.pieces;   // at least one tile, last row or short piece per warp
+    const uint64_t warps = (uint64_t)a.ntiles + (uint64_t)tab.nseg * (FLAT ? 2 : 1) + ss.pieces;   // at least one tile, last row or short piece per warp
     if (grid * kSrvWarps > warps) grid = (warps + kSrvWarps - 1) / kSrvWarps;
     return launch_pdl_smem(kernel, (unsigned)grid, kSrvThreads, kSmemBytes, stream, tab, ss, a, timeouts);
 }
 
 cudaError_t launch_server_tma_segments(const WorkerPtrs& ptrs, int W, int bits, const ServerSegHost* segs, int nseg,
                                        const SegmentTable* short_tab, int short_first, float* params, float lr,
-                                       cudaStream_t stream)
+                                       bool flat, cudaStream_t stream)
 {
     if (nseg < 1 || nseg > kMaxSrvSegs) return cudaErrorInvalidValue;
     ServerShortSegs ss;
@@ -1250,16 +1301,22 @@ cudaError_t launch_server_tma_segments(const WorkerPtrs& ptrs, int W, int bits, 
     for (int j = 0; j < nseg; ++j) {
         const ServerSegHost& h = segs[j];
         ServerSegEntry& e = tab.e[j];
-        const uint64_t nrows_full = h.n / 32;
-        if (nrows_full == 0 || nrows_full > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+        const uint64_t head = flat ? (0 - h.elem0) % 32 : 0;          // elements up to the next row of `params`
+        if (h.n < head + 32) return cudaErrorInvalidValue;
+        const uint64_t nrows_full = (h.n - head) / 32;
+        if (nrows_full > 0x7FFFFFFFull) return cudaErrorInvalidValue;
         const char* why = nullptr;
-        if (!encode_rows_map(&tab.map[j], params + h.elem0, nrows_full, 4, 32, kSrvTileRows, &why))
+        if (!encode_rows_map(&tab.map[j], params + h.elem0 + head, nrows_full, 4, 32, kSrvTileRows, &why))
             return cudaErrorNotSupported;
         e.tile_start = (uint32_t)tiles;
         e.nrows_full = (uint32_t)nrows_full;
         e.scale_idx = h.scale_idx;
-        e.ragged = (uint32_t)(h.n % 32);
-        e.code_word0 = h.code_word0;
+        e.ragged = (uint32_t)((h.n - head) % 32);
+        e.head = (uint32_t)head;
+        e.shift = (uint32_t)(head * bits) & 31u;
+        e.code_word0 = h.code_word0 + (head * bits >> 5);
+        e.words0 = h.code_word0;
+        e.words_end = h.code_word0 + (h.n * (uint64_t)bits + 31) / 32;
         e.elem0 = h.elem0;
         tiles += (nrows_full + kSrvTileRows - 1) / kSrvTileRows;
         if (tiles > 0x7FFFFFFFull) return cudaErrorInvalidValue;
@@ -1286,8 +1343,11 @@ cudaError_t launch_server_tma_segments(const WorkerPtrs& ptrs, int W, int bits, 
 #define MQG_SEGS_CASE(B) \
         case B: \
             if constexpr (UnitDecode<B, false>::kExists) \
-                if (sum_in_units<B>(a, -lr)) return launch_server_segs_inst<B, true>(tab, ss, a, timeouts, stream); \
-            return launch_server_segs_inst<B, false>(tab, ss, a, timeouts, stream)
+                if (sum_in_units<B>(a, -lr)) \
+                    return flat ? launch_server_segs_inst<B, true, true>(tab, ss, a, timeouts, stream) \
+                                : launch_server_segs_inst<B, true, false>(tab, ss, a, timeouts, stream); \
+            return flat ? launch_server_segs_inst<B, false, true>(tab, ss, a, timeouts, stream) \
+                        : launch_server_segs_inst<B, false, false>(tab, ss, a, timeouts, stream)
         MQG_SEGS_CASE(1); MQG_SEGS_CASE(2); MQG_SEGS_CASE(3); MQG_SEGS_CASE(4);
         MQG_SEGS_CASE(5); MQG_SEGS_CASE(6); MQG_SEGS_CASE(7); MQG_SEGS_CASE(8);
 #undef MQG_SEGS_CASE
