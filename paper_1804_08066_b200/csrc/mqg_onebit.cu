@@ -221,8 +221,7 @@ onebit_tma_kernel(const __grid_constant__ CUtensorMap map_g, const __grid_consta
         typename Shared::Stage& stage = sh.stage[s];
         const uint32_t row0 = tile * a.tile_rows, row = row0 + t, bar = smem_u32(&sh.bar[s]);
         const bool active = t < a.tile_rows && row < (uint32_t)a.nrows;
-        const bool ragged_warp = a.nrows > ta.nrows_full &&
-                                 warp_has_row(ta.nrows_full, row - (t & 31u), (int)(a.tile_rows - (t & ~31u)));
+        const bool ragged_warp = a.nrows > ta.nrows_full && tile + 1 == ta.ntiles && warp_has_row(ta.nrows_full, row - (t & 31u));
         const bool ragged = ragged_warp && active && row >= (uint32_t)ta.nrows_full;
         if (ragged_warp) {
             fetch_ragged_row(smem_u32(sh.ragged[0][t >> 5]), static_cast<const uint8_t*>(a.grad), ta.nrows_full,

@@ -323,6 +323,7 @@ int fill_tma_args(QuantizeArgs& a, TmaQuantizeConsts& c, uint64_t rpb)
         k0 += 0x9E3779B9u; k1 += 0xBB67AE85u;
     }
     c.rk.worker = a.key.worker; c.rk.step = a.key.step;
+    c.ragged_tile = a.nrows > a.nrows_full ? a.ntiles - 1 : 0xFFFFFFFFu;
     c.full_tiles = a.tile_rows == (uint32_t)threads ? (uint32_t)(a.nrows_full / a.tile_rows) : 0u;
     c.blk0_lo = (uint32_t)(a.elem_offset >> 3); c.blk0_hi = (uint32_t)(a.elem_offset >> 35);
     c.head = philox_head(c.blk0_hi, c.rk.worker, c.rk.k0[0]);

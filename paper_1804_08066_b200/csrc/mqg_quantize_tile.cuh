@@ -117,18 +117,37 @@ static __device__ __noinline__ void fetch_ragged_wide_row(uint32_t to, const uin
     fetch_ragged_row(to, grad, row, total_bytes, 128);
 }
 
-// Whether this thread's warp holds that row: `first` is the row of the warp's lane 0, `rows` the tile's rows from there on.
-__device__ __forceinline__ bool warp_has_row(uint64_t row, uint32_t first, int rows)
+// The warp moves that row into row `row` of the tile's stage, once the tile's copy, which fills it with zeros, has landed; its
+// owner reads it like any other.  (Read from where it is, after or instead of the stage's, the choice between the two cost
+// every row of the tiles that may have one 10 to 26 instructions.)
+static __device__ __noinline__ void put_ragged_row(uint8_t* stage, uint32_t row, const uint8_t* from, uint32_t row_bytes)
 {
-    return row >= first && row - first < (uint64_t)max(min(rows, 32), 0);
+    cp_async_wait_all();
+    __syncwarp();
+    const uint32_t lane = threadIdx.x & 31u, chunk = lane >> 2;
+    const uint32_t at = row_bytes == 128 ? row * 8 + (chunk ^ (row & 7u)) : row * 4 + (chunk ^ ((row >> 1) & 3u));
+    if (4 * lane < row_bytes)
+        reinterpret_cast<uint32_t*>(stage)[at * 4 + (lane & 3u)] = reinterpret_cast<const uint32_t*>(from)[lane];
+    fence_proxy_async();             // orders these stores before the bulk copy that refills the stage
+    __syncwarp();
 }
 
-// The stage and the row in it from which a thread reads its row: the ragged one is row 0 of a stage of its own (whose
-// swizzle leaves row 0 as it is).
-struct RowSource {
-    const uint8_t* stage;
-    int row;
-};
+// The same in one step, by its owner, for 128-byte rows whose launches are long (mqg_segments_workers.cu).
+static __device__ __noinline__ void stage_ragged_row(uint8_t* stage, uint32_t row, const uint8_t* grad, uint64_t from,
+                                                     uint64_t total_bytes)
+{
+    for (uint32_t w = 0; w < 32; ++w) {
+        const uint64_t at = from * 128 + 4 * w;
+        uint32_t v = 0u;
+        if (at + 4 <= total_bytes) v = *reinterpret_cast<const uint32_t*>(grad + at);
+        else if (at + 2 <= total_bytes) v = *reinterpret_cast<const uint16_t*>(grad + at);
+        reinterpret_cast<uint32_t*>(stage)[(row * 8 + ((w >> 2) ^ (row & 7u))) * 4 + (w & 3u)] = v;
+    }
+    fence_proxy_async();             // orders these stores before the bulk copy that refills the stage
+}
+
+// Whether this thread's warp holds that row, in the tile that does; `first` is the row of the warp's lane 0.
+__device__ __forceinline__ bool warp_has_row(uint64_t row, uint32_t first) { return (uint32_t)row - first < 32u; }
 
 // How the rows of a bucket are reduced: a bucket is an aligned power-of-two group of at most 32 rows (lane
 // shuffles), a whole number of warps (one shared-memory atomic per warp), or any other number of rows (one
@@ -182,6 +201,7 @@ __device__ __forceinline__ void load_tile_rows(uint32_t stage, const CUtensorMap
 struct TmaQuantizeConsts {
     RoundKeys rk;
     uint32_t full_tiles;         // leading tiles in which every thread has a complete row
+    uint32_t ragged_tile;        // the tile whose last row is shorter than the others; 2^32 - 1 if there is none
     uint32_t blk0_lo, blk0_hi;   // Philox block index of element 0: elem_offset / 8; the launch's blocks
                                  // all have the high half blk0_hi (tma_path_applies)
     PhiloxHead head;             // launch-wide part of the blocks of worker rk.worker
@@ -214,8 +234,7 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     const uint32_t t = threadIdx.x;
     const uint32_t row = tile * a.tile_rows + t;
     const bool active = FULL || (t < a.tile_rows && row < (uint32_t)a.nrows);
-    const bool ragged_warp = !FULL && a.nrows > a.nrows_full &&
-                             warp_has_row(a.nrows_full, row - (t & 31u), (int)(a.tile_rows - (t & ~31u)));
+    const bool tail = !FULL && tile == c.ragged_tile;            // a tile with a row that the copy does not cover
     const uint32_t stg = k % kQuantStages, parity = (k / kQuantStages) & 1;
     const uint32_t bar = smem_u32(&sh.bar[stg]);
     uint8_t* stage = sh.stage[stg];
@@ -231,11 +250,13 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     constexpr bool kEarlyDraw = !NORM && DTYPE == 0 && BITS >= 3;
     uint32_t h[16];
     if (kEarlyDraw && active) draw_row_blocks_head(wv.blk0_lo + 4u * row, wv.head, c.rk, h);
-    if (ragged_warp) fetch_ragged_row(smem_u32(sh.ragged[t >> 5]), static_cast<const uint8_t*>(wv.grad), a.nrows_full,
-                                      a.n * (DTYPE == 0 ? 4 : 2), DTYPE == 0 ? 128 : 64);
+    if (tail && warp_has_row(a.nrows_full, row - (t & 31u)))
+        fetch_ragged_row(smem_u32(sh.ragged[t >> 5]), static_cast<const uint8_t*>(wv.grad), a.nrows_full,
+                         a.n * (DTYPE == 0 ? 4 : 2), DTYPE == 0 ? 128 : 64);
     bool ok = mbar_try_wait(bar, parity);
     if (!ok) ok = mbar_wait(bar, parity, a.poll_limit);
-    if (ragged_warp) { cp_async_wait_all(); __syncwarp(); }
+    if (tail && warp_has_row(a.nrows_full, row - (t & 31u)))
+        put_ragged_row(stage, (uint32_t)a.nrows_full - tile * a.tile_rows, sh.ragged[t >> 5], DTYPE == 0 ? 128 : 64);
 
     // bf16 rows whose maximum is wanted stay packed until the encode: half the registers across the barrier, and the
     // maximum takes two elements per instruction (30.0 against 30.5 us per 50 M elements at K = 4)
@@ -243,10 +264,8 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
     float x[32];
     uint32_t raw[16];
     if (active) {
-        const RowSource src = ragged_warp && row >= (uint32_t)a.nrows_full ? RowSource{sh.ragged[t >> 5], 0}
-                                                                           : RowSource{stage, (int)t};
-        if (kPackedRow) read_row_words(src.stage, src.row, raw);
-        else read_row_swizzled<DTYPE>(src.stage, src.row, x);
+        if (kPackedRow) read_row_words(stage, (int)t, raw);
+        else read_row_swizzled<DTYPE>(stage, (int)t, x);
     } else {
 #pragma unroll
         for (int j = 0; j < 32; ++j) x[j] = 0.0f;
@@ -361,32 +380,32 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
 // ordered bits; the kernel initialises them to the identities.
 template <int BITS, int DTYPE, int THREADS, bool FULL, int RED, typename Refill>
 __device__ __forceinline__ bool range_quantize_tile(TmaQuantizeShared<DTYPE, THREADS>& sh, const WorkerView wv,
-                                                    const QuantizeArgs& a, uint32_t k, uint32_t rot, uint32_t tile,
-                                                    Refill&& refill, uint32_t local_bucket, bool scale_writer)
+                                                    const QuantizeArgs& a, const TmaQuantizeConsts& c, uint32_t k,
+                                                    uint32_t rot, uint32_t tile, Refill&& refill, uint32_t local_bucket,
+                                                    bool scale_writer)
 {
     constexpr int kQuantStages = TmaQuantizeShared<DTYPE, THREADS>::kStages;
     constexpr bool SHUFFLE = RED == kByShuffle;
     const uint32_t t = threadIdx.x;
     const uint32_t row = tile * a.tile_rows + t;
     const bool active = FULL || (t < a.tile_rows && row < (uint32_t)a.nrows);
-    const bool ragged_warp = !FULL && a.nrows > a.nrows_full &&
-                             warp_has_row(a.nrows_full, row - (t & 31u), (int)(a.tile_rows - (t & ~31u)));
+    const bool tail = !FULL && tile == c.ragged_tile;            // a tile with a row that the copy does not cover
     const uint32_t stg = k % kQuantStages, parity = (k / kQuantStages) & 1;
     const uint32_t bar = smem_u32(&sh.bar[stg]);
     uint8_t* stage = sh.stage[stg];
 
-    if (ragged_warp) fetch_ragged_row(smem_u32(sh.ragged[t >> 5]), static_cast<const uint8_t*>(wv.grad), a.nrows_full,
-                                      a.n * (DTYPE == 0 ? 4 : 2), DTYPE == 0 ? 128 : 64);
+    if (tail && warp_has_row(a.nrows_full, row - (t & 31u)))
+        fetch_ragged_row(smem_u32(sh.ragged[t >> 5]), static_cast<const uint8_t*>(wv.grad), a.nrows_full,
+                         a.n * (DTYPE == 0 ? 4 : 2), DTYPE == 0 ? 128 : 64);
     bool ok = mbar_try_wait(bar, parity);
     if (!ok) ok = mbar_wait(bar, parity, a.poll_limit);
-    if (ragged_warp) { cp_async_wait_all(); __syncwarp(); }
+    if (tail && warp_has_row(a.nrows_full, row - (t & 31u)))
+        put_ragged_row(stage, (uint32_t)a.nrows_full - tile * a.tile_rows, sh.ragged[t >> 5], DTYPE == 0 ? 128 : 64);
 
     float x[32];
     uint32_t mlo = kOrderedMinIdentity, mhi = kOrderedMaxIdentity;
     if (active) {
-        const RowSource src = ragged_warp && row >= (uint32_t)a.nrows_full ? RowSource{sh.ragged[t >> 5], 0}
-                                                                           : RowSource{stage, (int)t};
-        read_row_swizzled<DTYPE>(src.stage, src.row, x);
+        read_row_swizzled<DTYPE>(stage, (int)t, x);
         if (!FULL) {
             const uint64_t left = a.n - (uint64_t)row * 32;      // >= 1
 #pragma unroll
@@ -463,26 +482,25 @@ __device__ __forceinline__ bool quantize_wide_tile(TmaQuantizeShared<kBf16Wide, 
     const uint32_t t = threadIdx.x;
     const uint32_t row = tile * a.tile_rows + t;
     const bool active = FULL || (t < a.tile_rows && row < (uint32_t)a.nrows);
-    const bool ragged_warp = !FULL && a.nrows > a.nrows_full &&
-                             warp_has_row(a.nrows_full, row - (t & 31u), (int)(a.tile_rows - (t & ~31u)));
+    const bool tail = !FULL && tile == c.ragged_tile;            // a tile with a row that the copy does not cover
     const uint32_t stg = k % kQuantStages, parity = (k / kQuantStages) & 1;
     const uint32_t bar = smem_u32(&sh.bar[stg]);
     uint8_t* stage = sh.stage[stg];
 
-    if (ragged_warp)
+    if (tail && warp_has_row(a.nrows_full, row - (t & 31u)))
         fetch_ragged_wide_row(smem_u32(sh.ragged[t >> 5]), static_cast<const uint8_t*>(wv.grad), a.nrows_full, a.n * 2);
     bool ok = mbar_try_wait(bar, parity);
     if (!ok) ok = mbar_wait(bar, parity, a.poll_limit);
-    if (ragged_warp) { cp_async_wait_all(); __syncwarp(); }
+    if (tail) { cp_async_wait_all(); __syncwarp(); }
 
     uint32_t raw[2][16];
     if (active) {
-        const RowSource src = ragged_warp && row >= (uint32_t)a.nrows_full ? RowSource{sh.ragged[t >> 5], 0}
-                                                                           : RowSource{stage, (int)t};
-        const uint4* s = reinterpret_cast<const uint4*>(src.stage);
+        // the ragged row is read where it is, as row 0 of a stage of its own (put into its stage first: 110 against 108 us)
+        const bool apart = tail && row >= (uint32_t)a.nrows_full;
+        const uint4* s = reinterpret_cast<const uint4*>(apart ? sh.ragged[t >> 5] : stage);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const uint4 v = s[swz(src.row, i)];
+            const uint4 v = s[swz(apart ? 0 : (int)t, i)];
             uint32_t* to = &raw[i >> 2][(i & 3) * 4];
             to[0] = v.x; to[1] = v.y; to[2] = v.z; to[3] = v.w;
         }
@@ -546,7 +564,7 @@ __device__ __forceinline__ bool mode_tile(TmaQuantizeShared<DTYPE, THREADS>& sh,
     if constexpr (DTYPE == kBf16Wide)
         return quantize_wide_tile<BITS, THREADS, FULL, RED>(sh, wv, a, c, k, rot, tile, refill, local_bucket, scale_writer);
     else if constexpr (MODE == kRange)
-        return range_quantize_tile<BITS, DTYPE, THREADS, FULL, RED>(sh, wv, a, k, rot, tile, refill, local_bucket,
+        return range_quantize_tile<BITS, DTYPE, THREADS, FULL, RED>(sh, wv, a, c, k, rot, tile, refill, local_bucket,
                                                                     scale_writer);
     else
         return quantize_tile<BITS, DTYPE, THREADS, FULL, RED, MODE == kNorm>(sh, wv, a, c, k, rot, tile, refill,

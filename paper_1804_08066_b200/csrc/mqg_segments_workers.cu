@@ -73,7 +73,6 @@ encode_entries_kernel(const __grid_constant__ SegEntryTable<CAP> T, unsigned int
     constexpr int kHalves = DTYPE == 0 ? 1 : 2, kElems = 32 * kHalves, kWords = BITS * kHalves;
     struct Shared {
         alignas(1024) uint8_t stage[kStages][kTileBytes];
-        alignas(16) uint8_t ragged[kWarps][128];
         alignas(8) uint64_t bar[kStages];
         uint32_t read[kStages];        // warps that have read the stage, over all its uses
     };
@@ -128,28 +127,16 @@ encode_entries_kernel(const __grid_constant__ SegEntryTable<CAP> T, unsigned int
         const uint32_t bar = smem_u32(&sh.bar[s]);
         uint32_t h[16];
         draw_row_blocks_head(blk0 + 4u * kHalves * row, head, T.rk, h);
-        const bool active = row < rows, ragged_warp = u + 1 == end && rows > rows_full && warp_has_row(rows_full, row - lane, 32);
-        if (ragged_warp) {
-            const uint32_t to = smem_u32(sh.ragged[t >> 5]);
-            const uint8_t* grad = static_cast<const uint8_t*>(T.e[e].grad);
-            if constexpr (DTYPE == 0) fetch_ragged_row(to, grad, rows_full, T.e[e].n * 4, 128);
-            else fetch_ragged_wide_row(to, grad, rows_full, T.e[e].n * 2);
-        }
+        const bool active = row < rows;
         ok = mbar_try_wait(bar, (k / kStages) & 1);
         if (!ok) ok = mbar_wait(bar, (k / kStages) & 1, T.poll_limit);
         if (!__all_sync(0xFFFFFFFFu, ok)) { ok = false; break; }
+        if (active && row >= rows_full)    // a last row that the copy does not cover
+            stage_ragged_row(stage, t, static_cast<const uint8_t*>(T.e[e].grad), row, T.e[e].n * (DTYPE == 0 ? 4 : 2));
 
         uint4 v[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[i] = reinterpret_cast<const uint4*>(stage)[swz((int)t, i)];
-        if (ragged_warp) {
-            cp_async_wait_all();
-            __syncwarp();
-            if (row >= rows_full) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) v[i] = reinterpret_cast<const uint4*>(sh.ragged[t >> 5])[i];
-            }
-        }
         __syncwarp();                      // every lane has read the stage
         bool last = false;
         if (lane == 0) {
@@ -243,7 +230,6 @@ encode_flat_kernel(const __grid_constant__ FlatTable<CAP> T, unsigned int* __res
     struct Shared {
         alignas(1024) uint8_t stage[kStages][kTileBytes];
         alignas(16) uint32_t out[kFlatWarps][32 * kWords];
-        alignas(16) uint8_t ragged[kFlatWarps][128];
         alignas(8) uint64_t bar[kStages];
         uint32_t read[kStages];        // warps that have read the stage, over all its uses
     };
@@ -301,28 +287,15 @@ encode_flat_kernel(const __grid_constant__ FlatTable<CAP> T, unsigned int* __res
         const uint32_t bar = smem_u32(&sh.bar[s]);
         uint32_t h[16];
         draw_row_blocks_head(blk0 + 4u * kHalves * row, head, T.rk, h);
-        const bool ragged_warp = u + 1 == end && rows > rows_full && warp_has_row(rows_full, row0, 32);
-        if (ragged_warp) {
-            const uint32_t to = smem_u32(sh.ragged[wid]);
-            const uint8_t* grad = static_cast<const uint8_t*>(T.e[e].base);
-            if constexpr (DTYPE == 0) fetch_ragged_row(to, grad, rows_full, T.e[e].bytes, 128);
-            else fetch_ragged_wide_row(to, grad, rows_full, T.e[e].bytes);
-        }
         ok = mbar_try_wait(bar, (k / kStages) & 1);
         if (!ok) ok = mbar_wait(bar, (k / kStages) & 1, T.poll_limit);
         if (!__all_sync(0xFFFFFFFFu, ok)) { ok = false; break; }
+        if (row < rows && row >= rows_full)        // as in encode_entries_kernel (two warps may share it: both put the same there)
+            stage_ragged_row(stage, at, static_cast<const uint8_t*>(T.e[e].base), row, T.e[e].bytes);
 
         uint4 v[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[i] = reinterpret_cast<const uint4*>(stage)[swz((int)at, i)];
-        if (ragged_warp) {
-            cp_async_wait_all();
-            __syncwarp();
-            if (row >= rows_full) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) v[i] = reinterpret_cast<const uint4*>(sh.ragged[wid])[i];
-            }
-        }
         __syncwarp();                      // every lane has read the stage
         bool refill = false;
         if (lane == 0) {
