@@ -91,7 +91,7 @@ mqg_status mqg_quantize(const void* grad, uint64_t n, int bits, uint64_t bucket,
  *                         buffer as in mqg_quantize; the outputs are what mqg_server_step and
  *                         mqg_dequant_accumulate take as codes[] / scales[]
  * Two kernels take all workers in one launch.  The first wants at least 2048 elements, elem_offset a multiple of 8 and
- * buckets of at most 8192 elements, those above 4096 a multiple of 1024.  The second takes buckets of up to 49152
+ * buckets of at most 16384 elements (the L2-norm variant 8192), those above 4096 a multiple of 1024.  The second takes buckets of up to 49152
  * elements (or one such gradient) with any elem_offset, a CTA to a bucket: used where the first does not apply for
  * buckets above 4096 elements, and below 65536 elements for up to 512 buckets.  Other shapes run as W launches (or more)
  * inside the call.
@@ -302,11 +302,12 @@ mqg_status mqg_quantize_segments_l2_static(const void* grad, int nseg, const uin
  *   codes     [out] code_off[nseg] words;  scales [out] nseg floats
  * Element i of segment j draws with position elem_offset + seg_off[j] + i.  Empty segments get
  * scale 0.
- * Performance note: a segment of at most 16384 elements is read once, a longer one twice; the longer ones are
- * encoded by the bulk-copy kernel when grad + seg_off[j] is 16-byte aligned and elem_offset + seg_off[j] is a
- * multiple of 8 (and, from 2^15 elements on, applied by mqg_server_step_segments' bulk-copy kernel when
- * params + seg_off[j] and every worker's codes + code_off[j] are 16-byte aligned); otherwise by the table-driven
- * kernels.  The results do not depend on which kernel ran.
+ * Performance note: a segment of at most 16384 elements is read once, and so are all of a call none of whose segments has
+ * more than 65536 (bf16: and at most 16 M elements in all); longer ones are read twice.  They are encoded by the bulk-copy
+ * kernels when elem_offset is a multiple of 8 and seg_off[0] one of 64 (or grad + seg_off[j] is 16-byte aligned and
+ * elem_offset + seg_off[j] a multiple of 8).  mqg_server_step_segments' bulk-copy kernel applies those of 2^15 elements and
+ * more, wherever they start from 2^19 (more than four workers: 2^20) elements in all on.  The results do not depend on
+ * which kernel ran.
  */
 mqg_status mqg_quantize_segments(const void* grad, int nseg, const uint64_t* seg_off,
                                  const uint64_t* code_off, int bits, uint64_t seed,
