@@ -99,7 +99,7 @@ constexpr int kBf16Wide = 2;                 // as DTYPE of the tile, the shared
 // row of the warp's beside the stages.  (Into the stage by its owner after the wait is one round trip more: 131,073 elements
 // 2.09 against 2.28 us, eight workers 2.86 against 3.15, the range 1.95 against 2.14.)  `row` is the gradient's, of row_bytes
 // bytes.
-__device__ __forceinline__ void fetch_ragged_row(uint32_t to, const uint8_t* grad, uint64_t row, uint64_t total_bytes,
+static __device__ __noinline__ void fetch_ragged_row(uint32_t to, const uint8_t* grad, uint64_t row, uint64_t total_bytes,
                                                  uint32_t row_bytes)
 {
     const uint32_t b = 4u * (threadIdx.x & 31u);
@@ -108,13 +108,6 @@ __device__ __forceinline__ void fetch_ragged_row(uint32_t to, const uint8_t* gra
     const uint32_t left = at < total_bytes ? (uint32_t)min(total_bytes - at, (uint64_t)4) : 0u;
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
                  ::"r"(to + b), "l"(grad + (left != 0 ? at : 0)), "r"(left) : "memory");
-}
-
-// For rows of 64, whose launches are long: in a function of its own, so that the code of the tiles without such a row stays
-// as it is (inlined, those took 2 % longer).
-static __device__ __noinline__ void fetch_ragged_wide_row(uint32_t to, const uint8_t* grad, uint64_t row, uint64_t total_bytes)
-{
-    fetch_ragged_row(to, grad, row, total_bytes, 128);
 }
 
 // The warp moves that row into row `row` of the tile's stage, once the tile's copy, which fills it with zeros, has landed; its
@@ -132,17 +125,20 @@ static __device__ __noinline__ void put_ragged_row(uint8_t* stage, uint32_t row,
     __syncwarp();
 }
 
-// The same in one step, by its owner, for 128-byte rows whose launches are long (mqg_segments_workers.cu).
+// The same in one step, by its owner, for 128-byte rows whose launches are long (rows of 64, and mqg_segments_workers.cu):
+// there the other tiles' code decides, which the forms above lengthened (50 M bf16 elements 28.7 against 28.0 us).
 static __device__ __noinline__ void stage_ragged_row(uint8_t* stage, uint32_t row, const uint8_t* grad, uint64_t from,
                                                      uint64_t total_bytes)
 {
-    for (uint32_t w = 0; w < 32; ++w) {
-        const uint64_t at = from * 128 + 4 * w;
-        uint32_t v = 0u;
-        if (at + 4 <= total_bytes) v = *reinterpret_cast<const uint32_t*>(grad + at);
-        else if (at + 2 <= total_bytes) v = *reinterpret_cast<const uint16_t*>(grad + at);
-        reinterpret_cast<uint32_t*>(stage)[(row * 8 + ((w >> 2) ^ (row & 7u))) * 4 + (w & 3u)] = v;
-    }
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(grad + from * 128);
+    const uint32_t left = (uint32_t)(total_bytes - from * 128);              // fewer than 128
+    uint32_t v[32];                  // all in flight at once
+#pragma unroll
+    for (uint32_t w = 0; w < 32; ++w) v[w] = 4 * w + 4 <= left ? __ldcg(src + w) : 0u;
+    const uint32_t half = left % 4 >= 2 ? *reinterpret_cast<const uint16_t*>(src + left / 4) : 0u;
+#pragma unroll
+    for (uint32_t w = 0; w < 32; ++w)
+        reinterpret_cast<uint32_t*>(stage)[(row * 8 + ((w >> 2) ^ (row & 7u))) * 4 + (w & 3u)] = w == left / 4 ? half : v[w];
     fence_proxy_async();             // orders these stores before the bulk copy that refills the stage
 }
 
@@ -482,25 +478,21 @@ __device__ __forceinline__ bool quantize_wide_tile(TmaQuantizeShared<kBf16Wide, 
     const uint32_t t = threadIdx.x;
     const uint32_t row = tile * a.tile_rows + t;
     const bool active = FULL || (t < a.tile_rows && row < (uint32_t)a.nrows);
-    const bool tail = !FULL && tile == c.ragged_tile;            // a tile with a row that the copy does not cover
     const uint32_t stg = k % kQuantStages, parity = (k / kQuantStages) & 1;
     const uint32_t bar = smem_u32(&sh.bar[stg]);
     uint8_t* stage = sh.stage[stg];
 
-    if (tail && warp_has_row(a.nrows_full, row - (t & 31u)))
-        fetch_ragged_wide_row(smem_u32(sh.ragged[t >> 5]), static_cast<const uint8_t*>(wv.grad), a.nrows_full, a.n * 2);
     bool ok = mbar_try_wait(bar, parity);
     if (!ok) ok = mbar_wait(bar, parity, a.poll_limit);
-    if (tail) { cp_async_wait_all(); __syncwarp(); }
 
     uint32_t raw[2][16];
     if (active) {
-        // the ragged row is read where it is, as row 0 of a stage of its own (put into its stage first: 110 against 108 us)
-        const bool apart = tail && row >= (uint32_t)a.nrows_full;
-        const uint4* s = reinterpret_cast<const uint4*>(apart ? sh.ragged[t >> 5] : stage);
+        if (!FULL && row >= (uint32_t)a.nrows_full)      // a row that the copy does not cover
+            stage_ragged_row(stage, t, static_cast<const uint8_t*>(wv.grad), row, a.n * 2);
+        const uint4* s = reinterpret_cast<const uint4*>(stage);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const uint4 v = s[swz(apart ? 0 : (int)t, i)];
+            const uint4 v = s[swz((int)t, i)];
             uint32_t* to = &raw[i >> 2][(i & 3) * 4];
             to[0] = v.x; to[1] = v.y; to[2] = v.z; to[3] = v.w;
         }
