@@ -249,7 +249,7 @@ mqg_status mqg_quantize_workers(const void* const* grads, int W, uint64_t n, int
         if (!aligned4(scales[w])) return fail(MQG_ERR_ALIGN, "worker %d: scales not 4-byte aligned", w);
     }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    if (mqg::quantize_workers_applies(W, n, bucket, elem_offset)) {
+    if (mqg::quantize_workers_applies(W, n, bucket, elem_offset, 0)) {
         const cudaError_t err = mqg::launch_quantize_workers(grads, W, n, bits, bucket, seed, codes, scales,
                                                              (int)dtype, first_worker, step, elem_offset,
                                                              0, stream);
@@ -311,7 +311,7 @@ mqg_status mqg_quantize_workers_minmax(const void* const* grads, int W, uint64_t
         if (!aligned8(ranges[w])) return fail(MQG_ERR_ALIGN, "worker %d: ranges not 8-byte aligned", w);
     }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    if (mqg::quantize_workers_applies(W, n, bucket, 0)) {
+    if (mqg::quantize_workers_applies(W, n, bucket, 0, 1)) {
         const cudaError_t err = mqg::launch_quantize_workers(grads, W, n, bits, bucket, 0, codes, ranges,
                                                              (int)dtype, 0, 0, 0, 1, stream);
         if (err != cudaSuccess) return cuda_fail("mqg_quantize_workers_minmax", err);
@@ -536,7 +536,7 @@ mqg_status mqg_quantize_workers_l2(const void* const* grads, int W, uint64_t n, 
         if (!aligned4(scales[w])) return fail(MQG_ERR_ALIGN, "worker %d: scales not 4-byte aligned", w);
     }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    if (mqg::quantize_workers_applies(W, n, bucket, elem_offset)) {
+    if (mqg::quantize_workers_applies(W, n, bucket, elem_offset, 2)) {
         const cudaError_t err = mqg::launch_quantize_workers(grads, W, n, bits, bucket, seed, codes, scales,
                                                              (int)dtype, first_worker, step, elem_offset,
                                                              2, stream);

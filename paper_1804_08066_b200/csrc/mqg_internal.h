@@ -42,7 +42,7 @@ cudaError_t launch_quantize_fused(const void* grad, uint64_t n, int bits, uint64
 // worker w draws as worker id first_worker + w.  Only when quantize_workers_applies() holds.
 // mode: 0 = the main codec, 1 = the (min, max) variant (`scales[w]` then points at worker w's ranges, two floats
 // per bucket; seed, first_worker, step and elem_offset are not used), 2 = the L2-norm scale variant.
-bool quantize_workers_applies(int W, uint64_t n, uint64_t bucket, uint64_t elem_offset);
+bool quantize_workers_applies(int W, uint64_t n, uint64_t bucket, uint64_t elem_offset, int mode);
 cudaError_t launch_quantize_workers(const void* const* grads, int W, uint64_t n, int bits,
                                     uint64_t bucket, uint64_t seed, uint32_t* const* codes,
                                     float* const* scales, int dtype, uint32_t first_worker,

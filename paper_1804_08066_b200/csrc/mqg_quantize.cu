@@ -384,7 +384,7 @@ cudaError_t launch_quantize_range_fused(const void* grad, uint64_t n, int bits, 
 // ---- L2-norm scale variant on the TMA kernel (block-aligned draws) ----
 bool quantize_norm_fused_applies(uint64_t n, uint64_t bucket, uint64_t elem_offset)
 {
-    if (n == 0) return false;
+    if (n == 0 || (bucket < n ? bucket : n) > (uint64_t)kMaxFusedBucket) return false;
     return tma_path_applies(n, bucket >= n ? (n + 31) / 32 : bucket / 32, elem_offset);
 }
 

@@ -164,12 +164,12 @@ static cudaError_t launch_workers_bits(const WorkerTable& tab, const QuantizeArg
 #undef MQG_WORKERS_MODE
 }
 
-bool quantize_workers_applies(int W, uint64_t n, uint64_t bucket, uint64_t elem_offset)
+bool quantize_workers_applies(int W, uint64_t n, uint64_t bucket, uint64_t elem_offset, int mode)
 {
     if (W < 2 || W > kMaxWorkers || n == 0) return false;
     const uint64_t nrows = (n + 31) / 32;
     const uint64_t rpb = (bucket >= n) ? nrows : bucket / 32;
-    if ((bucket < n ? bucket : n) > (uint64_t)kMaxTmaBucket) return false;
+    if ((bucket < n ? bucket : n) > (uint64_t)(mode == kNorm ? kMaxFusedBucket : kMaxTmaBucket)) return false;
     if (!tma_path_applies(n, rpb, elem_offset)) return false;
     const uint64_t tile_rows = rpb <= 128 ? (128 / rpb) * rpb : rpb;
     const uint64_t nt = (nrows + tile_rows - 1) / tile_rows;
