@@ -40,12 +40,18 @@ struct SpanTable {
 cudaError_t launch_spans(const TableArgs& a, const SpanTable& tab, unsigned nspan, uint64_t most, int mode, int bits,
                          int dtype, cudaStream_t stream);
 
-// Spans of a list (no clears) of up to kMaxJoinedElems elements, kSpanMaxAbs or kSpanNorm: those of more than
-// kJoinedChunk are a cluster's each.
+// Spans of a list (no clears) of up to kMaxJoinedElems elements, kSpanMaxAbs or kSpanNorm: those of more than `alone`
+// elements (kJoinedChunk .. 16384) are several CTAs' of a cluster, one for every kJoinedChunk elements.
 constexpr unsigned kMaxCluster = 8;                                  // CTAs, the portable limit
 constexpr uint64_t kJoinedChunk = (uint64_t)kMaxTileRows * 32;       // elements per CTA, a power of two of rows
 constexpr uint64_t kMaxJoinedElems = kMaxCluster * kJoinedChunk;
-cudaError_t launch_joined_spans(const TableArgs& a, const SpanTable& tab, uint64_t most, int mode, int bits, int dtype,
+constexpr uint32_t kNoPart = 0xFFFF;
+struct JoinedTable {
+    SpanTable spans;
+    uint16_t cta[kMaxCluster * kMaxSegmentsPerLaunch];       // span of a CTA + 256 times its part; kNoPart: fills a cluster up
+    uint8_t parts[kMaxSegmentsPerLaunch];                    // CTAs of a span
+};
+cudaError_t launch_joined_spans(const TableArgs& a, const SpanTable& tab, uint64_t alone, int mode, int bits, int dtype,
                                 cudaStream_t stream);
 
 // The same in the main codec together with the max pass over `longs`, whose scales launch_clear_scales has cleared.

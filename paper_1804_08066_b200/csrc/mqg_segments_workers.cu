@@ -481,6 +481,25 @@ bool flat_applies(const void* const* grads, int W, uint64_t begin, uint64_t end,
     return begin % 64 == 0 && elem_offset % 8 == 0 && first >> 32 == last >> 32 && (end + 31) / 32 <= 0x7FFFFFFFull;
 }
 
+// Whether a call's segments, none longer than a cluster's, are quantized by launch_joined_spans and not by a launch that clears
+// the scales, the max pass with the short segments beside it, and the encode; per worker: elements, those in segments of several
+// CTAs and those in segments of more than five.
+bool joined_spans_pay(int W, uint64_t elements, uint64_t in_joined, uint64_t in_long_joined, int dtype)
+{
+    const uint64_t all = elements * (uint64_t)W;
+    // A long launch with next to nothing that joins gains nothing from it and loses where clusters do not fill the SMs: 63 tensors of
+    // 9,000 and one of 60,000, 32 workers, 30.6 against 28.9 us (8 workers 10.5 / 13.9).
+    if (all > (16u << 20) && 8 * in_joined < elements) return false;
+    // bf16, whose two passes read half as much: short launches, and those of segments of up to five CTAs.  Against the three
+    // launches, us: 8 of 65,000, 4 / 8 / 32 workers 5.7 / 10.6 / 29.7 against 7.2 / 8.4 / 24.0; 20 of 41,000, 4 / 8 / 32
+    // workers 9.7 / 15.0 / 50.1 against 9.8 / 14.7 / 47.6; 20 of 33,000, 4 / 8 / 32 workers 6.3 / 11.2 / 39.1 against 9.6 / 14.2 /
+    // 44.9; 63 of 17,000 and one of 60,000, 8 workers 23.9 against 30.7.
+    // fp32: 40 of 60,000, 1 / 8 / 32 workers 6.0 / 33.3 / 132 against 8.5 / 41.4 / 181; 20 of 33,000, 1 / 8 / 32 workers 4.0 / 10.5 /
+    // 38.3 against 5.6 / 13.8 / 47.4.  (Parts of 512 and 1024 rows, for tensors of up to 262,144 elements, one worker: 4.9 and 6.8
+    // against 5.1 for 100,000 and 200,000.)
+    return dtype == 0 || all <= (3u << 20) || 3 * in_long_joined <= elements;
+}
+
 }  // namespace
 
 cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, const uint64_t* seg_off,
@@ -498,35 +517,36 @@ cudaError_t launch_quantize_segments(const void* const* grads, int W, int nseg, 
         return true;
     };
     uint64_t long_tiles = 0, longest = 0;             // tiles of 256 rows
+    uint64_t in_joined = 0, in_long_joined = 0;       // elements of the segments of several CTAs, of more than five
     bool any_span = false, aligned = true;            // aligned: the long segments, as the gradients are
     for (int j = 0; j < nseg; ++j) {
         const uint64_t len = seg_off[j + 1] - seg_off[j];
         if (len > longest) longest = len;
         if (len <= kSegmentSpanElems) { any_span = true; continue; }
+        in_joined += len;
+        if (len > 5 * kJoinedChunk) in_long_joined += len;
         long_tiles += (len + kMaxTileRows * 32 - 1) / (kMaxTileRows * 32);
         aligned = aligned && (seg_off[j] * esz) % 16 == 0;
     }
-    // Nothing longer than a cluster's: one launch for every 64 segments instead of three launches.  One CTA per 8192 elements
-    // and one row per thread: fp32, four bits, one tensor of 20,000 / 60,000 elements 3.6 / 3.8 against 5.0 us (with the norm 3.7
-    // against 7.5), 40 tensors of 60,000 and 100, 1 / 8 / 32 workers 5.4 / 20.7 / 80 against 9.2 / 24.2 / 90 us.  In bf16, whose
-    // two passes read half as much, up to 16 M elements: those 40 and 8 / 12 / 32 workers 23 / 33 / 90 against 27 / 33 / 78 us.
-    // (Parts of 512 and 1024 rows, for tensors of up to 262,144 elements: 4.9 and 6.8 against 5.1 us for 100,000 and
-    // 200,000, and 89 against 66 us for twenty of 200,000 and 8 workers.)
-    const uint64_t elements = (uint64_t)W * (seg_off[nseg] - seg_off[0]);
-    if (longest > kSegmentSpanElems && longest <= kMaxJoinedElems && (dtype == 0 || elements <= (16u << 20))) {
+    // Nothing longer than a cluster's: one launch for every 64 segments instead of three launches, where that pays.
+    if (longest > kSegmentSpanElems && longest <= kMaxJoinedElems &&
+        (workspace || joined_spans_pay(W, seg_off[nseg] - seg_off[0], in_joined, in_long_joined, dtype))) {
         for (int first = 0; first < nseg; first += kMaxSegmentsPerLaunch) {
             SpanTable spans;
             memset(&spans, 0, sizeof(spans));
             spans.first = first;
-            uint64_t most = 0;
+            uint64_t parts = 0;
             for (int j = first; j < nseg && j < first + kMaxSegmentsPerLaunch; ++j) {
                 const int k = spans.nspan++;
                 spans.elem0[k] = seg_off[j]; spans.len[k] = seg_off[j + 1] - seg_off[j]; spans.code0[k] = code_off[j];
                 spans.scale_idx[k] = (uint32_t)j;
-                if (spans.len[k] > most) most = spans.len[k];
+                parts += (spans.len[k] + kJoinedChunk - 1) / kJoinedChunk;
             }
-            const cudaError_t err = launch_joined_spans(a, spans, most, workspace ? kSpanNorm : kSpanMaxAbs, bits, dtype,
-                                                        stream);
+            // A CTA of two rows per thread for those it holds (20 tensors of 12,000 and one of 20,000, 16 workers 6.6 against 9.7
+            // us), unless the launch has at most two CTAs of one row per thread per SM (8,192 to 16,384 elements, 40 of 16,000, one
+            // worker 3.9 against 4.3 us; 32 of 9,000 and 32 of 33,000 5.0 against 6.0).
+            const cudaError_t err = launch_joined_spans(a, spans, parts * (uint64_t)W <= 2 * 148 ? kJoinedChunk : kSegmentSpanElems,
+                                                        workspace ? kSpanNorm : kSpanMaxAbs, bits, dtype, stream);
             if (err != cudaSuccess) return err;
         }
         return cudaSuccess;

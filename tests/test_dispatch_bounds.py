@@ -1,6 +1,7 @@
-"""Which shapes the one-pass quantizers take, asked of the library's own predicates (no GPU): the L2-norm kernels have tiles of
-at most 256 rows, the others of 512."""
+"""What the library's host code decides before it launches, asked of its own functions (no GPU): the shapes that the one-pass
+quantizers take (the L2-norm kernels have tiles of at most 256 rows, the others of 512), and the CTAs of a table's tensors."""
 import ctypes as C
+import random
 
 import pytest
 
@@ -35,3 +36,42 @@ def test_bucket_bounds(n, bucket, norm, others):
     assert _one("quantize_range_fused_applies", n, bucket) == others
     assert _workers(n, bucket, 0) == _workers(n, bucket, 1) == others
     assert not _workers(n, bucket, 0, offset=3) and not _one("quantize_norm_fused_applies", n, bucket, 3)
+
+
+class _Spans(C.Structure):
+    _fields_ = [("bucket", C.c_uint64), ("n", C.c_uint64), ("nspan", C.c_int), ("first", C.c_int), ("clear", C.c_uint32 * 2),
+                ("scale_idx", C.c_uint32 * 64), ("elem0", C.c_uint64 * 64), ("len", C.c_uint64 * 64), ("code0", C.c_uint64 * 64)]
+
+
+class _Joined(C.Structure):
+    _fields_ = [("spans", _Spans), ("cta", C.c_uint16 * 512), ("parts", C.c_uint8 * 64)]
+
+
+def _random_sizes(seed):
+    rng = random.Random(seed)
+    return [rng.choice((0, 1, 8192, 8193, 16384, 16385, 65536, rng.randrange(65537))) for _ in range(rng.randint(1, 64))]
+
+
+@pytest.mark.parametrize("alone", [8192, 16384])
+@pytest.mark.parametrize("sizes", [[9000] * 63 + [60000], [17000] * 63 + [60000], [9000] * 32 + [33000] * 32, [20000], [65536] * 64,
+                                   [100, 40000, 0], *map(_random_sizes, range(20))])
+def test_ctas_of_joined_tensors(sizes, alone):
+    """Every tensor once, in CTAs of one cluster, none of them shared, and no more CTAs than the parts and what fills clusters up."""
+    spans, tab, cluster = _Spans(nspan=len(sizes)), _Joined(), C.c_uint()
+    for j, n in enumerate(sizes):
+        spans.len[j] = n
+    place = C.CDLL(mqg.LIB_PATH)["_ZN3mqg18place_joined_spansERKNS_9SpanTableEmRNS_11JoinedTableERj"]
+    place.restype, place.argtypes = C.c_uint, [C.c_void_p, C.c_uint64, C.c_void_p, C.c_void_p]
+    ctas = place(C.byref(spans), alone, C.byref(tab), C.byref(cluster))
+    need = [1 if n <= alone else -(-n // 8192) for n in sizes]
+    size = cluster.value
+    assert size == max(need) and ctas % size == 0 and list(tab.parts[:len(sizes)]) == need
+    seen = []
+    for first in range(0, ctas, size):
+        placed = [divmod(c, 256)[::-1] for c in tab.cta[first:first + size] if c != 0xFFFF]
+        seen += placed
+        spans_here = [j for j, part in placed if part == 0]
+        assert placed == [(j, part) for j in spans_here for part in range(need[j])]       # whole tensors, parts in order
+        assert len({need[j] == 1 for j in spans_here}) == 1                               # none that waits for a lone one
+    assert sorted(seen) == [(j, part) for j in range(len(sizes)) for part in range(need[j])]
+    assert ctas <= 2 * sum(need) + 2 * size                                               # half of every cluster but the last

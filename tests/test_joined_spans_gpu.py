@@ -20,6 +20,8 @@ SIZES = {
     "the_longest": [262_144, 7, 262_143, 196_609],
     "one_more": [262_145, 100, 30_000],
     "two_tables": [20_000, 96] * 40,
+    "shared_clusters": [20_000, 17_000, 60_000, 9_000, 12_000, 33_000, 41_000, 0, 5, 8193],
+    "two_rows_per_thread": [9_000, 16_384, 8193, 100] * 12 + [20_000, 60_001, 33_000] * 5,
 }
 
 
