@@ -631,34 +631,24 @@ mqg_status mqg_server_step_segments(const uint32_t* const* codes, const float* c
     }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     // A long segment is a gradient with a single bucket: the long segments go to the TMA-fed server kernel together, in one
-    // launch (its form for segments that start anywhere, if one of them is off a 16-byte boundary); all other segments share
-    // the table-driven launch.  The results are the same bit for bit either way.
+    // launch, those off a 16-byte boundary in another of its form for segments that start anywhere (flat_server_form); all other
+    // segments share the table-driven launch.  The results are the same bit for bit either way.
     constexpr uint64_t kOwnLaunchElems = mqg::kEntrySegmentElems;
     auto is_long = [&](int j) {
         const uint64_t len = seg_off[j + 1] - seg_off[j];
         return !acc_out && len >= kOwnLaunchElems && mqg::server_tma_applies(len, len);
     };
-    auto aligned = [&](int j) {
-        bool all = aligned16(params + seg_off[j]);
-        for (int w = 0; w < W && all; ++w) all = aligned16(codes[w] + code_off[j]);
-        return all;
-    };
+    bool alike = true;                   // the workers' buffers start at the same place between two 16-byte boundaries
+    for (int w = 1; w < W; ++w) alike = alike && ((reinterpret_cast<uintptr_t>(codes[w]) ^ reinterpret_cast<uintptr_t>(codes[0])) & 15u) == 0;
+    auto aligned = [&](int j) { return alike && aligned16(params + seg_off[j]) && aligned16(codes[0] + code_off[j]); };
     if (mqg_status st = check_segments(nseg, seg_off, code_off, bits)) return st;
-    // That form takes over from the table-driven launch at half a million elements (more than four workers: a million): one
-    // tensor off the boundary, table / that form, one worker 3.4 / 3.9, 4.7 / 4.0, 9.9 / 4.9 us for 0.2, 0.4 and 1.6 M
-    // elements, eight 3.8 / 5.2, 6.4 / 6.6, 10.5 / 7.6 us for 0.2, 0.8 and 1.6 M, sixteen 8.2 / 9.6, 12.9 / 11.2 us for 0.8 and
-    // 1.6 M; 50 M elements and eight workers 631 / 110 us.
-    uint64_t longs_total = 0;
-    bool any_long = false, any_off = false;
-    for (int j = 0; j < nseg; ++j) {
-        if (!is_long(j)) continue;
-        longs_total += seg_off[j + 1] - seg_off[j];
-        if (aligned(j)) any_long = true;
-        else any_off = true;
-    }
-    const bool flat = any_off && longs_total >= (W <= 4 ? 1ull << 19 : 1ull << 20);
-    any_long = any_long || flat;
-    auto own = [&](int j) { return is_long(j) && (flat || aligned(j)); };
+    uint64_t on = 0, off = 0;            // elements of the long segments on and off the boundaries
+    for (int j = 0; j < nseg; ++j)
+        if (is_long(j)) (aligned(j) ? on : off) += seg_off[j + 1] - seg_off[j];
+    const int flat = mqg::flat_server_form(on, off, W, bits);
+    const bool any_long = on != 0 || flat != 0;
+    enum { kTable, kBulk, kFlat };
+    auto form = [&](int j) { return !is_long(j) ? kTable : aligned(j) ? (flat == 2 ? kFlat : kBulk) : flat != 0 ? kFlat : kTable; };
     // The other segments: table-driven launches - except that ONE table of short segments rides along
     // with the (first) launch of the long ones, so that a typical layered step is a single launch.
     mqg::SegmentTable folded;
@@ -673,20 +663,24 @@ mqg_status mqg_server_step_segments(const uint32_t* const* codes, const float* c
             }
             const cudaError_t err = mqg::launch_server_segments(ptrs, W, bits, tab, first, params, lr, acc_out, stream);
             return err == cudaSuccess ? MQG_OK : cuda_fail("mqg_server_step_segments", err);
-        }, own);
+        }, [&](int j) { return form(j) != kTable; });
     if (st != MQG_OK) return st;
     // The long ones, a launch for every kMaxServerSegsPerLaunch of them.  No heap here: the C ABI throws nothing.
     mqg::ServerSegHost longs[mqg::kMaxServerSegsPerLaunch];
-    int count = 0;
-    for (int j = 0; j <= nseg && any_long; ++j) {
-        if (j < nseg && own(j))
-            longs[count++] = {seg_off[j + 1] - seg_off[j], seg_off[j], code_off[j], (uint32_t)j};
-        if (count == 0 || (count < mqg::kMaxServerSegsPerLaunch && j < nseg)) continue;
-        const cudaError_t err = mqg::launch_server_tma_segments(ptrs, W, bits, longs, count, folded_first >= 0 ? &folded : nullptr,
-                                                                folded_first, params, lr, flat, stream);
-        if (err != cudaSuccess) return cuda_fail("mqg_server_step_segments", err);
-        folded_first = -1;
-        count = 0;
+    for (const auto which : {kBulk, kFlat}) {
+        if (which == kBulk ? on == 0 || flat == 2 : flat == 0) continue;
+        int count = 0;
+        for (int j = 0; j <= nseg; ++j) {
+            if (j < nseg && form(j) == which)
+                longs[count++] = {seg_off[j + 1] - seg_off[j], seg_off[j], code_off[j], (uint32_t)j};
+            if (count == 0 || (count < mqg::kMaxServerSegsPerLaunch && j < nseg)) continue;
+            const cudaError_t err = mqg::launch_server_tma_segments(ptrs, W, bits, longs, count,
+                                                                    folded_first >= 0 ? &folded : nullptr, folded_first, params,
+                                                                    lr, which == kFlat, stream);
+            if (err != cudaSuccess) return cuda_fail("mqg_server_step_segments", err);
+            folded_first = -1;
+            count = 0;
+        }
     }
     return MQG_OK;
 }

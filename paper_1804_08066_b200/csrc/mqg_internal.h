@@ -134,6 +134,9 @@ struct ServerSegHost {
     uint32_t scale_idx;      // index of its scale in every worker's scale array
 };
 constexpr int kMaxServerSegsPerLaunch = 16;
+// Which long segments of a call with `on` elements on and `off` elements off 16-byte boundaries take the `flat` form: 0 = none
+// (those off the boundaries go to the table-driven launch), 1 = those off the boundaries, 2 = all.
+int flat_server_form(uint64_t on, uint64_t off, int W, int bits);
 // short_tab (may be null): the table of the step's other segments, updated by the same launch with plain
 // loads; short_first = index of the table's first segment in the scale arrays.
 cudaError_t launch_server_tma_segments(const WorkerPtrs& ptrs, int W, int bits, const ServerSegHost* segs, int nseg,

@@ -1280,6 +1280,21 @@ static cudaError_t launch_server_segs_inst(const ServerSegTable& tab, const Serv
     return launch_pdl_smem(kernel, (unsigned)grid, kSrvThreads, kSmemBytes, stream, tab, ss, a, timeouts);
 }
 
+int flat_server_form(uint64_t on, uint64_t off, int W, int bits)
+{
+    // The table-driven launch is for short calls: one tensor, that launch / this form, one worker 3.4 / 3.9, 4.7 / 4.0, 9.9 / 4.9
+    // us for 0.2, 0.4 and 1.6 M elements, eight 3.8 / 5.2, 6.4 / 6.6, 10.5 / 7.6 us for 0.2, 0.8 and 1.6 M, sixteen 8.2 / 9.6,
+    // 12.9 / 11.2 us for 0.8 and 1.6 M; 50 M elements and eight workers 631 / 110 us.  (A table of a few long tensors that rides
+    // along with the launch of the others is a tail of 6 us: 16 M elements, 40,000 of them off the boundaries, one worker 24.4
+    // against 18.5 us.)
+    if (off == 0 || on + off < (W <= 4 ? 1ull << 19 : 1ull << 20)) return 0;
+    // Those on the boundaries go along, which saves 2 to 4 us for a second launch, unless their codes are many: the flat form
+    // copies them four bytes at a time.  Apart / together, 1.5 M elements off the boundaries: eight workers, four bits, 1, 8
+    // and 16 M on them 11.0 / 9.3, 21.5 / 21.1, 40.3 / 42.8 us, eight bits and 8 M 29.9 / 31.6, sixteen workers, four bits, 16 M
+    // 58.3 / 67.3 us.  Up to four workers the parameters are most of the bytes: four bits, four workers, 40 M 70.8 / 69.9 us.
+    return W >= 8 && on * (uint64_t)(W * bits) >= 512ull << 20 ? 1 : 2;
+}
+
 cudaError_t launch_server_tma_segments(const WorkerPtrs& ptrs, int W, int bits, const ServerSegHost* segs, int nseg,
                                        const SegmentTable* short_tab, int short_first, float* params, float lr,
                                        bool flat, cudaStream_t stream)

@@ -75,3 +75,15 @@ def test_ctas_of_joined_tensors(sizes, alone):
         assert len({need[j] == 1 for j in spans_here}) == 1                               # none that waits for a lone one
     assert sorted(seen) == [(j, part) for j in range(len(sizes)) for part in range(need[j])]
     assert ctas <= 2 * sum(need) + 2 * size                                               # half of every cluster but the last
+
+
+@pytest.mark.parametrize("on,off,W,bits,form", [
+    (50_000_000, 40_000, 8, 4, 1), (50_000_000, 40_000, 8, 8, 1), (16_777_216, 40_000, 16, 4, 1),
+    (8_388_608, 40_000, 8, 4, 2), (8_388_607, 2_000_000, 8, 8, 2), (100_000_000, 40_000, 4, 8, 2), (0, 50_000_000, 8, 8, 2),
+    (50_000_000, 0, 8, 8, 0), (0, 0, 1, 1, 0), (400_000, 600_000, 8, 8, 0), (400_000, 700_000, 8, 8, 2), (0, 524_288, 4, 2, 2),
+    (0, 524_287, 4, 2, 0)])
+def test_tensors_off_the_boundaries(on, off, W, bits, form):
+    """A few elements off the 16-byte boundaries do not take many away from the kernel for those on them."""
+    f = C.CDLL(mqg.LIB_PATH)["_ZN3mqg16flat_server_formEmmii"]
+    f.argtypes = [C.c_uint64, C.c_uint64, C.c_int, C.c_int]
+    assert f(on, off, W, bits) == form

@@ -57,3 +57,9 @@ def test_more_tensors_than_a_launch_holds():
 
 def test_many_tiles_per_warp():
     _run([3_000_001, 5_000_003], 4, 8)
+
+
+def test_only_those_off_the_boundaries():
+    """So many codes on the 16-byte boundaries that they keep their own launch, and the short tensors ride along with it."""
+    _run([8_388_608, 6, 40_002, 33_000, 500, 1_000_005, 9], 8, 8)
+    _run([300, 33_000, 8_388_600 + 32_768] + [32_769] * 17, 8, 8)
