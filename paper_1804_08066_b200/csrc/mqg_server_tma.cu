@@ -1189,21 +1189,28 @@ static int requantize_warps(uint64_t rpb)
 
 // At least 512 complete rows, fewer than 2^30 (so the draws' block numbers have no high half), buckets as above, those
 // below 32 rows few enough per tile for the warp's table; and where it is the faster one.  Against a CTA per tile
-// (mqg_requantize.cu) a warp's copies and constants are ahead of their use, which short launches gain from - at two bits 2.7 /
-// 4.3 against 2.9 / 7.5 us for 130,001 elements and 1 / 16 workers, 5.5 against 7.1 us for a million and 16 - and long ones
-// when there is much to sum: 25 M elements, bucket 2048, four bits, 8 / 16 workers 44 / 68 against 52 / 86 us, eight bits, 4
-// workers 35 against 39 us, two bits, 16 workers 69 against 72 us.  Otherwise the other's smaller CTAs with fewer
-// registers win: one bit, 4 / 16 workers 28 / 54 against 32 / 62 us, two bits, 4 / 8 workers 32 / 43.4 against 35 / 44.1 us,
-// eight bits, 2 workers 28 against 30 us; no difference at four bits.  Three warps: bucket 768, four bits, 4 / 8 workers 40 / 50
-// against 36 / 55 us, eight bits, 4 / 8 42 / 56 against 40 / 63 us.
+// (mqg_requantize.cu) a warp's copies and constants are ahead of their use, which short launches gain from - bucket 1024, two
+// bits, 1 / 8 / 16 workers 0.88 / 0.83 / 0.77 of the other's time at 1.5 M elements - and long ones when there is much to sum:
+// 25 M elements, bucket 2048, four bits, 8 / 16 workers 44 / 68 against 52 / 86 us, eight bits, 4 workers 35 against 39 us.
+// Otherwise the other's smaller CTAs with fewer registers win: 25 M elements, one bit, 4 / 16 workers 28 / 54 against 32 / 62 us,
+// two bits, 4 workers 32 against 35 us; 1 M elements, six bits, one worker 0.93.  Three warps, whose CTAs are smaller still: 24 and 48
+// rows, 0.7 M elements, four bits, 1 / 8 / 16 workers 1.02 / 0.88 / 0.84, 4 M 1.06 / 0.90 / 0.86; 96 rows 0.94 to 0.64 at 1 M.  Eight
+// warps: a bucket to a CTA, two CTAs to an SM, so that a launch of 2.2 to 2.8 rounds of 296 waits for its third: 6 M elements,
+// four bits, 4 / 8 workers 1.19 / 1.06, at 4 and 7 M and 8 workers 0.89 and 0.93.
 bool requantize_warp_applies(uint64_t n, uint64_t bucket, int W, int bits)
 {
     if (n / 32 < 512 || n / 32 >= (1ull << 30) - 1 || bucket >= n || bucket % 32 != 0) return false;
     const uint64_t rpb = bucket / 32;
     const int warps = requantize_warps(rpb);
     if (warps == 0 || (rpb < 24 && (uint64_t)W * (32 / rpb) > 2 * (uint64_t)kMaxWorkers)) return false;
-    if (n < (1u << 20)) return true;
-    return warps == 3 ? W >= 8 && W * bits >= 32 : bits == 4 || (bits >= 2 && W * bits >= 24);
+    const bool several = W >= 8 && bits >= 2, six = bits == 6 && W <= 2;
+    const bool much = several && W * bits >= 32 && (bits != 6 || W >= 16) && (bits >= 3 || n < 5ull << 19);
+    if (rpb == 24 || rpb == 48) return n < 1ull << 20 ? several : much;
+    if (n < 1ull << 20) return warps != 8 || !six;
+    if (n < 3ull << 19) return !six;
+    if (warps == 3) return much;
+    if (warps == 8) return several && W * bits >= 24 && (n < 660 * 8192 || n >= 840 * 8192);
+    return bits == 4 || (bits >= 2 && W * bits >= 24) || (several && n < 16ull << 20);
 }
 
 cudaError_t launch_requantize_warp(const WorkerPtrs& ptrs, int W, int bits, uint64_t n, uint64_t bucket,

@@ -87,3 +87,15 @@ def test_tensors_off_the_boundaries(on, off, W, bits, form):
     f = C.CDLL(mqg.LIB_PATH)["_ZN3mqg16flat_server_formEmmii"]
     f.argtypes = [C.c_uint64, C.c_uint64, C.c_int, C.c_int]
     assert f(on, off, W, bits) == form
+
+
+@pytest.mark.parametrize("n,bucket,W,bits,warps", [
+    (1_100_000, 2048, 8, 2, True), (1_500_000, 1024, 1, 3, True), (1_100_000, 1024, 1, 6, False), (1_600_000, 1024, 1, 3, False),
+    (25_000_000, 2048, 8, 4, True), (25_000_000, 2048, 4, 2, False), (9_000_000, 2048, 8, 2, True), (25_000_000, 2048, 8, 2, False),
+    (6_000_000, 8192, 4, 4, False), (6_000_000, 8192, 16, 4, False), (4_000_000, 8192, 8, 4, True), (8_000_000, 8192, 8, 4, True),
+    (8_000_000, 8192, 4, 8, False), (700_000, 768, 1, 4, False), (700_000, 768, 8, 4, True), (700_000, 3072, 1, 4, True),
+    (4_000_000, 1536, 8, 4, True), (4_000_000, 1536, 8, 3, False), (25_000_000, 1056, 8, 4, False)])
+def test_kernel_of_the_requantization(n, bucket, W, bits, warps):
+    f = C.CDLL(mqg.LIB_PATH)["_ZN3mqg23requantize_warp_appliesEmmii"]
+    f.restype, f.argtypes = C.c_bool, [C.c_uint64, C.c_uint64, C.c_int, C.c_int]
+    assert f(n, bucket, W, bits) == warps
