@@ -103,12 +103,12 @@ quantize_pack_kernel(const __grid_constant__ QuantizeArgs a)
 
 
 
-template <int BITS, int DTYPE, int THREADS, int RED, int MODE>
+template <int BITS, int DTYPE, int THREADS, int RED, int MODE, bool RAGGED, int STAGES>
 __global__ void __launch_bounds__(THREADS, quantize_min_ctas<DTYPE, THREADS>())
 quantize_tma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ QuantizeArgs a,
                     const __grid_constant__ TmaQuantizeConsts c, unsigned int* __restrict__ timeouts)
 {
-    using Shared = TmaQuantizeShared<DTYPE, THREADS>;
+    using Shared = TmaQuantizeShared<DTYPE, THREADS, STAGES>;
     constexpr int kQuantStages = Shared::kStages;
     Shared& sh = tile_shared<Shared>();
     constexpr bool kHalves = THREADS == 512;       // more rows than the box of a copy
@@ -150,10 +150,11 @@ quantize_tma_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_const
                     load_tile_rows(stage, &tmap, next_tile * a.tile_rows, a.tile_rows, Shared::kRowBytes, kHalves, bar);
             }
         };
-        ok = tile < c.full_tiles ? mode_tile<BITS, DTYPE, THREADS, true, RED, MODE>(sh, wv, a, c, k, rot, tile, refill,
-                                                                                    local_bucket, scale_writer)
-                                 : mode_tile<BITS, DTYPE, THREADS, false, RED, MODE>(sh, wv, a, c, k, rot, tile, refill,
-                                                                                     local_bucket, scale_writer);
+        ok = tile < c.full_tiles
+            ? mode_tile<BITS, DTYPE, THREADS, true, RED, MODE, RAGGED>(sh, wv, a, c, k, rot, tile, refill, local_bucket,
+                                                                       scale_writer)
+            : mode_tile<BITS, DTYPE, THREADS, false, RED, MODE, RAGGED>(sh, wv, a, c, k, rot, tile, refill, local_bucket,
+                                                                        scale_writer);
     }
     if (!ok) {
         // A copy never landed: record it, then give the copies still in flight (the one that was
@@ -181,13 +182,13 @@ static cudaError_t launch_bits(const QuantizeArgs& a, int dtype, bool aligned, u
                    : launch_pdl(quantize_pack_kernel<BITS, 1, false>, grid, kMaxTileRows, stream, a);
 }
 
-template <int BITS, int DTYPE, int THREADS, int RED, int MODE>
+template <int BITS, int DTYPE, int THREADS, int RED, int MODE, bool RAGGED, int STAGES>
 static cudaError_t launch_tma_inst(const CUtensorMap& map, const QuantizeArgs& a,
                                    const TmaQuantizeConsts& c, unsigned int* timeouts,
                                    cudaStream_t stream)
 {
-    auto kernel = quantize_tma_kernel<BITS, DTYPE, THREADS, RED, MODE>;
-    constexpr size_t kSmem = dynamic_bytes<TmaQuantizeShared<DTYPE, THREADS>>();
+    auto kernel = quantize_tma_kernel<BITS, DTYPE, THREADS, RED, MODE, RAGGED, STAGES>;
+    constexpr size_t kSmem = dynamic_bytes<TmaQuantizeShared<DTYPE, THREADS, STAGES>>();
     static std::atomic<int> grid_cap[64];                  // per device; 0 = not yet queried (zero-initialised)
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
@@ -214,13 +215,27 @@ template <int BITS, int DTYPE, int MODE>
 static cudaError_t launch_tma_shape(const CUtensorMap& map, const QuantizeArgs& a, const TmaQuantizeConsts& c, int threads,
                                     unsigned int* timeouts, cudaStream_t stream)
 {
+    auto launch = [&](auto cta, auto reduction) {
+        constexpr int kThreads = decltype(cta)::value, kRed = decltype(reduction)::value;
+        constexpr bool kKeeps = keeps_ragged_code<DTYPE, kThreads, kRed, MODE>();
+        auto rows = [&](auto stages) {
+            constexpr int kStages = decltype(stages)::value;
+            if (a.nrows > a.nrows_full)
+                return launch_tma_inst<BITS, DTYPE, kThreads, kRed, MODE, true, kStages>(map, a, c, timeouts, stream);
+            return launch_tma_inst<BITS, DTYPE, kThreads, kRed, MODE, kKeeps, kStages>(map, a, c, timeouts, stream);
+        };
+        if constexpr (DTYPE == 0 && kThreads == 256)
+            if (one_stage((uint64_t)a.ntiles * a.tile_rows)) return rows(Int<1>());
+        return rows(Int<2>());
+    };
     const int red = reduction_of(a.rows_per_bucket);
-    if (threads == 256) return launch_tma_inst<BITS, DTYPE, 256, kByWarps, MODE>(map, a, c, timeouts, stream);
+    if (threads == 256) return launch(Int<256>(), Int<kByWarps>());
     if constexpr (DTYPE != kBf16Wide && MODE != kNorm)       // 256 rows of 64 hold every bucket; no norm of longer ones
-        if (threads == 512) return launch_tma_inst<BITS, DTYPE, 512, kByWarps, MODE>(map, a, c, timeouts, stream);
-    if (red == kByShuffle) return launch_tma_inst<BITS, DTYPE, 128, kByShuffle, MODE>(map, a, c, timeouts, stream);
-    if (red == kByRows) return launch_tma_inst<BITS, DTYPE, 128, kByRows, MODE>(map, a, c, timeouts, stream);
-    return launch_tma_inst<BITS, DTYPE, 128, kByWarps, MODE>(map, a, c, timeouts, stream);
+        if (threads == 512) return launch(Int<512>(), Int<kByWarps>());
+    if (threads != 128) return cudaErrorInvalidValue;
+    if (red == kByShuffle) return launch(Int<128>(), Int<kByShuffle>());
+    if (red == kByRows) return launch(Int<128>(), Int<kByRows>());
+    return launch(Int<128>(), Int<kByWarps>());
 }
 
 // One worker on the TMA kernel (tma_path_applies() holds).

@@ -2,6 +2,8 @@
 // draws, encode, pack), shared by the kernels of mqg_quantize.cu, mqg_quantize_workers.cu and mqg_segments_workers.cu.
 #pragma once
 
+#include <type_traits>
+
 #include "mqg_common.cuh"
 #include "mqg_internal.h"
 #include "mqg_tma.cuh"
@@ -149,15 +151,14 @@ __device__ __forceinline__ bool warp_has_row(uint64_t row, uint32_t first) { ret
 // shuffles), a whole number of warps (one shared-memory atomic per warp), or any other number of rows (one
 // shared-memory atomic per row; at least three rows, so at most 42 buckets per tile of 128).
 enum : int { kByShuffle = 0, kByWarps = 1, kByRows = 2 };
+enum : int { kMaxAbs = 0, kRange = 1, kNorm = 2 };
 constexpr int kSlots = 44;
 
-template <int DTYPE, int THREADS>
+// STAGES: depth of the shared-memory ring, two but for short launches of 256 fp32 rows to a tile (one_stage).
+template <int DTYPE, int THREADS, int STAGES = 2>
 struct TmaQuantizeShared {
     static constexpr int kRowBytes = DTYPE == 1 ? 64 : 128;
-    // depth of the shared-memory ring: two stages where they fit in 32 KB, else one (the refill
-    // of a single stage still hides behind the tile's arithmetic)
-    // (512 threads: two, and one CTA per SM)
-    static constexpr int kStages = 2 * THREADS * kRowBytes <= 32768 || THREADS == 512 || (DTYPE == kBf16Wide && THREADS == 256) ? 2 : 1;
+    static constexpr int kStages = STAGES;
     alignas(1024) uint8_t stage[kStages][THREADS * kRowBytes];
     uint32_t slots[3][kSlots];             // bucket maxima, rotating so no reset races a use
     uint32_t slots_lo[3][kSlots];          // bucket minima of the (min, max) variant, as ordered bits
@@ -180,6 +181,19 @@ __device__ __forceinline__ Shared& tile_shared()
         return *reinterpret_cast<Shared*>(tile_smem + ((1024u - (smem_u32(tile_smem) & 1023u)) & 1023u));
     }
 }
+// Gradients of whole rows run kernels without the code for a last row that is shorter (it costs 1 to 6 % of a launch, 0.1 us of
+// a short one) - but for the range of fp32 rows by shuffles or warps, which the compiler makes 3 to 16 % slower without it.
+template <int DTYPE, int THREADS, int RED, int MODE>
+constexpr bool keeps_ragged_code() { return MODE == kRange && DTYPE == 0 && THREADS == 128 && RED != kByRows; }
+template <int N>
+using Int = std::integral_constant<int, N>;
+
+// Whether tiles of up to 256 fp32 rows keep to one stage, refilled behind the tile's arithmetic, instead of two.  Two pay when the
+// gradients come from DRAM and cost when they are in L2, i.e. from 18 M elements on; bucket 8192, four bits, one / two stages
+// against the one stage of before: 4, 12 and 33 M elements 0.99 / 1.07, 0.99 / 1.05 and 1.00 / 0.87 of the time, the range 0.98 / 1.02,
+// 1.00 / 1.02 and 1.00 / 0.93, the norm 1.00 / 0.99, 0.98 / 0.98 and 0.98 / 0.88.
+inline bool one_stage(uint64_t rows) { return rows < (18u << 20) / 32; }
+
 template <int DTYPE, int THREADS>
 constexpr int quantize_min_ctas() { return DTYPE == kBf16Wide ? (THREADS == 128 ? 5 : 2) : THREADS == 512 ? 1 : 512 / THREADS; }
 
@@ -218,19 +232,19 @@ struct WorkerView {
 // One tile, the k-th of this CTA, tile `tile` of worker `wv`.  FULL: every thread owns a complete
 // row (no bounds checks).  RED: how a bucket's rows are reduced.  After the tile's rows are in registers thread 0 calls
 // `refill(stage, bar)` to start the copy that uses the stage next.  Returns false if the tile's copy never landed.
-template <int BITS, int DTYPE, int THREADS, bool FULL, int RED, bool NORM = false,
-          typename Refill>
-__device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>& sh, const WorkerView wv,
+template <int BITS, int DTYPE, int THREADS, bool FULL, int RED, bool RAGGED, bool NORM = false,
+          typename Shared, typename Refill>
+__device__ __forceinline__ bool quantize_tile(Shared& sh, const WorkerView wv,
                                               const QuantizeArgs& a, const TmaQuantizeConsts& c,
                                               uint32_t k, uint32_t rot, uint32_t tile, Refill&& refill,
                                               uint32_t local_bucket, bool scale_writer)
 {
-    constexpr int kQuantStages = TmaQuantizeShared<DTYPE, THREADS>::kStages;
+    constexpr int kQuantStages = Shared::kStages;
     constexpr bool SHUFFLE = RED == kByShuffle;
     const uint32_t t = threadIdx.x;
     const uint32_t row = tile * a.tile_rows + t;
     const bool active = FULL || (t < a.tile_rows && row < (uint32_t)a.nrows);
-    const bool tail = !FULL && tile == c.ragged_tile;            // a tile with a row that the copy does not cover
+    const bool tail = RAGGED && !FULL && tile == c.ragged_tile;  // a tile with a row that the copy does not cover
     const uint32_t stg = k % kQuantStages, parity = (k / kQuantStages) & 1;
     const uint32_t bar = smem_u32(&sh.bar[stg]);
     uint8_t* stage = sh.stage[stg];
@@ -374,18 +388,18 @@ __device__ __forceinline__ bool quantize_tile(TmaQuantizeShared<DTYPE, THREADS>&
 // take part in the range: the elements a ragged row lacks repeat its first element, and threads
 // without a row contribute the identities.  sh.slots holds maxima, sh.slots_lo minima, both as
 // ordered bits; the kernel initialises them to the identities.
-template <int BITS, int DTYPE, int THREADS, bool FULL, int RED, typename Refill>
-__device__ __forceinline__ bool range_quantize_tile(TmaQuantizeShared<DTYPE, THREADS>& sh, const WorkerView wv,
+template <int BITS, int DTYPE, int THREADS, bool FULL, int RED, bool RAGGED, typename Shared, typename Refill>
+__device__ __forceinline__ bool range_quantize_tile(Shared& sh, const WorkerView wv,
                                                     const QuantizeArgs& a, const TmaQuantizeConsts& c, uint32_t k,
                                                     uint32_t rot, uint32_t tile, Refill&& refill, uint32_t local_bucket,
                                                     bool scale_writer)
 {
-    constexpr int kQuantStages = TmaQuantizeShared<DTYPE, THREADS>::kStages;
+    constexpr int kQuantStages = Shared::kStages;
     constexpr bool SHUFFLE = RED == kByShuffle;
     const uint32_t t = threadIdx.x;
     const uint32_t row = tile * a.tile_rows + t;
     const bool active = FULL || (t < a.tile_rows && row < (uint32_t)a.nrows);
-    const bool tail = !FULL && tile == c.ragged_tile;            // a tile with a row that the copy does not cover
+    const bool tail = RAGGED && !FULL && tile == c.ragged_tile;  // a tile with a row that the copy does not cover
     const uint32_t stg = k % kQuantStages, parity = (k / kQuantStages) & 1;
     const uint32_t bar = smem_u32(&sh.bar[stg]);
     uint8_t* stage = sh.stage[stg];
@@ -459,7 +473,6 @@ __device__ __forceinline__ bool range_quantize_tile(TmaQuantizeShared<DTYPE, THR
 
 // MODE: kMaxAbs = the main codec, kRange = the (min, max) variant, kNorm = the L2-norm scale variant.  (Rows of 64 bf16
 // elements below exist for the main codec only: the variants' long bf16 launches were not tried with them.)
-enum : int { kMaxAbs = 0, kRange = 1, kNorm = 2 };
 
 // ---------------------------------------------------------------------------------------
 // bf16 gradients long enough to fill the device: a thread owns 64 consecutive elements, 128 bytes of the stage as in
@@ -468,13 +481,13 @@ enum : int { kMaxAbs = 0, kRange = 1, kNorm = 2 };
 // here instead of once per 32.  (122 to 128 registers left to itself: four CTAs per SM, 28.3 us per 50 M elements at
 // K = 4; held to 102, five CTAs, 27.8 us; to 85, six CTAs, 29.5 us; rows of 32 29.8 us.)
 // ---------------------------------------------------------------------------------------
-template <int BITS, int THREADS, bool FULL, int RED, typename Refill>
-__device__ __forceinline__ bool quantize_wide_tile(TmaQuantizeShared<kBf16Wide, THREADS>& sh, const WorkerView wv,
+template <int BITS, int THREADS, bool FULL, int RED, bool RAGGED, typename Shared, typename Refill>
+__device__ __forceinline__ bool quantize_wide_tile(Shared& sh, const WorkerView wv,
                                                    const QuantizeArgs& a, const TmaQuantizeConsts& c, uint32_t k,
                                                    uint32_t rot, uint32_t tile, Refill&& refill, uint32_t local_bucket,
                                                    bool scale_writer)
 {
-    constexpr int kQuantStages = TmaQuantizeShared<kBf16Wide, THREADS>::kStages;
+    constexpr int kQuantStages = Shared::kStages;
     const uint32_t t = threadIdx.x;
     const uint32_t row = tile * a.tile_rows + t;
     const bool active = FULL || (t < a.tile_rows && row < (uint32_t)a.nrows);
@@ -487,7 +500,7 @@ __device__ __forceinline__ bool quantize_wide_tile(TmaQuantizeShared<kBf16Wide, 
 
     uint32_t raw[2][16];
     if (active) {
-        if (!FULL && row >= (uint32_t)a.nrows_full)      // a row that the copy does not cover
+        if (RAGGED && !FULL && row >= (uint32_t)a.nrows_full)      // a row that the copy does not cover
             stage_ragged_row(stage, t, static_cast<const uint8_t*>(wv.grad), row, a.n * 2);
         const uint4* s = reinterpret_cast<const uint4*>(stage);
 #pragma unroll
@@ -548,24 +561,24 @@ __device__ __forceinline__ bool quantize_wide_tile(TmaQuantizeShared<kBf16Wide, 
 }
 
 // One tile in the given mode.
-template <int BITS, int DTYPE, int THREADS, bool FULL, int RED, int MODE, typename Refill>
-__device__ __forceinline__ bool mode_tile(TmaQuantizeShared<DTYPE, THREADS>& sh, const WorkerView& wv, const QuantizeArgs& a,
+template <int BITS, int DTYPE, int THREADS, bool FULL, int RED, int MODE, bool RAGGED, typename Shared, typename Refill>
+__device__ __forceinline__ bool mode_tile(Shared& sh, const WorkerView& wv, const QuantizeArgs& a,
                                           const TmaQuantizeConsts& c, uint32_t k, uint32_t rot, uint32_t tile,
                                           Refill&& refill, uint32_t local_bucket, bool scale_writer)
 {
     if constexpr (DTYPE == kBf16Wide)
-        return quantize_wide_tile<BITS, THREADS, FULL, RED>(sh, wv, a, c, k, rot, tile, refill, local_bucket, scale_writer);
+        return quantize_wide_tile<BITS, THREADS, FULL, RED, RAGGED>(sh, wv, a, c, k, rot, tile, refill, local_bucket, scale_writer);
     else if constexpr (MODE == kRange)
-        return range_quantize_tile<BITS, DTYPE, THREADS, FULL, RED>(sh, wv, a, c, k, rot, tile, refill, local_bucket,
+        return range_quantize_tile<BITS, DTYPE, THREADS, FULL, RED, RAGGED>(sh, wv, a, c, k, rot, tile, refill, local_bucket,
                                                                     scale_writer);
     else
-        return quantize_tile<BITS, DTYPE, THREADS, FULL, RED, MODE == kNorm>(sh, wv, a, c, k, rot, tile, refill,
+        return quantize_tile<BITS, DTYPE, THREADS, FULL, RED, RAGGED, MODE == kNorm>(sh, wv, a, c, k, rot, tile, refill,
                                                                              local_bucket, scale_writer);
 }
 
 // First contents of a CTA's slots: the identities of the reductions.
-template <int DTYPE, int THREADS>
-__device__ __forceinline__ void init_slots(TmaQuantizeShared<DTYPE, THREADS>& sh)
+template <int DTYPE, int THREADS, typename Shared>
+__device__ __forceinline__ void init_slots(Shared& sh)
 {
     for (uint32_t i = threadIdx.x; i < 3u * kSlots; i += THREADS) {
         (&sh.slots[0][0])[i] = 0u;         // = kOrderedMaxIdentity

@@ -23,13 +23,13 @@ struct WorkerTable {
     PhiloxHead head[kMaxWorkers];
 };
 
-template <int BITS, int DTYPE, int THREADS, int RED, int MODE>
+template <int BITS, int DTYPE, int THREADS, int RED, int MODE, bool RAGGED, int STAGES>
 __global__ void __launch_bounds__(THREADS, quantize_min_ctas<DTYPE, THREADS>())
 quantize_workers_kernel(const __grid_constant__ WorkerTable tab, const __grid_constant__ QuantizeArgs a,
                         const __grid_constant__ TmaQuantizeConsts c, uint32_t total_tiles,
                         unsigned int* __restrict__ timeouts)
 {
-    using Shared = TmaQuantizeShared<DTYPE, THREADS>;
+    using Shared = TmaQuantizeShared<DTYPE, THREADS, STAGES>;
     constexpr int kQuantStages = Shared::kStages;
     Shared& sh = tile_shared<Shared>();
     constexpr bool kHalves = THREADS == 512;       // more rows than the box of a copy
@@ -85,10 +85,11 @@ quantize_workers_kernel(const __grid_constant__ WorkerTable tab, const __grid_co
             auto refill = [&](uint32_t stage, uint32_t bar) {
                 if (vfill < total_tiles) load_tile(fill, stage, bar);
             };
-            ok = tile < c.full_tiles ? mode_tile<BITS, DTYPE, THREADS, true, RED, MODE>(sh, wv, a, c, k, rot, tile, refill,
-                                                                                        local_bucket, scale_writer)
-                                     : mode_tile<BITS, DTYPE, THREADS, false, RED, MODE>(sh, wv, a, c, k, rot, tile,
-                                                                                         refill, local_bucket, scale_writer);
+            ok = tile < c.full_tiles
+                ? mode_tile<BITS, DTYPE, THREADS, true, RED, MODE, RAGGED>(sh, wv, a, c, k, rot, tile, refill, local_bucket,
+                                                                           scale_writer)
+                : mode_tile<BITS, DTYPE, THREADS, false, RED, MODE, RAGGED>(sh, wv, a, c, k, rot, tile, refill, local_bucket,
+                                                                            scale_writer);
             vfill += stride;
             if (vfill < total_tiles) advance(fill, stride);
         }
@@ -105,13 +106,13 @@ quantize_workers_kernel(const __grid_constant__ WorkerTable tab, const __grid_co
     }
 }
 
-template <int BITS, int DTYPE, int THREADS, int RED, int MODE>
+template <int BITS, int DTYPE, int THREADS, int RED, int MODE, bool RAGGED, int STAGES>
 static cudaError_t launch_workers_inst(const WorkerTable& tab, const QuantizeArgs& a,
                                        const TmaQuantizeConsts& c, uint32_t total_tiles,
                                        unsigned int* timeouts, cudaStream_t stream)
 {
-    auto kernel = quantize_workers_kernel<BITS, DTYPE, THREADS, RED, MODE>;
-    constexpr size_t kSmem = dynamic_bytes<TmaQuantizeShared<DTYPE, THREADS>>();
+    auto kernel = quantize_workers_kernel<BITS, DTYPE, THREADS, RED, MODE, RAGGED, STAGES>;
+    constexpr size_t kSmem = dynamic_bytes<TmaQuantizeShared<DTYPE, THREADS, STAGES>>();
     static std::atomic<int> grid_cap[64];                  // per device; 0 = not yet queried (zero-initialised)
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
@@ -138,15 +139,27 @@ template <int BITS, int DTYPE, int MODE>
 static cudaError_t launch_workers_shape(const WorkerTable& tab, const QuantizeArgs& a, const TmaQuantizeConsts& c,
                                         uint32_t total_tiles, int threads, unsigned int* timeouts, cudaStream_t stream)
 {
+    auto launch = [&](auto cta, auto reduction) {
+        constexpr int kThreads = decltype(cta)::value, kRed = decltype(reduction)::value;
+        constexpr bool kKeeps = keeps_ragged_code<DTYPE, kThreads, kRed, MODE>();
+        auto rows = [&](auto stages) {
+            constexpr int kStages = decltype(stages)::value;
+            if (a.nrows > a.nrows_full)
+                return launch_workers_inst<BITS, DTYPE, kThreads, kRed, MODE, true, kStages>(tab, a, c, total_tiles, timeouts, stream);
+            return launch_workers_inst<BITS, DTYPE, kThreads, kRed, MODE, kKeeps, kStages>(tab, a, c, total_tiles, timeouts, stream);
+        };
+        if constexpr (DTYPE == 0 && kThreads == 256)
+            if (one_stage((uint64_t)total_tiles * a.tile_rows)) return rows(Int<1>());
+        return rows(Int<2>());
+    };
     const int red = reduction_of(a.rows_per_bucket);
-    if (threads == 256)
-        return launch_workers_inst<BITS, DTYPE, 256, kByWarps, MODE>(tab, a, c, total_tiles, timeouts, stream);
+    if (threads == 256) return launch(Int<256>(), Int<kByWarps>());
     if constexpr (DTYPE != kBf16Wide && MODE != kNorm)       // 256 rows of 64 hold every bucket; no norm of longer ones
-        if (threads == 512)
-            return launch_workers_inst<BITS, DTYPE, 512, kByWarps, MODE>(tab, a, c, total_tiles, timeouts, stream);
-    if (red == kByShuffle) return launch_workers_inst<BITS, DTYPE, 128, kByShuffle, MODE>(tab, a, c, total_tiles, timeouts, stream);
-    if (red == kByRows) return launch_workers_inst<BITS, DTYPE, 128, kByRows, MODE>(tab, a, c, total_tiles, timeouts, stream);
-    return launch_workers_inst<BITS, DTYPE, 128, kByWarps, MODE>(tab, a, c, total_tiles, timeouts, stream);
+        if (threads == 512) return launch(Int<512>(), Int<kByWarps>());
+    if (threads != 128) return cudaErrorInvalidValue;
+    if (red == kByShuffle) return launch(Int<128>(), Int<kByShuffle>());
+    if (red == kByRows) return launch(Int<128>(), Int<kByRows>());
+    return launch(Int<128>(), Int<kByWarps>());
 }
 
 template <int BITS>

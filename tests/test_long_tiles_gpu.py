@@ -1,5 +1,6 @@
 """Buckets of 8193 to 16384 elements in the bulk-copy kernels (tiles of more rows than one copy's box holds), fp32, bf16 in
-rows of 32 and of 64, one worker and several, whole and ragged ends: bit for bit against the CPU checker."""
+rows of 32 and of 64, one worker and several, whole and ragged ends, and buckets of 8192 in launches long enough for two stages:
+bit for bit against the CPU checker."""
 import numpy as np
 import pytest
 import torch
@@ -19,6 +20,8 @@ pytestmark = pytest.mark.gpu
     (9216 * 6 + 33, 9216, 3, 1),                     # 288 rows (of 64: 144, no whole warps)
     (16384, 16384, 2, 5),                            # one bucket
     (16384 * 700 + 17, 16384, 2, 4),                 # more tiles than CTAs; bf16: rows of 64
+    (8192 * 2305, 8192, 1, 4),                       # from 18 M elements on
+    (8192 * 1160 + 17, 8192, 2, 5),
 ])
 @pytest.mark.parametrize("bf16", [False, True])
 def test_long_tiles(n, bucket, W, bits, bf16):
@@ -51,3 +54,16 @@ def test_long_tiles(n, bucket, W, bits, bf16):
         assert bits_equal(ranges[w].numpy(np.float32), r_ref.reshape(-1)) == 0
         assert np.array_equal(codes[w].numpy(np.uint32), c_ref)
     assert mqg.mqg_device_timeouts() == 0
+
+
+@pytest.mark.parametrize("n", [8192 * 2305, 8192 * 2305 + 5])
+def test_norm_in_two_stages(n):
+    bits, bucket = 6, 8192
+    x = wl.laplace(n, 1e-4, config=13, worker=1)
+    codes, scales = Guarded(mqg.mqg_code_words(n, bits), torch.int32), Guarded(mqg.mqg_num_buckets(n, bucket), torch.float32)
+    mqg.mqg_quantize_l2(to_dev(x), n, bits, bucket, 9, codes.view, scales.view, worker=1)
+    torch.cuda.synchronize()
+    codes.check_guards(), scales.check_guards()
+    c_ref, s_ref = O.quantize_l2(x, bits, bucket, 9, worker=1)
+    assert bits_equal(scales.numpy(np.float32), s_ref) == 0
+    assert np.array_equal(codes.numpy(np.uint32), c_ref)
