@@ -113,11 +113,9 @@ mqg_status quantize_segments(const void* const* grads, int W, int nseg, const ui
 // calls fn(table, first_segment_index) for each chunk.  Segments for which skip(j) holds get no
 // tiles in the tables, exactly like empty segments: another launch takes care of them.  skip is
 // only called once the table has been checked.
-struct SkipNone { bool operator()(int) const { return false; } };
-
-template <typename Fn, typename Skip = SkipNone>
+template <typename Fn, typename Skip>
 mqg_status for_each_chunk(int nseg, const uint64_t* seg_off, const uint64_t* code_off, int bits,
-                          Fn&& fn, Skip&& skip = Skip())
+                          Fn&& fn, Skip&& skip)
 {
     if (mqg_status st = check_segments(nseg, seg_off, code_off, bits)) return st;
     const uint64_t tile_elems = (uint64_t)mqg::kMaxTileRows * 32;

@@ -841,8 +841,9 @@ __device__ __forceinline__ void add_decoded_row(const uint32_t (&w)[BITS], const
 // For |h| (step, lo) in [2^-86, 2^18] or 0 that changes no rounding: all x^ and all sums are multiples of 2^-109, in units
 // of 2^40 multiples of 2^-149, so a result that is subnormal there is exact there, and exact in 24 bits here; the largest
 // is below 2^32.  A tile with any other scale is summed by add_decoded_row.
-// What it gives (against the three instructions): 16 workers of 250 M elements at four bits, encode and update 2987 against
-// 3035 us, eight of 25 M re-quantized and applied 75.2 against 77.4 us, the update at two bits 43.6 against 44.5 us.
+// What it gives (against the three instructions): eight workers of 25 M elements at four bits re-quantized and applied 75.2
+// against 77.4 us.  Where the launch moves more bytes than that it is about the runs' own spread: the update of 25 M at two
+// bits 43.9 against 44.8 us, 16 workers of 250 M at four bits, encode and update, 3031 against 3053 us.
 constexpr float kSumUnit = 1099511627776.0f, kPerSumUnit = 1.0f / kSumUnit;     // 2^40
 __host__ __device__ inline bool fits_sum_unit(float factor) { return factor > -0x1p80f && factor < 0x1p80f; }
 

@@ -49,7 +49,7 @@ cudaError_t launch_quantize_workers(const void* const* grads, int W, uint64_t n,
                                     uint32_t step, uint64_t elem_offset, int mode, cudaStream_t stream);
 
 // (min, max) nearest-rounding variant.  ranges[2b] = lo, ranges[2b + 1] = hi of bucket b.
-// One-pass kernel for buckets of at most kMaxFusedBucket elements (mqg_quantize.cu), a CTA per bucket for those it does not
+// One-pass kernel for buckets of at most kMaxTmaBucket elements (mqg_quantize.cu), a CTA per bucket for those it does not
 // take and up to 49152 elements (launch_bucket_spans), the general launches for longer ones (ranges by atomics on ordered
 // bits, then encode).
 bool quantize_range_fused_applies(uint64_t n, uint64_t bucket);
@@ -104,8 +104,8 @@ cudaError_t launch_bucket_spans(const void* const* grads, int W, uint64_t n, int
                                 uint32_t* const* codes, float* const* scales, int mode, int dtype, uint32_t first_worker,
                                 uint32_t step, uint64_t elem_offset, cudaStream_t stream);
 
-// Two-pass quantize with uniform large buckets (bucket > kMaxFusedBucket, or a single bucket
-// whose length is not a multiple of 32).
+// Two-pass quantize with uniform large buckets (those that quantize_long_fused_applies and
+// bucket_spans_apply do not take: bucket > kMaxFusedBucket, or a single bucket whose length is not a multiple of 32).
 cudaError_t launch_quantize_big_buckets(const void* grad, uint64_t n, int bits, uint64_t bucket,
                                         uint64_t seed, uint32_t* codes, float* scales, int dtype,
                                         uint32_t worker, uint32_t step, uint64_t elem_offset,
@@ -152,7 +152,8 @@ cudaError_t launch_requantize(const WorkerPtrs& ptrs, int W, int bits, uint64_t 
                               float mean_scale, uint64_t seed, uint32_t* codes_out, float* scales_out,
                               uint32_t worker, uint32_t step, cudaStream_t stream);
 
-// The same on the warp-pipelined kernel of mqg_server_tma.cu (whole rows, buckets of 2^k rows up to 128).
+// The same on the warp-pipelined kernel of mqg_server_tma.cu (buckets of 2^k rows up to 256, or of
+// 24, 48 or 96; a last row may be short).
 bool requantize_warp_applies(uint64_t n, uint64_t bucket, int W, int bits);
 cudaError_t launch_requantize_warp(const WorkerPtrs& ptrs, int W, int bits, uint64_t n, uint64_t bucket,
                                    float mean_scale, uint64_t seed, uint32_t* codes_out, float* scales_out,

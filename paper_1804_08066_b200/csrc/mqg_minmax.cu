@@ -1,6 +1,6 @@
 // General kernels of the (min, max) nearest-rounding codec variant (the scheme the footnote of Section 3.2 refers to, a
 // bucket's range [min, max] mapped linearly onto the 2^K codes) for buckets of more than 49152 elements: the range tile of
-// mqg_quantize_tile.cuh takes buckets of up to 8192, a CTA to a bucket (mqg_segments.cu) the rest.  A thread owns a row of 32
+// mqg_quantize_tile.cuh takes buckets of up to 16384, a CTA to a bucket (mqg_segments.cu) the rest.  A thread owns a row of 32
 // elements throughout; buckets are whole rows (multiples of 32 elements, or one bucket).  Ordinary launches, four to a call.
 #include "mqg_common.cuh"
 #include "mqg_internal.h"

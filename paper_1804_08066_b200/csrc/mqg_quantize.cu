@@ -308,7 +308,7 @@ uint64_t fill_args(QuantizeArgs& a, const void* grad, uint64_t n, int bits, uint
     a.nbuckets = (n + bucket - 1) / bucket;
     a.ncode_words = (n * (uint64_t)bits + 31) / 32;
     a.elem_offset = elem_offset;
-    // bucket % 32 == 0 and bucket <= 8192, or a single bucket of at most 8192 elements
+    // bucket % 32 == 0 and bucket <= kMaxTmaBucket (the norm kMaxFusedBucket), or a single bucket of at most that many elements
     const uint64_t rpb = (bucket >= n) ? a.nrows : bucket / row_elems;
     a.rows_per_bucket = (uint32_t)rpb;
     a.buckets_per_tile = (uint32_t)(kMaxTileRows / rpb);

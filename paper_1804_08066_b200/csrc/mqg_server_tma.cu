@@ -11,7 +11,7 @@
 //     cost about a dozen instructions of the warp per copy - the operands of a bulk copy travel
 //     through the uniform datapath - and with eight of them per tile a third of the kernel's
 //     instructions were overhead: 40.1 executed instructions per parameter at four bits and eight
-//     workers against 31.4 now.)
+//     workers against 31.4 without it, before sums in units of 2^40.)
 // A warp therefore never waits for DRAM latency in steady state and there is no CTA-wide barrier
 // anywhere.  Per-(worker, bucket) de-quantization constants are computed once per tile into the
 // warp's small shared table, one tile ahead.
@@ -320,16 +320,13 @@ __device__ __forceinline__ void fill_code_stage_flat(const ServerTmaArgs& a, uin
 template <int BITS>
 constexpr int server_min_ctas() { return 4; }
 
-// MODE 1: dst = params, dst <- fma(-lr, sum, dst).  MODE 0: dst = acc, dst <- sum.
-// MODE 2: dst = acc, the sum continues from the value already there.
-// RANGE: the (min, max) nearest-rounding variant (x^ = fma(q, step, lo)).
 // The one row of a gradient that has fewer than 32 elements (row `row`, the last one): a warp, lane j on
 // element j, with plain loads and stores.  What bounds it is one round trip to memory and the chain of the sum: the code
 // words of eight workers are requested at a time, and lane w divides for worker w (at most 32).  131,073 parameters, 1 / 8 / 16
 // workers: 2.4 / 3.2 / 4.2 us, against 3.1 / 4.7 / 7.0 us with a division per worker and element, after the warp's tile.
 // `params` is the row's first parameter, `count` its length; its codes start at bit `bit0` of word `word0` of every worker's
 // buffer, and their stream ends before word `words_end`; `bucket` is the index of the row's scale.
-// SEGS: every lane divides for every worker.  (With the shuffles in a function that a grid over segments calls, its main loop
+// MODE and RANGE as in server_tma_body.  SEGS: every lane divides for every worker.  (With the shuffles in a function that a grid over segments calls, its main loop
 // is compiled to something 2.5 % slower at four bits and eight workers.)
 template <int BITS, int MODE, bool RANGE, bool SEGS>
 __device__ __noinline__ void server_ragged_row(const ServerTmaArgs& a, float* params, uint32_t count, uint64_t word0,
@@ -383,6 +380,9 @@ __device__ __noinline__ void server_ragged_row(const ServerTmaArgs& a, float* pa
     if (in) params[lane] = MODE == 1 ? __fmaf_rn(a.neg_lr, v.x, old) : v.x;
 }
 
+// MODE 1: dst = params, dst <- fma(-lr, sum, dst).  MODE 0: dst = acc, dst <- sum.
+// MODE 2: dst = acc, the sum continues from the value already there.
+// RANGE: the (min, max) nearest-rounding variant (x^ = fma(q, step, lo)).
 template <int BITS, int MODE, bool RANGE, bool SEGS, bool kUnit, bool FLAT = false>
 __device__ __forceinline__ void server_tma_body(const CUtensorMap* map_full, const ServerTmaArgs& a,
                                                 const ServerSegTable* segs, unsigned int* __restrict__ timeouts)
@@ -765,7 +765,8 @@ server_tma_segments_kernel(const __grid_constant__ ServerSegTable segs, const __
 
 // Whether a launch sums in units of 2^40, and its arguments for that; `factor`: what the sum is multiplied with.  From a
 // whole code stage of workers on: with fewer, what it saves is less than what the second form of the decode costs a launch
-// (three workers, four bits: 7.9 against 7.5 us for 5 M parameters, 2.85 against 2.7 us for 131,072).
+// (three workers, four bits: 7.9 against 7.5 us for 5 M parameters, 2.85 against 2.7 us for 131,072; four to seven workers at
+// two to four bits stay with those: not measured).
 template <int BITS>
 static bool sum_in_units(ServerTmaArgs& a, float factor)
 {
